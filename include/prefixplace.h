@@ -71,7 +71,8 @@ typedef struct {
                                       worker, which is the same DP, so it is not run again) */
     int64_t dp_cells;              /* out: sum over executed DPs of n * k_h (Eq. 9 cells) */
     int32_t kernel_launches;       /* out: kernels launched by this call */
-    int64_t dp_rows_swept;         /* out: rows the DPs actually swept (pruned sweep), summed */
+    int64_t dp_rows_swept;         /* out: rows the DPs actually swept (after reduction and
+                                      pruning), summed */
     int32_t time_phases;           /* in: nonzero = time the phases below with CUDA events */
     float phase_ms[3];             /* out (if time_phases): device time of the marginal,
                                       tree-DP (with its row pruning) and traceback launches,
@@ -206,7 +207,8 @@ pp_status pp_marginals(pp_instance *inst, int32_t batch, const int32_t *worker,
  * pp_traceback reads for `batch` items whose budgets are at most
  * `max_budget`: the decision bits plus the rows of the pruned sweep (rows
  * strictly below a chunk whose strict descendants all have profit <= 0 never
- * change a kept row's value or decision, so the DP skips them).  Returns 0 for
+ * change a kept row's value or decision, so the DP skips them) and of the
+ * exact reduction (chunks that are the same in every optimal set need no DP).  Returns 0 for
  * batch <= 0 or an invalid max_budget.
  */
 size_t pp_dp_bits_size(const pp_instance *inst, int32_t batch, int32_t max_budget);
@@ -268,7 +270,7 @@ pp_status pp_tree_dp_noalloc(pp_instance *inst, int32_t batch, const int64_t *pr
 /*
  * pp_dp_rows_swept -- for the last pp_tree_dp / pp_tree_dp_noalloc on
  * `workspace` (same batch and max_budget), the number of rows each item's DP
- * actually swept after pruning (host [batch] out).  Synchronises `stream`.
+ * actually swept after the exact reduction and the pruning (host [batch] out).  Synchronises `stream`.
  * Errors: PP_EINVAL, PP_ECUDA.
  */
 pp_status pp_dp_rows_swept(const pp_instance *inst, int32_t batch, int32_t max_budget,

@@ -33,6 +33,7 @@
 // per (warp, c) gives the word ((item * P + g) * n + i) * C + c whose bit
 // `lane` is column (g * 32 + lane) * C + c + 1.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <mutex>
 
@@ -197,7 +198,8 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
                const int32_t *__restrict__ item_budget, int32_t max_budget,
                const int32_t *__restrict__ item_active, int64_t *__restrict__ best,
                uint32_t *__restrict__ bits, int64_t *__restrict__ gstack, int L_smem, int L_glob,
-               int32_t *__restrict__ status, int32_t batch, int32_t slot_base, int32_t ranked)
+               int32_t *__restrict__ status, int32_t batch, int32_t slot_base, int32_t ranked,
+               const int32_t *__restrict__ red, const int32_t *__restrict__ left, const int64_t *__restrict__ base)
 {
     using namespace wavecfg;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -212,7 +214,7 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
         __shared__ int s_item;
         if (threadIdx.x < 32) {
             const int x = threadIdx.x;
-            const int key = x < batch && (!item_active || item_active[x]) ? nkept[x] : -1;
+            const int key = x < batch && (!item_active || item_active[x]) && !(red && red[x] == 1) ? nkept[x] : -1;
             int rank = 0;
             for (int y = 0; y < batch; ++y) {
                 const int ky = __shfl_sync(kFull, key, y);
@@ -228,12 +230,13 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
     const int NT = blockDim.x;
     const int WPC = NT >> 5;
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int P = CL * WPC;
     const int g = cr * WPC + wl;
-    const int kpad = P * 32 * C;
+    const int kpad = CL * WPC * 32 * C;
 
     // uniform over the whole cluster: return before any DSMEM traffic
     if (item_active && !item_active[item]) return;
+    const int state = red ? red[item] : 0;     // of the reduction
+    if (state == 1) return;                    // solved by it
     const int32_t kreq = item_budget[item];
     if (kreq < 0 || kreq > max_budget) {
         if (cr == 0 && threadIdx.x == 0) {
@@ -242,7 +245,12 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
         }
         return;
     }
-    const int k = kreq < kpad ? kreq : kpad;   // kpad covers min(max_budget, total weight)
+    const int kall = state == 2 ? left[item] : kreq;
+    const int k = kall < kpad ? kall : kpad;   // kpad covers min(max_budget, total weight)
+    // only the warps that hold columns up to k work (what the reduction leaves
+    // of a budget is a fraction of it); P is their number, PB the bit layout's
+    const int PB = CL * WPC;
+    const int P = k > 32 * C ? (k + 32 * C - 1) / (32 * C) : 1;
 
     uint64_t *ring = reinterpret_cast<uint64_t *>(smem);                           // [WPC][kRing][WMAX]
     int64_t *pstage = reinterpret_cast<int64_t *>(ring + (size_t)WPC * kRing * WMAX);  // [WPC][2][32] profits
@@ -253,6 +261,10 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
     if (threadIdx.x < WPC) ack[threadIdx.x] = 0;
     cluster_sync_all();     // every CTA initialised before any remote write
 
+    if (g >= P) {               // no columns: only the last cluster barrier is waited for
+        cluster_sync_all();
+        return;
+    }
     const bool has_prev = g > 0, has_next = g < P - 1;
     const bool prev_remote = has_prev && wl == 0;
     // the previous warp's acknowledgement word, as a generic cluster address
@@ -275,7 +287,7 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
 
     // decision bits in block pairs: the words of 32-row blocks 2b and 2b+1
     // of one column sit side by side (one 8-byte word per 64 rows)
-    uint32_t *Bw = bits + ((size_t)item * P + g) * (size_t)nblk * C * 32 + 2 * lane;
+    uint32_t *Bw = bits + ((size_t)item * PB + g) * (size_t)nblk * C * 32 + 2 * lane;
     int64_t *gst = gstack + (((size_t)item * L_glob) * CL + cr) * (size_t)C * NT;
     int64_t *const my_gst = gst + threadIdx.x;
     // this warp's shared-memory stack levels: a column's word of a level sits
@@ -506,7 +518,7 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
     asm volatile("cp.async.wait_all;" ::: "memory");   // nothing in flight into this CTA's shared memory
     if (!aborted) {
         if (k == 0) {
-            if (g == 0 && lane == 0) best[item] = 0;
+            if (g == 0 && lane == 0) best[item] = state == 2 ? base[item] : 0;
         } else {
             const int q = k - 1;
             const int tt = q / C;
@@ -514,14 +526,17 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
             int64_t v = cur[0];
 #pragma unroll
             for (int c = 1; c < C; ++c) v = cc == c ? cur[c] : v;
-            if (g == (tt >> 5) && lane == (tt & 31)) best[item] = v;
+            if (g == (tt >> 5) && lane == (tt & 31)) best[item] = state == 2 ? base[item] + v : v;
         }
     }
     cluster_sync_all();     // no CTA leaves while a neighbour may still write its shared memory
 }
 
 // ===========================================================================
-// General kernel (any chunk weight): one CTA, one barrier per row.
+// General kernel (any chunk weight): one CTA, one barrier per row.  It sweeps
+// the same kept rows by the same stack plan as the wavefront kernel, the top
+// of the skip-row stack in registers.  Only the warps that hold columns up to
+// the item's budget take part (a narrower barrier).
 // ===========================================================================
 constexpr int kMetaRows = 256;
 
@@ -532,23 +547,21 @@ static size_t flat_smem_fixed(int kpad)
 
 template <int C>
 __global__ void __launch_bounds__(1024, 1)
-k_tree_dp_flat(int32_t n, const int32_t *__restrict__ rowlist, const int32_t *__restrict__ nkept,
-               const int64_t *__restrict__ profit, const int32_t *__restrict__ order,
-               const int32_t *__restrict__ wpre, const int32_t *__restrict__ meta,
+k_tree_dp_flat(int32_t n, DpWork work, const int32_t *__restrict__ wpre,
                const int32_t *__restrict__ item_budget, int32_t max_budget,
                const int32_t *__restrict__ item_active, int64_t *__restrict__ best,
-               uint32_t *__restrict__ bits, int64_t *__restrict__ gstack, int L_smem, int L_glob,
-               int32_t *__restrict__ status)
+               int64_t *__restrict__ gstack, int L_smem, int L_glob, int32_t *__restrict__ status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int T = blockDim.x;
+    const int TB = blockDim.x;                                  // threads of the bit layout
     const int t = threadIdx.x;
     const int lane = t & 31, warp = t >> 5;
-    const int P = T >> 5;
     const int item = blockIdx.x;
-    const int kpad = T * C;
+    const int kpad = TB * C;
 
     if (item_active && !item_active[item]) return;
+    const int state = work.red ? work.red[item] : 0;            // of the reduction
+    if (state == 1) return;                                     // solved by it
     const int32_t kreq = item_budget[item];
     if (kreq < 0 || kreq > max_budget) {
         if (t == 0) {
@@ -557,64 +570,67 @@ k_tree_dp_flat(int32_t n, const int32_t *__restrict__ rowlist, const int32_t *__
         }
         return;
     }
-    const int k = kreq < kpad ? kreq : kpad;
+    const int kall = state == 2 ? work.left[item] : kreq;
+    const int k = kall < kpad ? kall : kpad;
+    const int T = k > 32 * C ? (k + 32 * C - 1) / (32 * C) * 32 : 32;    // threads at work
+    if (t >= T) return;
 
-    int64_t *srow = reinterpret_cast<int64_t *>(smem);          // [2][C][T]
-    int64_t *sstk = srow + 2 * (size_t)kpad;                    // [L_smem][C][T]
+    int64_t *srow = reinterpret_cast<int64_t *>(smem);          // [2][C][TB]
+    int64_t *sstk = srow + 2 * (size_t)kpad;                    // [L_smem][C][TB]
     int64_t *sp = sstk + (size_t)L_smem * kpad;                 // [2][kMetaRows]
     int32_t *sw = reinterpret_cast<int32_t *>(sp + 2 * kMetaRows);
     int32_t *sm = sw + 2 * kMetaRows;
     int64_t *gst = gstack + (size_t)item * L_glob * kpad;
-    const int64_t *Pp = profit + (size_t)item * n;
     const int nblk = (n + 63) / 64 * 2;                      // 32-row blocks, in pairs
-    uint32_t *Bw = bits + ((size_t)item * P + warp) * (size_t)nblk * C * 32 + 2 * lane;
-    const int nrows = rowlist ? nkept[item] : n;
-    const int32_t *rows = rowlist ? rowlist + (size_t)item * n : nullptr;
+    uint32_t *Bw = work.bits + ((size_t)item * (TB >> 5) + warp) * (size_t)nblk * C * 32 + 2 * lane;
+    const int nrows = work.nkept[item];
+    const int32_t *rows = work.rowlist + (size_t)item * n;
+    const int64_t *Rp = work.rowp + (size_t)item * n;
+    const int32_t *Rm = work.rowm + (size_t)item * n;
     uint32_t wbits[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) wbits[c] = 0;
 
-    int64_t cur[C];
+    int64_t cur[C], top[C];
 #pragma unroll
     for (int c = 0; c < C; ++c) {
-        cur[c] = 0;
-        srow[c * T + t] = 0;
+        cur[c] = top[c] = 0;
+        srow[c * TB + t] = 0;
     }
-    for (int x = t; x < kMetaRows && x < nrows; x += T) {
-        const int i = rows ? rows[x] : n - 1 - x;
-        sp[x] = Pp[order ? order[i] : i];
-        sw[x] = wpre[i];
-        sm[x] = meta[i];
-    }
-    __syncthreads();
+    // rows are staged 256 at a time, a block ahead, with asynchronous copies
+    auto stage = [&](int blk) {
+        const int buf = (blk & 1) * kMetaRows;
+        for (int x = t; x < kMetaRows && blk * kMetaRows + x < nrows; x += T) {
+            const int r = blk * kMetaRows + x;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(sp + buf + x)),
+                         "l"(__cvta_generic_to_global(Rp + r)) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sm + buf + x)),
+                         "l"(__cvta_generic_to_global(Rm + r)) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(sw + buf + x)),
+                         "l"(__cvta_generic_to_global(wpre + rows[r])) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto staged = [&] { asm volatile("cp.async.wait_all;" ::: "memory"); };
+    auto barrier = [&] { asm volatile("bar.sync 1, %0;" ::"r"(T) : "memory"); };
+    stage(0);
+    staged();
+    barrier();
 
-    int64_t nx_p = 0;
-    int32_t nx_w = 0, nx_m = 0;
     for (int r = 0; r < nrows; ++r) {
         const int blk = r / kMetaRows, off = r - blk * kMetaRows, buf = (blk & 1) * kMetaRows;
-        if (off == 0) {
-            const int x = (blk + 1) * kMetaRows + t;
-            if (t < kMetaRows && x < nrows) {
-                const int ii = rows ? rows[x] : n - 1 - x;
-                nx_p = Pp[order ? order[ii] : ii];
-                nx_w = wpre[ii];
-                nx_m = meta[ii];
-            }
-        }
+        if (off == 0) stage(blk + 1);
         const int64_t p = sp[buf + off];
         const int w = sw[buf + off];
         const int32_t m = sm[buf + off];
-        const int skip = meta_skip(m), push = meta_push(m);
+        const bool from_cur = (m & (3 << 3)) == (kWaveCur << 3);
+        const int lvl = (int)((uint32_t)m >> 16);
         const int64_t *prev = srow + (r & 1) * kpad;
         int64_t *outr = srow + ((r + 1) & 1) * kpad;
         const uint32_t mrow = 1u << (r & 31);
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-            int64_t s;
-            if (skip == kSkipCur) s = cur[c];
-            else if (skip == kSkipZero) s = 0;
-            else if (skip < L_smem) s = sstk[((size_t)skip * C + c) * T + t];
-            else s = gst[((size_t)(skip - L_smem) * C + c) * T + t];
+            const int64_t s = from_cur ? cur[c] : top[c];
             const int jj = t * C + c + 1 - w;
             bool take = false;
             int64_t v = s;
@@ -622,7 +638,7 @@ k_tree_dp_flat(int32_t n, const int32_t *__restrict__ rowlist, const int32_t *__
                 int64_t base = 0;
                 if (jj > 0) {
                     const int q = jj - 1;
-                    base = prev[(q % C) * T + q / C];
+                    base = prev[(q % C) * TB + q / C];
                 }
                 const int64_t tv = p + base;
                 if (tv > s) {
@@ -631,7 +647,7 @@ k_tree_dp_flat(int32_t n, const int32_t *__restrict__ rowlist, const int32_t *__
                 }
             }
             cur[c] = v;
-            outr[c * T + t] = v;
+            outr[c * TB + t] = v;
             if (take) wbits[c] |= mrow;
         }
         if ((r & 31) == 31 || r == nrows - 1) {
@@ -641,32 +657,36 @@ k_tree_dp_flat(int32_t n, const int32_t *__restrict__ rowlist, const int32_t *__
                 wbits[c] = 0;
             }
         }
-        if (push >= 0) {
+        if (m & kWavePush) {
 #pragma unroll
             for (int c = 0; c < C; ++c) {
-                if (push < L_smem) sstk[((size_t)push * C + c) * T + t] = cur[c];
-                else gst[((size_t)(push - L_smem) * C + c) * T + t] = cur[c];
+                top[c] = cur[c];
+                if (lvl < L_smem) sstk[((size_t)lvl * C + c) * TB + t] = cur[c];
+                else gst[((size_t)(lvl - L_smem) * C + c) * TB + t] = cur[c];
             }
-        }
-        if (off == kMetaRows - 1) {
-            const int x = (blk + 1) * kMetaRows + t;
-            const int nb = ((blk + 1) & 1) * kMetaRows;
-            if (t < kMetaRows && x < nrows) {
-                sp[nb + t] = nx_p;
-                sw[nb + t] = nx_w;
-                sm[nb + t] = nx_m;
+        } else if (m & kWaveReload) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                if (lvl < L_smem) top[c] = sstk[((size_t)lvl * C + c) * TB + t];
+                else top[c] = gst[((size_t)(lvl - L_smem) * C + c) * TB + t];
             }
+        } else if (m & kWaveZeroTop) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) top[c] = 0;
         }
-        __syncthreads();
+        if (off == kMetaRows - 1) staged();
+        barrier();
     }
+    staged();                                   // no copy outlives the block
+    const int64_t add = state == 2 ? work.base[item] : 0;
     if (k == 0) {
-        if (t == 0) best[item] = 0;
+        if (t == 0) best[item] = add;
     } else {
         const int q = k - 1;
         if (q / C == t) {
 #pragma unroll
             for (int c = 0; c < C; ++c)
-                if (c == q % C) best[item] = cur[c];
+                if (c == q % C) best[item] = cur[c] + add;
         }
     }
 }
@@ -684,8 +704,11 @@ constexpr int kPruneCluster = 8;         // CTAs per item of the pruned-sweep ke
 // has a positive strict descendant iff cnt[next(x)] - cnt[x + 1] > 0, and row
 // i is kept iff it is a root or its parent has one.  A kept row i that is
 // itself an identity (p_i <= 0 and no positive strict descendant: D[i] =
-// D[next(i)], all bits "skip") is dropped as well (for the one-CTA kernel,
-// which follows the host's stack plan, only if it has no stack operation).
+// D[next(i)], all bits "skip") is dropped as well.  For an item that the
+// reduction has cut down (red = 2) the rows are the undecided ones: decided
+// rows inside the optimal set are closed upwards and those outside it
+// downwards, so the undecided rows in preorder form a forest of their own,
+// with the same subtree ends.
 // Kept rows are listed in sweep order (decreasing i); every position records
 // the first kept row at or after it in preorder, so a skip to a dropped row
 // lands where the all-"skip" walk through it would.
@@ -755,8 +778,8 @@ template <bool BYNODE>
 __global__ void __launch_bounds__(1024)
 k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict__ order,
         const int32_t *__restrict__ next, const int2 *__restrict__ pspan,
-        const int32_t *__restrict__ wpre, const int32_t *__restrict__ wmeta,
-        const int32_t *__restrict__ item_active, DpWork w, int prune, int wave, int stack_depth,
+        const int32_t *__restrict__ wpre,
+        const int32_t *__restrict__ item_active, DpWork w, int prune, int stack_depth,
         int32_t *__restrict__ status, unsigned long long *__restrict__ rows_kept)
 {
     constexpr int V = 4;
@@ -765,6 +788,9 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
     const int CL = (int)cluster_nctarank(), cr = (int)cluster_ctarank();
     const int item = blockIdx.x / CL;
     if (item_active && !item_active[item]) return;       // uniform over the cluster
+    const int state = w.red ? w.red[item] : 0;           // of the reduction
+    if (state == 1) return;                              // solved by it
+    const uint32_t *ud = state == 2 ? w.undecided + (size_t)item * ((n + 31) / 32) : nullptr;
     const int64_t *Pp = profit + (size_t)item * n;
     int32_t *cnt = w.cnt + (size_t)item * (n + 1);
     int32_t *rl = w.rowlist + (size_t)item * n;
@@ -778,8 +804,9 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
     };
     int lo, hi, total;
 
-    // prefix counts of positive profits, preorder
-    slice(n, lo, hi);
+    // prefix counts of positive profits, preorder (the reduction has already
+    // chosen the rows otherwise)
+    slice(ud ? 0 : n, lo, hi);
     int mine = 0;
     for (int i = lo + t; i < hi; i += T) mine += pval(i) > 0;
     block_exclusive_scan(mine, &total, sh);
@@ -805,22 +832,20 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
         }
         carry += tt;
     }
-    if (cr == 0 && t == 0) cnt[n] = npos;
+    if (cr == 0 && t == 0 && !ud) cnt[n] = npos;
     cluster_sync_all();                                   // cnt complete for every CTA
 
     // kept rows in sweep order r = n - 1 - i, their kept index, their total weight
     auto keep = [&](int r) -> bool {
         if (!prune) return true;
         const int i = n - 1 - r;
+        if (ud) return (ud[i >> 5] >> (i & 31)) & 1u;
         const int2 sp = pspan[i];
         if (!(sp.x < 0 || cnt[sp.y] - cnt[sp.x] > 0)) return false;
         // an identity row (p <= 0 and no positive strict descendant, so D[i] =
         // D[next(i)] and every bit is "skip") is dropped too: a skip to it
-        // lands on the first kept row after it, which holds the same values.
-        // The one-CTA kernel reads the host's stack plan and keeps the ones
-        // with a stack operation; the wavefront kernel's plan is rebuilt below
-        const bool ident = cnt[next[i]] - cnt[i + 1] == 0 && pval(i) <= 0;
-        return !(ident && (wave || (wmeta[i] & kWaveStackOps) == 0));
+        // lands on the first kept row after it, which holds the same values
+        return cnt[next[i]] - cnt[i + 1] != 0 || pval(i) > 0;
     };
     slice(n, lo, hi);
     int kmine = 0;
@@ -884,8 +909,7 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
                 sk[q] = nx < n ? kx[nx] : -1;
                 wq[v] = wpre[i];
                 rp[q] = pval(i);
-                rm[q] = wmeta[i];               // the wavefront kernel's is rebuilt below
-                if (wave) cnt[q] = -1;          // cnt (done with) becomes last_top_reader
+                cnt[q] = -1;                    // cnt (done with) becomes last_top_reader
             }
             wl += wq[v];
         }
@@ -902,11 +926,9 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
         wcarry += tt;
     }
     if (cr == 0 && t == 0) ws[nk] = 0;
-    if (!wave) return;
 
-    // Skip-row stack plan of the wavefront kernel over the kept rows (the
-    // host's plan is for the whole tree; after pruning many of its pushes
-    // have no reader left).  Kept row q reads row sk[q]: the row just
+    // Skip-row stack plan over the kept rows (the host's plan is for the
+    // whole tree; after pruning many of its pushes have no reader left).  Kept row q reads row sk[q]: the row just
     // computed when sk[q] = q - 1, else the stack top (the zero row when the
     // stack is empty, which is the case whenever sk[q] = -1).  A row read
     // through the stack is pushed when computed and popped after its last
@@ -984,40 +1006,58 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t dp_work_bytes(int batch, int n, int words)
+static std::atomic<bool> g_injected[64];      // pp_test_inject has silenced a warp, per device
+
+bool reduce_on(const pp_instance *inst)
 {
-    const size_t nb = (size_t)(n + 63) / 64 * 64, B = (size_t)std::max(batch, 1), N = (size_t)std::max(n, 1);
-    return align256(B * nb * words * 4) + 4 * align256(B * N * 4) + 2 * align256(B * (N + 1) * 4) +
-           align256(B * 4) + align256(B * N * 8);
+    return inst->red.CL > 0 && !inst->tune_noprune && !(inst->device < 64 && g_injected[inst->device].load());
 }
 
-DpWork dp_work_split(void *base, int batch, int n, int words)
+size_t dp_work_bytes(const pp_instance *inst, int batch, int words)
 {
+    const int n = inst->n;
+    const size_t nb = (size_t)(n + 63) / 64 * 64, B = (size_t)std::max(batch, 1), N = (size_t)std::max(n, 1);
+    return align256(B * nb * words * 4) + 4 * align256(B * N * 4) + 2 * align256(B * (N + 1) * 4) +
+           align256(B * 4) + align256(B * N * 8) +
+           (inst->red.CL ? 2 * align256(B * 4) + align256(B * 8) + 2 * align256(B * ((N + 31) / 32) * 4) +
+                               B * reduce_item_bytes(inst)
+                         : 0);
+}
+
+DpWork dp_work_split(const pp_instance *inst, void *base, int batch, int words)
+{
+    const int n = inst->n;
     const size_t nb = (size_t)(n + 63) / 64 * 64, B = (size_t)std::max(batch, 1), N = (size_t)std::max(n, 1);
     char *p = reinterpret_cast<char *>(base);
+    auto take = [&](size_t bytes) {
+        char *q = p;
+        p += align256(bytes);
+        return q;
+    };
     DpWork w;
-    w.bits = reinterpret_cast<uint32_t *>(p);
-    p += align256(B * nb * words * 4);
-    w.rowlist = reinterpret_cast<int32_t *>(p);
-    p += align256(B * N * 4);
-    w.kidx = reinterpret_cast<int32_t *>(p);
-    p += align256(B * N * 4);
-    w.cnt = reinterpret_cast<int32_t *>(p);
-    p += align256(B * (N + 1) * 4);
-    w.nkept = reinterpret_cast<int32_t *>(p);
-    p += align256(B * 4);
-    w.skip = reinterpret_cast<int32_t *>(p);
-    p += align256(B * N * 4);
-    w.wsuf = reinterpret_cast<int32_t *>(p);
-    p += align256(B * (N + 1) * 4);
-    w.rowp = reinterpret_cast<int64_t *>(p);
-    p += align256(B * N * 8);
-    w.rowm = reinterpret_cast<int32_t *>(p);
+    w.bits = reinterpret_cast<uint32_t *>(take(B * nb * words * 4));
+    w.rowlist = reinterpret_cast<int32_t *>(take(B * N * 4));
+    w.kidx = reinterpret_cast<int32_t *>(take(B * N * 4));
+    w.cnt = reinterpret_cast<int32_t *>(take(B * (N + 1) * 4));
+    w.nkept = reinterpret_cast<int32_t *>(take(B * 4));
+    w.skip = reinterpret_cast<int32_t *>(take(B * N * 4));
+    w.wsuf = reinterpret_cast<int32_t *>(take(B * (N + 1) * 4));
+    w.rowp = reinterpret_cast<int64_t *>(take(B * N * 8));
+    w.rowm = reinterpret_cast<int32_t *>(take(B * N * 4));
+    if (reduce_on(inst)) {
+        w.red = reinterpret_cast<int32_t *>(take(B * 4));
+        w.left = reinterpret_cast<int32_t *>(take(B * 4));
+        w.base = reinterpret_cast<int64_t *>(take(B * 8));
+        w.taken = reinterpret_cast<uint32_t *>(take(B * ((N + 31) / 32) * 4));
+        w.undecided = reinterpret_cast<uint32_t *>(take(B * ((N + 31) / 32) * 4));
+        w.red_scratch = p;
+    }
     return w;
 }
 
-DpWork dp_work_item(const DpWork &w, int item, int n, int words)
+DpWork dp_work_item(const pp_instance *inst, const DpWork &w, int item, int words)
 {
+    const int n = inst->n;
     const size_t nb = (size_t)(n + 63) / 64 * 64, N = (size_t)std::max(n, 1), it = (size_t)item;
     DpWork o;
     o.bits = w.bits + it * nb * words;
@@ -1029,6 +1069,14 @@ DpWork dp_work_item(const DpWork &w, int item, int n, int words)
     o.wsuf = w.wsuf + it * (N + 1);
     o.rowp = w.rowp + it * N;
     o.rowm = w.rowm + it * N;
+    if (w.red) {
+        o.red = w.red + it;
+        o.left = w.left + it;
+        o.base = w.base + it;
+        o.taken = w.taken + it * ((N + 31) / 32);
+        o.undecided = w.undecided + it * ((N + 31) / 32);
+        o.red_scratch = w.red_scratch + it * reduce_item_bytes(inst);
+    }
     return o;
 }
 
@@ -1247,18 +1295,13 @@ static pp_status ensure_split_streams(pp_instance *inst)
 }
 
 template <int C>
-static pp_status launch_flat_c(pp_instance *inst, int batch, const int64_t *profit, bool by_node,
-                               const int32_t *item_budget, int32_t max_budget,
+static pp_status launch_flat_c(pp_instance *inst, int batch, const int32_t *item_budget, int32_t max_budget,
                                const int32_t *item_active, const DpGeom &g, int64_t *best,
                                const DpWork &work, int64_t *gstack, int L_glob, cudaStream_t st)
 {
-    uint32_t *bits = work.bits;
     PP_CUDA(cudaFuncSetAttribute(k_tree_dp_flat<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
-    k_tree_dp_flat<C><<<batch, g.T, g.smem, st>>>(inst->n, work.rowlist, work.nkept, profit,
-                                                   by_node ? inst->d_order : nullptr,
-                                                   inst->d_wpre, inst->d_meta, item_budget, max_budget,
-                                                   item_active, best, bits, gstack, g.L_smem, L_glob,
-                                                   inst->d_status);
+    k_tree_dp_flat<C><<<batch, g.T, g.smem, st>>>(inst->n, work, inst->d_wpre, item_budget, max_budget,
+                                                   item_active, best, gstack, g.L_smem, L_glob, inst->d_status);
     PP_CUDA(cudaGetLastError());
     return PP_OK;
 }
@@ -1272,7 +1315,13 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
                                    int32_t max_budget, int64_t *gstack, int L_glob,
                                    unsigned long long *rows_kept)
 {
-    // the pruned sweep of every item, then the DP over its kept rows
+    // the exact reduction; then, for the items it leaves, the pruned sweep
+    // and the DP over its kept rows
+    if (work.red) {
+        pp_status s = launch_reduce(inst, batch, profit, by_node, item_budget, item_active, best, work, st, max_budget,
+                                    rows_kept);
+        if (s != PP_OK) return s;
+    }
     {
         cudaLaunchConfig_t pc = {};
         pc.gridDim = dim3(kPruneCluster * batch);
@@ -1285,16 +1334,16 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
         pa[0].val.clusterDim.z = 1;
         pc.attrs = pa;
         pc.numAttrs = 1;
-        const int32_t *ord = inst->d_order, *nxt = inst->d_next, *wp = inst->d_wpre, *wm = inst->d_wave;
+        const int32_t *ord = inst->d_order, *nxt = inst->d_next, *wp = inst->d_wpre;
         const int2 *psp = inst->d_pspan;
-        const int pr = !inst->tune_noprune, wv = g.wave, sd = inst->stack_depth;
+        const int pr = !inst->tune_noprune, sd = inst->stack_depth;
         int32_t *stt = inst->d_status;
         if (by_node)
-            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<true>, inst->n, profit, ord, nxt, psp, wp, wm, item_active,
-                                       work, pr, wv, sd, stt, rows_kept));
+            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<true>, inst->n, profit, ord, nxt, psp, wp, item_active,
+                                       work, pr, sd, stt, rows_kept));
         else
-            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<false>, inst->n, profit, ord, nxt, psp, wp, wm, item_active,
-                                       work, pr, wv, sd, stt, rows_kept));
+            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<false>, inst->n, profit, ord, nxt, psp, wp, item_active,
+                                       work, pr, sd, stt, rows_kept));
     }
     PP_CUDA(cudaGetLastError());
     uint32_t *bits = work.bits;
@@ -1326,7 +1375,7 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
             int32_t Lg = L_glob, ranked = g.split > 0;
             void *args[] = {&n, &nblk, (void *)&rowp, (void *)&rowm, (void *)&nkept, (void *)&item_budget,
                             &max_budget, (void *)&item_active, &best, &bits, &gstack, &L_smem, &Lg, &status,
-                            &nb, &slot_base, &ranked};
+                            &nb, &slot_base, &ranked, (void *)&work.red, (void *)&work.left, (void *)&work.base};
             PP_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
             return PP_OK;
         };
@@ -1347,12 +1396,12 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
         return PP_OK;
     }
     switch (g.C) {
-    case 1: return launch_flat_c<1>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
-    case 2: return launch_flat_c<2>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
-    case 4: return launch_flat_c<4>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
-    case 8: return launch_flat_c<8>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
-    case 16: return launch_flat_c<16>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
-    case 32: return launch_flat_c<32>(inst, batch, profit, by_node, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 1: return launch_flat_c<1>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 2: return launch_flat_c<2>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 4: return launch_flat_c<4>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 8: return launch_flat_c<8>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 16: return launch_flat_c<16>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
+    case 32: return launch_flat_c<32>(inst, batch, item_budget, max_budget, item_active, g, best, work, gstack, L_glob, st);
     default: return fail(PP_EINVAL, "unsupported DP geometry");
     }
 }
@@ -1398,7 +1447,7 @@ extern "C" size_t pp_dp_bits_size(const pp_instance *inst, int32_t batch, int32_
 {
     DpGeom g;
     if (!inst || batch <= 0 || !dp_geometry(inst, max_budget, &g, batch)) return 0;
-    return dp_work_bytes(batch, inst->n, g.words);
+    return dp_work_bytes(inst, batch, g.words);
 }
 
 extern "C" pp_status pp_tree_dp(pp_instance *inst, int32_t batch, const int64_t *profit,
@@ -1413,13 +1462,16 @@ extern "C" pp_status pp_tree_dp(pp_instance *inst, int32_t batch, const int64_t 
     if (!budget || !best || (inst->n > 0 && (!profit || !bits)))
         return fail(PP_EINVAL, "null device pointer");
     return launch_tree_dp(inst, batch, profit, true, budget, nullptr, g, best,
-                          dp_work_split(bits, batch, inst->n, g.words), (cudaStream_t)stream, max_budget);
+                          dp_work_split(inst, bits, batch, g.words), (cudaStream_t)stream, max_budget);
 }
 
 extern "C" pp_status pp_test_inject(int32_t kind, int32_t value)
 {
     if (kind != 1) return fail(PP_EINVAL, "unknown injection kind");
     PP_CUDA(cudaMemcpyToSymbol(g_drop_publish_warp, &value, sizeof(value)));
+    int dev = 0;
+    PP_CUDA(cudaGetDevice(&dev));
+    if (dev < 64) g_injected[dev].store(value >= 0);    // the reduction would leave nothing to wait for
     return PP_OK;
 }
 
@@ -1530,7 +1582,7 @@ extern "C" pp_status pp_tree_dp_noalloc(pp_instance *inst, int32_t batch, const 
                                    std::to_string(kStaticStackBytes) +
                                    " bytes; use a smaller batch or pp_tree_dp");
     return launch_dp_kernels(inst, batch, profit, true, budget, nullptr, g, best,
-                             dp_work_split(bits, batch, inst->n, g.words), st, max_budget, scratch, L_glob,
+                             dp_work_split(inst, bits, batch, g.words), st, max_budget, scratch, L_glob,
                              nullptr);
 }
 
@@ -1553,7 +1605,7 @@ extern "C" pp_status pp_dp_rows_swept(const pp_instance *inst, int32_t batch, in
         return PP_OK;
     }
     if (!workspace) return fail(PP_EINVAL, "null workspace");
-    const DpWork w = dp_work_split(const_cast<uint32_t *>(workspace), batch, inst->n, g.words);
+    const DpWork w = dp_work_split(inst, const_cast<uint32_t *>(workspace), batch, g.words);
     PP_CUDA(cudaMemcpyAsync(rows, w.nkept, sizeof(int32_t) * batch, cudaMemcpyDeviceToHost, (cudaStream_t)stream));
     PP_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
     return PP_OK;

@@ -218,8 +218,6 @@ extern "C" pp_status pp_instance_destroy(pp_instance *inst)
     cudaFree(inst->d_order);
     cudaFree(inst->d_next);
     cudaFree(inst->d_wpre);
-    cudaFree(inst->d_meta);
-    cudaFree(inst->d_wave);
     cudaFree(inst->d_pspan);
     cudaFree(inst->d_budget);
     cudaFree(inst->d_a);
@@ -230,6 +228,7 @@ extern "C" pp_status pp_instance_destroy(pp_instance *inst)
     cudaFree(inst->d_tr);
     cudaFree(inst->d_g);
     cudaFree(inst->d_status);
+    cudaFree(inst->d_red);
     free_scratch(inst->stack);
     free_scratch(inst->plan);
     free_scratch(inst->plan_bits);
@@ -261,7 +260,7 @@ static pp_status upload(T **dst, const T *src, size_t count, cudaStream_t st)
 // The tree's host tables of an instance: preorder, next, weights by
 // position, the traceback's skip depth, the skip-row stack plan, budgets.
 static pp_status build_host_tables(int32_t n, int32_t W, const int32_t *parent, const int32_t *weight,
-                                   int32_t mode, const int32_t *budget, pp_instance *inst)
+                                   int32_t mode, const int32_t *budget, pp_instance *inst, ReduceTables *red)
 {
     inst->n = n;
     inst->W = W;
@@ -290,9 +289,21 @@ static pp_status build_host_tables(int32_t n, int32_t W, const int32_t *parent, 
         }
         inst->trace_skips = s1 > 0 && s2 > 5 * s1 ? 3 : 1;
     }
-    if (!build_row_meta(n, inst->h_next, inst->h_meta, &inst->stack_depth, &inst->h_wpre, &inst->h_wave))
+    std::vector<int32_t> meta;
+    if (!build_row_meta(n, inst->h_next, meta, &inst->stack_depth))
         return fail(PP_EINVAL, "skip-row stack deeper than supported");
     inst->h_budget.assign(budget, budget + W);
+    inst->h_par.resize(n);
+    {
+        std::vector<int32_t> pos(n);
+        for (int32_t i = 0; i < n; ++i) pos[inst->h_order[i]] = i;
+        for (int32_t i = 0; i < n; ++i) {
+            const int32_t p = parent[inst->h_order[i]];
+            inst->h_par[i] = p < 0 ? -1 : pos[p];
+        }
+    }
+    if (build_reduce_tables(n, inst->h_par, inst->h_next, inst->h_wpre, inst->total_weight, inst->max_weight, red))
+        inst->red = reduce_shape(*red);
     return PP_OK;
 }
 
@@ -360,7 +371,8 @@ static pp_status create_impl(int32_t n, int32_t W, const int32_t *parent, const 
         pool.reserve(nth);
         for (int q = 0; q < nth; ++q) pool.emplace_back(check, q);
     }
-    const pp_status tables = build_host_tables(n, W, parent, weight, mode, budget, inst);
+    ReduceTables red;
+    const pp_status tables = build_host_tables(n, W, parent, weight, mode, budget, inst, &red);
     for (auto &th : pool) th.join();
     u128 total = 0, sum_demand = 0, sum_recompute = 0;
     uint64_t dr_bits = 0, t_bits = 0;
@@ -385,19 +397,24 @@ static pp_status create_impl(int32_t n, int32_t W, const int32_t *parent, const 
     if ((s = upload(&inst->d_order, inst->h_order.data(), n, st))) return s;
     if ((s = upload(&inst->d_next, inst->h_next.data(), n, st))) return s;
     if ((s = upload(&inst->d_wpre, inst->h_wpre.data(), n, st))) return s;
-    if ((s = upload(&inst->d_meta, inst->h_meta.data(), n, st))) return s;
-    if ((s = upload(&inst->d_wave, inst->h_wave.data(), n, st))) return s;
     {
         // for the parent x of each position: the preorder range [x + 1, next(x))
         // of x's strict descendants (the pruned sweep's test)
-        std::vector<int32_t> pos(n);
         std::vector<int2> span(n);
-        for (int32_t i = 0; i < n; ++i) pos[inst->h_order[i]] = i;
         for (int32_t i = 0; i < n; ++i) {
-            const int32_t par = parent[inst->h_order[i]];
-            span[i] = par < 0 ? make_int2(-1, -1) : make_int2(pos[par] + 1, inst->h_next[pos[par]]);
+            const int32_t par = inst->h_par[i];
+            span[i] = par < 0 ? make_int2(-1, -1) : make_int2(par + 1, inst->h_next[par]);
         }
         if ((s = upload(&inst->d_pspan, span.data(), n, st))) return s;
+        std::vector<char> rt;
+        if (inst->red.CL) {
+            rt.resize(reduce_tables_bytes(red));
+            reduce_tables_pack(red, rt.data());
+            char *d = nullptr;
+            s = upload(&d, rt.data(), rt.size(), st);
+            inst->d_red = d;
+            if (s) return s;
+        }
         PP_CUDA(cudaStreamSynchronize(st));          // the host vectors die here
     }
     if ((s = upload(&inst->d_budget, budget, W, st))) return s;

@@ -44,7 +44,6 @@ inline int32_t meta_pack(int skip, int push)
 // 16-31 level.
 constexpr int kWaveCur = 0, kWaveTop = 2;
 constexpr int kWaveReload = 1 << 5, kWavePush = 1 << 6, kWaveZeroTop = 1 << 7;
-constexpr int kWaveStackOps = kWaveReload | kWavePush | kWaveZeroTop;
 __host__ __device__ inline int32_t wave_pack(int w, int kind, int flags, int level)
 {
     return (int32_t)((uint32_t)(w - 1) | ((uint32_t)kind << 3) | (uint32_t)flags | ((uint32_t)level << 16));
@@ -104,14 +103,45 @@ struct DpWork {
     int32_t *wsuf = nullptr;       // [batch][n + 1]
     int64_t *rowp = nullptr;       // [batch][n] profit of each kept row, sweep order
     int32_t *rowm = nullptr;       // [batch][n] wave-kernel metadata of each kept row
+    // exact reduction (pp_reduce.cu), null when the launch does without it.
+    // red[item] = 1: solved, the optimal set is `taken` and nkept[item] the
+    // number of rows that were undecided; the pruned sweep's kernels leave
+    // it alone.  2: those kernels sweep only the rows in `undecided`, with the
+    // budget left[item]; base[item] is the value of the decided rows, which
+    // are in `taken`.  0: they sweep all rows.
+    int32_t *red = nullptr;        // [batch]
+    int32_t *left = nullptr;       // [batch]
+    int64_t *base = nullptr;       // [batch]
+    uint32_t *taken = nullptr;     // [batch][ceil(n / 32)] by preorder position
+    uint32_t *undecided = nullptr; // [batch][ceil(n / 32)]
+    char *red_scratch = nullptr;   // [batch][reduce_item_bytes]
 };
-size_t dp_work_bytes(int batch, int n, int words);
-DpWork dp_work_split(void *base, int batch, int n, int words);
+size_t dp_work_bytes(const pp_instance *inst, int batch, int words);
+DpWork dp_work_split(const pp_instance *inst, void *base, int batch, int words);
 // the same workspace seen as a batch of one: item `item` of `w`
-DpWork dp_work_item(const DpWork &w, int item, int n, int words);
+DpWork dp_work_item(const pp_instance *inst, const DpWork &w, int item, int words);
 
 // Status word values written by kernels (same numbering as pp_status).
 constexpr int32_t kDevOk = PP_OK;
+
+// Layout of the exact reduction (pp_reduce.cu): host tables while an instance
+// is built, and their sizes.  CL = 0: this tree is not reduced.
+constexpr int32_t kReduceMinRows = 1024;    // below, the sweep is as short as the reduction
+struct ReduceTables {
+    struct Slot {
+        int32_t pos, code, acc, par;
+    };
+    struct Stream {
+        int32_t tile, tiles;
+    };
+    int CL = 0;
+    std::vector<Slot> slot;
+    std::vector<Stream> stream;
+    std::vector<int32_t> lev, binlev, binslot, nacc;
+};
+struct ReduceShape {
+    int CL = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_acc = 0, acc_smem = 0;
+};
 
 struct Scratch {
     void *ptr = nullptr;
@@ -132,13 +162,11 @@ struct pp_instance {
     int32_t trace_skips = 1;            // skips the traceback speculates per step beyond the first
     // DP launch-shape overrides of this instance (pp_tune_dp; 0 = automatic)
     int32_t tune_cl = 0, tune_c = 0, tune_flat = 0, tune_noprune = 0;
-    std::vector<int32_t> h_order, h_next, h_budget, h_wpre, h_meta, h_wave;
+    std::vector<int32_t> h_order, h_next, h_par, h_budget, h_wpre;
     // device tables, preorder-indexed unless noted
     int32_t *d_order = nullptr;         // [n] position -> node id
     int32_t *d_next = nullptr;          // [n]
     int32_t *d_wpre = nullptr;          // [n] chunk weight
-    int32_t *d_meta = nullptr;          // [n] packed skip / push codes
-    int32_t *d_wave = nullptr;          // [n] wavefront-kernel row metadata
     int2 *d_pspan = nullptr;            // [n] parent x's strict-descendant range (x+1, next(x)); roots -1
     int32_t *d_budget = nullptr;        // [W]
     int64_t *d_a = nullptr;             // mode 0: [W][n] a_m(b)       (Eq. 2)
@@ -149,6 +177,8 @@ struct pp_instance {
     int64_t *d_tr = nullptr;            // by node id: mode 0 [W][n] f_m(b), mode 1 [W][W][n] f_{m<-h}(b)
     int64_t *d_g = nullptr;             // mode 1: [W][W][n] Lambda_m(b) q_{m<-h}(b) at [h][m][i] (Eq. 5)
     int32_t *d_status = nullptr;        // device status word
+    pp::ReduceShape red;                // exact reduction's layout (pp_reduce.cu); CL = 0: none
+    void *d_red = nullptr;              // its tables
     pp::Scratch stack;                  // skip-row stack spill of pp_tree_dp
     pp::Scratch plan;                   // pp_plan_run working set
     pp::Scratch plan_bits;              // pp_plan_run decision bits
@@ -194,6 +224,20 @@ pp_status launch_tree_dp(pp_instance *inst, int batch, const int64_t *profit, bo
                          const int32_t *item_budget, const int32_t *item_active,
                          const DpGeom &g, int64_t *best, const DpWork &work, cudaStream_t st,
                          int32_t max_budget, unsigned long long *rows_kept = nullptr, int stack_item = 0);
+// The exact reduction (pp_reduce.cu).  `par` is the parent's position (-1: root).
+bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::vector<int32_t> &next,
+                         const std::vector<int32_t> &wpre, int64_t total_weight, int32_t max_weight,
+                         ReduceTables *out);
+size_t reduce_tables_bytes(const ReduceTables &R);
+void reduce_tables_pack(const ReduceTables &R, char *dst);
+ReduceShape reduce_shape(const ReduceTables &R);
+size_t reduce_item_bytes(const pp_instance *inst);
+// whether launches of this instance try the reduction first (not without
+// pruning, and not while pp_test_inject makes a warp of the sweep silent)
+bool reduce_on(const pp_instance *inst);
+pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, bool by_node,
+                        const int32_t *item_budget, const int32_t *item_active, int64_t *best, const DpWork &work,
+                        cudaStream_t st, int32_t max_budget, unsigned long long *rows_kept);
 // scratch for the skip-row stack of `items` item slots of geometry g
 pp_status ensure_dp_stack(pp_instance *inst, const DpGeom &g, int items);
 

@@ -134,10 +134,10 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     PlanBuffers pb;
     pp_status s = plan_buffers(inst, B, &pb);
     if (s != PP_OK) return s;
-    s = ensure_scratch(inst->plan_bits, std::max(dp_work_bytes(S, n, g.words), dp_work_bytes(W, n, gw.words)));
+    s = ensure_scratch(inst->plan_bits, std::max(dp_work_bytes(inst, S, g.words), dp_work_bytes(inst, W, gw.words)));
     if (s != PP_OK) return s;
-    const DpWork work = dp_work_split(inst->plan_bits.ptr, S, n, g.words);
-    const DpWork work_w = dp_work_split(inst->plan_bits.ptr, W, n, gw.words);
+    const DpWork work = dp_work_split(inst, inst->plan_bits.ptr, S, g.words);
+    const DpWork work_w = dp_work_split(inst, inst->plan_bits.ptr, W, gw.words);
     unsigned long long *rows_kept = pb.rows;
     PP_CUDA(cudaMemsetAsync(rows_kept, 0, sizeof(unsigned long long), st));
 
@@ -196,7 +196,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 return s;
             if ((s = mark())) return s;
             if ((s = mark())) return s;   // no traceback for the standalone scores
-            launches += 3 + (gw.split ? 1 : 0);     // a split DP is two launches
+            launches += 3 + (gw.split ? 1 : 0) + (work.red ? 1 : 0);     // a split DP is two launches
             dp_launches += 1;
             std::vector<int64_t> score(W);
             standalone_cells = (int64_t)n * sumk;
@@ -326,7 +326,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
             a.greedy = greedy;
             if ((r = launch_traceback(inst, S, work, g, kb, nullptr, &a, st))) return r;
             if ((r = mark())) return r;
-            launches += 4 + (g.split ? 1 : 0);
+            launches += 4 + (g.split ? 1 : 0) + (work.red ? 1 : 0);
             dp_launches += 1;
             return PP_OK;
         };
@@ -423,7 +423,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 }
                 if (s) return s;
                 if ((s = smark(x, sx))) return s;
-                const DpWork wx = dp_work_item(work, x, n, g.words);
+                const DpWork wx = dp_work_item(inst, work, x, g.words);
                 if ((s = launch_tree_dp(inst, 1, pf, false, kb, pb.active + x, g1, pb.best + x, wx, sx, maxk,
                                         rows_kept, x)))
                     return s;
@@ -439,7 +439,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 a.greedy = pass == 0;
                 if ((s = launch_traceback(inst, 1, wx, g1, kb, nullptr, &a, sx))) return s;
                 if ((s = smark(x, sx))) return s;
-                launches += 4;
+                launches += 4 + (work.red ? 1 : 0);
                 if (pass > 0 && t == W - 1) {
                     k_sweep_end<<<1, 32, 0, sx>>>(1, pb.active + x, pb.improved + x, pb.sweeps + x);
                     PP_CUDA(cudaGetLastError());

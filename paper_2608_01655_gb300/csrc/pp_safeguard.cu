@@ -73,7 +73,7 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
     const size_t o_rows = 0, o_cand = o_rows + a256(4 * N * B), o_prof = o_cand + a256(4 * N * 3);
     const size_t o_best = o_prof + a256(8 * N * B), o_obj = o_best + a256(8 * (size_t)B);
     const size_t o_int = o_obj + a256(8 * 3), o_work = o_int + a256(4 * 5 * (size_t)B);
-    const size_t wbytes = std::max(dp_work_bytes(B, n, gB.words), dp_work_bytes(1, n, g1.words));
+    const size_t wbytes = std::max(dp_work_bytes(inst, B, gB.words), dp_work_bytes(inst, 1, g1.words));
     pp_status s = ensure_scratch(inst->sg, o_work + wbytes);
     if (s != PP_OK) return s;
     char *base = reinterpret_cast<char *>(inst->sg.ptr);
@@ -100,8 +100,8 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
     if (n > 0 && W > 0) {
         int bx = (n + 255) / 256;
         if (bx > 2 * inst->sm_count) bx = 2 * inst->sm_count;
-        const DpWork wB = dp_work_split(base + o_work, B, n, gB.words);
-        const DpWork w1 = dp_work_split(base + o_work, 1, n, g1.words);
+        const DpWork wB = dp_work_split(inst, base + o_work, B, gB.words);
+        const DpWork w1 = dp_work_split(inst, base + o_work, 1, g1.words);
         // Independent and Popularity: 2W independent DPs, one batch
         k_sg_profit<<<dim3(bx, B), 256, 0, st>>>(n, kind, worker, nullptr, inst->d_a, inst->d_own, inst->d_pop,
                                                  profit);
@@ -116,7 +116,7 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
         if ((s = launch_traceback(inst, B, wB, gB, kb, nullptr, &acc, st))) return s;
         k_or_rows<<<dim3(bx, 2), 256, 0, st>>>(n, W, 2, rows, cand);
         PP_CUDA(cudaGetLastError());
-        nl += 5 + (gB.split ? 1 : 0);             // a split DP is two launches
+        nl += 5 + (gB.split ? 1 : 0) + (wB.red ? 1 : 0);             // a split DP is two launches
         // LocalDedup: worker m sees the chunks of workers 0..m-1 in cand[2]
         uint32_t *dd = cand + 2 * N;
         for (int m = 0; m < W; ++m) {
@@ -131,7 +131,7 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
             a1.mask = dd;
             a1.greedy = 1;
             if ((s = launch_traceback(inst, 1, w1, g1, kb + m, nullptr, &a1, st))) return s;
-            nl += 4;
+            nl += 4 + (w1.red ? 1 : 0);
         }
     }
     if ((s = launch_objective(inst, 3, cand, nullptr, objd, st))) return s;

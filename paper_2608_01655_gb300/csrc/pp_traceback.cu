@@ -133,6 +133,8 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
             uint8_t *__restrict__ chosen, AcceptArgs acc)
 {
     const int item = blockIdx.x;
+    const int bi = acc.bits_item ? acc.bits_item[item] : item;   // the DP item whose bits this walks
+    const int state = w.red ? w.red[bi] : 0;   // of the reduction: 1 its set is a bitmap, 2 joins the walk's
     uint32_t hbit = 0;
     uint32_t *M = nullptr;
     if (acc.mask) {
@@ -145,11 +147,32 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
         M = acc.mask + (size_t)item * n;
         // fire-and-forget reductions: no thread waits for the old mask words
         // (in the greedy pass T_h is still empty: nothing to clear)
-        if (!acc.greedy)
+        if (!acc.greedy && !state)
             for (int32_t x = threadIdx.x; x < n; x += blockDim.x) atomicAnd(M + x, ~hbit);
     } else {
         uint8_t *ch = chosen + (size_t)item * n;
         for (int32_t x = threadIdx.x; x < n; x += blockDim.x) ch[x] = 0;
+    }
+    if (state) {
+        const uint32_t *tk = w.taken + (size_t)bi * ((n + 31) / 32);
+        __syncthreads();                      // chosen[] is cleared
+        for (int32_t x = threadIdx.x; x < n; x += blockDim.x) {
+            const bool in = (tk[x >> 5] >> (x & 31)) & 1u;
+            if (BYNODE) {
+                if (in) chosen[(size_t)item * n + order[x]] = 1;
+            } else if (in) {
+                atomicOr(M + x, hbit);
+            } else if (!acc.greedy) {
+                atomicAnd(M + x, ~hbit);
+            }
+        }
+        if (state == 1) {
+            if (acc.mask && !acc.greedy && threadIdx.x == 0) {
+                acc.improved[item] = 1;
+                acc.accepted[item] += 1;
+            }
+            return;
+        }
     }
     __shared__ int s_walk[3];                 // walker's tile row, tile column, done
     if (threadIdx.x == 0) {
@@ -159,8 +182,7 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
     }
     __syncthreads();
     volatile int *walk = s_walk;
-    const int32_t kq = item_budget[item];
-    const int bi = acc.bits_item ? acc.bits_item[item] : item;   // the DP item whose bits this walks
+    const int32_t kq = state == 2 ? w.left[bi] : item_budget[item];
     const int npair = (n + 63) / 64;                          // 64-row block pairs per chain warp
     const uint64_t *Bi = reinterpret_cast<const uint64_t *>(w.bits) + (size_t)bi * P * (size_t)npair * C * 32;
     const int32_t *rl = w.rowlist + (size_t)bi * n;
@@ -347,6 +369,6 @@ extern "C" pp_status pp_traceback(pp_instance *inst, int32_t batch, const uint32
     if (!dp_geometry(inst, max_budget, &g, std::max(batch, 1))) return fail(PP_EINVAL, "max_budget out of range");
     if (batch == 0 || inst->n == 0) return PP_OK;
     if (!bits || !budget || !chosen) return fail(PP_EINVAL, "null device pointer");
-    return launch_traceback(inst, batch, dp_work_split(const_cast<uint32_t *>(bits), batch, inst->n, g.words), g,
+    return launch_traceback(inst, batch, dp_work_split(inst, const_cast<uint32_t *>(bits), batch, g.words), g,
                             budget, chosen, nullptr, (cudaStream_t)stream);
 }

@@ -1,0 +1,99 @@
+"""The exact reduction before the tree DP's sweep (csrc/pp_reduce.cu), bit for
+bit against the oracle: trees around its tile, stream and cluster boundaries,
+budgets that bind or do not, ties that leave it more undecided rows than it
+takes, and paths too long for it.  Everything is integer: equality."""
+import numpy as np
+import pytest
+
+from paper_2608_01655_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def pp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_01655_gb300 import build
+    build.build()
+    from paper_2608_01655_gb300 import binding
+    return binding
+
+
+def _tree(rng, shape, n):
+    if shape == "random":
+        return np.array([-1] + [int(rng.integers(v)) if rng.random() < 0.98 else -1 for v in range(1, n)], np.int32)
+    if shape == "star":
+        return np.full(n, -1, np.int32)
+    if shape == "chain":
+        return np.arange(-1, n - 1, dtype=np.int32)
+    if shape == "caterpillar":                   # a spine of n / 2 nodes, a leaf on each
+        return np.array([-1] + [v - 1 if v % 2 else max(v - 2, 0) for v in range(1, n)], np.int32)
+    return wl._mixed_tree(rng, n)                # chains under a bushy prefix
+
+
+def _check(pp, oracle_lib, parent, weight, profits, budgets, by_rows):
+    n, B = len(parent), len(profits)
+    inst = wl.Instance("t", n, 1, parent, weight, np.ones((1, n), np.int64), np.ones((1, n), np.int64),
+                       np.ones((1, n), np.int64), 0, np.array([1], np.int32), 1, 1)
+    maxb = int(max(budgets))
+    with pp.Instance.from_workload(inst) as ppi:
+        prof = torch.from_numpy(np.ascontiguousarray(profits, np.int64)).cuda()
+        bud = torch.from_numpy(np.asarray(budgets, np.int32)).cuda()
+        best = torch.zeros(B, dtype=torch.int64, device="cuda")
+        bits = torch.randint(0, 1 << 30, (pp.pp_dp_bits_size(ppi, B, maxb) // 4,), dtype=torch.int32, device="cuda")
+        chosen = torch.zeros((B, n), dtype=torch.uint8, device="cuda")
+        for _ in range(2):                       # the workspace holds anything, then the last call's
+            pp.pp_tree_dp(ppi, prof, bud, maxb, best, bits)
+            pp.pp_traceback(ppi, bits, bud, maxb, chosen)
+            ppi.sync()
+            for b in range(B):
+                ob, oc = oracle_lib.rooted_dp(parent, weight, profits[b], int(budgets[b]))
+                assert int(best[b]) == ob, b
+                np.testing.assert_array_equal(chosen[b].cpu().numpy(), oc, err_msg=str(b))
+        by_rows(pp.pp_dp_rows_swept(ppi, B, maxb, bits))
+
+
+@pytest.mark.parametrize("shape", ["random", "star", "caterpillar", "mixed"])
+@pytest.mark.parametrize("n,wmax", [(1024, 1), (1055, 3), (6144, 1), (6145, 2), (12289, 9), (24577, 1)])
+def test_reduced_optimum_and_set(pp, oracle_lib, shape, n, wmax):
+    """One CTA to eight, weights on and above the wavefront kernel's limit;
+    per batch: profits over several decades, few values (ties), mostly zero,
+    negative ones, a budget of one slot and one that does not bind."""
+    rng = np.random.default_rng(n + wmax)
+    parent = _tree(rng, shape, n)
+    weight = rng.integers(1, wmax + 1, size=n).astype(np.int32)
+    wide = np.exp(rng.uniform(0, 18, size=(6, n))).astype(np.int64)
+    wide[1] = rng.integers(0, 4, size=n)
+    wide[2][rng.random(n) < 0.9] = 0
+    wide[3] -= int(np.quantile(wide[3], 0.6))
+    tw = int(weight.sum())
+    budgets = [n // 9 + 1, n // 20, n // 7, n // 11 + 3, 1, min(tw + 5, 8192)]
+
+    def rows(r):
+        assert r[5] == 0 or tw > 8192            # nothing is undecided without a limit
+        if shape != "caterpillar":               # (whose spine is taken in long runs: any count)
+            assert r[0] <= 1024                  # reduced
+    _check(pp, oracle_lib, parent, weight, wide, budgets, rows)
+
+
+def test_ties_and_zero_budget_and_long_paths(pp, oracle_lib):
+    """Equal profits on a star leave every row undecided (the pruned sweep
+    takes over), a budget of 0 takes nothing, profits near 2^61 are beyond the
+    price's range, and a path above 4,096 rows is not reduced at all."""
+    rng = np.random.default_rng(5)
+    n = 3000
+    one = np.ones(n, np.int32)
+    profits = np.stack([np.full(n, 7), rng.integers(1, 99, n), np.where(np.arange(n) == 5, 1 << 61, 3)]).astype(np.int64)
+
+    def rows(r):
+        assert r[0] == n and r[1] == 0 and r[2] > 1024
+    _check(pp, oracle_lib, np.full(n, -1, np.int32), one, profits, [100, 0, 50], rows)
+    for m, want in ((4096, False), (4097, True)):
+        p = rng.integers(1, 99, size=(1, m)).astype(np.int64)
+
+        def swept(r, want=want, m=m):
+            assert (r[0] == m) == want
+        _check(pp, oracle_lib, _tree(rng, "chain", m), np.ones(m, np.int32), p, [m], swept)
