@@ -134,13 +134,13 @@ struct ReduceTables {
     struct Stream {
         int32_t tile, tiles;
     };
-    int CL = 0;
+    int CL = 0, max_kids = 0;
     std::vector<Slot> slot;
     std::vector<Stream> stream;
     std::vector<int32_t> lev, binlev, binslot, nacc;
 };
 struct ReduceShape {
-    int CL = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_acc = 0, acc_smem = 0;
+    int CL = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_acc = 0, acc_smem = 0, max_kids = 0;
 };
 
 struct Scratch {

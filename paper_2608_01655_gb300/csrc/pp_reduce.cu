@@ -36,9 +36,10 @@
 // log2(n) + 1 for every tree shape (6 to 9 on the prefix trees here, whose
 // depth is 72 and more).  Rows are laid out by (bin, level, path), bottom of
 // the path first, in tiles of 32 (one per warp step).  A bin is a set of
-// whole subtrees of at most n / (4 CL) rows, one bin per CTA of the cluster,
+// whole subtrees of at most n / (2 CL) rows, one bin per CTA of the cluster,
 // so that levels are separated by block barriers only; the few nodes above
-// all bins form a last bin that the first CTA walks after a cluster barrier.
+// all bins form a last bin that one warp of every CTA walks for itself, after
+// the cluster barrier that ends an evaluation.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -50,8 +51,9 @@ namespace pp {
 namespace {
 
 constexpr unsigned kAll = 0xffffffffu;
-constexpr int kThreads = 512;               // per CTA
+constexpr int kThreads = 1024;              // per CTA
 constexpr int kWarps = kThreads / 32;
+constexpr int kMaxLevels = 20;              // of a bin (heavy paths: log2 of its rows, plus one)
 constexpr int kMaxEvals = 16;               // prices tried per item
 constexpr int kPasses = 4;                  // thresholds tried per item
 constexpr int kRowCap = 1024;               // undecided rows the on-chip DP takes
@@ -62,8 +64,13 @@ constexpr int kKeyBase = (127 << 5) - 1;    // float bits >> 18 of 1.0, minus 1
 constexpr int kBins = 2048;                 // keys of 0 .. 2^62
 constexpr int kKeyPad = 0xffff;
 constexpr int64_t kBig = (int64_t)1 << 61;
-constexpr int kMaxWeight = (1 << 22);       // weights ride in the slot code
+constexpr int kMaxWeight = 1 << 22;         // weights ride in the slot code
 constexpr int kMaxPathRows = 4096;          // longer heavy paths are left to the sweep
+constexpr int kMaxKids = 65535;             // light children of a row: its 16-bit limbs add up in 32 bits
+constexpr int kMaxTop = 256;                // rows of the last bin (every CTA walks it)
+// the search's 32-bit units: the first price is 2^11 to 2^12 of them
+constexpr int kUnitBits = 11;
+constexpr int kClipRow = 1 << 24, kClipPath = 1 << 26, kClipPrice = 1 << 19;
 
 // slot code: bits 0-4 lanes to the left in the same path and tile, 5 the path
 // comes from the previous tile, 6 top of its path, 8.. weight
@@ -81,7 +88,7 @@ struct Tab {
 
 struct Scal {                    // per item, zeroed by the kernel
     unsigned long long maxp;
-    unsigned long long sumL[kMaxEvals];
+    unsigned long long sumL;
     unsigned long long sumZ[kMaxEvals];
     unsigned long long vfix[kPasses];
     unsigned long long wfix[kPasses];
@@ -100,23 +107,43 @@ struct Args {
     unsigned long long *rows_kept;
     DpWork w;
     size_t item_bytes;           // of w.red_scratch
-    int acc_smem;                // accumulators in shared memory
     int64_t total_weight;
     int32_t max_weight;
+    int32_t clip_kid;            // the search's bound on what a light child adds
 };
 
 __host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
+// Accumulators: what a row's light children add to it.  The search adds
+// 32-bit values and sizes; the exact evaluation adds four 16-bit limbs,
+// because shared memory adds 32-bit words natively and 64-bit ones in a
+// compare-and-swap loop.  Integer sums do not depend on the order of the
+// additions.  `down` is what the light children read on the way down.
+constexpr size_t kAccBytes = 8 + 16 + 8;
+struct Acc {
+    int4 *limb;
+    int2 *s;                     // search: value, size
+    float2 *down;                // lin, lout
+};
+__host__ __device__ inline Acc acc_at(char *base, size_t count)
+{
+    Acc a;
+    a.limb = (int4 *)base;
+    a.s = (int2 *)(base + count * 16);
+    a.down = (float2 *)(base + count * 24);
+    return a;
+}
+
 // one item's scratch
 struct Scratch1 {
     Scal *s;
-    unsigned *hist;              // [kBins]
+    unsigned *hist;              // [2][kBins] profits per slot (weights), losses (rows)
     int64_t *prof, *f;           // [nslots]
+    int *unit;                   // [nslots] profits in the search's units
     uint16_t *key;               // [nslots]
-    long long *topY, *topLin, *topLout;      // [ntop]
-    int *topZ;
-    long long *accY, *accLin, *accLout;      // [nslots] when not in shared memory
-    int *accZ;
+    int2 *tops;                  // [3][ntop] what the bins add to the last one: search (three prices in turn)
+    int4 *topl;                  // [ntop] exact evaluation
+    char *own;                   // accumulators of the bins when they are not in shared memory
 };
 __host__ __device__ inline size_t carve(char *base, int nslots, int ntop, bool acc_global, Scratch1 *o)
 {
@@ -128,19 +155,14 @@ __host__ __device__ inline size_t carve(char *base, int nslots, int ntop, bool a
     };
     Scratch1 x;
     x.s = (Scal *)take(sizeof(Scal));
-    x.hist = (unsigned *)take(kBins * 4);
-    x.topY = (long long *)take((size_t)ntop * 8);
-    x.topZ = (int *)take((size_t)ntop * 4);
-    x.topLin = (long long *)take((size_t)ntop * 8);
-    x.topLout = (long long *)take((size_t)ntop * 8);
+    x.hist = (unsigned *)take(2 * kBins * 4);
     x.prof = (int64_t *)take((size_t)nslots * 8);
     x.f = (int64_t *)take((size_t)nslots * 8);
+    x.unit = (int *)take((size_t)nslots * 4);
     x.key = (uint16_t *)take((size_t)nslots * 2);
-    const size_t na = acc_global ? (size_t)nslots : 0;
-    x.accY = (long long *)take(na * 8);
-    x.accZ = (int *)take(na * 4);
-    x.accLin = (long long *)take(na * 8);
-    x.accLout = (long long *)take(na * 8);
+    x.tops = (int2 *)take((size_t)ntop * 3 * 8);
+    x.topl = (int4 *)take((size_t)ntop * 16);
+    x.own = take(acc_global ? (size_t)(nslots + 32) * kAccBytes : 0);
     if (o) *o = x;
     return off;
 }
@@ -156,150 +178,382 @@ __device__ __forceinline__ int cluster_rank()
     return (int)r;
 }
 
-// order-preserving code of a loss >= 0, in [0, kBins)
-__device__ __forceinline__ int loss_key(int64_t loss)
+// order-preserving code of a value >= 0, in [0, kBins): 32 codes per octave
+__device__ __forceinline__ int code_of(int64_t v)
 {
-    if (loss <= 0) return 0;
-    return (int)(__float_as_uint(__ll2float_rd(loss)) >> 18) - kKeyBase;
+    if (v <= 0) return 0;
+    return (int)(__float_as_uint(__ll2float_rd(v)) >> 18) - kKeyBase;
+}
+__device__ __forceinline__ float code_edge(int code) { return __uint_as_float((unsigned)(code + kKeyBase) << 18); }
+
+
+__device__ __forceinline__ int64_t limbs(const int4 l)
+{
+    return (int64_t)((unsigned long long)(unsigned)l.x + ((unsigned long long)(unsigned)l.y << 16) +
+                     ((unsigned long long)(unsigned)l.z << 32) + ((unsigned long long)(unsigned)l.w << 48));
+}
+__device__ __forceinline__ void limb_add(int4 *a, int64_t v)
+{
+    int *l = (int *)a;
+    atomicAdd(l, (int)(v & 0xffff));
+    atomicAdd(l + 1, (int)((v >> 16) & 0xffff));
+    atomicAdd(l + 2, (int)((v >> 32) & 0xffff));
+    atomicAdd(l + 3, (int)(v >> 48));
+}
+__device__ __forceinline__ void pair_add(int2 *a, int y, int z)
+{
+    atomicAdd((int *)a, y);
+    atomicAdd((int *)a + 1, z);
+}
+// accumulators in global memory are added to in L2: read there
+template <bool GLOBAL, typename T>
+__device__ __forceinline__ T acc_ld(const T *p)
+{
+    if constexpr (GLOBAL) return __ldcg(p);
+    else return *p;
 }
 
-__device__ __forceinline__ int64_t sat(int64_t x) { return x < kBig ? x : kBig; }
+// The stream that this warp walks at level l of a bin: (first tile, tiles)
+__device__ __forceinline__ int2 stream_of(const Tab &t, int l0, int l)
+{
+    const int s = __ldg(t.lev + l0 + l) + (int)(threadIdx.x >> 5);
+    return s < __ldg(t.lev + l0 + l + 1) ? __ldg(t.stream + s) : make_int2(0, 0);
+}
 
-// f, and the values and sizes of the best closed sets, of one bin at price lam
-struct BinAcc {
-    volatile long long *y, *lin, *lout;
-    volatile int *z;
+// ---- one tile of the search: f, and the size of the best closed set below
+// (and with) every row, at a price of `lam` units; `out` the lanes with f <= 0
+struct STile {
+    int f, z;
+    unsigned out;
 };
+__device__ __forceinline__ STile search_tile(int code, int p, int2 kids, int lam, int &carryY, int &carryZ)
+{
+    const int lane = threadIdx.x & 31;
+    const int off = code & 31, w = code >> kWeightShift;
+    const int d = min(p - min(lam * min(w, 4095), kClipRow) + kids.x, kClipRow);
+    const bool cont = code & kCont;
+    const int cy = cont ? carryY : 0;
+    int ps = w + kids.y;
+    // inclusive scan of x -> max(m, s + x) along the path
+    int m = 0, sm = d;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int m2 = __shfl_up_sync(kAll, m, o), s2 = __shfl_up_sync(kAll, sm, o), p2 = __shfl_up_sync(kAll, ps, o);
+        if (off >= o) {
+            m = max(m, sm + m2);
+            sm += s2;
+        }
+        if (lane >= o) ps += p2;
+    }
+    const int y = min(max(m, sm + cy), kClipPath);
+    const int yp = __shfl_up_sync(kAll, y, 1);
+    STile r;
+    r.f = d + (off ? yp : cy);
+    r.out = __ballot_sync(kAll, r.f <= 0);
+    const unsigned neg = r.out & ((2u << lane) - (1u << (lane - off)));    // in this path, up to here
+    const int at = neg ? 31 - __clz((int)neg) : lane - off - 1;
+    const int pb = __shfl_sync(kAll, ps, at & 31);
+    r.z = ps - (at >= 0 ? pb : 0) + (!neg && cont ? carryZ : 0);
+    carryY = __shfl_sync(kAll, y, 31);
+    carryZ = __shfl_sync(kAll, r.z, 31);
+    return r;
+}
 
-__device__ void eval_bin(const Tab &t, int b, const Scratch1 &g, const BinAcc &own, const BinAcc &top, int64_t lam,
-                         int64_t &rootY, int &rootZ)
+// The search over a bin: levels from the leaves up, a block barrier between
+// them, the next tile's loads in flight while a tile is scanned (also across
+// levels).  A tile without a row of positive f has none at any higher price:
+// `live` holds the tiles (of the first 32 of a stream) still to be walked,
+// and `cand` what it becomes if this price turns out to be a lower bound.
+// own.s[na] stays zero (rows without light children read it).
+template <bool GLOBAL>
+__device__ __forceinline__ void search_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
+                                           int na, int2 *tops, int lam, int clip, unsigned *live, unsigned *cand,
+                                           bool use_cand, int &rootZ)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int l0 = t.binlev[b], l1 = t.binlev[b + 1] - 1;
-    for (int l = l0; l < l1; ++l) {
-        const int s1 = t.lev[l + 1];
-        for (int s = t.lev[l] + warp; s < s1; s += kWarps) {
-            const int2 st = t.stream[s];
-            int64_t carryY = 0;
-            int carryZ = 0;
-            for (int q = 0; q < st.y; ++q) {
-                const int slot = (st.x + q) * 32 + lane;
-                const int4 e = t.slot[slot];
-                const int off = e.y & 31, w = e.y >> kWeightShift;
-                const bool cont = e.y & kCont;
-                int64_t d = g.prof[slot] - lam * w;
-                int zz = w;
-                if (e.z >= 0) {
-                    d += own.y[e.z];
-                    zz += own.z[e.z];
-                    own.y[e.z] = 0;            // for the next price
-                    own.z[e.z] = 0;
-                }
-                // inclusive scan of x -> max(m, s + x) along the path
-                int64_t m = 0, sm = d;
-                int ps = zz;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int64_t m2 = __shfl_up_sync(kAll, m, o), s2 = __shfl_up_sync(kAll, sm, o);
-                    const int p2 = __shfl_up_sync(kAll, ps, o);
-                    if (off >= o) {
-                        const int64_t v = sm + m2;
-                        m = m > v ? m : v;
-                        sm += s2;
-                    }
-                    if (lane >= o) ps += p2;
-                }
-                const int64_t v = sm + (cont ? carryY : 0);
-                const int64_t y = m > v ? m : v;
-                int64_t yp = __shfl_up_sync(kAll, y, 1);
-                if (off == 0) yp = cont ? carryY : 0;
-                const int64_t f = d + yp;
-                g.f[slot] = f;
-                // size of the best closed set below (and with) this row
-                const bool in = f > 0;
-                const unsigned seg = (2u << lane) - (1u << (lane - off));
-                const unsigned neg = __ballot_sync(kAll, !in) & seg;
-                const int at = neg ? 31 - __clz((int)neg) : lane - off - 1;
-                const int pp = __shfl_sync(kAll, ps, at & 31);
-                int z = ps - (at >= 0 ? pp : 0);
-                if (!neg && cont) z += carryZ;
-                if ((e.y & kTop) && in) {
-                    if (e.w == -1) {
-                        rootY += f;
-                        rootZ += z;
-                    } else {
-                        const BinAcc &to = e.w >= 0 ? own : top;
-                        const int id = e.w >= 0 ? e.w : -2 - e.w;
-                        atomicAdd((unsigned long long *)(to.y + id), (unsigned long long)f);
-                        atomicAdd((int *)(to.z + id), z);
-                    }
-                }
-                carryY = __shfl_sync(kAll, y, 31);
-                carryZ = __shfl_sync(kAll, z, 31);
+    int2 st = make_int2(0, 0);
+    unsigned todo = 0, opened = 0;
+    int fl = -1, q = 0, late = 32;           // level and tile in flight; tiles past 32 are always walked
+    int4 e = make_int4(-1, 0, -1, -1);
+    int p = 0;
+    auto advance = [&] {                     // the next tile, its loads started
+        while (!todo && late >= st.y) {
+            if (++fl >= nlev) return;
+            const int i = fl * kWarps + warp;
+            st = strm[i];
+            late = 32;
+            todo = opened = use_cand ? cand[i] : live[i];
+            if (use_cand && lane == 0) live[i] = todo;
+        }
+        if (todo) {
+            q = __ffs((int)todo) - 1;
+            todo &= todo - 1;
+        } else {
+            q = late++;
+        }
+        const int slot = (st.x + q) * 32 + lane;
+        e = __ldg(t.slot + slot);
+        p = g.unit[slot];
+    };
+    advance();
+    for (int l = 0; l < nlev; ++l) {
+        int carryY = 0, carryZ = 0, prev = -1;
+        unsigned keep = fl == l ? opened : 0;
+        while (fl == l) {
+            const int4 c = e;
+            const int pc = p, at = q;
+            const int2 kids = acc_ld<GLOBAL>(own.s + (c.z < 0 ? na : c.z));
+            if (at != prev + 1) carryY = carryZ = 0;
+            prev = at;
+            advance();
+            const STile r = search_tile(c.y, pc, kids, lam, carryY, carryZ);
+            if (at < 32 && r.out == kAll) keep &= ~(1u << at);
+            if ((c.y & kTop) && r.f > 0) {
+                if (c.w >= 0) pair_add(own.s + c.w, min(r.f, clip), r.z);
+                else if (c.w == -1) rootZ += r.z;
+                else pair_add(tops - 2 - c.w, min(r.f, clip), r.z);
             }
         }
-        __syncthreads();
+        __syncwarp();                        // every lane has read its masks
+        if (lane == 0) cand[l * kWarps + warp] = keep;
+        if (l + 1 < nlev) __syncthreads();
     }
 }
 
-// losses of one bin, levels from the top down; keys to g.key, histogram in sh
-__device__ void loss_bin(const Tab &t, int b, const Scratch1 &g, const BinAcc &own, const BinAcc &top, unsigned *hist)
+// The last bin, by one warp (every CTA does it for itself): its tiles in
+// order; `loc`: what the bins have added, then its own paths.
+__device__ __forceinline__ int search_top(const Tab &t, const Scratch1 &g, const int2 *tops, int2 *loc, int lam, int clip)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(tops + i);
+    __syncwarp();
+    int rootZ = 0, carryY = 0, carryZ = 0;
+    const int s0 = t.binslot[t.CL];
+    int4 e = __ldg(t.slot + s0 + lane);
+    int p = __ldcg(g.unit + s0 + lane);
+    for (int s = s0; s < t.nslots; s += 32) {
+        const int4 c = e;
+        const int pc = p;
+        if (s + 32 < t.nslots) {
+            e = __ldg(t.slot + s + 32 + lane);
+            p = __ldcg(g.unit + s + 32 + lane);
+        }
+        int2 kids = make_int2(0, 0);
+        if (c.z >= 0) kids = loc[c.z];
+        const STile r = search_tile(c.y, pc, kids, lam, carryY, carryZ);
+        if ((c.y & kTop) && r.f > 0) {
+            if (c.w == -1) rootZ += r.z;
+            else pair_add(loc + c.w, min(r.f, clip), r.z);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rootZ += __shfl_xor_sync(kAll, rootZ, o);
+    return rootZ;
+}
+
+// ---- one tile of the exact evaluation at the price lam
+__device__ __forceinline__ int64_t exact_tile(const int4 c, int64_t p, int64_t kids, int64_t lam, int64_t &carryY)
+{
+    const int off = c.y & 31;
+    const bool cont = c.y & kCont;
+    const int64_t d = p - lam * (c.y >> kWeightShift) + kids;
+    int64_t m = 0, sm = d;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t m2 = __shfl_up_sync(kAll, m, o), s2 = __shfl_up_sync(kAll, sm, o);
+        if (off >= o) {
+            const int64_t v = sm + m2;
+            m = m > v ? m : v;
+            sm += s2;
+        }
+    }
+    const int64_t v = sm + (cont ? carryY : 0);
+    const int64_t y = m > v ? m : v;
+    int64_t yp = __shfl_up_sync(kAll, y, 1);
+    if (off == 0) yp = cont ? carryY : 0;
+    carryY = __shfl_sync(kAll, y, 31);
+    return d + yp;
+}
+
+// f of every row of a bin to g.f, the roots' share of L to rootY
+template <bool GLOBAL>
+__device__ __forceinline__ void exact_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
+                                          int64_t lam, int64_t &rootY)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int l0 = t.binlev[b], l1 = t.binlev[b + 1] - 1;
-    for (int l = l1 - 1; l >= l0; --l) {
-        const int s1 = t.lev[l + 1];
-        for (int s = t.lev[l] + warp; s < s1; s += kWarps) {
-            const int2 st = t.stream[s];
-            int64_t ca = 0, cb = kBig;
-            for (int q = st.y - 1; q >= 0; --q) {
-                const int slot = (st.x + q) * 32 + lane;
-                const int4 e = t.slot[slot];
-                const int64_t f = g.f[slot];
-                const unsigned starts = __ballot_sync(kAll, (e.y & 31) == 0);
-                const unsigned tops = __ballot_sync(kAll, (e.y & kTop) != 0);
-                const unsigned after = lane < 31 ? starts >> (lane + 1) : 0u;
-                const int rem = after ? __ffs((int)after) - 1 : 31 - lane;    // lanes to the right in this path
-                int64_t a = f < 0 ? sat(-f) : 0, bb = f;
-                if (e.y & kTop) {
-                    int64_t bl = 0, bo = kBig;
-                    if (e.w != -1) {
-                        const BinAcc &to = e.w >= 0 ? own : top;
-                        const int id = e.w >= 0 ? e.w : -2 - e.w;
-                        bl = to.lin[id];
-                        bo = to.lout[id];
-                    }
-                    a = sat(a + bl);
-                    bb = bb < bo ? bb : bo;
-                }
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int64_t a2 = __shfl_down_sync(kAll, a, o), b2 = __shfl_down_sync(kAll, bb, o);
-                    if (rem >= o) {
-                        a = sat(a + a2);
-                        bb = bb < b2 ? bb : b2;
-                    }
-                }
-                if (!((tops >> (lane + rem)) & 1u)) {       // the path goes on in the next tile
-                    a = sat(a + ca);
-                    bb = bb < cb ? bb : cb;
-                }
-                if (e.z >= 0) {
-                    own.lin[e.z] = a;
-                    own.lout[e.z] = bb;
-                }
-                int code = kKeyPad;
-                if (e.x >= 0) {
-                    const int k = loss_key(bb > 0 ? bb : a);
-                    code = k | (bb > 0 ? 0x8000 : 0);
-                    atomicAdd(hist + k, 1u);
-                }
-                g.key[slot] = (uint16_t)code;
-                ca = __shfl_sync(kAll, a, 0);
-                cb = __shfl_sync(kAll, bb, 0);
+    int2 st = make_int2(0, 0);
+    int fl = -1, q = 0;                      // level and tile in flight
+    int4 e = make_int4(-1, 0, -1, -1);
+    int64_t p = 0;
+    auto advance = [&] {
+        ++q;
+        while (q >= st.y) {
+            if (++fl >= nlev) return;
+            st = strm[fl * kWarps + warp];
+            q = 0;
+        }
+        const int slot = (st.x + q) * 32 + lane;
+        e = __ldg(t.slot + slot);
+        p = g.prof[slot];
+    };
+    advance();
+    for (int l = 0; l < nlev; ++l) {
+        int64_t carryY = 0;
+        while (fl == l) {
+            const int4 c = e;
+            const int64_t pc = p;
+            const int slot = (st.x + q) * 32 + lane;
+            advance();
+            const int64_t kids = c.z >= 0 ? limbs(acc_ld<GLOBAL>(own.limb + c.z)) : 0;
+            const int64_t f = exact_tile(c, pc, kids, lam, carryY);
+            g.f[slot] = f;
+            if ((c.y & kTop) && f > 0) {
+                if (c.w >= 0) limb_add(own.limb + c.w, f);
+                else if (c.w == -1) rootY += f;
+                else limb_add(g.topl - 2 - c.w, f);
             }
         }
-        __syncthreads();
+        if (l + 1 < nlev) __syncthreads();
+    }
+}
+// the last bin, by one warp of every CTA (they write the same f)
+__device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, int4 *loc, int64_t lam, int64_t *ftop)
+{
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(g.topl + i);
+    __syncwarp();
+    int64_t rootY = 0, carryY = 0;
+    const int s0 = t.binslot[t.CL];
+    int4 e = __ldg(t.slot + s0 + lane);
+    int64_t pn = __ldcg(g.prof + s0 + lane);
+    for (int s = s0; s < t.nslots; s += 32) {
+        const int4 c = e;
+        const int64_t p = pn;
+        if (s + 32 < t.nslots) {
+            e = __ldg(t.slot + s + 32 + lane);
+            pn = __ldcg(g.prof + s + 32 + lane);
+        }
+        const int64_t kids = c.z >= 0 ? limbs(loc[c.z]) : 0;
+        const int64_t f = exact_tile(c, p, kids, lam, carryY);
+        ftop[s - s0 + lane] = f;
+        if ((c.y & kTop) && f > 0) {
+            if (c.w == -1) rootY += f;
+            else limb_add(loc + c.w, f);
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rootY += __shfl_xor_sync(kAll, rootY, o);
+    return rootY;
+}
+
+// ---- one tile of the losses, from the top of a path down: `a` the sum of
+// max(0, -f) over the path from the root, `b` the smallest f on it.  In
+// floats rounded down: a loss is only ever underestimated, which keeps rows.
+__device__ __forceinline__ void loss_tile(const int4 c, int64_t f, float2 up, float &ca, float &cb, float &a, float &b)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned starts = __ballot_sync(kAll, (c.y & 31) == 0);
+    const unsigned tops = __ballot_sync(kAll, (c.y & kTop) != 0);
+    const unsigned after = lane < 31 ? starts >> (lane + 1) : 0u;
+    const int rem = after ? __ffs((int)after) - 1 : 31 - lane;    // lanes to the right in this path
+    b = __ll2float_rd(f);
+    a = f < 0 ? __ll2float_rd(-f) : 0.f;
+    if ((c.y & kTop) && c.w != -1) {
+        a = __fadd_rd(a, up.x);
+        b = fminf(b, up.y);
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float a2 = __shfl_down_sync(kAll, a, o), b2 = __shfl_down_sync(kAll, b, o);
+        if (rem >= o) {
+            a = __fadd_rd(a, a2);
+            b = fminf(b, b2);
+        }
+    }
+    if (!((tops >> (lane + rem)) & 1u)) {       // the path goes on in the next tile
+        a = __fadd_rd(a, ca);
+        b = fminf(b, cb);
+    }
+    ca = __shfl_sync(kAll, a, 0);
+    cb = __shfl_sync(kAll, b, 0);
+}
+// key of a row (15 bits) and whether it is in S (bit 15)
+__device__ __forceinline__ int loss_code(float a, float b)
+{
+    const float v = b > 0.f ? b : a;
+    const int k = v < 1.f ? 0 : min((int)(__float_as_uint(v) >> 18) - kKeyBase, kBins - 1);
+    return k | (b > 0.f ? 0x8000 : 0);
+}
+
+// losses of one bin, levels from the top down; keys to g.key, histogram in sh
+template <bool GLOBAL>
+__device__ __forceinline__ void loss_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
+                                         const float2 *topd, unsigned *hist)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int2 st = make_int2(0, 0);
+    int fl = nlev, q = 0;
+    int4 e = make_int4(-1, 0, -1, -1);
+    int64_t f = 0;
+    auto advance = [&] {
+        --q;
+        while (q < 0) {
+            if (--fl < 0) return;
+            st = strm[fl * kWarps + warp];
+            q = st.y - 1;
+        }
+        const int slot = (st.x + q) * 32 + lane;
+        e = __ldg(t.slot + slot);
+        f = g.f[slot];
+    };
+    advance();
+    for (int l = nlev - 1; l >= 0; --l) {
+        float ca = 0.f, cb = 0.f;
+        while (fl == l) {
+            const int4 c = e;
+            const int64_t fc = f;
+            const int slot = (st.x + q) * 32 + lane;
+            advance();
+            float2 up = make_float2(0.f, 0.f);
+            if ((c.y & kTop) && c.w != -1) up = c.w >= 0 ? acc_ld<GLOBAL>(own.down + c.w) : topd[-2 - c.w];
+            float a, b;
+            loss_tile(c, fc, up, ca, cb, a, b);
+            if (c.z >= 0) own.down[c.z] = make_float2(a, b);
+            int code = kKeyPad;
+            if (c.x >= 0) {
+                code = loss_code(a, b);
+                atomicAdd(hist + (code & 0x7fff), 1u);
+            }
+            g.key[slot] = (uint16_t)code;
+        }
+        if (l > 0) __syncthreads();
+    }
+}
+// the last bin, by one warp; one CTA (`write`) keeps its keys
+__device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, const int64_t *ftop, float2 *topd, unsigned *hist,
+                                         bool write)
+{
+    const int lane = threadIdx.x & 31;
+    float ca = 0.f, cb = 0.f;
+    const int s0 = t.binslot[t.CL];
+    for (int s = t.nslots - 32; s >= s0; s -= 32) {
+        const int4 c = __ldg(t.slot + s + lane);
+        float2 up = make_float2(0.f, 0.f);
+        if ((c.y & kTop) && c.w >= 0) up = topd[c.w];
+        float a, b;
+        loss_tile(c, ftop[s - s0 + lane], up, ca, cb, a, b);
+        if (c.z >= 0) topd[c.z] = make_float2(a, b);
+        if (write) {
+            int code = kKeyPad;
+            if (c.x >= 0) {
+                code = loss_code(a, b);
+                atomicAdd(hist + (code & 0x7fff), 1u);
+            }
+            g.key[s + lane] = (uint16_t)code;
+        }
+        __syncwarp();
     }
 }
 
@@ -315,74 +569,204 @@ __device__ int block_scan(int v, int *total, int *sh)
     }
     if (lane == 31) sh[wid] = x;
     __syncthreads();
-    int before = 0, tot = 0;
+    int w = lane < kWarps ? sh[lane] : 0;    // every warp scans the warps' totals
+    const int mine = w;
 #pragma unroll
-    for (int i = 0; i < kWarps; ++i) {
-        before += i < wid ? sh[i] : 0;
-        tot += sh[i];
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, w, o);
+        if (lane >= o) w += y;
     }
-    *total = tot;
+    *total = __shfl_sync(kAll, w, 31);
+    const int before = __shfl_sync(kAll, w - mine, wid);
     __syncthreads();
     return before + x - v;
 }
 
-// what the price search knows: a price with |S| > k and one with |S| <= k
-struct Bracket {
-    double x0, y0, z0, x1, y1, z1;
+// ---------------------------------------------------------------------------
+// The price.  |S| falls with the price; the one wanted is where it passes k.
+// Its first guess is the k-th largest profit per slot (chunks taken without
+// their prefixes: within ~15% on the prefix trees here), the second scales
+// that curve through the first point, then the bracket is closed by
+// interpolating logarithms (|S| falls like a power).  3 to 6 prices; a search
+// from price 0 by the tangents of L took 9 to 10.
+// ---------------------------------------------------------------------------
+enum : int { kGo = 0, kStop = 1, kSlack = 2 };
+
+struct Search {                              // prices in units
+    float x0, x1, z0, z1;                    // price and |S| of the ends with |S| > k and <= k
+    int have, side;                          // bit 0, 1: that end is there; steps in a row to one side
 };
 
-enum : int { kGo = 0, kStop = 1, kBack = 2, kSlack = 3 };
+// weight of the rows worth at least lam per slot, and its inverse (cum[c]:
+// weight of the codes >= c)
+__device__ float rank_at(const int *cum, float lam)
+{
+    const int c = lam < 1.f ? 0 : min((int)(__float_as_uint(lam) >> 18) - kKeyBase, kBins - 1);
+    const float lo = code_edge(c), hi = code_edge(c + 1);
+    const int n0 = cum[c], n1 = c + 1 < kBins ? cum[c + 1] : 0;
+    return n0 - (n0 - n1) * ((lam - lo) / (hi - lo));
+}
+__device__ float price_of_rank(const int *cum, float rank)
+{
+    int a = 1, b = kBins;                    // the last code with cum >= rank
+    while (b - a > 1) {
+        const int m = (a + b) >> 1;
+        if (cum[m] >= rank) a = m;
+        else b = m;
+    }
+    const float lo = code_edge(a), hi = code_edge(a + 1);
+    const int n0 = cum[a], n1 = a + 1 < kBins ? cum[a + 1] : 0;
+    float fr = n0 > n1 ? (n0 - rank) / (n0 - n1) : 0.f;
+    fr = fminf(fmaxf(fr, 0.f), 1.f);
+    return lo + (hi - lo) * fr;
+}
 
-// what to do after the price lam gave L and |S| = Z: try `nx` (kGo), stop
-// here (kStop), or go back to the better end of the bracket `nx` (kBack)
-__device__ int next_price(Bracket &b, double k, int evals, int64_t lam, double L, double Z, int64_t &nx_out)
+// what to do after the price `lam` (units of 2^shift) gave |S| = Z: try `nx`
+// (kGo), stop and use `nx` (kStop), or the budget does not bind (kSlack)
+__device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int lam, float Z, int &nx)
 {
     if (Z > k) {
-        b.x0 = (double)lam;
-        b.y0 = L;
+        b.x0 = (float)lam;
         b.z0 = Z;
+        b.side = b.side > 0 ? b.side + 1 : 1;
+        b.have |= 1;
     } else {
-        b.x1 = (double)lam;
-        b.y1 = L;
+        if (lam == 0) return kSlack;
+        b.x1 = (float)lam;
         b.z1 = Z;
+        b.side = b.side < 0 ? b.side - 1 : -1;
+        b.have |= 2;
     }
-    // L is convex in the price: its minimum lies above the crossing of the
-    // two tangents, so L - y bounds what a better price could still give
-    const double x = ((b.y0 - (k - b.z0) * b.x0) - (b.y1 - (k - b.z1) * b.x1)) / (b.z0 - b.z1);
-    const double y = b.y0 + (k - b.z0) * (x - b.x0);
-    const double best = b.y0 < b.y1 ? b.y0 : b.y1;
-    if (evals > 1 && (best - y <= 0.03 * x || b.x1 - b.x0 <= 1.0 || evals >= kMaxEvals - 1)) {
-        nx_out = (int64_t)(b.y0 < b.y1 ? b.x0 : b.x1);
-        return nx_out == lam ? kStop : kBack;
+    if ((Z - k) * (Z - k) <= 0.05f * k) {    // |S| is so near k that L is flat
+        nx = lam;
+        return kStop;
     }
-    double nx = x;
-    if (b.x0 > 0 && b.z1 > 0 && evals <= 5) {
-        // |S| falls roughly like a power of the price: interpolate the logarithms
-        const float s = __log2f((float)(b.z0 / k)) / __log2f((float)(b.z0 / b.z1));
-        nx = b.x0 * (double)exp2f(__log2f((float)(b.x1 / b.x0)) * s);
+    float x;
+    if (b.have == 3) {
+        // L's slope is k - |S|, so these bound what a better price could still give
+        const float d = b.x1 - b.x0, e0 = (b.z0 - k) * d, e1 = (k - b.z1) * d;
+        if (fminf(e0, e1) <= 0.1f * b.x0 || d <= 1.f || evals >= kMaxEvals) {
+            nx = (int)(e0 < e1 ? b.x0 : b.x1);
+            return kStop;
+        }
+        if (b.x0 > 0.f) {
+            float s = __log2f(b.z0 / k) / __log2f(b.z0 / fmaxf(b.z1, 1.f));
+            if (b.side >= 2 || b.side <= -2) s = 0.5f * s + 0.25f;      // creeping from one side
+            if (evals > 5) s = fminf(fmaxf(s, 0.2f), 0.8f);
+            x = b.x0 * exp2f(__log2f(b.x1 / b.x0) * s);
+        } else {
+            x = 0.5f * b.x1;
+        }
+        x = fminf(fmaxf(x, b.x0 + 1.f), b.x1 - 1.f);
+    } else {
+        if (evals >= kMaxEvals) {
+            nx = lam;
+            return kStop;
+        }
+        const bool above = Z > k;            // the price has to rise
+        const float l1 = fmaxf((float)lam, 1.f), c = rank_at(cum, l1 * unit);
+        if (Z > 0.f && c > 0.f && evals < 6) {
+            x = price_of_rank(cum, k * c / Z) / unit;
+            x = above ? fmaxf(x, l1) * 1.01f : fminf(x, l1) * 0.99f;
+            if (evals > 2) x *= above ? 1.3f : 0.7f;
+        } else {
+            x = above ? (float)maxlam : 0.f;
+        }
+        x = above ? fmaxf(x, b.x0 + 1.f) : fminf(x, b.x1 - 1.f);
     }
-    nx = nx < b.x0 + 1.0 ? b.x0 + 1.0 : nx;
-    nx = nx > b.x1 - 1.0 ? b.x1 - 1.0 : nx;
-    nx_out = (int64_t)nx > 0 ? (int64_t)nx : 1;
+    nx = min(max((int)x, 0), maxlam);
     return kGo;
 }
 
-struct Rows {                                // undecided rows, in sweep order (last position first)
-    int pos[kRowCap], w[kRowCap], skip[kRowCap], info[kRowCap], last[kRowCap];
-    int64_t p[kRowCap];
+// ---------------------------------------------------------------------------
+// Eq. 9 over the undecided rows, in shared memory
+// ---------------------------------------------------------------------------
+struct __align__(16) Row {
+    int64_t p;
+    int w, info;                             // flags below, stack level << 8
 };
-constexpr int kPush = 1, kReload = 2, kZeroTop = 4, kFromCur = 8;      // info flags, level << 8
+struct Rows {                                // in sweep order (last position first)
+    Row row[kRowCap + 1];
+    int pos[kRowCap], skip[kRowCap], last[kRowCap];
+    unsigned leaf[kRowCap / 32];             // bit: skip[r] = r - 1
+};
+constexpr int kPush = 1, kReload = 2, kZeroTop = 4, kFromCur = 8;
+
+// `act` warps, C columns per thread (column j = 1 + thread + c * threads).
+// The row just computed goes through shared memory (any weight is then one
+// load at j - w; `guard` words left of column 0 read as never worth taking),
+// a row's own scalars are loaded one row ahead, and decision bits are packed
+// per thread over 32 rows.
+template <int C>
+__device__ __forceinline__ void dp_rows(const Rows &R, int T, int act, int guard, int64_t *rowb, int64_t *stk,
+                                        uint32_t *bits, int64_t *result, int kc)
+{
+    const int tid = threadIdx.x, nt = act * 32, cols = nt * C, pitch = cols + 1 + guard;
+    int64_t cur[C], top[C];
+    uint32_t wb[C];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        cur[c] = top[c] = 0;
+        wb[c] = 0;
+    }
+    const int64_t *prev = rowb + guard;
+    int64_t *out = rowb + pitch + guard;
+    Row nx = R.row[0];
+    for (int r = 0; r < T; ++r) {
+        const Row x = nx;
+        nx = R.row[r + 1];
+        int64_t in[C];                       // all loads before any store
+#pragma unroll
+        for (int c = 0; c < C; ++c) in[c] = prev[1 + tid - x.w + c * nt];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int64_t sk = (x.info & kFromCur) ? cur[c] : top[c];
+            const int64_t tv = x.p + in[c];
+            const bool take = tv > sk;
+            cur[c] = take ? tv : sk;
+            out[1 + tid + c * nt] = cur[c];
+            if (take) wb[c] |= 1u << (r & 31);
+        }
+        if (x.info & (kPush | kReload | kZeroTop)) {
+            int64_t *sl = stk + (x.info >> 8) * cols + tid;
+            if (x.info & kPush) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) sl[c * nt] = top[c] = cur[c];
+            } else {
+#pragma unroll
+                for (int c = 0; c < C; ++c) top[c] = (x.info & kReload) ? sl[c * nt] : 0;
+            }
+        }
+        if ((r & 31) == 31 || r == T - 1) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                bits[(r >> 5) * cols + tid + c * nt] = wb[c];
+                wb[c] = 0;
+            }
+        }
+        if (act == 1) __syncwarp();
+        else asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+        const int64_t *sw = prev;
+        prev = out;
+        out = const_cast<int64_t *>(sw);
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+        if (kc == 1 + tid + c * nt) *result = cur[c];
+}
 
 }  // namespace
 
+template <bool SMEM>                         // accumulators of the bins in shared memory
 __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int2 strm[kMaxLevels * kWarps];
+    __shared__ unsigned live[kMaxLevels * kWarps], cand[kMaxLevels * kWarps];
+    __shared__ int4 s_top[kMaxTop];          // the last bin's own sums, then what it passes down
     __shared__ int sh[kWarps];
-    __shared__ long long shL[kWarps];
-    __shared__ int64_t s_lam;
-    __shared__ int s_key, s_flag, s_T;
-    __shared__ long long s_val;
+    __shared__ int s_a, s_b, s_flag, s_lam;
+    __shared__ int64_t s_val;
     const Tab &t = A.t;
     const int CL = t.CL, cr = CL > 1 ? cluster_rank() : 0;
     const int item = blockIdx.x / CL;
@@ -396,45 +780,11 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     }
     const int64_t k = kreq < A.total_weight ? kreq : A.total_weight;     // more changes nothing
     Scratch1 g;
-    carve(A.w.red_scratch + (size_t)item * A.item_bytes, t.nslots, t.ntop, !A.acc_smem, &g);
+    carve(A.w.red_scratch + (size_t)item * A.item_bytes, t.nslots, t.ntop, !SMEM, &g);
     const int words = (n + 31) / 32;
     uint32_t *taken = A.w.taken + (size_t)item * words, *freeb = A.w.undecided + (size_t)item * words;
     const int64_t *P = A.profit + (size_t)item * n;
-
-    // accumulators of this CTA's bin
-    BinAcc own, top;
-    const int na = t.nacc[cr];
-    if (A.acc_smem) {
-        own.y = (long long *)smem;
-        own.lin = own.y + na;
-        own.lout = own.lin + na;
-        own.z = (int *)(own.lout + na);
-    } else {
-        const int s0 = t.binslot[cr];
-        own.y = g.accY + s0;
-        own.lin = g.accLin + s0;
-        own.lout = g.accLout + s0;
-        own.z = g.accZ + s0;
-    }
-    top.y = g.topY;
-    top.lin = g.topLin;
-    top.lout = g.topLout;
-    top.z = g.topZ;
-
-    // ---- gather the profits, clear what is added to
-    for (int i = tid; i < na; i += kThreads) {
-        own.y[i] = 0;
-        own.z[i] = 0;
-    }
-    if (cr == 0) {
-        for (int i = tid; i < t.ntop; i += kThreads) {
-            top.y[i] = 0;
-            top.z[i] = 0;
-        }
-        for (int i = tid; i < (int)(sizeof(Scal) / 8); i += kThreads) ((unsigned long long *)g.s)[i] = 0;
-        for (int i = tid; i < kBins; i += kThreads) g.hist[i] = 0;
-    }
-    for (int i = cr * kThreads + tid; i < words; i += CL * kThreads) taken[i] = 0;
+    for (int i = cr * kThreads + tid; i < words; i += CL * kThreads) taken[i] = freeb[i] = 0;
     if (k == 0) {                            // nothing fits
         if (cr == 0 && tid == 0) {
             A.best[item] = 0;
@@ -443,172 +793,249 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         }
         return;
     }
-    const bool has_top = t.ntop > 0 || t.binslot[CL] < t.nslots;
+    const int na = t.nacc[cr];
+    const int lo = t.binslot[cr], hi = t.binslot[cr + 1];
+    const Acc own = acc_at(SMEM ? (char *)smem : g.own + (size_t)(lo + cr) * kAccBytes, na + 1);   // (one reads as zero)
+    unsigned *hist = (unsigned *)(smem + (SMEM ? up16((size_t)(na + 1) * kAccBytes) : 0));
+    const bool has_top = t.binslot[CL] < t.nslots;
+    const int l0 = t.binlev[cr], nlev = t.binlev[cr + 1] - 1 - l0;
+    const int top0 = t.binslot[CL];
+    auto sync_all = [&] {
+        if (CL > 1) cluster_sync();
+        else __syncthreads();
+    };
+
+    // ---- clear what is added to; this bin's streams
+    if (cr == 0) {
+        for (int i = tid; i < (int)(sizeof(Scal) / 8); i += kThreads) ((unsigned long long *)g.s)[i] = 0;
+        for (int i = tid; i < 2 * kBins; i += kThreads) g.hist[i] = 0;
+        for (int i = tid; i < 3 * t.ntop; i += kThreads) g.tops[i] = make_int2(0, 0);
+        for (int i = tid; i < t.ntop; i += kThreads) g.topl[i] = make_int4(0, 0, 0, 0);
+    }
+    for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+    for (int l = 0; l < nlev; ++l) {
+        const int2 x = stream_of(t, l0, l);
+        if (lane == 0) {
+            strm[l * kWarps + warp] = x;
+            live[l * kWarps + warp] = x.y >= 32 ? kAll : (1u << x.y) - 1;
+        }
+    }
+    sync_all();
+
+    // ---- gather the profits into the slots; weights by profit per slot
+    // (from every tile up to 16,384 slots, then from a sample of the tiles)
     int64_t mx = 0;
-    auto gather = [&](int lo, int hi) {
-        for (int s = lo + tid; s < hi; s += kThreads) {
-            const int x = t.slot[s].x;
-            const int64_t p = x >= 0 ? P[A.order ? A.order[x] : x] : 0;
-            g.prof[s] = p;
-            mx = p > mx ? p : mx;
+    const int every = t.nslots > 16384 ? 31 - __clz(t.nslots >> 13) : 0;
+    auto gather = [&](int from, int to) {
+        constexpr int U = 4;                 // loads in flight per thread
+        for (int s0 = from + tid; s0 < to; s0 += U * kThreads) {
+            int4 e[U];
+            int64_t p[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                e[u] = s0 + u * kThreads < to ? __ldg(t.slot + s0 + u * kThreads) : make_int4(-1, 0, -1, -1);
+            if (A.order)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (e[u].x >= 0) e[u].x = __ldg(A.order + e[u].x);
+#pragma unroll
+            for (int u = 0; u < U; ++u) p[u] = e[u].x >= 0 ? P[e[u].x] : 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int s = s0 + u * kThreads;
+                if (s >= to) break;
+                g.prof[s] = p[u];
+                mx = p[u] > mx ? p[u] : mx;
+                if (p[u] > 0 && ((s >> 5) & ((1 << every) - 1)) == 0) {
+                    const int w = e[u].y >> kWeightShift;
+                    const int c = w == 1 ? code_of(p[u]) : code_of((int64_t)((float)p[u] / (float)w));
+                    atomicAdd(hist + c, (unsigned)w << every);
+                }
+            }
         }
     };
-    const int lo = t.binslot[cr], hi = t.binslot[cr + 1];
     gather(lo, hi);
     if (cr == 0 && has_top) gather(t.binslot[CL], t.nslots);
-    if (CL > 1) cluster_sync();              // the scalars are clear
-    else __syncthreads();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const int64_t y = __shfl_xor_sync(kAll, mx, o);
         mx = y > mx ? y : mx;
     }
     if (lane == 0 && mx > 0) atomicMax(&g.s->maxp, (unsigned long long)mx);
-    auto sync_all = [&] {
-        if (CL > 1) cluster_sync();
-        else __syncthreads();
-    };
+    __syncthreads();
+    for (int i = tid; i < kBins; i += kThreads)
+        if (hist[i]) atomicAdd(g.hist + i, hist[i]);
     sync_all();
-    const int64_t maxp = (int64_t) * (volatile unsigned long long *)&g.s->maxp;
-
-    // ---- the price: |S| <= k at price 0 means that the budget does not bind
-    int64_t lam = 0, L = 0;
-    bool slack = false, give_up = maxp > kBig / (k > A.max_weight ? k : A.max_weight);
-    Bracket br;
-    br.x1 = (double)maxp;
-    br.y1 = (double)maxp * (double)k;
-    br.z1 = 0;
-    br.x0 = br.y0 = br.z0 = 0;
-    // one price: f of every row to g.f, the sums over the roots to slot `ev`
-    auto evaluate = [&](int ev) {
-        int64_t ry = 0;
-        int rz = 0;
-        eval_bin(t, cr, g, own, top, lam, ry, rz);
-        if (has_top) {
-            sync_all();
-            if (cr == 0) eval_bin(t, CL, g, top, top, lam, ry, rz);
-        }
+    const int64_t maxp = (int64_t)__ldcg(&g.s->maxp);
+    int *cum = (int *)hist;                  // weight of the codes >= c
+    {
+        constexpr int V = kBins / kThreads;
+        int c[V], sum = 0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ry += __shfl_xor_sync(kAll, ry, o);
-            rz += __shfl_xor_sync(kAll, rz, o);
+        for (int v = V - 1; v >= 0; --v) {
+            c[v] = sum;                      // of the codes above, in this thread's run
+            sum += (int)__ldcg(g.hist + tid * V + v);
         }
-        if (lane == 0) {
-            shL[warp] = ry;
-            sh[warp] = rz;
+        int tot;
+        const int before = block_scan(sum, &tot, sh);
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            const int mine = (int)__ldcg(g.hist + tid * V + v);
+            cum[tid * V + v] = tot - before - sum + c[v] + mine;
         }
         __syncthreads();
-        if (tid == 0) {
-            unsigned long long a = 0, z = 0;
-            for (int i = 0; i < kWarps; ++i) {
-                a += (unsigned long long)shL[i];
-                z += (unsigned long long)sh[i];
+    }
+
+    // ---- the price
+    const bool give_up = maxp > kBig / (k > A.max_weight ? k : A.max_weight);
+    int64_t lam = 0, L = 0;
+    if (!give_up) {
+        const float guess = cum[0] <= k ? 0.f : fminf(fmaxf(price_of_rank(cum, (float)k), 1.f), (float)maxp);
+        const int shift = max(0, (int)(__float_as_uint(fmaxf(guess, 1.f)) >> 23) - 127 - kUnitBits);
+        const int maxlam = (int)min((maxp >> shift) + 1, (int64_t)kClipPrice);
+        int price = (int)(guess * exp2f((float)-shift));
+        Search sr;
+        sr.have = sr.side = 0;
+        sr.x0 = sr.x1 = sr.z0 = sr.z1 = 0.f;
+        auto to_units = [&](int from, int to) {
+            for (int s = from + tid; s < to; s += kThreads) {
+                const int64_t p = g.prof[s] >> shift;
+                g.unit[s] = (int)(p > kClipRow ? kClipRow : p < -kClipRow ? -kClipRow : p);
             }
-            if (a) atomicAdd(&g.s->sumL[ev], a);
-            if (z) atomicAdd(&g.s->sumZ[ev], z);
+        };
+        to_units(lo, hi);
+        if (cr == 0 && has_top) to_units(top0, t.nslots);
+        bool low = false;                    // the last price was a lower bound
+        for (int ev = 0;; ++ev) {
+            for (int i = tid; i <= na; i += kThreads) own.s[i] = make_int2(0, 0);
+            // (the set that the last price but one's sums were read from)
+            if (cr == 0)
+                for (int i = tid; i < t.ntop; i += kThreads) g.tops[(ev + 1) % 3 * t.ntop + i] = make_int2(0, 0);
+            int2 *tops = g.tops + ev % 3 * t.ntop;
+            int rz = 0;
+            __syncthreads();
+            search_bin<!SMEM>(t, strm, nlev, g, own, na, tops, price, A.clip_kid, live, cand, low, rz);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(kAll, rz, o);
+            if (lane == 0 && rz) atomicAdd(&g.s->sumZ[ev], (unsigned long long)rz);
+            sync_all();
+            if (warp == 0) {
+                int z = has_top ? search_top(t, g, tops, (int2 *)s_top, price, A.clip_kid) : 0;
+                if (lane == 0) {
+                    z += (int)__ldcg(&g.s->sumZ[ev]);
+                    int nx = price;
+                    s_flag = next_price(sr, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
+                    s_lam = nx;
+                    s_a = z > k;
+                }
+            }
+            __syncthreads();
+            price = s_lam;
+            low = s_a;
+            if (s_flag != kGo) break;
+            __syncthreads();
         }
+        if (s_flag == kSlack) price = 0;
+        lam = (int64_t)price << shift;
+        // ---- exactly there: f of every row, L
+        for (int i = tid; i < na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
+        __syncthreads();
+        int64_t ry = 0;
+        exact_bin<!SMEM>(t, strm, nlev, g, own, lam, ry);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ry += __shfl_xor_sync(kAll, ry, o);
+        if (lane == 0 && ry) atomicAdd(&g.s->sumL, (unsigned long long)ry);
         sync_all();
-    };
-    for (int ev = 0; !give_up; ++ev) {
-        evaluate(ev);
-        if (tid == 0) {
-            const int64_t sl = (int64_t) * (volatile unsigned long long *)&g.s->sumL[ev] + lam * k;
-            const int64_t sz = (int64_t) * (volatile unsigned long long *)&g.s->sumZ[ev];
-            int64_t nx = 0;
-            s_flag = lam == 0 && sz <= k ? kSlack : next_price(br, (double)k, ev + 1, lam, (double)sl, (double)sz, nx);
-            s_val = sl;
-            s_lam = nx;
+        if (warp == 0) {
+            ry = has_top ? exact_top(t, g, s_top, lam, g.f + top0) : 0;
+            if (lane == 0) s_val = (int64_t)__ldcg(&g.s->sumL) + ry + lam * k;
         }
         __syncthreads();
         L = s_val;
-        const int todo = s_flag;
-        if (todo == kGo || todo == kBack) lam = s_lam;
-        __syncthreads();
-        if (todo == kGo) continue;           // (never at the last but one slot: next_price stops there)
-        slack = todo == kSlack;
-        if (todo == kBack) {
-            evaluate(kMaxEvals - 1);
-            L = (int64_t) * (volatile unsigned long long *)&g.s->sumL[kMaxEvals - 1] + lam * k;
-        }
-        break;
     }
 
     // ---- losses and their histogram
-    unsigned *hist = (unsigned *)(smem + (A.acc_smem ? up16((size_t)na * 28) : 0));
+    unsigned *ghist = g.hist + kBins;
     if (!give_up) {
         for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
         __syncthreads();
         if (has_top) {
-            if (cr == 0) loss_bin(t, CL, g, top, top, hist);
-            sync_all();
+            if (warp == 0) loss_top(t, g, g.f + top0, (float2 *)s_top, hist, cr == 0);
+            __syncthreads();
         }
-        loss_bin(t, cr, g, own, top, hist);
+        loss_bin<!SMEM>(t, strm, nlev, g, own, (const float2 *)s_top, hist);
+        __syncthreads();
         for (int i = tid; i < kBins; i += kThreads)
-            if (hist[i]) atomicAdd(g.hist + i, hist[i]);
+            if (hist[i]) atomicAdd(ghist + i, hist[i]);
         sync_all();
     }
-    // largest key whose rows, and all below, are at most `rows` (but at least key 0)
-    auto key_of_rank = [&](int rows) {
+    // the largest key up to `most` whose rows, and all below, are at most
+    // `rows` (but at least key 0), and their number
+    auto up_to = [&](int rows, int most, int &key_out) {
         constexpr int V = kBins / kThreads;
         int c[V], sum = 0;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
-            c[v] = (int)*(volatile unsigned *)(g.hist + tid * V + v);
+            c[v] = (int)__ldcg(ghist + tid * V + v);
             sum += c[v];
         }
+        if (tid == 0) s_a = s_b = 0;
         int tot;
-        int ex = block_scan(sum, &tot, sh);
-        if (tid == 0) s_key = 0;
-        __syncthreads();
-        int last = -1;
+        int ex = block_scan(sum, &tot, sh);              // (orders the line above too)
+        int last = -1, cnt = 0;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             ex += c[v];
-            if (ex <= rows) last = tid * V + v;
+            const int q = tid * V + v;
+            if (q == 0 || (q <= most && ex <= rows)) {
+                last = q;
+                cnt = ex;
+            }
         }
-        if (last > 0) atomicMax(&s_key, last);
+        if (last >= 0) {
+            atomicMax(&s_a, last);
+            atomicMax(&s_b, cnt);
+        }
         __syncthreads();
-        const int r = s_key;
+        key_out = s_a;
+        const int r = s_b;
         __syncthreads();
         return r;
     };
-    auto rows_up_to = [&](int key) {
-        constexpr int V = kBins / kThreads;
-        int sum = 0;
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-            if (tid * V + v <= key) sum += (int)*(volatile unsigned *)(g.hist + tid * V + v);
-        int tot;
-        block_scan(sum, &tot, sh);
-        return tot;
-    };
 
-    int verdict = 3, key = 0, pass = 0;
+    int verdict = 3, key = 0, pass = 0, vkey = -1;      // vkey: the smallest sure key so far (first CTA)
     bool sure = false;           // the key comes from a V: no row above it is undecided
     if (!give_up) {
-        key = slack ? -1 : key_of_rank(kFirstRows);
-        for (pass = 0; pass < kPasses; ++pass) {
-            const int T = key < 0 ? 0 : rows_up_to(key);
+        int T = 0;
+        // first the rows whose loss is within a tenth of a slot's price (most
+        // gaps are), at most kFirstRows; none at price 0 (see kleft < 0 below)
+        if (lam == 0) {
+            key = -1;
+        } else {
+            T = up_to(kFirstRows, code_of(lam / 10), key);
+        }
+        for (; pass < kPasses; ++pass) {
             const bool big = T > kRowCap;                         // the same in every CTA
-            if (big && !sure) {
-                verdict = 3;
-                break;
-            }
+            verdict = 3;
+            if (big && !sure) break;
             // ---- decided rows: value and weight of those in; the others' positions
-            for (int i = cr * kThreads + tid; i < words; i += CL * kThreads) freeb[i] = 0;
-            sync_all();
+            if (pass > 0) {
+                for (int i = cr * kThreads + tid; i < words; i += CL * kThreads) freeb[i] = 0;
+                sync_all();
+            }
             unsigned long long vf = 0, wf = 0;
             auto classify = [&](int a, int b) {
+#pragma unroll 4
                 for (int s = a + tid; s < b; s += kThreads) {
                     const int c = g.key[s];
-                    if (c == kKeyPad) continue;
                     const int kk = c & 0x7fff;
+                    if (c == kKeyPad) continue;
                     if (kk <= key) {
-                        const int x = t.slot[s].x;
+                        const int x = __ldg(&t.slot[s].x);
                         atomicOr(freeb + (x >> 5), 1u << (x & 31));
                     } else if (c & 0x8000) {
                         vf += (unsigned long long)g.prof[s];
-                        wf += (unsigned)(t.slot[s].y >> kWeightShift);
+                        wf += (unsigned)(__ldg(&t.slot[s].y) >> kWeightShift);
                     }
                 }
             };
@@ -631,53 +1058,61 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             // ---- the first CTA: DP over the undecided rows, on chip
             if (cr == 0) {
                 Rows &R = *(Rows *)smem;
-                unsigned char *pool = smem + sizeof(Rows);
-                const int64_t vfix = (int64_t) * (volatile unsigned long long *)&g.s->vfix[pass];
-                const int64_t wfix = (int64_t) * (volatile unsigned long long *)&g.s->wfix[pass];
-                const int64_t kleft = k - wfix;
-                int out = 0, okey = 0;       // 1 solved, 2 again with okey (5: which is sure), 3 not reducible
+                unsigned char *pool = smem + up16(sizeof(Rows));
+                const int64_t vfix = (int64_t)__ldcg(&g.s->vfix[pass]);
+                const int64_t kleft = k - (int64_t)__ldcg(&g.s->wfix[pass]);
+                int out = 0, okey = 0;       // 1 solved, 2 again with okey (5: which is sure), 3 not reducible, 4 to the sweep
                 if (kleft < 0) {                        // too few rows undecided: take more by rank
                     out = 2;
-                    okey = key_of_rank(pass == 0 ? 2 * kFirstRows : kRowCap);
+                    up_to(kFirstRows, kBins, okey);
+                    if (okey <= key) up_to(kRowCap, kBins, okey);
                     if (okey <= key) out = 3;
                 } else {
                     // rows in sweep order from the bitmap
                     const int per = (words + kThreads - 1) / kThreads;
                     const int w0 = min(words, tid * per), w1 = min(words, w0 + per);
                     int c = 0;
-                    for (int i = w0; i < w1; ++i) c += __popc(*(volatile uint32_t *)(freeb + i));
+#pragma unroll 4
+                    for (int i = w0; i < w1; ++i) c += __popc(__ldcg(freeb + i));
                     int tot;
                     int ex = block_scan(c, &tot, sh);
-                    for (int i = w0; i < w1; ++i) {
-                        uint32_t m = *(volatile uint32_t *)(freeb + i);
-                        while (m) {
-                            const int x = i * 32 + __ffs((int)m) - 1;
-                            m &= m - 1;
-                            R.pos[T - 1 - ex] = x;
-                            ++ex;
+                    if (c)
+                        for (int i = w0; i < w1; ++i) {
+                            uint32_t m = __ldcg(freeb + i);
+                            while (m) {
+                                const int x = i * 32 + __ffs((int)m) - 1;
+                                m &= m - 1;
+                                R.pos[T - 1 - ex] = x;
+                                ++ex;
+                            }
                         }
-                    }
                     __syncthreads();
-                    int64_t wsum = 0;
-                    for (int r = tid; r < T; r += kThreads) {
-                        const int x = R.pos[r];
-                        R.p[r] = P[A.order ? A.order[x] : x];
-                        R.w[r] = A.wpre[x];
-                        wsum += R.w[r];
-                        R.last[r] = -1;
-                        // the first undecided row at or after next(x), -1: none
-                        const int nx = A.next[x];
-                        int a = 0, b = r;               // rows 0..a-1 have pos >= nx
-                        while (a < b) {
-                            const int mid = (a + b) >> 1;
-                            if (R.pos[mid] >= nx) a = mid + 1;
-                            else b = mid;
+                    int wsum = 0;                       // capped: far above every column cap
+                    for (int r = tid; r < (T + 31 & ~31); r += kThreads) {
+                        bool leaf = false;
+                        if (r < T) {
+                            const int x = R.pos[r];
+                            const int w = __ldg(A.wpre + x);
+                            R.row[r].p = P[A.order ? __ldg(A.order + x) : x];
+                            R.row[r].w = w;
+                            wsum += min(w, 1 << 18);
+                            R.last[r] = -1;
+                            // the first undecided row at or after next(x), -1: none
+                            const int nx = __ldg(A.next + x);
+                            int a = 0, b = r;           // rows 0..a-1 have pos >= nx
+                            while (a < b) {
+                                const int mid = (a + b) >> 1;
+                                if (R.pos[mid] >= nx) a = mid + 1;
+                                else b = mid;
+                            }
+                            R.skip[r] = a - 1;
+                            leaf = a == r;
                         }
-                        R.skip[r] = a - 1;
+                        const unsigned lm = __ballot_sync(kAll, leaf);
+                        if (lane == 0) R.leaf[r >> 5] = lm;
                     }
-                    wsum = wsum < (1 << 30) ? wsum : (1 << 30);
                     int wtot;
-                    block_scan((int)min(wsum, (int64_t)(1 << 20)), &wtot, sh);   // (2^20 is above every column cap)
+                    block_scan(wsum, &wtot, sh);
                     const int kc = (int)(kleft < wtot ? kleft : wtot);
                     // stack plan, as the pruned sweep's: a row read through the
                     // stack is pushed when computed and popped after its last reader
@@ -685,13 +1120,15 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                         const int sk = R.skip[r];
                         if (sk >= 0 && sk != r - 1) atomicMax(&R.last[sk], r);
                     }
+                    if (tid == 0) s_a = 0;
                     __syncthreads();
-                    int depth = 0, deepest = 0;
+                    int depth = 0;
                     for (int base = 0; base < T; base += kThreads) {
                         const int r = base + tid;
+                        int sk = -1;
                         bool pop = false, push = false;
                         if (r < T) {
-                            const int sk = R.skip[r];
+                            sk = R.skip[r];
                             pop = sk >= 0 && sk != r - 1 && R.last[sk] == r;
                             push = R.last[r] >= 0;
                         }
@@ -703,95 +1140,76 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                             if (push) {
                                 fl = kPush;
                                 lvl = dd;
+                                atomicMax(&s_a, dd + 1);
                             } else if (pop && dd > 0) {
                                 fl = kReload;
                                 lvl = dd - 1;
                             } else if (pop) {
                                 fl = kZeroTop;
                             }
-                            const int sk = R.skip[r];
                             if (sk >= 0 && sk == r - 1 && R.last[r - 1] < 0) fl |= kFromCur;
-                            R.info[r] = fl | (lvl << 8);
-                            deepest = max(deepest, push ? dd + 1 : 0);
+                            R.row[r].info = fl | (lvl << 8);
                         }
                         depth += dt;
                     }
-                    if (tid == 0) s_T = 0;
                     __syncthreads();
-                    if (deepest) atomicMax(&s_T, deepest);
-                    __syncthreads();
-                    const int levels = s_T;
-                    const int nw = (kc + 31) / 32;                   // warps that hold columns
-                    const size_t need = (size_t)T * nw * 4 + (size_t)(levels + 2) * nw * 32 * 8;
+                    const int levels = s_a;
+                    // one warp up to 256 columns, then 4 columns per thread
+                    const int C = kc <= 32 ? 1 : kc <= 64 ? 2 : kc <= 128 ? 4 : kc <= 256 ? 8 : 4;
+                    const int act = kc <= 256 ? 1 : (kc + 127) / 128;
+                    const int cols = act * 32 * C;
+                    const int guard = min(A.max_weight, cols);
+                    const int pitch = cols + 1 + guard;
+                    const size_t need = (size_t)2 * pitch * 8 + (size_t)levels * cols * 8 + (size_t)((T + 31) / 32) * cols * 4;
                     if (kc > kColCap || need > (size_t)kPool) {
-                        out = 3;
+                        out = sure ? 4 : 3;
                     } else {
-                        // one column per thread (two above 512); column j = c + 1
-                        int64_t *rowb = (int64_t *)pool;             // [2][nw * 32]
-                        int64_t *stk = rowb + 2 * nw * 32;           // [levels][nw * 32]
-                        uint32_t *bits = (uint32_t *)(stk + (size_t)levels * nw * 32);   // [T][nw]
-                        const int cols = nw * 32;
-                        const int act = min(nw, kWarps);             // warps in the loop
-                        if (tid == 0) s_val = 0;
-                        for (int c2 = tid; c2 < cols; c2 += kThreads) rowb[c2] = 0;
+                        int64_t *rowb = (int64_t *)pool;             // [2][guard + 1 + cols]
+                        int64_t *stk = rowb + 2 * pitch;             // [levels][cols]
+                        uint32_t *bits = (uint32_t *)(stk + (size_t)levels * cols);   // [T / 32][cols]
+                        if (tid == 0) {
+                            s_val = 0;
+                            R.row[T].p = 0;
+                            R.row[T].w = R.row[T].info = 0;
+                        }
+                        for (int i = tid; i < 2 * pitch; i += kThreads) rowb[i] = i % pitch < guard ? -2 * kBig : 0;
+                        for (int r = tid; r < T; r += kThreads)
+                            if (R.row[r].w > cols) R.row[r].w = cols + 1;    // never fits: column 0's guard
                         __syncthreads();
                         if (warp < act) {
-                            int64_t cur[2] = {0, 0}, tp[2] = {0, 0};
-                            const bool two = tid + kThreads < cols;  // uniform over the warp
-                            for (int r = 0; r < T; ++r) {
-                                const int64_t p = R.p[r];
-                                const int w = R.w[r], info = R.info[r];
-                                const int64_t *prev = rowb + (r & 1) * cols;
-                                int64_t *outr = rowb + ((r + 1) & 1) * cols;
-#pragma unroll
-                                for (int h = 0; h < 2; ++h) {
-                                    if (h == 1 && !two) break;
-                                    const int j = tid + h * kThreads + 1;
-                                    const int64_t sk = (info & kFromCur) ? cur[h] : tp[h];
-                                    bool take = false;
-                                    int64_t v = sk;
-                                    if (j >= w) {
-                                        const int64_t tv = p + (j > w ? prev[j - w - 1] : 0);
-                                        take = tv > sk;
-                                        v = take ? tv : sk;
-                                    }
-                                    cur[h] = v;
-                                    outr[j - 1] = v;
-                                    const unsigned m = __ballot_sync(kAll, take);
-                                    if (lane == 0) bits[r * nw + ((j - 1) >> 5)] = m;
-                                    const int lvl = info >> 8;
-                                    if (info & kPush) {
-                                        stk[lvl * cols + j - 1] = v;
-                                        tp[h] = v;
-                                    } else if (info & kReload) {
-                                        tp[h] = stk[lvl * cols + j - 1];
-                                    } else if (info & kZeroTop) {
-                                        tp[h] = 0;
-                                    }
-                                }
-                                if (act == 1) __syncwarp();
-                                else asm volatile("bar.sync 1, %0;" ::"r"(act * 32) : "memory");
-                            }
-                            if (kc > 0) {
-                                if (tid == (kc - 1) % kThreads) s_val = cur[(kc - 1) / kThreads];
-                            }
+                            if (act > 1) dp_rows<4>(R, T, act, guard, rowb, stk, bits, &s_val, kc);
+                            else if (C == 1) dp_rows<1>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
+                            else if (C == 2) dp_rows<2>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
+                            else if (C == 4) dp_rows<4>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
+                            else dp_rows<8>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
                         }
                         __syncthreads();
                         const int64_t V = vfix + s_val;
-                        const int need_key = slack ? -1 : loss_key(L - V);
-                        if (slack || need_key <= key) {
+                        // at price 0 with |S| <= k, S is Eq. 9's set: a chunk is
+                        // taken iff what it brings is positive
+                        const int need_key = key < 0 ? -1 : code_of(L - V);
+                        if (need_key <= key) {
                             out = 1;
-                            // walk the decisions
+                            // walk the decisions: in a 32-row word of the column, the
+                            // next row that is taken or whose skip is no leaf's
                             if (tid == 0) {
                                 int r = T - 1, j = kc;
                                 while (r >= 0 && j > 0) {
-                                    if ((bits[r * nw + ((j - 1) >> 5)] >> ((j - 1) & 31)) & 1u) {
-                                        const int x = R.pos[r];
+                                    const int blk = r >> 5;
+                                    const uint32_t word = bits[blk * cols + j - 1];
+                                    const uint32_t cand = (word | ~R.leaf[blk]) & ((2u << (r & 31)) - 1u);
+                                    if (cand == 0) {
+                                        r = blk * 32 - 1;
+                                        continue;
+                                    }
+                                    const int q = 31 - __clz((int)cand), rr = blk * 32 + q;
+                                    if ((word >> q) & 1u) {
+                                        const int x = R.pos[rr];
                                         atomicOr(taken + (x >> 5), 1u << (x & 31));
-                                        j -= R.w[r];
-                                        --r;
+                                        j -= R.row[rr].w;
+                                        r = rr - 1;
                                     } else {
-                                        r = R.skip[r];
+                                        r = R.skip[rr];
                                     }
                                 }
                                 A.best[item] = V;
@@ -800,9 +1218,23 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                             }
                         } else {
                             out = 5;
-                            okey = need_key;
+                            okey = vkey = vkey < 0 ? need_key : min(vkey, need_key);
+                            int same;
+                            if (pass == 0 && up_to(INT_MAX, okey, same) > kRowCap) {
+                                // a V from more rows may need fewer
+                                int more;
+                                up_to(2 * kFirstRows, kBins, more);
+                                if (more > key) {
+                                    out = 2;
+                                    okey = more;
+                                }
+                            }
                         }
                     }
+                }
+                if (out == 3 && vkey >= 0) {
+                    out = 5;
+                    okey = vkey;
                 }
                 if (tid == 0) {
                     g.s->key[pass] = okey;
@@ -810,20 +1242,23 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 }
             }
             sync_all();
-            verdict = *(volatile int *)&g.s->verdict[pass];
+            verdict = __ldcg(&g.s->verdict[pass]);
             if (verdict != 2 && verdict != 5) break;
             sure = verdict == 5;
-            key = *(volatile int *)&g.s->key[pass];
+            key = __ldcg(&g.s->key[pass]);
+            int same;
+            T = up_to(INT_MAX, key, same);
         }
     }
     const int state = verdict == 1 ? 1 : verdict == 4 ? 2 : 0;
     // ---- the decided "in" rows join the set
     if (state) {
         auto mark = [&](int a, int b) {
+#pragma unroll 4
             for (int s = a + tid; s < b; s += kThreads) {
                 const int c = g.key[s];
                 if (c == kKeyPad || !(c & 0x8000) || (c & 0x7fff) <= key) continue;
-                const int x = t.slot[s].x;
+                const int x = __ldg(&t.slot[s].x);
                 atomicOr(taken + (x >> 5), 1u << (x & 31));
             }
         };
@@ -833,8 +1268,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     if (cr == 0 && tid == 0) {
         *red = state;
         if (state == 2) {
-            A.w.left[item] = (int32_t)(k - (int64_t) * (volatile unsigned long long *)&g.s->wfix[pass]);
-            A.w.base[item] = (int64_t) * (volatile unsigned long long *)&g.s->vfix[pass];
+            A.w.left[item] = (int32_t)(k - (int64_t)__ldcg(&g.s->wfix[pass]));
+            A.w.base[item] = (int64_t)__ldcg(&g.s->vfix[pass]);
         }
     }
 }
@@ -842,8 +1277,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 // ---------------------------------------------------------------------------
 // host: the layout (see the top of the file), one device block per instance
 // ---------------------------------------------------------------------------
-// CTAs of an item's cluster: one per 6,144 rows (12 tiles per warp), at most 8
-static int cluster_of(int n) { return n <= 6144 ? 1 : n <= 12288 ? 2 : n <= 24576 ? 4 : 8; }
+// CTAs of an item's cluster
+static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 2 : n <= 98304 ? 4 : 8; }
 
 bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::vector<int32_t> &next,
                          const std::vector<int32_t> &wpre, int64_t total_weight, int32_t max_weight,
@@ -852,11 +1287,33 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     ReduceTables &R = *out;
     R = ReduceTables();
     if (n < kReduceMinRows || max_weight > kMaxWeight || total_weight >= ((int64_t)1 << 30)) return false;
-    const int CL = cluster_of(n);
-    const int limit = CL == 1 ? n : std::max(64, n / (4 * CL));      // rows of a subtree that stays in one bin
+    int CL = cluster_of(n);
+    // rows of a subtree that stays in one bin: half a CTA's share, more
+    // if that leaves too many rows above the bins
+    std::vector<int32_t> kids(n, 0), heavy(n, -1), best(n, 0);
+    for (int32_t i = 0; i < n; ++i) {
+        const int p = par[i];
+        if (p < 0) continue;
+        if (++kids[p] > kMaxKids) return false;
+        R.max_kids = std::max(R.max_kids, kids[p]);
+    }
+    int limit = n;
+    if (CL > 1) {
+        limit = std::max(64, n / (2 * CL));
+        for (;; limit *= 2) {
+            int above = 0;
+            for (int32_t i = 0; i < n; ++i) above += next[i] - i > limit;
+            if (above <= kMaxTop) break;
+            if (limit >= n / 2) {
+                CL = 1;
+                limit = n;
+                break;
+            }
+        }
+    }
     auto is_top = [&](int i) { return next[i] - i > limit; };
     // bins: subtrees below the limit, each to the emptiest bin
-    std::vector<int32_t> bin(n), heavy(n, -1), best(n, 0), level(n, 0), acc(n, -1);
+    std::vector<int32_t> bin(n), level(n, 0), acc(n, -1);
     std::vector<int64_t> load(CL, 0);
     for (int32_t i = 0; i < n; ++i) {
         const int p = par[i];
@@ -885,6 +1342,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     }
     // path tops grouped by (bin, level)
     const int nl = maxlev + 1;
+    if (nl > kMaxLevels) return false;
     std::vector<int32_t> start((size_t)(CL + 1) * nl + 1, 0), rows((size_t)(CL + 1) * nl, 0), tops, len(n, 0);
     for (int32_t i = n - 1; i >= 0; --i) len[i] = 1 + (heavy[i] >= 0 ? len[heavy[i]] : 0);
     auto path_top = [&](int i) { return par[i] < 0 || heavy[par[i]] != i; };
@@ -913,7 +1371,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
             const size_t q = (size_t)b * nl + l;
             R.lev.push_back((int32_t)R.stream.size());
             // streams of about equal length, one per warp of the CTA when there are rows for all
-            const int ns = std::max(1, std::min(kWarps, (rows[q] + 63) / 64));
+            const int ns = std::max(1, std::min(kWarps, (rows[q] + 31) / 32));
             const int want = (rows[q] + ns - 1) / ns;
             int in_stream = 0, tile0 = (int)(R.slot.size() / 32);
             auto close = [&] {
@@ -1006,9 +1464,9 @@ ReduceShape reduce_shape(const ReduceTables &R)
     s.nstreams = (int)R.stream.size();
     s.nlev = (int)R.lev.size();
     s.ntop = R.nacc[R.CL];
+    s.max_kids = R.max_kids;
     s.max_acc = *std::max_element(R.nacc.begin(), R.nacc.end() - 1);
-    // two CTAs fit on one SM: at most 104 KB each
-    s.acc_smem = up16((size_t)s.max_acc * 28) + kBins * 4 <= (size_t)(104 << 10);
+    s.acc_smem = up16((size_t)(s.max_acc + 1) * kAccBytes) + kBins * 4 <= (size_t)(192 << 10);
     return s;
 }
 
@@ -1037,12 +1495,13 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.rows_kept = rows_kept;
     a.w = work;
     a.item_bytes = reduce_item_bytes(inst);
-    a.acc_smem = r.acc_smem;
     a.total_weight = inst->total_weight;
     a.max_weight = inst->max_weight;
-    const size_t scan = (r.acc_smem ? up16((size_t)r.max_acc * 28) : 0) + kBins * 4;
-    const size_t smem = std::max(scan, sizeof(Rows) + kPool);
-    PP_CUDA(cudaFuncSetAttribute(k_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
+    const size_t scan = (r.acc_smem ? up16((size_t)(r.max_acc + 1) * kAccBytes) : 0) + kBins * 4;
+    const size_t smem = std::max(scan, up16(sizeof(Rows)) + kPool);
+    const auto kern = r.acc_smem ? k_reduce<true> : k_reduce<false>;
+    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r.CL * batch);
     cfg.blockDim = dim3(kThreads);
@@ -1055,7 +1514,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    PP_CUDA(cudaLaunchKernelEx(&cfg, k_reduce, a));
+    PP_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
     return PP_OK;
 }
 

@@ -74,8 +74,8 @@ def test_reduced_optimum_and_set(pp, oracle_lib, shape, n, wmax):
 
     def rows(r):
         assert r[5] == 0 or tw > 8192            # nothing is undecided without a limit
-        if shape != "caterpillar":               # (whose spine is taken in long runs: any count)
-            assert r[0] <= 1024                  # reduced
+        if shape == "mixed":
+            assert r[0] <= n // 4                # few rows are left undecided
     _check(pp, oracle_lib, parent, weight, wide, budgets, rows)
 
 
