@@ -128,14 +128,15 @@ constexpr int32_t kDevOk = PP_OK;
 // is built, and their sizes.  CL = 0: this tree is not reduced.
 constexpr int32_t kReduceMinRows = 1024;    // below, the sweep is as short as the reduction
 struct ReduceTables {
-    struct Slot {
-        int32_t pos, code, acc, par;
+    struct Info {
+        int32_t x, y;
     };
     struct Stream {
         int32_t tile, tiles;
     };
     int CL = 0, max_kids = 0;
-    std::vector<Slot> slot;
+    std::vector<Info> info;
+    std::vector<int32_t> pos;
     std::vector<Stream> stream;
     std::vector<int32_t> lev, binlev, binslot, nacc;
 };

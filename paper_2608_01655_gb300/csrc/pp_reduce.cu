@@ -65,20 +65,27 @@ constexpr int kBins = 2048;                 // keys of 0 .. 2^62
 constexpr int kKeyPad = 0xffff;
 constexpr int64_t kBig = (int64_t)1 << 61;
 constexpr int kMaxWeight = 1 << 22;         // weights ride in the slot code
-constexpr int kMaxPathRows = 4096;          // longer heavy paths are left to the sweep
+constexpr int kMaxPathRows = 1024;          // trees with longer heavy paths are left to the sweep
 constexpr int kMaxKids = 65535;             // light children of a row: its 16-bit limbs add up in 32 bits
+constexpr int kRing = 3;                    // tiles of a warp in flight or in use
+constexpr int kMaxTiles = 64;               // of a warp, all levels together
+constexpr size_t kRingBytes = (size_t)kWarps * kRing * 512;
 constexpr int kMaxTop = 256;                // rows of the last bin (every CTA walks it)
 // the search's 32-bit units: the first price is 2^11 to 2^12 of them
 constexpr int kUnitBits = 11;
 constexpr int kClipRow = 1 << 24, kClipPath = 1 << 26, kClipPrice = 1 << 19;
 
-// slot code: bits 0-4 lanes to the left in the same path and tile, 5 the path
-// comes from the previous tile, 6 top of its path, 8.. weight
-constexpr int kCont = 32, kTop = 64, kWeightShift = 8;
+// slot info.  x: bits 0-4 lanes to the left in the same path and tile, 5 the
+// path comes from the previous tile, 6 top of its path, 7 its parent is in
+// the last bin, 8.. weight.  y: accumulator (low half), the parent's
+// accumulator for a path's top (high half); kNone: none, a root
+constexpr int kCont = 32, kTop = 64, kUp = 128, kWeightShift = 8;
+constexpr int kNone = 0xffff;
 
 struct Tab {
     int n, CL, nslots, ntop;
-    const int4 *slot;            // position (-1 pad), code, accumulator (-1 none), parent
+    const int2 *info;
+    const int *pos;              // position of the slot's row (-1 pad)
     const int2 *stream;          // first tile, tiles: what one warp walks in sequence
     const int *lev;              // stream boundaries of the levels
     const int *binlev;           // [CL + 2] boundaries of a bin's entries in lev
@@ -213,12 +220,53 @@ __device__ __forceinline__ T acc_ld(const T *p)
     else return *p;
 }
 
-// The stream that this warp walks at level l of a bin: (first tile, tiles)
-__device__ __forceinline__ int2 stream_of(const Tab &t, int l0, int l)
-{
-    const int s = __ldg(t.lev + l0 + l) + (int)(threadIdx.x >> 5);
-    return s < __ldg(t.lev + l0 + l + 1) ? __ldg(t.stream + s) : make_int2(0, 0);
-}
+// The tiles that a warp walks, (level << 16) + tile, its lanes' slots (info
+// and a value) copied to shared memory two tiles ahead.  Asynchronous copies:
+// registers loaded for the next trip of a loop are waited for at its back
+// edge, which puts L2's latency (300 to 500 cycles) on every tile.
+template <typename V, int DIR>
+struct Feed {
+    const int2 *info;                        // of this lane's slot of the bin's first tile
+    const V *val;
+    const unsigned *list;
+    int2 *ri;                                // this lane's column of the ring
+    V *rv;
+    int n, i, h;                             // tiles, the one in hand, its ring slot
+
+    __device__ __forceinline__ Feed(const int2 *info_, const V *val_, const unsigned *list_, int n_, unsigned char *ring)
+        : info(info_ + (threadIdx.x & 31)), val(val_ + (threadIdx.x & 31)), list(list_), n(n_)
+    {
+        ri = (int2 *)(ring + (threadIdx.x >> 5) * (kRing * 512)) + (threadIdx.x & 31);
+        rv = (V *)(ring + (threadIdx.x >> 5) * (kRing * 512) + kRing * 256) + (threadIdx.x & 31);
+        i = DIR > 0 ? 0 : n - 1;
+        h = 0;
+        issue(i, 0);
+        issue(i + DIR, 1);
+    }
+    __device__ __forceinline__ void issue(int x, int to)
+    {
+        if (x >= 0 && x < n) {
+            const int slot = (int)(list[x] & 0xffffu) * 32;
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(ri + to * 32)),
+                         "l"(__cvta_generic_to_global(info + slot)) : "memory");
+            asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(rv + to * 32)),
+                         "l"(__cvta_generic_to_global(val + slot)), "n"((int)sizeof(V)) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    __device__ __forceinline__ bool more() const { return DIR > 0 ? i < n : i >= 0; }
+    __device__ __forceinline__ unsigned entry() const { return list[i]; }
+    // the slots of the tile in hand; the one after next is started
+    __device__ __forceinline__ void take(int2 &c, V &v)
+    {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        c = ri[h * 32];
+        v = rv[h * 32];
+        issue(i + 2 * DIR, h == 0 ? 2 : h - 1);
+        h = h == 2 ? 0 : h + 1;
+        i += DIR;
+    }
+};
 
 // ---- one tile of the search: f, and the size of the best closed set below
 // (and with) every row, at a price of `lam` units; `out` the lanes with f <= 0
@@ -260,64 +308,42 @@ __device__ __forceinline__ STile search_tile(int code, int p, int2 kids, int lam
 }
 
 // The search over a bin: levels from the leaves up, a block barrier between
-// them, the next tile's loads in flight while a tile is scanned (also across
-// levels).  A tile without a row of positive f has none at any higher price:
-// `live` holds the tiles (of the first 32 of a stream) still to be walked,
-// and `cand` what it becomes if this price turns out to be a lower bound.
-// own.s[na] stays zero (rows without light children read it).
+// them.  A tile without a row of positive f has none at any higher price:
+// `keep` gets the others, the list to walk if this price turns out to be a
+// lower bound; their number is returned.  own.s[na] stays zero (rows without
+// light children read it).
 template <bool GLOBAL>
-__device__ __forceinline__ void search_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
-                                           int na, int2 *tops, int lam, int clip, unsigned *live, unsigned *cand,
-                                           bool use_cand, int &rootZ)
+__device__ __forceinline__ int search_bin(const int2 *info, const int *val, const unsigned *list, int n, unsigned *keep,
+                                          int nlev, const Acc &own, int na, int2 *tops, int lam, int clip,
+                                          unsigned char *ring, int &rootZ)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int2 st = make_int2(0, 0);
-    unsigned todo = 0, opened = 0;
-    int fl = -1, q = 0, late = 32;           // level and tile in flight; tiles past 32 are always walked
-    int4 e = make_int4(-1, 0, -1, -1);
-    int p = 0;
-    auto advance = [&] {                     // the next tile, its loads started
-        while (!todo && late >= st.y) {
-            if (++fl >= nlev) return;
-            const int i = fl * kWarps + warp;
-            st = strm[i];
-            late = 32;
-            todo = opened = use_cand ? cand[i] : live[i];
-            if (use_cand && lane == 0) live[i] = todo;
+    const int lane = threadIdx.x & 31;
+    Feed<int, 1> feed(info, val, list, n, ring);
+    int lev = 0, carryY = 0, carryZ = 0, kept = 0;
+    unsigned prev = 0;
+    while (feed.more()) {
+        const unsigned en = feed.entry();
+        for (; lev < (int)(en >> 16); ++lev) __syncthreads();
+        int2 c;
+        int p;
+        feed.take(c, p);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const int2 kids = acc_ld<GLOBAL>(own.s + min(ac, na));
+        if (en != prev + 1) carryY = carryZ = 0;         // not the same path's next tile
+        prev = en;
+        const STile r = search_tile(c.x, p, kids, lam, carryY, carryZ);
+        if (r.out != kAll) {
+            if (lane == 0) keep[kept] = en;
+            ++kept;
         }
-        if (todo) {
-            q = __ffs((int)todo) - 1;
-            todo &= todo - 1;
-        } else {
-            q = late++;
+        if ((c.x & kTop) && r.f > 0) {
+            if (up == kNone) rootZ += r.z;
+            else if (c.x & kUp) pair_add(tops + up, min(r.f, clip), r.z);
+            else pair_add(own.s + up, min(r.f, clip), r.z);
         }
-        const int slot = (st.x + q) * 32 + lane;
-        e = __ldg(t.slot + slot);
-        p = g.unit[slot];
-    };
-    advance();
-    for (int l = 0; l < nlev; ++l) {
-        int carryY = 0, carryZ = 0, prev = -1;
-        unsigned keep = fl == l ? opened : 0;
-        while (fl == l) {
-            const int4 c = e;
-            const int pc = p, at = q;
-            const int2 kids = acc_ld<GLOBAL>(own.s + (c.z < 0 ? na : c.z));
-            if (at != prev + 1) carryY = carryZ = 0;
-            prev = at;
-            advance();
-            const STile r = search_tile(c.y, pc, kids, lam, carryY, carryZ);
-            if (at < 32 && r.out == kAll) keep &= ~(1u << at);
-            if ((c.y & kTop) && r.f > 0) {
-                if (c.w >= 0) pair_add(own.s + c.w, min(r.f, clip), r.z);
-                else if (c.w == -1) rootZ += r.z;
-                else pair_add(tops - 2 - c.w, min(r.f, clip), r.z);
-            }
-        }
-        __syncwarp();                        // every lane has read its masks
-        if (lane == 0) cand[l * kWarps + warp] = keep;
-        if (l + 1 < nlev) __syncthreads();
     }
+    for (++lev; lev < nlev; ++lev) __syncthreads();
+    return kept;
 }
 
 // The last bin, by one warp (every CTA does it for itself): its tiles in
@@ -328,22 +354,14 @@ __device__ __forceinline__ int search_top(const Tab &t, const Scratch1 &g, const
     for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(tops + i);
     __syncwarp();
     int rootZ = 0, carryY = 0, carryZ = 0;
-    const int s0 = t.binslot[t.CL];
-    int4 e = __ldg(t.slot + s0 + lane);
-    int p = __ldcg(g.unit + s0 + lane);
-    for (int s = s0; s < t.nslots; s += 32) {
-        const int4 c = e;
-        const int pc = p;
-        if (s + 32 < t.nslots) {
-            e = __ldg(t.slot + s + 32 + lane);
-            p = __ldcg(g.unit + s + 32 + lane);
-        }
-        int2 kids = make_int2(0, 0);
-        if (c.z >= 0) kids = loc[c.z];
-        const STile r = search_tile(c.y, pc, kids, lam, carryY, carryZ);
-        if ((c.y & kTop) && r.f > 0) {
-            if (c.w == -1) rootZ += r.z;
-            else pair_add(loc + c.w, min(r.f, clip), r.z);
+    for (int s = t.binslot[t.CL] + lane; s < t.nslots; s += 32) {
+        const int2 c = __ldg(t.info + s);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const int2 kids = ac != kNone ? loc[ac] : make_int2(0, 0);
+        const STile r = search_tile(c.x, __ldcg(g.unit + s), kids, lam, carryY, carryZ);
+        if ((c.x & kTop) && r.f > 0) {
+            if (up == kNone) rootZ += r.z;
+            else pair_add(loc + up, min(r.f, clip), r.z);
         }
         __syncwarp();
     }
@@ -353,11 +371,11 @@ __device__ __forceinline__ int search_top(const Tab &t, const Scratch1 &g, const
 }
 
 // ---- one tile of the exact evaluation at the price lam
-__device__ __forceinline__ int64_t exact_tile(const int4 c, int64_t p, int64_t kids, int64_t lam, int64_t &carryY)
+__device__ __forceinline__ int64_t exact_tile(int code, int64_t p, int64_t kids, int64_t lam, int64_t &carryY)
 {
-    const int off = c.y & 31;
-    const bool cont = c.y & kCont;
-    const int64_t d = p - lam * (c.y >> kWeightShift) + kids;
+    const int off = code & 31;
+    const bool cont = code & kCont;
+    const int64_t d = p - lam * (code >> kWeightShift) + kids;
     int64_t m = 0, sm = d;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -376,70 +394,53 @@ __device__ __forceinline__ int64_t exact_tile(const int4 c, int64_t p, int64_t k
     return d + yp;
 }
 
-// f of every row of a bin to g.f, the roots' share of L to rootY
+// f of every row of a bin to f, the roots' share of L to rootY
 template <bool GLOBAL>
-__device__ __forceinline__ void exact_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
-                                          int64_t lam, int64_t &rootY)
+__device__ __forceinline__ void exact_bin(const int2 *info, const int64_t *val, int64_t *fout, int4 *topl,
+                                          const unsigned *list, int n, int nlev, const Acc &own, int na, int64_t lam,
+                                          unsigned char *ring, int64_t &rootY)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int2 st = make_int2(0, 0);
-    int fl = -1, q = 0;                      // level and tile in flight
-    int4 e = make_int4(-1, 0, -1, -1);
-    int64_t p = 0;
-    auto advance = [&] {
-        ++q;
-        while (q >= st.y) {
-            if (++fl >= nlev) return;
-            st = strm[fl * kWarps + warp];
-            q = 0;
+    const int lane = threadIdx.x & 31;
+    Feed<int64_t, 1> feed(info, val, list, n, ring);
+    int lev = 0;
+    int64_t carryY = 0;
+    unsigned prev = 0;
+    while (feed.more()) {
+        const unsigned en = feed.entry();
+        for (; lev < (int)(en >> 16); ++lev) __syncthreads();
+        int2 c;
+        int64_t p;
+        feed.take(c, p);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const int64_t kids = limbs(acc_ld<GLOBAL>(own.limb + min(ac, na)));
+        if (en != prev + 1) carryY = 0;
+        prev = en;
+        const int64_t f = exact_tile(c.x, p, kids, lam, carryY);
+        fout[(en & 0xffffu) * 32 + lane] = f;
+        if ((c.x & kTop) && f > 0) {
+            if (up == kNone) rootY += f;
+            else if (c.x & kUp) limb_add(topl + up, f);
+            else limb_add(own.limb + up, f);
         }
-        const int slot = (st.x + q) * 32 + lane;
-        e = __ldg(t.slot + slot);
-        p = g.prof[slot];
-    };
-    advance();
-    for (int l = 0; l < nlev; ++l) {
-        int64_t carryY = 0;
-        while (fl == l) {
-            const int4 c = e;
-            const int64_t pc = p;
-            const int slot = (st.x + q) * 32 + lane;
-            advance();
-            const int64_t kids = c.z >= 0 ? limbs(acc_ld<GLOBAL>(own.limb + c.z)) : 0;
-            const int64_t f = exact_tile(c, pc, kids, lam, carryY);
-            g.f[slot] = f;
-            if ((c.y & kTop) && f > 0) {
-                if (c.w >= 0) limb_add(own.limb + c.w, f);
-                else if (c.w == -1) rootY += f;
-                else limb_add(g.topl - 2 - c.w, f);
-            }
-        }
-        if (l + 1 < nlev) __syncthreads();
     }
+    for (++lev; lev < nlev; ++lev) __syncthreads();
 }
 // the last bin, by one warp of every CTA (they write the same f)
-__device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, int4 *loc, int64_t lam, int64_t *ftop)
+__device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, int4 *loc, int64_t lam)
 {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(g.topl + i);
     __syncwarp();
     int64_t rootY = 0, carryY = 0;
-    const int s0 = t.binslot[t.CL];
-    int4 e = __ldg(t.slot + s0 + lane);
-    int64_t pn = __ldcg(g.prof + s0 + lane);
-    for (int s = s0; s < t.nslots; s += 32) {
-        const int4 c = e;
-        const int64_t p = pn;
-        if (s + 32 < t.nslots) {
-            e = __ldg(t.slot + s + 32 + lane);
-            pn = __ldcg(g.prof + s + 32 + lane);
-        }
-        const int64_t kids = c.z >= 0 ? limbs(loc[c.z]) : 0;
-        const int64_t f = exact_tile(c, p, kids, lam, carryY);
-        ftop[s - s0 + lane] = f;
-        if ((c.y & kTop) && f > 0) {
-            if (c.w == -1) rootY += f;
-            else limb_add(loc + c.w, f);
+    for (int s = t.binslot[t.CL] + lane; s < t.nslots; s += 32) {
+        const int2 c = __ldg(t.info + s);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const int64_t kids = ac != kNone ? limbs(loc[ac]) : 0;
+        const int64_t f = exact_tile(c.x, __ldcg(g.prof + s), kids, lam, carryY);
+        g.f[s] = f;
+        if ((c.x & kTop) && f > 0) {
+            if (up == kNone) rootY += f;
+            else limb_add(loc + up, f);
         }
         __syncwarp();
     }
@@ -451,16 +452,17 @@ __device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, in
 // ---- one tile of the losses, from the top of a path down: `a` the sum of
 // max(0, -f) over the path from the root, `b` the smallest f on it.  In
 // floats rounded down: a loss is only ever underestimated, which keeps rows.
-__device__ __forceinline__ void loss_tile(const int4 c, int64_t f, float2 up, float &ca, float &cb, float &a, float &b)
+__device__ __forceinline__ void loss_tile(int code, int64_t f, bool child, float2 up, float &ca, float &cb, float &a,
+                                          float &b)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned starts = __ballot_sync(kAll, (c.y & 31) == 0);
-    const unsigned tops = __ballot_sync(kAll, (c.y & kTop) != 0);
+    const unsigned starts = __ballot_sync(kAll, (code & 31) == 0);
+    const unsigned tops = __ballot_sync(kAll, (code & kTop) != 0);
     const unsigned after = lane < 31 ? starts >> (lane + 1) : 0u;
     const int rem = after ? __ffs((int)after) - 1 : 31 - lane;    // lanes to the right in this path
     b = __ll2float_rd(f);
     a = f < 0 ? __ll2float_rd(-f) : 0.f;
-    if ((c.y & kTop) && c.w != -1) {
+    if (child) {                             // a path's top below some row: `up` is that row's
         a = __fadd_rd(a, up.x);
         b = fminf(b, up.y);
     }
@@ -487,71 +489,54 @@ __device__ __forceinline__ int loss_code(float a, float b)
     return k | (b > 0.f ? 0x8000 : 0);
 }
 
-// losses of one bin, levels from the top down; keys to g.key, histogram in sh
+// losses of one bin, levels from the top down, and their histogram
 template <bool GLOBAL>
-__device__ __forceinline__ void loss_bin(const Tab &t, const int2 *strm, int nlev, const Scratch1 &g, const Acc &own,
-                                         const float2 *topd, unsigned *hist)
+__device__ __forceinline__ void loss_bin(const int2 *info, const int64_t *fin, uint16_t *key, const unsigned *list, int n,
+                                         int nlev, const Acc &own, const float2 *topd, unsigned char *ring,
+                                         unsigned *hist)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int2 st = make_int2(0, 0);
-    int fl = nlev, q = 0;
-    int4 e = make_int4(-1, 0, -1, -1);
-    int64_t f = 0;
-    auto advance = [&] {
-        --q;
-        while (q < 0) {
-            if (--fl < 0) return;
-            st = strm[fl * kWarps + warp];
-            q = st.y - 1;
+    const int lane = threadIdx.x & 31;
+    Feed<int64_t, -1> feed(info, fin, list, n, ring);
+    int lev = nlev - 1;
+    float ca = 0.f, cb = 0.f;
+    while (feed.more()) {
+        const unsigned en = feed.entry();
+        for (; lev > (int)(en >> 16); --lev) __syncthreads();
+        int2 c;
+        int64_t f;
+        feed.take(c, f);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const bool child = (c.x & kTop) && up != kNone;
+        float2 from = make_float2(0.f, 0.f);
+        if (child) {
+            if (c.x & kUp) from = topd[up];
+            else from = acc_ld<GLOBAL>(own.down + up);
         }
-        const int slot = (st.x + q) * 32 + lane;
-        e = __ldg(t.slot + slot);
-        f = g.f[slot];
-    };
-    advance();
-    for (int l = nlev - 1; l >= 0; --l) {
-        float ca = 0.f, cb = 0.f;
-        while (fl == l) {
-            const int4 c = e;
-            const int64_t fc = f;
-            const int slot = (st.x + q) * 32 + lane;
-            advance();
-            float2 up = make_float2(0.f, 0.f);
-            if ((c.y & kTop) && c.w != -1) up = c.w >= 0 ? acc_ld<GLOBAL>(own.down + c.w) : topd[-2 - c.w];
-            float a, b;
-            loss_tile(c, fc, up, ca, cb, a, b);
-            if (c.z >= 0) own.down[c.z] = make_float2(a, b);
-            int code = kKeyPad;
-            if (c.x >= 0) {
-                code = loss_code(a, b);
-                atomicAdd(hist + (code & 0x7fff), 1u);
-            }
-            g.key[slot] = (uint16_t)code;
-        }
-        if (l > 0) __syncthreads();
+        float a, b;                          // (a path that goes on does so in the tile just done)
+        loss_tile(c.x, f, child, from, ca, cb, a, b);
+        if (ac != kNone) own.down[ac] = make_float2(a, b);
+        const int code = (c.x >> kWeightShift) ? loss_code(a, b) : kKeyPad;      // (a pad weighs nothing)
+        if (code != kKeyPad) atomicAdd(hist + (code & 0x7fff), 1u);
+        key[(en & 0xffffu) * 32 + lane] = (uint16_t)code;
     }
+    for (; lev > 0; --lev) __syncthreads();
 }
 // the last bin, by one warp; one CTA (`write`) keeps its keys
-__device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, const int64_t *ftop, float2 *topd, unsigned *hist,
-                                         bool write)
+__device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, float2 *topd, unsigned *hist, bool write)
 {
     const int lane = threadIdx.x & 31;
     float ca = 0.f, cb = 0.f;
-    const int s0 = t.binslot[t.CL];
-    for (int s = t.nslots - 32; s >= s0; s -= 32) {
-        const int4 c = __ldg(t.slot + s + lane);
-        float2 up = make_float2(0.f, 0.f);
-        if ((c.y & kTop) && c.w >= 0) up = topd[c.w];
+    for (int s = t.nslots - 32 + lane; s >= t.binslot[t.CL]; s -= 32) {
+        const int2 c = __ldg(t.info + s);
+        const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
+        const bool child = (c.x & kTop) && up != kNone;
         float a, b;
-        loss_tile(c, ftop[s - s0 + lane], up, ca, cb, a, b);
-        if (c.z >= 0) topd[c.z] = make_float2(a, b);
+        loss_tile(c.x, g.f[s], child, child ? topd[up] : make_float2(0.f, 0.f), ca, cb, a, b);
+        if (ac != kNone) topd[ac] = make_float2(a, b);
         if (write) {
-            int code = kKeyPad;
-            if (c.x >= 0) {
-                code = loss_code(a, b);
-                atomicAdd(hist + (code & 0x7fff), 1u);
-            }
-            g.key[s + lane] = (uint16_t)code;
+            const int code = (c.x >> kWeightShift) ? loss_code(a, b) : kKeyPad;
+            if (code != kKeyPad) atomicAdd(hist + (code & 0x7fff), 1u);
+            g.key[s] = (uint16_t)code;
         }
         __syncwarp();
     }
@@ -651,6 +636,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         }
         if (b.x0 > 0.f) {
             float s = __log2f(b.z0 / k) / __log2f(b.z0 / fmaxf(b.z1, 1.f));
+            s = fminf(fmaxf(s, 0.15f), 0.85f);
             if (b.side >= 2 || b.side <= -2) s = 0.5f * s + 0.25f;      // creeping from one side
             if (evals > 5) s = fminf(fmaxf(s, 0.2f), 0.8f);
             x = b.x0 * exp2f(__log2f(b.x1 / b.x0) * s);
@@ -667,8 +653,8 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         const float l1 = fmaxf((float)lam, 1.f), c = rank_at(cum, l1 * unit);
         if (Z > 0.f && c > 0.f && evals < 6) {
             x = price_of_rank(cum, k * c / Z) / unit;
-            x = above ? fmaxf(x, l1) * 1.01f : fminf(x, l1) * 0.99f;
-            if (evals > 2) x *= above ? 1.3f : 0.7f;
+            const float step = evals == 1 ? 0.015f : evals == 2 ? 0.04f : evals == 3 ? 0.1f : 0.3f;
+            x = above ? fmaxf(x, l1) * (1.f + step) : fminf(x, l1) * (1.f - step);
         } else {
             x = above ? (float)maxlam : 0.f;
         }
@@ -686,73 +672,56 @@ struct __align__(16) Row {
     int w, info;                             // flags below, stack level << 8
 };
 struct Rows {                                // in sweep order (last position first)
-    Row row[kRowCap + 1];
-    int pos[kRowCap], skip[kRowCap], last[kRowCap];
-    unsigned leaf[kRowCap / 32];             // bit: skip[r] = r - 1
+    Row row[kRowCap + 4];                    // (read four at a time)
+    int2 step[kRowCap];                      // the walk's: weight, row that a skip goes to (-1 past the last)
+    int pos[kRowCap], last[kRowCap];
+    unsigned leaf[kRowCap / 32];             // bit: a skip goes to the next row
 };
 constexpr int kPush = 1, kReload = 2, kZeroTop = 4, kFromCur = 8;
 
-// `act` warps, C columns per thread (column j = 1 + thread + c * threads).
+// One column per thread (column j = 1 + thread), as many warps as that takes.
 // The row just computed goes through shared memory (any weight is then one
 // load at j - w; `guard` words left of column 0 read as never worth taking),
-// a row's own scalars are loaded one row ahead, and decision bits are packed
-// per thread over 32 rows.
-template <int C>
+// a barrier of these warps per row; the scalars of four rows are read at once
+// and decision bits packed per thread over 32 rows.  Several columns per
+// thread of one warp took 100 (2 columns) to 310 ns (8) a row: a single warp
+// issues every instruction of a row in turn.
 __device__ __forceinline__ void dp_rows(const Rows &R, int T, int act, int guard, int64_t *rowb, int64_t *stk,
                                         uint32_t *bits, int64_t *result, int kc)
 {
-    const int tid = threadIdx.x, nt = act * 32, cols = nt * C, pitch = cols + 1 + guard;
-    int64_t cur[C], top[C];
-    uint32_t wb[C];
+    const int tid = threadIdx.x, cols = act * 32, pitch = cols + 1 + guard;
+    int64_t cur = 0, top = 0;
+    uint32_t wb = 0;
+    int64_t *const b0 = rowb + guard + 1 + tid, *const b1 = b0 + pitch;     // this column in the two row buffers
+    for (int r0 = 0; r0 < T; r0 += 4) {
+        Row x[4];
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-        cur[c] = top[c] = 0;
-        wb[c] = 0;
-    }
-    const int64_t *prev = rowb + guard;
-    int64_t *out = rowb + pitch + guard;
-    Row nx = R.row[0];
-    for (int r = 0; r < T; ++r) {
-        const Row x = nx;
-        nx = R.row[r + 1];
-        int64_t in[C];                       // all loads before any store
+        for (int u = 0; u < 4; ++u) x[u] = R.row[r0 + u];
 #pragma unroll
-        for (int c = 0; c < C; ++c) in[c] = prev[1 + tid - x.w + c * nt];
-#pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int64_t sk = (x.info & kFromCur) ? cur[c] : top[c];
-            const int64_t tv = x.p + in[c];
+        for (int u = 0; u < 4; ++u) {
+            if (r0 + u >= T) break;
+            const int64_t *prev = u & 1 ? b1 : b0;
+            int64_t *out = u & 1 ? b0 : b1;
+            const int64_t tv = x[u].p + prev[-x[u].w];
+            const int64_t sk = (x[u].info & kFromCur) ? cur : top;
             const bool take = tv > sk;
-            cur[c] = take ? tv : sk;
-            out[1 + tid + c * nt] = cur[c];
-            if (take) wb[c] |= 1u << (r & 31);
-        }
-        if (x.info & (kPush | kReload | kZeroTop)) {
-            int64_t *sl = stk + (x.info >> 8) * cols + tid;
-            if (x.info & kPush) {
-#pragma unroll
-                for (int c = 0; c < C; ++c) sl[c * nt] = top[c] = cur[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < C; ++c) top[c] = (x.info & kReload) ? sl[c * nt] : 0;
+            cur = take ? tv : sk;
+            *out = cur;
+            if (take) wb |= 1u << ((r0 + u) & 31);
+            if (x[u].info & (kPush | kReload | kZeroTop)) {
+                int64_t *sl = stk + (x[u].info >> 8) * cols + tid;
+                if (x[u].info & kPush) *sl = top = cur;
+                else top = (x[u].info & kReload) ? *sl : 0;
             }
+            if (act == 1) __syncwarp();
+            else asm volatile("bar.sync 1, %0;" ::"r"(cols) : "memory");
         }
-        if ((r & 31) == 31 || r == T - 1) {
-#pragma unroll
-            for (int c = 0; c < C; ++c) {
-                bits[(r >> 5) * cols + tid + c * nt] = wb[c];
-                wb[c] = 0;
-            }
+        if ((r0 & 31) == 28 || r0 + 4 >= T) {
+            bits[(r0 >> 5) * cols + tid] = wb;
+            wb = 0;
         }
-        if (act == 1) __syncwarp();
-        else asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
-        const int64_t *sw = prev;
-        prev = out;
-        out = const_cast<int64_t *>(sw);
     }
-#pragma unroll
-    for (int c = 0; c < C; ++c)
-        if (kc == 1 + tid + c * nt) *result = cur[c];
+    if (kc == 1 + tid) *result = cur;
 }
 
 }  // namespace
@@ -761,8 +730,7 @@ template <bool SMEM>                         // accumulators of the bins in shar
 __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int2 strm[kMaxLevels * kWarps];
-    __shared__ unsigned live[kMaxLevels * kWarps], cand[kMaxLevels * kWarps];
+    __shared__ unsigned lists[3][kWarps][kMaxTiles];    // a warp's tiles: all; two that the search shortens in turn
     __shared__ int4 s_top[kMaxTop];          // the last bin's own sums, then what it passes down
     __shared__ int sh[kWarps];
     __shared__ int s_a, s_b, s_flag, s_lam;
@@ -796,8 +764,10 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     const int na = t.nacc[cr];
     const int lo = t.binslot[cr], hi = t.binslot[cr + 1];
     const Acc own = acc_at(SMEM ? (char *)smem : g.own + (size_t)(lo + cr) * kAccBytes, na + 1);   // (one reads as zero)
-    unsigned *hist = (unsigned *)(smem + (SMEM ? up16((size_t)(na + 1) * kAccBytes) : 0));
+    unsigned char *ring = smem + (SMEM ? up16((size_t)(na + 1) * kAccBytes) : 0);
+    unsigned *hist = (unsigned *)(ring + kRingBytes);
     const bool has_top = t.binslot[CL] < t.nslots;
+    const int2 *info = t.info + lo;
     const int l0 = t.binlev[cr], nlev = t.binlev[cr + 1] - 1 - l0;
     const int top0 = t.binslot[CL];
     auto sync_all = [&] {
@@ -813,12 +783,14 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         for (int i = tid; i < t.ntop; i += kThreads) g.topl[i] = make_int4(0, 0, 0, 0);
     }
     for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
+    int tiles = 0;                           // of this warp
     for (int l = 0; l < nlev; ++l) {
-        const int2 x = stream_of(t, l0, l);
-        if (lane == 0) {
-            strm[l * kWarps + warp] = x;
-            live[l * kWarps + warp] = x.y >= 32 ? kAll : (1u << x.y) - 1;
-        }
+        const int q = __ldg(t.lev + l0 + l) + warp;
+        if (q >= __ldg(t.lev + l0 + l + 1)) continue;
+        const int2 x = __ldg(t.stream + q);
+        for (int i = lane; i < x.y; i += 32)
+            lists[0][warp][tiles + i] = lists[1][warp][tiles + i] = ((unsigned)l << 16) + (unsigned)(x.x - (lo >> 5) + i);
+        tiles += x.y;
     }
     sync_all();
 
@@ -829,17 +801,16 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     auto gather = [&](int from, int to) {
         constexpr int U = 4;                 // loads in flight per thread
         for (int s0 = from + tid; s0 < to; s0 += U * kThreads) {
-            int4 e[U];
+            int x[U];
             int64_t p[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                e[u] = s0 + u * kThreads < to ? __ldg(t.slot + s0 + u * kThreads) : make_int4(-1, 0, -1, -1);
+            for (int u = 0; u < U; ++u) x[u] = s0 + u * kThreads < to ? __ldg(t.pos + s0 + u * kThreads) : -1;
             if (A.order)
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (e[u].x >= 0) e[u].x = __ldg(A.order + e[u].x);
+                    if (x[u] >= 0) x[u] = __ldg(A.order + x[u]);
 #pragma unroll
-            for (int u = 0; u < U; ++u) p[u] = e[u].x >= 0 ? P[e[u].x] : 0;
+            for (int u = 0; u < U; ++u) p[u] = x[u] >= 0 ? P[x[u]] : 0;
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int s = s0 + u * kThreads;
@@ -847,7 +818,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 g.prof[s] = p[u];
                 mx = p[u] > mx ? p[u] : mx;
                 if (p[u] > 0 && ((s >> 5) & ((1 << every) - 1)) == 0) {
-                    const int w = e[u].y >> kWeightShift;
+                    const int w = __ldg(&t.info[s].x) >> kWeightShift;
                     const int c = w == 1 ? code_of(p[u]) : code_of((int64_t)((float)p[u] / (float)w));
                     atomicAdd(hist + c, (unsigned)w << every);
                 }
@@ -906,15 +877,21 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         to_units(lo, hi);
         if (cr == 0 && has_top) to_units(top0, t.nslots);
         bool low = false;                    // the last price was a lower bound
+        int at = 1, alive = tiles, kept = 0;
         for (int ev = 0;; ++ev) {
             for (int i = tid; i <= na; i += kThreads) own.s[i] = make_int2(0, 0);
             // (the set that the last price but one's sums were read from)
+            if (low) {                       // fewer tiles to walk from now on
+                at ^= 3;
+                alive = kept;
+            }
             if (cr == 0)
                 for (int i = tid; i < t.ntop; i += kThreads) g.tops[(ev + 1) % 3 * t.ntop + i] = make_int2(0, 0);
             int2 *tops = g.tops + ev % 3 * t.ntop;
             int rz = 0;
             __syncthreads();
-            search_bin<!SMEM>(t, strm, nlev, g, own, na, tops, price, A.clip_kid, live, cand, low, rz);
+            kept = search_bin<!SMEM>(info, g.unit + lo, lists[at][warp], alive, lists[at ^ 3][warp], nlev, own, na, tops,
+                                     price, A.clip_kid, ring, rz);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(kAll, rz, o);
             if (lane == 0 && rz) atomicAdd(&g.s->sumZ[ev], (unsigned long long)rz);
@@ -938,16 +915,16 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         if (s_flag == kSlack) price = 0;
         lam = (int64_t)price << shift;
         // ---- exactly there: f of every row, L
-        for (int i = tid; i < na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
+        for (int i = tid; i <= na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
         __syncthreads();
         int64_t ry = 0;
-        exact_bin<!SMEM>(t, strm, nlev, g, own, lam, ry);
+        exact_bin<!SMEM>(info, g.prof + lo, g.f + lo, g.topl, lists[0][warp], tiles, nlev, own, na, lam, ring, ry);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ry += __shfl_xor_sync(kAll, ry, o);
         if (lane == 0 && ry) atomicAdd(&g.s->sumL, (unsigned long long)ry);
         sync_all();
         if (warp == 0) {
-            ry = has_top ? exact_top(t, g, s_top, lam, g.f + top0) : 0;
+            ry = has_top ? exact_top(t, g, s_top, lam) : 0;
             if (lane == 0) s_val = (int64_t)__ldcg(&g.s->sumL) + ry + lam * k;
         }
         __syncthreads();
@@ -960,10 +937,10 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
         __syncthreads();
         if (has_top) {
-            if (warp == 0) loss_top(t, g, g.f + top0, (float2 *)s_top, hist, cr == 0);
+            if (warp == 0) loss_top(t, g, (float2 *)s_top, hist, cr == 0);
             __syncthreads();
         }
-        loss_bin<!SMEM>(t, strm, nlev, g, own, (const float2 *)s_top, hist);
+        loss_bin<!SMEM>(info, g.f + lo, g.key + lo, lists[0][warp], tiles, nlev, own, (const float2 *)s_top, ring, hist);
         __syncthreads();
         for (int i = tid; i < kBins; i += kThreads)
             if (hist[i]) atomicAdd(ghist + i, hist[i]);
@@ -1031,11 +1008,11 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                     const int kk = c & 0x7fff;
                     if (c == kKeyPad) continue;
                     if (kk <= key) {
-                        const int x = __ldg(&t.slot[s].x);
+                        const int x = __ldg(t.pos + s);
                         atomicOr(freeb + (x >> 5), 1u << (x & 31));
                     } else if (c & 0x8000) {
                         vf += (unsigned long long)g.prof[s];
-                        wf += (unsigned)(__ldg(&t.slot[s].y) >> kWeightShift);
+                        wf += (unsigned)(__ldg(&t.info[s].x) >> kWeightShift);
                     }
                 }
             };
@@ -1105,7 +1082,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                                 if (R.pos[mid] >= nx) a = mid + 1;
                                 else b = mid;
                             }
-                            R.skip[r] = a - 1;
+                            R.step[r] = make_int2(w, a - 1);
                             leaf = a == r;
                         }
                         const unsigned lm = __ballot_sync(kAll, leaf);
@@ -1117,7 +1094,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                     // stack plan, as the pruned sweep's: a row read through the
                     // stack is pushed when computed and popped after its last reader
                     for (int r = tid; r < T; r += kThreads) {
-                        const int sk = R.skip[r];
+                        const int sk = R.step[r].y;
                         if (sk >= 0 && sk != r - 1) atomicMax(&R.last[sk], r);
                     }
                     if (tid == 0) s_a = 0;
@@ -1128,7 +1105,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                         int sk = -1;
                         bool pop = false, push = false;
                         if (r < T) {
-                            sk = R.skip[r];
+                            sk = R.step[r].y;
                             pop = sk >= 0 && sk != r - 1 && R.last[sk] == r;
                             push = R.last[r] >= 0;
                         }
@@ -1154,10 +1131,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                     }
                     __syncthreads();
                     const int levels = s_a;
-                    // one warp up to 256 columns, then 4 columns per thread
-                    const int C = kc <= 32 ? 1 : kc <= 64 ? 2 : kc <= 128 ? 4 : kc <= 256 ? 8 : 4;
-                    const int act = kc <= 256 ? 1 : (kc + 127) / 128;
-                    const int cols = act * 32 * C;
+                    const int act = max(1, (kc + 31) / 32);          // warps that hold columns
+                    const int cols = act * 32;
                     const int guard = min(A.max_weight, cols);
                     const int pitch = cols + 1 + guard;
                     const size_t need = (size_t)2 * pitch * 8 + (size_t)levels * cols * 8 + (size_t)((T + 31) / 32) * cols * 4;
@@ -1167,22 +1142,16 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                         int64_t *rowb = (int64_t *)pool;             // [2][guard + 1 + cols]
                         int64_t *stk = rowb + 2 * pitch;             // [levels][cols]
                         uint32_t *bits = (uint32_t *)(stk + (size_t)levels * cols);   // [T / 32][cols]
-                        if (tid == 0) {
-                            s_val = 0;
-                            R.row[T].p = 0;
-                            R.row[T].w = R.row[T].info = 0;
+                        if (tid == 0) s_val = 0;
+                        if (tid < 4) {
+                            R.row[T + tid].p = 0;
+                            R.row[T + tid].w = R.row[T + tid].info = 0;
                         }
                         for (int i = tid; i < 2 * pitch; i += kThreads) rowb[i] = i % pitch < guard ? -2 * kBig : 0;
                         for (int r = tid; r < T; r += kThreads)
                             if (R.row[r].w > cols) R.row[r].w = cols + 1;    // never fits: column 0's guard
                         __syncthreads();
-                        if (warp < act) {
-                            if (act > 1) dp_rows<4>(R, T, act, guard, rowb, stk, bits, &s_val, kc);
-                            else if (C == 1) dp_rows<1>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
-                            else if (C == 2) dp_rows<2>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
-                            else if (C == 4) dp_rows<4>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
-                            else dp_rows<8>(R, T, 1, guard, rowb, stk, bits, &s_val, kc);
-                        }
+                        if (warp < act) dp_rows(R, T, act, guard, rowb, stk, bits, &s_val, kc);
                         __syncthreads();
                         const int64_t V = vfix + s_val;
                         // at price 0 with |S| <= k, S is Eq. 9's set: a chunk is
@@ -1197,20 +1166,16 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                                 while (r >= 0 && j > 0) {
                                     const int blk = r >> 5;
                                     const uint32_t word = bits[blk * cols + j - 1];
-                                    const uint32_t cand = (word | ~R.leaf[blk]) & ((2u << (r & 31)) - 1u);
-                                    if (cand == 0) {
-                                        r = blk * 32 - 1;
-                                        continue;
-                                    }
-                                    const int q = 31 - __clz((int)cand), rr = blk * 32 + q;
-                                    if ((word >> q) & 1u) {
+                                    const uint32_t cand = (word | ~R.leaf[blk]) & (0xffffffffu >> (31 - (r & 31)));
+                                    const int rr = (r & ~31) + 31 - __clz((int)cand);      // below the block if none
+                                    const int2 st = R.step[max(rr, 0)];
+                                    const bool none = cand == 0, take = (cand & word) >> (rr & 31) & 1u;
+                                    if (!none && take) {
                                         const int x = R.pos[rr];
                                         atomicOr(taken + (x >> 5), 1u << (x & 31));
-                                        j -= R.row[rr].w;
-                                        r = rr - 1;
-                                    } else {
-                                        r = R.skip[rr];
                                     }
+                                    j -= !none && take ? st.x : 0;
+                                    r = none || take ? rr - !none : st.y;
                                 }
                                 A.best[item] = V;
                                 A.w.nkept[item] = T;
@@ -1258,7 +1223,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             for (int s = a + tid; s < b; s += kThreads) {
                 const int c = g.key[s];
                 if (c == kKeyPad || !(c & 0x8000) || (c & 0x7fff) <= key) continue;
-                const int x = __ldg(&t.slot[s].x);
+                const int x = __ldg(t.pos + s);
                 atomicOr(taken + (x >> 5), 1u << (x & 31));
             }
         };
@@ -1278,7 +1243,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 // host: the layout (see the top of the file), one device block per instance
 // ---------------------------------------------------------------------------
 // CTAs of an item's cluster
-static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 2 : n <= 98304 ? 4 : 8; }
+static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 4 : n <= 98304 ? 5 : 8; }
 
 bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::vector<int32_t> &next,
                          const std::vector<int32_t> &wpre, int64_t total_weight, int32_t max_weight,
@@ -1340,6 +1305,8 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
         else if (bin[p] == bin[i]) level[p] = std::max(level[p], level[i] + 1);
         if (heavy[p] != i && acc[p] < 0) acc[p] = R.nacc[bin[p]]++;
     }
+    for (int b = 0; b <= CL; ++b)
+        if (R.nacc[b] >= kNone) return false;
     // path tops grouped by (bin, level)
     const int nl = maxlev + 1;
     if (nl > kMaxLevels) return false;
@@ -1360,24 +1327,40 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
         for (int32_t i = 0; i < n; ++i)
             if (path_top(i)) tops[at[(size_t)bin[i] * nl + level[i]]++] = i;
     }
-    R.slot.reserve((size_t)n + 32 * 64);
+    R.info.reserve((size_t)n + 32 * 64);
+    R.pos.reserve((size_t)n + 32 * 64);
     std::vector<int32_t> path;
     for (int b = 0; b <= CL; ++b) {
-        R.binslot.push_back((int32_t)R.slot.size());
+        R.binslot.push_back((int32_t)R.info.size());
         R.binlev.push_back((int32_t)R.lev.size());
         int levels = nl;
         while (levels > 0 && rows[(size_t)b * nl + levels - 1] == 0) --levels;
         for (int l = 0; l < levels; ++l) {
             const size_t q = (size_t)b * nl + l;
             R.lev.push_back((int32_t)R.stream.size());
-            // streams of about equal length, one per warp of the CTA when there are rows for all
-            const int ns = std::max(1, std::min(kWarps, (rows[q] + 31) / 32));
-            const int want = (rows[q] + ns - 1) / ns;
-            int in_stream = 0, tile0 = (int)(R.slot.size() / 32);
+            // streams, at most one per warp of the CTA: the fewest tiles each
+            // (one, where the level has rows for no more) that take every path,
+            // next fit; a longer path has a stream of its own
+            int room = (rows[q] + 32 * kWarps - 1) / (32 * kWarps) * 32;
+            for (;; room += 32) {
+                int streams = 0, used = room + 1;
+                for (int x = start[q]; x < start[q + 1] && streams <= kWarps; ++x) {
+                    if (used + len[tops[x]] > room) {
+                        ++streams;
+                        used = 0;
+                    }
+                    used += len[tops[x]];
+                }
+                if (streams <= kWarps) break;
+            }
+            int in_stream = 0, tile0 = (int)(R.info.size() / 32);
             auto close = [&] {
                 if (in_stream == 0) return;
-                while (R.slot.size() % 32) R.slot.push_back({-1, 0, -1, -1});
-                const int tile1 = (int)(R.slot.size() / 32);
+                while (R.info.size() % 32) {
+                    R.info.push_back({0, kNone | (int)((unsigned)kNone << 16)});
+                    R.pos.push_back(-1);
+                }
+                const int tile1 = (int)(R.info.size() / 32);
                 R.stream.push_back({tile0, tile1 - tile0});
                 tile0 = tile1;
                 in_stream = 0;
@@ -1386,36 +1369,47 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
                 const int topn = tops[x];
                 path.clear();
                 for (int v = topn; v >= 0; v = heavy[v]) path.push_back(v);
-                int first = (int)R.slot.size();            // the path's first slot
+                if (in_stream > 0 && in_stream + (int)path.size() > room) close();
+                int first = (int)R.info.size();            // the path's first slot
                 for (int y = (int)path.size() - 1; y >= 0; --y) {
                     const int v = path[y];
-                    const int s = (int)R.slot.size(), t0 = s & ~31;
+                    const int s = (int)R.info.size(), t0 = s & ~31;
                     int code = (s - std::max(first, t0)) | (first < t0 ? kCont : 0) | (v == topn ? kTop : 0) |
                                (wpre[v] << kWeightShift);
-                    int pr = -1;
-                    if (v == topn && par[v] >= 0)
-                        pr = bin[par[v]] == bin[v] ? acc[par[v]] : -2 - acc[par[v]];
-                    R.slot.push_back({v, code, acc[v], pr});
+                    int up = kNone;
+                    if (v == topn && par[v] >= 0) {
+                        up = acc[par[v]];
+                        if (bin[par[v]] != bin[v]) code |= kUp;
+                    }
+                    R.info.push_back({code, (acc[v] < 0 ? kNone : acc[v]) | (int)((unsigned)up << 16)});
+                    R.pos.push_back(v);
                 }
                 in_stream += (int)path.size();
-                if (in_stream >= want) close();
             }
             close();
         }
         R.lev.push_back((int32_t)R.stream.size());
     }
-    R.binslot.push_back((int32_t)R.slot.size());
+    R.binslot.push_back((int32_t)R.info.size());
     R.binlev.push_back((int32_t)R.lev.size());
+    // a warp's tiles have to fit its list
+    for (int b = 0; b < CL; ++b)
+        for (int w = 0; w < kWarps; ++w) {
+            int tiles = 0;
+            for (int l = R.binlev[b]; l + 1 < R.binlev[b + 1]; ++l)
+                if (R.lev[l] + w < R.lev[l + 1]) tiles += R.stream[R.lev[l] + w].tiles;
+            if (tiles > kMaxTiles) return false;
+        }
     R.CL = CL;
     return true;
 }
 
 static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// device block: slots | streams | levels | binlev | binslot | nacc
+// device block: info | positions | streams | levels | binlev | binslot | nacc
 size_t reduce_tables_bytes(const ReduceTables &R)
 {
-    return al(R.slot.size() * 16) + al(R.stream.size() * 8) + al(R.lev.size() * 4) + al(R.binlev.size() * 4) +
+    return al(R.info.size() * 8) + al(R.info.size() * 4) + al(R.stream.size() * 8) + al(R.lev.size() * 4) + al(R.binlev.size() * 4) +
            al(R.binslot.size() * 4) + al(R.nacc.size() * 4);
 }
 
@@ -1425,7 +1419,8 @@ void reduce_tables_pack(const ReduceTables &R, char *dst)
         std::memcpy(dst, src, bytes);
         dst += al(bytes);
     };
-    put(R.slot.data(), R.slot.size() * 16);
+    put(R.info.data(), R.info.size() * 8);
+    put(R.pos.data(), R.info.size() * 4);
     put(R.stream.data(), R.stream.size() * 8);
     put(R.lev.data(), R.lev.size() * 4);
     put(R.binlev.data(), R.binlev.size() * 4);
@@ -1447,7 +1442,8 @@ static Tab device_tab(const pp_instance *inst)
     t.CL = r.CL;
     t.nslots = r.nslots;
     t.ntop = r.ntop;
-    t.slot = (const int4 *)take((size_t)r.nslots * 16);
+    t.info = (const int2 *)take((size_t)r.nslots * 8);
+    t.pos = (const int *)take((size_t)r.nslots * 4);
     t.stream = (const int2 *)take((size_t)r.nstreams * 8);
     t.lev = (const int *)take((size_t)r.nlev * 4);
     t.binlev = (const int *)take((size_t)(r.CL + 2) * 4);
@@ -1460,13 +1456,13 @@ ReduceShape reduce_shape(const ReduceTables &R)
 {
     ReduceShape s;
     s.CL = R.CL;
-    s.nslots = (int)R.slot.size();
+    s.nslots = (int)R.info.size();
     s.nstreams = (int)R.stream.size();
     s.nlev = (int)R.lev.size();
     s.ntop = R.nacc[R.CL];
     s.max_kids = R.max_kids;
     s.max_acc = *std::max_element(R.nacc.begin(), R.nacc.end() - 1);
-    s.acc_smem = up16((size_t)(s.max_acc + 1) * kAccBytes) + kBins * 4 <= (size_t)(192 << 10);
+    s.acc_smem = up16((size_t)(s.max_acc + 1) * kAccBytes) + kRingBytes + kBins * 4 <= (size_t)(192 << 10);
     return s;
 }
 
@@ -1498,7 +1494,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.total_weight = inst->total_weight;
     a.max_weight = inst->max_weight;
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
-    const size_t scan = (r.acc_smem ? up16((size_t)(r.max_acc + 1) * kAccBytes) : 0) + kBins * 4;
+    const size_t scan = (r.acc_smem ? up16((size_t)(r.max_acc + 1) * kAccBytes) : 0) + kRingBytes + kBins * 4;
     const size_t smem = std::max(scan, up16(sizeof(Rows)) + kPool);
     const auto kern = r.acc_smem ? k_reduce<true> : k_reduce<false>;
     PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

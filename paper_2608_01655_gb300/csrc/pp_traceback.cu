@@ -5,6 +5,8 @@
 // offset c, the 8-byte word ((item * P + g) * nblk / 2 + r / 64) * C + c) * 32
 // + lane holds the take decisions of kept rows r (sweep order, 64 rows, bit
 // r % 64) at column (g * 32 + lane) * C + c + 1.
+#include <algorithm>
+
 #include "pp_internal.cuh"
 
 namespace pp {
@@ -135,6 +137,10 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
     const int item = blockIdx.x;
     const int bi = acc.bits_item ? acc.bits_item[item] : item;   // the DP item whose bits this walks
     const int state = w.red ? w.red[bi] : 0;   // of the reduction: 1 its set is a bitmap, 2 joins the walk's
+    // (only a bitmap is spread over the CTAs of an item)
+    const int part = state == 1 ? blockIdx.y : 0, parts = state == 1 ? gridDim.y : 1;
+    if (state != 1 && blockIdx.y) return;
+    const int32_t x0 = part * blockDim.x + threadIdx.x, dx = parts * blockDim.x;
     uint32_t hbit = 0;
     uint32_t *M = nullptr;
     if (acc.mask) {
@@ -151,12 +157,17 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
             for (int32_t x = threadIdx.x; x < n; x += blockDim.x) atomicAnd(M + x, ~hbit);
     } else {
         uint8_t *ch = chosen + (size_t)item * n;
+        if (state == 1) {
+            const uint32_t *tk = w.taken + (size_t)bi * ((n + 31) / 32);
+            for (int32_t x = x0; x < n; x += dx) ch[order[x]] = (tk[x >> 5] >> (x & 31)) & 1u;
+            return;
+        }
         for (int32_t x = threadIdx.x; x < n; x += blockDim.x) ch[x] = 0;
     }
     if (state) {
         const uint32_t *tk = w.taken + (size_t)bi * ((n + 31) / 32);
         __syncthreads();                      // chosen[] is cleared
-        for (int32_t x = threadIdx.x; x < n; x += blockDim.x) {
+        for (int32_t x = x0; x < n; x += dx) {
             const bool in = (tk[x >> 5] >> (x & 31)) & 1u;
             if (BYNODE) {
                 if (in) chosen[(size_t)item * n + order[x]] = 1;
@@ -167,7 +178,7 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
             }
         }
         if (state == 1) {
-            if (acc.mask && !acc.greedy && threadIdx.x == 0) {
+            if (!acc.greedy && x0 == 0) {
                 acc.improved[item] = 1;
                 acc.accepted[item] += 1;
             }
@@ -341,8 +352,10 @@ pp_status launch_traceback(pp_instance *inst, int batch, const DpWork &work, con
     const int unit = inst->max_weight <= 1;
     const bool bynode = a.mask == nullptr;
     const int skips = inst->trace_skips >= 3 ? 3 : 1;
+    // CTAs per item to write out a set that the reduction has found: 8 chunks a thread
+    const int parts = work.red ? std::min(32, (inst->n + 2047) / 2048) : 1;
     auto go = [&](auto kern) {
-        kern<<<batch, 256, 0, st>>>(inst->n, work, g.C, g.P, g.kpad, item_budget, inst->d_order, chosen, a);
+        kern<<<dim3(batch, parts), 256, 0, st>>>(inst->n, work, g.C, g.P, g.kpad, item_budget, inst->d_order, chosen, a);
     };
     if (skips == 3) {
         if (bynode) unit ? go(k_traceback<3, true, true>) : go(k_traceback<3, true, false>);
