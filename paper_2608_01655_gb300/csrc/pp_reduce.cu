@@ -57,9 +57,9 @@ constexpr int kMaxLevels = 20;              // of a bin (heavy paths: log2 of it
 constexpr int kMaxEvals = 16;               // prices tried per item
 constexpr int kPasses = 4;                  // thresholds tried per item
 constexpr int kRowCap = 1024;               // undecided rows the on-chip DP takes
-constexpr int kFirstRows = 256;             // rows of the first threshold (by rank of the loss)
+constexpr int kFirstRows = 320;             // most rows of the first threshold
 constexpr int kColCap = 1024;               // its columns (budget left over)
-constexpr int kPool = 64 << 10;             // its decision bits, stack and row buffers, bytes
+constexpr int kPool = 96 << 10;             // its decisions, stack and row buffers, bytes
 constexpr int kKeyBase = (127 << 5) - 1;    // float bits >> 18 of 1.0, minus 1
 constexpr int kBins = 2048;                 // keys of 0 .. 2^62
 constexpr int kKeyPad = 0xffff;
@@ -672,7 +672,7 @@ struct __align__(16) Row {
     int w, info;                             // flags below, stack level << 8
 };
 struct Rows {                                // in sweep order (last position first)
-    Row row[kRowCap + 4];                    // (read four at a time)
+    Row row[kRowCap + 8];                    // (read up to eight at a time)
     int2 step[kRowCap];                      // the walk's: weight, row that a skip goes to (-1 past the last)
     int pos[kRowCap], last[kRowCap];
     unsigned leaf[kRowCap / 32];             // bit: a skip goes to the next row
@@ -724,12 +724,90 @@ __device__ __forceinline__ void dp_rows(const Rows &R, int T, int act, int guard
     if (kc == 1 + tid) *result = cur;
 }
 
+// Unit weights and at most 128 columns: one warp, C columns per lane (column
+// j = 1 + lane * C + c) in registers, the column shift a shuffle, no barrier:
+// 24 to 40 ns a row against 90 with a barrier per row.  Instead of decision
+// bits it keeps, per row and column, the first row taken from there on
+// (following skips changes nothing), so the walk takes one step per chunk.
+constexpr int kNoRow = 0xffff;
+constexpr int kUnitCols = 128;
+template <int C>
+__device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint16_t *stf, uint16_t *first,
+                                        int64_t *result, int kc)
+{
+    constexpr int cols = 32 * C;
+    const int lane = threadIdx.x & 31;
+    int64_t cur[C], top[C];
+    int fc[C], ft[C];                        // first row taken from the row just computed, from the top
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        cur[c] = top[c] = 0;
+        fc[c] = ft[c] = kNoRow;
+    }
+    constexpr int U = 4;                     // rows unrolled (no-op rows past the last)
+    constexpr int kOps = kPush | kReload | kZeroTop;
+    for (int r0 = 0; r0 < T; r0 += U) {
+        Row x[U];
+        int ops = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            x[u] = R.row[r0 + u];
+            ops |= x[u].info;
+        }
+        auto row = [&](const int u, const bool stack) {
+            int64_t up = __shfl_up_sync(kAll, cur[C - 1], 1);
+            up = lane ? up : 0;
+            const bool same = x[u].info & kFromCur;
+#pragma unroll
+            for (int c = C - 1; c >= 0; --c) {
+                const int64_t sk = same ? cur[c] : top[c];
+                const int64_t tv = x[u].p + (c ? cur[c > 0 ? c - 1 : 0] : up);
+                const bool take = tv > sk;
+                cur[c] = take ? tv : sk;
+                fc[c] = take ? r0 + u : same ? fc[c] : ft[c];
+            }
+            uint16_t *fo = first + (r0 + u) * cols + lane * C;
+            if (C == 4) *(uint2 *)fo = make_uint2(fc[0] | fc[C > 1 ? 1 : 0] << 16, fc[C > 2 ? 2 : 0] | fc[C > 3 ? 3 : 0] << 16);
+            else if (C == 2) *(unsigned *)fo = fc[0] | fc[C > 1 ? 1 : 0] << 16;
+            else *fo = (uint16_t)fc[0];
+            if (stack && (x[u].info & kOps)) {
+                const int at = (x[u].info >> 8) * cols + lane;       // (a lane's own cells: no exchange)
+                if (x[u].info & kPush) {
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        stk[at + 32 * c] = top[c] = cur[c];
+                        stf[at + 32 * c] = (uint16_t)(ft[c] = fc[c]);
+                    }
+                } else {
+                    const bool re = x[u].info & kReload;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        top[c] = re ? stk[at + 32 * c] : 0;
+                        ft[c] = re ? stf[at + 32 * c] : kNoRow;
+                    }
+                }
+            }
+        };
+        if ((ops & kOps) == 0) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) row(u, false);
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) row(u, true);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+        if (kc == 1 + lane * C + c) *result = cur[c];
+}
+
 }  // namespace
 
 template <bool SMEM>                         // accumulators of the bins in shared memory
 __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned char leaf[kWarps * kMaxTiles];   // tiles of level 0: see the gather
     __shared__ unsigned lists[3][kWarps][kMaxTiles];    // a warp's tiles: all; two that the search shortens in turn
     __shared__ int4 s_top[kMaxTop];          // the last bin's own sums, then what it passes down
     __shared__ int sh[kWarps];
@@ -788,10 +866,12 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         const int q = __ldg(t.lev + l0 + l) + warp;
         if (q >= __ldg(t.lev + l0 + l + 1)) continue;
         const int2 x = __ldg(t.stream + q);
-        for (int i = lane; i < x.y; i += 32)
-            lists[0][warp][tiles + i] = lists[1][warp][tiles + i] = ((unsigned)l << 16) + (unsigned)(x.x - (lo >> 5) + i);
+        for (int i = lane; i < x.y; i += 32) lists[0][warp][tiles + i] = ((unsigned)l << 16) + (unsigned)(x.x - (lo >> 5) + i);
         tiles += x.y;
     }
+    // the slots of level 0 (paths without light children) end here
+    const int leaf_end = nlev > 1 ? min(hi, __ldg(&t.stream[__ldg(t.lev + l0 + 1)].x) * 32) : hi;
+    for (int i = tid; i < (leaf_end - lo) >> 5; i += kThreads) leaf[i] = 0;
     sync_all();
 
     // ---- gather the profits into the slots; weights by profit per slot
@@ -817,6 +897,12 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 if (s >= to) break;
                 g.prof[s] = p[u];
                 mx = p[u] > mx ? p[u] : mx;
+                // a warp's slots are a tile; bit 0: no profit in it, bit 1: its
+                // first path comes from the tile before
+                if (!__any_sync(kAll, p[u] > 0) && s < leaf_end) {
+                    const bool cont = __any_sync(kAll, __ldg(&t.info[s].x) & kCont);
+                    if (lane == 0) leaf[(s - lo) >> 5] = cont ? 3 : 1;
+                }
                 if (p[u] > 0 && ((s >> 5) & ((1 << every) - 1)) == 0) {
                     const int w = __ldg(&t.info[s].x) >> kWeightShift;
                     const int c = w == 1 ? code_of(p[u]) : code_of((int64_t)((float)p[u] / (float)w));
@@ -838,6 +924,25 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         if (hist[i]) atomicAdd(g.hist + i, hist[i]);
     sync_all();
     const int64_t maxp = (int64_t)__ldcg(&g.s->maxp);
+    {
+        // leaf tiles without a profit leave the lists: at any price nothing in
+        // them is taken (on the planner's later sweeps, most of the tree)
+        int kept = 0;
+        unsigned prev = 0;
+        bool pd = false;
+        for (int i = 0; i < tiles; ++i) {
+            const unsigned en = lists[0][warp][i];
+            const int fl = en >> 16 ? 0 : leaf[en];
+            const bool d = (fl & 1) && (!(fl & 2) || (pd && en == prev + 1));
+            __syncwarp();
+            if (d) g.key[lo + en * 32 + lane] = kKeyPad;
+            else if (lane == 0) lists[0][warp][kept] = lists[1][warp][kept] = en;
+            kept += !d;
+            pd = d;
+            prev = en;
+        }
+        tiles = kept;
+    }
     int *cum = (int *)hist;                  // weight of the codes >= c
     {
         constexpr int V = kBins / kThreads;
@@ -984,12 +1089,13 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     bool sure = false;           // the key comes from a V: no row above it is undecided
     if (!give_up) {
         int T = 0;
-        // first the rows whose loss is within a tenth of a slot's price (most
-        // gaps are), at most kFirstRows; none at price 0 (see kleft < 0 below)
+        // first the rows whose loss is within 0.15 of the price of a chunk's
+        // slots (most gaps are), at most kFirstRows; none at price 0 (see
+        // kleft < 0 below)
         if (lam == 0) {
             key = -1;
         } else {
-            T = up_to(kFirstRows, code_of(lam / 10), key);
+            T = up_to(kFirstRows, code_of((int64_t)(0.15f * (float)lam * ((float)A.total_weight / (float)n))), key);
         }
         for (; pass < kPasses; ++pass) {
             const bool big = T > kRowCap;                         // the same in every CTA
@@ -1136,22 +1242,38 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                     const int guard = min(A.max_weight, cols);
                     const int pitch = cols + 1 + guard;
                     const size_t need = (size_t)2 * pitch * 8 + (size_t)levels * cols * 8 + (size_t)((T + 31) / 32) * cols * 4;
-                    if (kc > kColCap || need > (size_t)kPool) {
+                    const int C = kc <= 32 ? 1 : kc <= 64 ? 2 : 4;   // columns per lane of the one-warp kernel
+                    const size_t uneed = (size_t)levels * 32 * C * 10 + (size_t)(T + 4) * 32 * C * 2;
+                    const bool unit = A.max_weight == 1 && kc <= kUnitCols && uneed <= (size_t)kPool;
+                    const int ucols = 32 * C;
+                    if (kc > kColCap || (!unit && need > (size_t)kPool)) {
                         out = sure ? 4 : 3;
                     } else {
                         int64_t *rowb = (int64_t *)pool;             // [2][guard + 1 + cols]
                         int64_t *stk = rowb + 2 * pitch;             // [levels][cols]
                         uint32_t *bits = (uint32_t *)(stk + (size_t)levels * cols);   // [T / 32][cols]
+                        int64_t *ustk = (int64_t *)pool;             // [levels][ucols]
+                        uint16_t *first = (uint16_t *)(ustk + (size_t)levels * ucols);       // [T][ucols]
+                        uint16_t *stf = first + (size_t)(T + 4) * ucols;     // [levels][ucols]
+                        if (!unit) {
+                            for (int i = tid; i < 2 * pitch; i += kThreads) rowb[i] = i % pitch < guard ? -2 * kBig : 0;
+                            for (int r = tid; r < T; r += kThreads)
+                                if (R.row[r].w > cols) R.row[r].w = cols + 1;    // never fits: column 0's guard
+                        }
                         if (tid == 0) s_val = 0;
                         if (tid < 4) {
-                            R.row[T + tid].p = 0;
-                            R.row[T + tid].w = R.row[T + tid].info = 0;
+                            R.row[T + tid].p = -kBig;                // no-op rows: never taken
+                            R.row[T + tid].w = 0;
+                            R.row[T + tid].info = kFromCur;
                         }
-                        for (int i = tid; i < 2 * pitch; i += kThreads) rowb[i] = i % pitch < guard ? -2 * kBig : 0;
-                        for (int r = tid; r < T; r += kThreads)
-                            if (R.row[r].w > cols) R.row[r].w = cols + 1;    // never fits: column 0's guard
                         __syncthreads();
-                        if (warp < act) dp_rows(R, T, act, guard, rowb, stk, bits, &s_val, kc);
+                        if (!unit) {
+                            if (warp < act) dp_rows(R, T, act, guard, rowb, stk, bits, &s_val, kc);
+                        } else if (warp == 0) {
+                            if (C == 1) dp_unit<1>(R, T, ustk, stf, first, &s_val, kc);
+                            else if (C == 2) dp_unit<2>(R, T, ustk, stf, first, &s_val, kc);
+                            else dp_unit<4>(R, T, ustk, stf, first, &s_val, kc);
+                        }
                         __syncthreads();
                         const int64_t V = vfix + s_val;
                         // at price 0 with |S| <= k, S is Eq. 9's set: a chunk is
@@ -1163,23 +1285,34 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                             // next row that is taken or whose skip is no leaf's
                             if (tid == 0) {
                                 int r = T - 1, j = kc;
-                                while (r >= 0 && j > 0) {
+                                int m = 0;                   // rows taken, listed in R.last
+                                while (unit && r >= 0 && j > 0) {
+                                    const int f = first[r * ucols + j - 1];
+                                    if (f == kNoRow) break;
+                                    R.last[m++] = f;
+                                    r = f - 1;
+                                    --j;
+                                }
+                                while (!unit && r >= 0 && j > 0) {
                                     const int blk = r >> 5;
                                     const uint32_t word = bits[blk * cols + j - 1];
                                     const uint32_t cand = (word | ~R.leaf[blk]) & (0xffffffffu >> (31 - (r & 31)));
                                     const int rr = (r & ~31) + 31 - __clz((int)cand);      // below the block if none
                                     const int2 st = R.step[max(rr, 0)];
                                     const bool none = cand == 0, take = (cand & word) >> (rr & 31) & 1u;
-                                    if (!none && take) {
-                                        const int x = R.pos[rr];
-                                        atomicOr(taken + (x >> 5), 1u << (x & 31));
-                                    }
+                                    if (!none && take) R.last[m++] = rr;
                                     j -= !none && take ? st.x : 0;
                                     r = none || take ? rr - !none : st.y;
                                 }
+                                s_a = m;
                                 A.best[item] = V;
                                 A.w.nkept[item] = T;
                                 if (A.rows_kept) atomicAdd(A.rows_kept, (unsigned long long)T);
+                            }
+                            __syncthreads();
+                            for (int i = tid; i < s_a; i += kThreads) {
+                                const int x = R.pos[R.last[i]];
+                                atomicOr(taken + (x >> 5), 1u << (x & 31));
                             }
                         } else {
                             out = 5;
@@ -1243,7 +1376,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 // host: the layout (see the top of the file), one device block per instance
 // ---------------------------------------------------------------------------
 // CTAs of an item's cluster
-static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 4 : n <= 98304 ? 5 : 8; }
+static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 4 : n <= 98304 ? 6 : 8; }
 
 bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::vector<int32_t> &next,
                          const std::vector<int32_t> &wpre, int64_t total_weight, int32_t max_weight,
