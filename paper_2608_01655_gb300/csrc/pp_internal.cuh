@@ -249,15 +249,18 @@ pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,
 pp_status launch_objective(pp_instance *inst, int batch, const uint32_t *mask,
                            const uint8_t *chosen, int64_t *obj, cudaStream_t st);
 
-// Top-2 holder tables of the source-dependent marginals, per start (batch item):
-// v1, v2, l1 [batch][W][n] and the pre-update bit of the current worker [batch][n].
+// Top-2 holder tables of the source-dependent marginals, per start (batch
+// item), for the holder masks `seen`; every worker's marginals, and which of
+// them are stale (bit per worker).
 struct Top2 {
-    int64_t *v1 = nullptr;
-    int64_t *v2 = nullptr;
-    int8_t *l1 = nullptr;
-    uint8_t *oldbit = nullptr;
+    int64_t *v1 = nullptr;       // [batch][W][n]
+    int64_t *v2 = nullptr;       // [batch][W][n]
+    int64_t *marg = nullptr;     // [batch][W][n]
+    uint32_t *seen = nullptr;    // [batch][n]
+    uint32_t *stale = nullptr;   // [batch][n]
+    int8_t *l1 = nullptr;        // [batch][W][n]
 };
-pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *prev_worker, const int32_t *worker,
+pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *worker,
                                 const uint32_t *mask, const int32_t *item_active, const Top2 &t2,
                                 int64_t *profit, int64_t *oldsum, cudaStream_t st);
 

@@ -142,68 +142,86 @@ pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,
 // g_{l,m}(i), l1 = the first holder reaching it, v2 = the largest value among
 // the other holders (0 with fewer than two).  Then
 //   max_{l in H_b \ h} g_{l,m}(b) = (l1 == h) ? v2 : v1,
-// which is exact also under ties (then v2 = v1).  The marginal kernel records
-// each chunk's bit h before the update, and the next step's marginal pass
-// first applies the change of exactly the chunks whose bit h changed.
+// which is exact also under ties (then v2 = v1).  The tables hold for the
+// holder masks `seen`; a marginal pass first applies the change of the chunks
+// whose mask differs (the step before changed one worker's bit).
+// A marginal depends on the other workers' holdings alone, so each worker's
+// marginals are kept (`marg`), with a bit per worker and chunk that says
+// which are stale: a changed chunk makes every worker's stale but the changed
+// one's.  After the greedy pass few are, and a pass reads 28 bytes a chunk
+// instead of 17 W.
 // ---------------------------------------------------------------------------
-// Apply worker h's change at chunk i to the top-2 tables (tb = the start's
-// table base): h joined -> insert its values; h left -> rebuild the entries
-// where it was the top holder or tied the second.
-__device__ __forceinline__ void top2_apply(int32_t n, int32_t W, int32_t h, int32_t i, uint32_t mk, bool now,
-                                           size_t tb, const int64_t *__restrict__ g, int64_t *__restrict__ v1,
-                                           int64_t *__restrict__ v2, int8_t *__restrict__ l1)
+// Apply worker h's change at chunk i to the top-2 entry of requester m (tb =
+// the start's table base): h joined -> insert its value; h left -> rebuild the
+// entry where it was the top holder or tied the second.
+__device__ __forceinline__ void top2_apply(int32_t n, int32_t W, int32_t h, int32_t m, int32_t i, uint32_t mk, bool now,
+                                           size_t tb, const int64_t *__restrict__ g, const Top2 &t)
 {
-    for (int32_t m = 0; m < W; ++m) {
-        const size_t q = tb + (size_t)m * n + i;
-        const int64_t x = g[((size_t)h * W + m) * n + i];
-        if (now) {
-            if (l1[q] < 0 || x > v1[q]) {
-                v2[q] = l1[q] < 0 ? 0 : v1[q];
-                v1[q] = x;
-                l1[q] = (int8_t)h;
-            } else if (x > v2[q]) {
-                v2[q] = x;
-            }
-            continue;
+    const size_t q = tb + (size_t)m * n + i;
+    const int64_t x = g[((size_t)h * W + m) * n + i], a = t.v1[q], b = t.v2[q];
+    const int l1 = t.l1[q];
+    if (now) {
+        if (l1 < 0 || x > a) {
+            t.v2[q] = l1 < 0 ? 0 : a;
+            t.v1[q] = x;
+            t.l1[q] = (int8_t)h;
+        } else if (x > b) {
+            t.v2[q] = x;
         }
-        if (l1[q] != h && x < v2[q]) continue;
-        int64_t b1 = 0, b2 = 0;
-        int id1 = -1;
-        uint32_t o = mk;
-        while (o) {
-            const int l = __ffs(o) - 1;
-            o &= o - 1;
-            const int64_t y = g[((size_t)l * W + m) * n + i];
-            if (id1 < 0 || y > b1) {
-                b2 = id1 < 0 ? 0 : b1;
-                b1 = y;
-                id1 = l;
-            } else if (y > b2) {
-                b2 = y;
-            }
-        }
-        v1[q] = b1;
-        v2[q] = b2;
-        l1[q] = (int8_t)id1;
+        return;
     }
+    if (l1 != h && x < b) return;
+    int64_t b1 = 0, b2 = 0;
+    int id1 = -1;
+    for (uint32_t o = mk; o;) {
+        constexpr int U = 4;                 // holders whose loads are in flight
+        int id[U];
+        int64_t y[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            id[u] = o ? __ffs(o) - 1 : -1;
+            o &= o - 1;
+            if (id[u] >= 0) y[u] = g[((size_t)id[u] * W + m) * n + i];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (id[u] < 0) break;
+            if (id1 < 0 || y[u] > b1) {
+                b2 = id1 < 0 ? 0 : b1;
+                b1 = y[u];
+                id1 = id[u];
+            } else if (y[u] > b2) {
+                b2 = y[u];
+            }
+        }
+    }
+    t.v1[q] = b1;
+    t.v2[q] = b2;
+    t.l1[q] = (int8_t)id1;
 }
 
-// prev_worker (optional): the worker of the start's previous step, whose
-// change is applied to the tables first (the bit recorded then vs the mask now)
-__global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W,
-                                                         const int32_t *__restrict__ prev_worker,
-                                                         const int32_t *__restrict__ worker,
+// requester m's share of worker h's marginal at chunk i
+__device__ __forceinline__ int64_t top2_share(int32_t n, int32_t W, int32_t h, int32_t m, int32_t i, size_t tb,
+                                              const int64_t *__restrict__ g, const Top2 &t)
+{
+    const size_t q = tb + (size_t)m * n + i;
+    const int64_t a = g[((size_t)h * W + m) * n + i], b = t.v1[q], c = t.v2[q];
+    const int64_t other = t.l1[q] == h ? c : b;
+    return a > other ? a - other : 0;
+}
+
+// A lane per chunk; a changed chunk's tables, and a stale marginal unless many
+// lanes have one, are the whole warp's work, a lane per requester: one lane
+// alone waited for memory W times (and W times per holder in a rebuild), which
+// was 53 us a pass whatever n.
+__global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W, const int32_t *__restrict__ worker,
                                                          const uint32_t *__restrict__ mask,
-                                                         const int64_t *__restrict__ g,
-                                                         int64_t *__restrict__ v1,
-                                                         int64_t *__restrict__ v2,
-                                                         int8_t *__restrict__ l1,
+                                                         const int64_t *__restrict__ g, Top2 t,
                                                          const int32_t *__restrict__ item_active,
-                                                         int64_t *__restrict__ profit,
-                                                         int64_t *__restrict__ oldsum,
-                                                         uint8_t *__restrict__ oldbit,
+                                                         int64_t *__restrict__ profit, int64_t *__restrict__ oldsum,
                                                          int32_t *__restrict__ status)
 {
+    constexpr unsigned kAllLanes = 0xffffffffu;
     const int item = blockIdx.y;
     if (item_active && !item_active[item]) return;
     const int32_t h = worker[item];
@@ -214,31 +232,54 @@ __global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W,
         for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) P[i] = 0;
         return;
     }
+    const int lane = threadIdx.x & 31;
     const size_t tb = (size_t)item * W * n;
-    const int32_t hp = prev_worker ? prev_worker[item] : -1;
+    int64_t *marg = t.marg + tb + (size_t)h * n;
+    uint32_t *seen = t.seen + (size_t)item * n, *stale = t.stale + (size_t)item * n;
     int64_t held = 0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t mk = M[i];
-        if (hp >= 0 && hp < W) {
-            const bool now = (mk >> hp) & 1u;
-            if (now != (bool)oldbit[(size_t)item * n + i]) top2_apply(n, W, hp, i, mk, now, tb, g, v1, v2, l1);
+    for (int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
+        const int32_t i = i0 + lane;
+        const bool in = i < n;
+        const uint32_t mk = in ? M[i] : 0, was = in ? seen[i] : 0, st = in ? stale[i] : 0;
+        int64_t p = in ? marg[i] : 0;
+        uint32_t s = st;
+        if (mk != was) {
+            seen[i] = mk;
+            s |= ~(mk ^ was);
         }
-        int64_t p = 0;
-        for (int32_t m = 0; m < W; ++m) {
-            const size_t o = tb + (size_t)m * n + i;
-            const int64_t other = l1[o] == h ? v2[o] : v1[o];
-            const int64_t mine = g[((size_t)h * W + m) * n + i];
-            p += mine > other ? mine - other : 0;
+        for (unsigned c = __ballot_sync(kAllLanes, mk != was); c; c &= c - 1) {
+            const int src = __ffs((int)c) - 1;
+            const uint32_t now = __shfl_sync(kAllLanes, mk, src), x = now ^ __shfl_sync(kAllLanes, was, src);
+            if (lane < W) top2_apply(n, W, __ffs(x) - 1, lane, i0 + src, now, (now & x) != 0, tb, g, t);
         }
-        P[i] = p;
-        const bool hh = (mk >> h) & 1u;
-        oldbit[(size_t)item * n + i] = hh;
-        if (hh) held += p;
+        __syncwarp();                        // the tables' new entries, before the shares below
+        const bool old = (s >> h) & 1u;
+        const unsigned c = __ballot_sync(kAllLanes, old);
+        if (__popc(c) <= 8) {
+            for (unsigned o = c; o; o &= o - 1) {
+                const int src = __ffs((int)o) - 1;
+                int64_t v = lane < W ? top2_share(n, W, h, lane, i0 + src, tb, g, t) : 0;
+#pragma unroll
+                for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(kAllLanes, v, q);
+                if (lane == src) p = v;
+            }
+        } else if (old) {
+            p = 0;
+#pragma unroll 4
+            for (int32_t m = 0; m < W; ++m) p += top2_share(n, W, h, m, i, tb, g, t);
+        }
+        if (old) {
+            marg[i] = p;
+            s &= ~(1u << h);
+        }
+        if (s != st) stale[i] = s;
+        if (in) P[i] = p;
+        if ((mk >> h) & 1u) held += p;
     }
     if (oldsum) block_add64(held, oldsum + item);
 }
 
-pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *prev_worker, const int32_t *worker,
+pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *worker,
                                 const uint32_t *mask, const int32_t *item_active, const Top2 &t2,
                                 int64_t *profit, int64_t *oldsum, cudaStream_t st)
 {
@@ -248,10 +289,8 @@ pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *pre
     int cap = (2 * inst->sm_count * 8 + batch - 1) / batch;
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    k_marginals_top2<<<dim3(bx, batch), 256, 0, st>>>(inst->n, inst->W, prev_worker, worker, mask, inst->d_g,
-                                                      t2.v1, t2.v2,
-                                                      t2.l1, item_active, profit, oldsum, t2.oldbit,
-                                                      inst->d_status);
+    k_marginals_top2<<<dim3(bx, batch), 256, 0, st>>>(inst->n, inst->W, worker, mask, inst->d_g, t2, item_active,
+                                                      profit, oldsum, inst->d_status);
     PP_CUDA(cudaGetLastError());
     return PP_OK;
 }

@@ -16,8 +16,10 @@
 namespace pp {
 
 // automatic choice of the top-2 marginals: whenever the tables (17 bytes per
-// start, requester and chunk) fit in this much device memory
-constexpr size_t kTop2MaxBytes = (size_t)16 << 30;
+// start, requester and chunk, and 8 per start, worker and chunk for the kept
+// marginals) fit in this much device memory
+constexpr size_t kTop2MaxBytes = (size_t)24 << 30;
+constexpr size_t kTop2Bytes = 17 + 8;
 
 // per-sweep bookkeeping: a start that accepted nothing is done
 __global__ void k_sweep_end(int S, int32_t *active, int32_t *improved, int32_t *sweeps)
@@ -244,20 +246,27 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     const int mreq = stats ? stats->marginals : 0;
     if (mreq < 0 || mreq > 2) return fail(PP_EINVAL, "stats->marginals must be 0, 1 or 2");
     const bool use_top2 = inst->mode == PP_TRANSFER_SOURCE && n > 0 &&
-                          (mreq == 2 || (mreq == 0 && (size_t)S * W * n * 17 <= kTop2MaxBytes));
+                          (mreq == 2 || (mreq == 0 && (size_t)S * W * n * kTop2Bytes <= kTop2MaxBytes));
     Top2 t2;
     if (use_top2) {
-        const size_t tw = (size_t)S * W * n, a = 255;
-        const size_t b1 = (8 * tw + a) & ~a, b2 = b1 + ((8 * tw + a) & ~a), b3 = b2 + ((tw + a) & ~a);
-        if ((s = ensure_scratch(inst->top2, b3 + (size_t)S * n))) return s;
+        const size_t tw = (size_t)S * W * n, sn = (size_t)S * n;
+        if ((s = ensure_scratch(inst->top2, 3 * align_up(8 * tw) + 2 * align_up(4 * sn) + align_up(tw)))) return s;
         char *base = reinterpret_cast<char *>(inst->top2.ptr);
-        t2.v1 = reinterpret_cast<int64_t *>(base);
-        t2.v2 = reinterpret_cast<int64_t *>(base + b1);
-        t2.l1 = reinterpret_cast<int8_t *>(base + b2);
-        t2.oldbit = reinterpret_cast<uint8_t *>(base + b3);
-        PP_CUDA(cudaMemsetAsync(base, 0, b2, st));                 // v1 = v2 = 0: no holders yet
-        PP_CUDA(cudaMemsetAsync(t2.l1, 0xFF, tw, st));             // l1 = -1
-        PP_CUDA(cudaMemsetAsync(t2.oldbit, 0, (size_t)S * n, st)); // nobody holds anything yet
+        auto carve = [&](size_t bytes) {
+            char *q = base;
+            base += align_up(bytes);
+            return q;
+        };
+        t2.v1 = reinterpret_cast<int64_t *>(carve(8 * tw));
+        t2.v2 = reinterpret_cast<int64_t *>(carve(8 * tw));
+        t2.seen = reinterpret_cast<uint32_t *>(carve(4 * sn));
+        t2.stale = reinterpret_cast<uint32_t *>(carve(4 * sn));
+        t2.l1 = reinterpret_cast<int8_t *>(carve(tw));
+        t2.marg = reinterpret_cast<int64_t *>(carve(8 * tw));
+        // v1 = v2 = 0 and no masks seen: nobody holds anything yet; l1 = -1 and
+        // every marginal stale
+        PP_CUDA(cudaMemsetAsync(t2.v1, 0, (char *)t2.stale - (char *)t2.v1, st));
+        PP_CUDA(cudaMemsetAsync(t2.stale, 0xFF, (char *)t2.marg - (char *)t2.stale, st));
     }
     PP_CUDA(cudaMemsetAsync(pb.improved, 0, 4 * S, st));
     // The first greedy update of every start runs against an empty placement,
@@ -304,7 +313,6 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     int32_t start_steps = 0;            // per-start streams: updates launched per start
     std::vector<std::vector<cudaEvent_t>> sev;   // per-start streams: each start's phase events
     if (lockstep) {
-        const int32_t *prev_wk = nullptr;     // top-2: worker of the previous step, per start
         auto step = [&](int t, int greedy) -> pp_status {
             const int32_t *wk = pb.work + (size_t)t * B;
             const int32_t *kb = pb.kbud + (size_t)t * B;
@@ -312,8 +320,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
             if ((r = mark())) return r;
             if (use_top2) {
                 // the previous step's change is folded into this step's marginal pass
-                r = launch_marginals_top2(inst, S, prev_wk, wk, pb.mask, pb.active, t2, pb.profit, pb.oldsum, st);
-                prev_wk = wk;
+                r = launch_marginals_top2(inst, S, wk, pb.mask, pb.active, t2, pb.profit, pb.oldsum, st);
             } else {
                 r = launch_marginals(inst, S, wk, pb.mask, false, pb.active, pb.profit, pb.oldsum, st);
             }
@@ -342,7 +349,6 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         for (int32_t t = 0; t < W; ++t) {
             if (t == 0 && reuse) {
                 if ((s = first_from_standalone())) return s;
-                prev_wk = pb.work;        // top-2: step 0's change is folded in at step 1
                 continue;
             }
             if ((s = step(t, 1))) return s;
@@ -392,7 +398,6 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         if (reuse && (s = first_from_standalone())) return s;     // on the caller's stream, before the fork
         PP_CUDA(cudaEventRecord(inst->plan_fork, st));
         for (int x = 0; x < NS; ++x) PP_CUDA(cudaStreamWaitEvent(inst->plan_streams[x], inst->plan_fork, 0));
-        std::vector<const int32_t *> prev(S, nullptr);
         sev.resize(timing ? ngroups : 0);
         auto smark = [&](int x, cudaStream_t sx) -> pp_status {
             if (!timing) return PP_OK;
@@ -406,10 +411,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         const size_t N = (size_t)std::max(n, 1);
         for (int q = 0; q < W * (1 + R); ++q) {
             const int pass = q / W, t = q % W;
-            if (q == 0 && reuse) {
-                for (int x = 0; x < S; ++x) prev[x] = pb.work + x;    // top-2: folded in at step 1
-                continue;
-            }
+            if (q == 0 && reuse) continue;
             for (int q0 = 0; q0 < ngroups; ++q0) {
                 const int x = q0 * gs, b = std::min(gs, S - x);       // starts x .. x + b - 1
                 cudaStream_t sx = inst->plan_streams[q0 % NS];
@@ -423,9 +425,10 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                     tx.v1 += (size_t)x * W * N;
                     tx.v2 += (size_t)x * W * N;
                     tx.l1 += (size_t)x * W * N;
-                    tx.oldbit += (size_t)x * N;
-                    s = launch_marginals_top2(inst, b, prev[x], wk, mk, pb.active + x, tx, pf, pb.oldsum + x, sx);
-                    prev[x] = wk;
+                    tx.marg += (size_t)x * W * N;
+                    tx.seen += (size_t)x * N;
+                    tx.stale += (size_t)x * N;
+                    s = launch_marginals_top2(inst, b, wk, mk, pb.active + x, tx, pf, pb.oldsum + x, sx);
                 } else {
                     s = launch_marginals(inst, b, wk, mk, false, pb.active + x, pf, pb.oldsum + x, sx);
                 }
