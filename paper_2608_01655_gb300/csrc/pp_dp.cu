@@ -203,6 +203,8 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
 {
     using namespace wavecfg;
     extern __shared__ __align__(16) unsigned char smem[];
+    chain_wait();
+    chain_release();
     const int CL = (int)cluster_nctarank();
     const int cr = (int)cluster_ctarank();
     int item = blockIdx.x / CL;
@@ -553,6 +555,8 @@ k_tree_dp_flat(int32_t n, DpWork work, const int32_t *__restrict__ wpre,
                int64_t *__restrict__ gstack, int L_smem, int L_glob, int32_t *__restrict__ status)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    chain_wait();
+    chain_release();
     const int TB = blockDim.x;                                  // threads of the bit layout
     const int t = threadIdx.x;
     const int lane = t & 31, warp = t >> 5;
@@ -783,6 +787,8 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
         int32_t *__restrict__ status, unsigned long long *__restrict__ rows_kept)
 {
     constexpr int V = 4;
+    chain_wait();
+    chain_release();
     __shared__ int sh[32];
     __shared__ int slot, bcast[2];
     const int CL = (int)cluster_nctarank(), cr = (int)cluster_ctarank();
@@ -1300,9 +1306,8 @@ static pp_status launch_flat_c(pp_instance *inst, int batch, const int32_t *item
                                const DpWork &work, int64_t *gstack, int L_glob, cudaStream_t st)
 {
     PP_CUDA(cudaFuncSetAttribute(k_tree_dp_flat<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
-    k_tree_dp_flat<C><<<batch, g.T, g.smem, st>>>(inst->n, work, inst->d_wpre, item_budget, max_budget,
-                                                   item_active, best, gstack, g.L_smem, L_glob, inst->d_status);
-    PP_CUDA(cudaGetLastError());
+    PP_CUDA(launch_chained(k_tree_dp_flat<C>, dim3(batch), dim3(g.T), g.smem, st, 1, inst->n, work, inst->d_wpre,
+                           item_budget, max_budget, item_active, best, gstack, g.L_smem, L_glob, inst->d_status));
     return PP_OK;
 }
 
@@ -1323,29 +1328,14 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
         if (s != PP_OK) return s;
     }
     {
-        cudaLaunchConfig_t pc = {};
-        pc.gridDim = dim3(kPruneCluster * batch);
-        pc.blockDim = dim3(1024);
-        pc.stream = st;
-        cudaLaunchAttribute pa[1];
-        pa[0].id = cudaLaunchAttributeClusterDimension;
-        pa[0].val.clusterDim.x = kPruneCluster;
-        pa[0].val.clusterDim.y = 1;
-        pa[0].val.clusterDim.z = 1;
-        pc.attrs = pa;
-        pc.numAttrs = 1;
         const int32_t *ord = inst->d_order, *nxt = inst->d_next, *wp = inst->d_wpre;
         const int2 *psp = inst->d_pspan;
         const int pr = !inst->tune_noprune, sd = inst->stack_depth;
         int32_t *stt = inst->d_status;
-        if (by_node)
-            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<true>, inst->n, profit, ord, nxt, psp, wp, item_active,
-                                       work, pr, sd, stt, rows_kept));
-        else
-            PP_CUDA(cudaLaunchKernelEx(&pc, k_prune<false>, inst->n, profit, ord, nxt, psp, wp, item_active,
-                                       work, pr, sd, stt, rows_kept));
+        PP_CUDA(launch_chained(by_node ? k_prune<true> : k_prune<false>, dim3(kPruneCluster * batch), dim3(1024), 0, st,
+                               kPruneCluster, inst->n, profit, ord, nxt, psp, wp, item_active, work, pr, sd, stt,
+                               rows_kept));
     }
-    PP_CUDA(cudaGetLastError());
     uint32_t *bits = work.bits;
     const int32_t *nkept = work.nkept;
     if (g.wave) {
@@ -1365,13 +1355,15 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
             cfg.blockDim = dim3(WPC * 32);
             cfg.dynamicSmemBytes = smem;
             cfg.stream = s;
-            cudaLaunchAttribute attr[1];
+            cudaLaunchAttribute attr[2];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = CL;
             attr[0].val.clusterDim.y = 1;
             attr[0].val.clusterDim.z = 1;
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
             cfg.attrs = attr;
-            cfg.numAttrs = 1;
+            cfg.numAttrs = g.split ? 1 : 2;              // (the halves of a split follow events)
             int32_t Lg = L_glob, ranked = g.split > 0;
             void *args[] = {&n, &nblk, (void *)&rowp, (void *)&rowm, (void *)&nkept, (void *)&item_budget,
                             &max_budget, (void *)&item_active, &best, &bits, &gstack, &L_smem, &Lg, &status,

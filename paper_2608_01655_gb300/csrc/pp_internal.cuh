@@ -115,6 +115,7 @@ struct DpWork {
     uint32_t *taken = nullptr;     // [batch][ceil(n / 32)] by preorder position
     uint32_t *undecided = nullptr; // [batch][ceil(n / 32)]
     char *red_scratch = nullptr;   // [batch][reduce_item_bytes]
+    int64_t *clear = nullptr;      // [batch] or null: zeroed by the reduction (the planner's next held sums)
 };
 size_t dp_work_bytes(const pp_instance *inst, int batch, int words);
 DpWork dp_work_split(const pp_instance *inst, void *base, int batch, int words);
@@ -199,6 +200,34 @@ struct pp_instance {
 };
 
 namespace pp {
+
+// Kernels of one update follow each other on a stream within microseconds:
+// each is launched while the one before still runs (programmatic dependent
+// launch), waits for it to be complete with chain_wait() before it touches
+// memory, and lets the next one be launched with chain_release().
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, int cluster, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // error reporting (thread-local message)
 pp_status fail(pp_status s, const std::string &msg);

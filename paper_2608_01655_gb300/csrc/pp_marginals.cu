@@ -64,7 +64,7 @@ __device__ __forceinline__ int64_t marginal_at(int32_t n, int32_t W, int32_t h, 
 
 // grid: (blocks over positions, batch).  BYNODE: masks / profits indexed by
 // node id (ABI); otherwise by preorder position (planner).  oldsum (optional)
-// receives sum of p_h over the chunks worker h currently holds, which equals
+// is added the sum of p_h over the chunks worker h currently holds, which equals
 // G(T) - G(T_-h, {}) by Prop. 1 and is the refinement's acceptance threshold.
 template <bool BYNODE, int MODE>
 __global__ void __launch_bounds__(256) k_marginals(int32_t n, int32_t W,
@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(256) k_marginals(int32_t n, int32_t W,
                                                     int64_t *__restrict__ oldsum,
                                                     int32_t *__restrict__ status)
 {
+    chain_wait();
+    chain_release();
     const int item = blockIdx.y;
     if (item_active && !item_active[item]) return;
     const int32_t h = worker[item];
@@ -102,19 +104,13 @@ __global__ void __launch_bounds__(256) k_marginals(int32_t n, int32_t W,
     if (oldsum) block_add64(held, oldsum + item);
 }
 
-template <bool BYNODE>
-static void marg_dispatch(pp_instance *inst, dim3 grid, int batch, const int32_t *worker,
-                          const uint32_t *mask, const int32_t *item_active, int64_t *profit,
-                          int64_t *oldsum, cudaStream_t st)
+template <bool BYNODE, int MODE>
+static cudaError_t marg_launch(pp_instance *inst, dim3 grid, const int32_t *worker, const uint32_t *mask,
+                               const int32_t *item_active, int64_t *profit, int64_t *oldsum, cudaStream_t st)
 {
-    if (inst->mode == 0)
-        k_marginals<BYNODE, 0><<<grid, 256, 0, st>>>(inst->n, inst->W, worker, mask, inst->d_order,
-                                                     inst->d_a, inst->d_delta, inst->d_g,
-                                                     item_active, profit, oldsum, inst->d_status);
-    else
-        k_marginals<BYNODE, 1><<<grid, 256, 0, st>>>(inst->n, inst->W, worker, mask, inst->d_order,
-                                                     inst->d_a, inst->d_delta, inst->d_g,
-                                                     item_active, profit, oldsum, inst->d_status);
+    return launch_chained(k_marginals<BYNODE, MODE>, grid, dim3(256), 0, st, 1, inst->n, inst->W, worker, mask,
+                          inst->d_order, inst->d_a, inst->d_delta, inst->d_g, item_active, profit, oldsum,
+                          inst->d_status);
 }
 
 pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,
@@ -122,15 +118,14 @@ pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,
                            int64_t *profit, int64_t *oldsum, cudaStream_t st)
 {
     if (batch <= 0 || inst->n == 0) return PP_OK;
-    if (oldsum) PP_CUDA(cudaMemsetAsync(oldsum, 0, sizeof(int64_t) * batch, st));
     int bx = (inst->n + 255) / 256;
     int cap = (2 * inst->sm_count * 8 + batch - 1) / batch;   // ~16 blocks per SM overall
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
     dim3 grid(bx, batch);
-    if (by_node) marg_dispatch<true>(inst, grid, batch, worker, mask, item_active, profit, oldsum, st);
-    else marg_dispatch<false>(inst, grid, batch, worker, mask, item_active, profit, oldsum, st);
-    PP_CUDA(cudaGetLastError());
+    const auto go = inst->mode == 0 ? (by_node ? marg_launch<true, 0> : marg_launch<false, 0>)
+                                    : (by_node ? marg_launch<true, 1> : marg_launch<false, 1>);
+    PP_CUDA(go(inst, grid, worker, mask, item_active, profit, oldsum, st));
     return PP_OK;
 }
 
@@ -222,6 +217,8 @@ __global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W, co
                                                          int32_t *__restrict__ status)
 {
     constexpr unsigned kAllLanes = 0xffffffffu;
+    chain_wait();
+    chain_release();
     const int item = blockIdx.y;
     if (item_active && !item_active[item]) return;
     const int32_t h = worker[item];
@@ -284,14 +281,12 @@ pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *wor
                                 int64_t *profit, int64_t *oldsum, cudaStream_t st)
 {
     if (batch <= 0 || inst->n == 0) return PP_OK;
-    if (oldsum) PP_CUDA(cudaMemsetAsync(oldsum, 0, sizeof(int64_t) * batch, st));
     int bx = (inst->n + 255) / 256;
     int cap = (2 * inst->sm_count * 8 + batch - 1) / batch;
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    k_marginals_top2<<<dim3(bx, batch), 256, 0, st>>>(inst->n, inst->W, worker, mask, inst->d_g, t2, item_active,
-                                                      profit, oldsum, inst->d_status);
-    PP_CUDA(cudaGetLastError());
+    PP_CUDA(launch_chained(k_marginals_top2, dim3(bx, batch), dim3(256), 0, st, 1, inst->n, inst->W, worker, mask,
+                           inst->d_g, t2, item_active, profit, oldsum, inst->d_status));
     return PP_OK;
 }
 

@@ -72,7 +72,7 @@ struct PlanBuffers {
     uint32_t *mask;      // [B][n]
     int64_t *profit;     // [B][n]
     int64_t *best;       // [B]
-    int64_t *oldsum;     // [B]
+    int64_t *oldsum;     // [2][B] held sums of the current update, and of the next (zero)
     int64_t *obj;        // [B]
     int32_t *active;     // [B]
     int32_t *improved;   // [B]
@@ -90,7 +90,7 @@ static pp_status plan_buffers(pp_instance *inst, int B, PlanBuffers *pb)
     const size_t n = (size_t)std::max(inst->n, 1);
     const int W = inst->W;
     size_t off[12], tot = 0;
-    const size_t sz[12] = {4 * n * B, 8 * n * B, 8 * (size_t)B, 8 * (size_t)B, 8 * (size_t)B,
+    const size_t sz[12] = {4 * n * B, 8 * n * B, 8 * (size_t)B, 16 * (size_t)B, 8 * (size_t)B,
                            4 * (size_t)B, 4 * (size_t)B, 4 * (size_t)B, 4 * (size_t)B,
                            4 * (size_t)(W + 1) * B, 4 * (size_t)(W + 1) * B, 8};
     for (int x = 0; x < 12; ++x) {
@@ -269,6 +269,18 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         PP_CUDA(cudaMemsetAsync(t2.stale, 0xFF, (char *)t2.marg - (char *)t2.stale, st));
     }
     PP_CUDA(cudaMemsetAsync(pb.improved, 0, 4 * S, st));
+    PP_CUDA(cudaMemsetAsync(pb.oldsum, 0, 16 * (size_t)B, st));
+    // The held sums of an update are added to by its marginal pass and read by
+    // its traceback; two sets alternate, and the reduction of an update zeroes
+    // the other set (without it, a memset does)
+    int parity = 0;
+    auto held_sums = [&](int first, int count, cudaStream_t sx, DpWork *w, int64_t **cur) -> pp_status {
+        *cur = pb.oldsum + (size_t)parity * B + first;
+        int64_t *other = pb.oldsum + (size_t)(parity ^ 1) * B + first;
+        if (w->red) w->clear = other;
+        else PP_CUDA(cudaMemsetAsync(other, 0, sizeof(int64_t) * count, sx));
+        return PP_OK;
+    };
     // The first greedy update of every start runs against an empty placement,
     // so its marginals and its DP are exactly the standalone-score DP of its
     // worker, computed above for the default orders: the start walks those
@@ -317,22 +329,26 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
             const int32_t *wk = pb.work + (size_t)t * B;
             const int32_t *kb = pb.kbud + (size_t)t * B;
             pp_status r;
+            DpWork wx = work;
+            int64_t *held = nullptr;
+            if ((r = held_sums(0, S, st, &wx, &held))) return r;
+            parity ^= 1;
             if ((r = mark())) return r;
             if (use_top2) {
                 // the previous step's change is folded into this step's marginal pass
-                r = launch_marginals_top2(inst, S, wk, pb.mask, pb.active, t2, pb.profit, pb.oldsum, st);
+                r = launch_marginals_top2(inst, S, wk, pb.mask, pb.active, t2, pb.profit, held, st);
             } else {
-                r = launch_marginals(inst, S, wk, pb.mask, false, pb.active, pb.profit, pb.oldsum, st);
+                r = launch_marginals(inst, S, wk, pb.mask, false, pb.active, pb.profit, held, st);
             }
             if (r) return r;
             if ((r = mark())) return r;
-            if ((r = launch_tree_dp(inst, S, pb.profit, false, kb, pb.active, g, pb.best, work, st, maxk, rows_kept)))
+            if ((r = launch_tree_dp(inst, S, pb.profit, false, kb, pb.active, g, pb.best, wx, st, maxk, rows_kept)))
                 return r;
             if ((r = mark())) return r;
             AcceptArgs a;
             a.worker = wk;
             a.best = pb.best;
-            a.oldsum = pb.oldsum;
+            a.oldsum = held;
             a.active = pb.active;
             a.improved = pb.improved;
             a.accepted = pb.accepted;
@@ -419,6 +435,9 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 const int32_t *kb = pb.kbud + (size_t)t * B + x;
                 uint32_t *mk = pb.mask + (size_t)x * N;
                 int64_t *pf = pb.profit + (size_t)x * N;
+                DpWork wx = dp_work_item(inst, work, x, g.words);
+                int64_t *held = nullptr;
+                if ((s = held_sums(x, b, sx, &wx, &held))) return s;
                 if ((s = smark(q0, sx))) return s;
                 if (use_top2) {
                     Top2 tx = t2;
@@ -428,13 +447,12 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                     tx.marg += (size_t)x * W * N;
                     tx.seen += (size_t)x * N;
                     tx.stale += (size_t)x * N;
-                    s = launch_marginals_top2(inst, b, wk, mk, pb.active + x, tx, pf, pb.oldsum + x, sx);
+                    s = launch_marginals_top2(inst, b, wk, mk, pb.active + x, tx, pf, held, sx);
                 } else {
-                    s = launch_marginals(inst, b, wk, mk, false, pb.active + x, pf, pb.oldsum + x, sx);
+                    s = launch_marginals(inst, b, wk, mk, false, pb.active + x, pf, held, sx);
                 }
                 if (s) return s;
                 if ((s = smark(q0, sx))) return s;
-                const DpWork wx = dp_work_item(inst, work, x, g.words);
                 if ((s = launch_tree_dp(inst, b, pf, false, kb, pb.active + x, g1, pb.best + x, wx, sx, maxk,
                                         rows_kept, x)))
                     return s;
@@ -442,7 +460,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 AcceptArgs a;
                 a.worker = wk;
                 a.best = pb.best + x;
-                a.oldsum = pb.oldsum + x;
+                a.oldsum = held;
                 a.active = pb.active + x;
                 a.improved = pb.improved + x;
                 a.accepted = pb.accepted + x;
@@ -457,6 +475,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                     launches += 1;
                 }
             }
+            parity ^= 1;
         }
         start_steps = W * (1 + R);
         for (int x = 0; x < NS; ++x) {

@@ -816,6 +816,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     const Tab &t = A.t;
     const int CL = t.CL, cr = CL > 1 ? cluster_rank() : 0;
     const int item = blockIdx.x / CL;
+    chain_wait();
+    if (A.w.clear && cr == 0 && threadIdx.x == 0) A.w.clear[item] = 0;
     const int n = t.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int32_t *red = A.w.red + item;
     if (A.item_active && !A.item_active[item]) return;      // uniform over the cluster
@@ -1349,6 +1351,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         }
     }
     const int state = verdict == 1 ? 1 : verdict == 4 ? 2 : 0;
+    chain_release();
     // ---- the decided "in" rows join the set
     if (state) {
         auto mark = [&](int a, int b) {
@@ -1631,19 +1634,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     const size_t smem = std::max(scan, up16(sizeof(Rows)) + kPool);
     const auto kern = r.acc_smem ? k_reduce<true> : k_reduce<false>;
     PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(r.CL * batch);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = r.CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    PP_CUDA(cudaLaunchKernelEx(&cfg, kern, a));
+    PP_CUDA(launch_chained(kern, dim3(r.CL * batch), dim3(kThreads), smem, st, r.CL, a));
     return PP_OK;
 }
 

@@ -134,6 +134,8 @@ k_traceback(int32_t n, DpWork w, int C, int P, int kpad,
             const int32_t *__restrict__ item_budget, const int32_t *__restrict__ order,
             uint8_t *__restrict__ chosen, AcceptArgs acc)
 {
+    chain_wait();
+    chain_release();
     const int item = blockIdx.x;
     const int bi = acc.bits_item ? acc.bits_item[item] : item;   // the DP item whose bits this walks
     const int state = w.red ? w.red[bi] : 0;   // of the reduction: 1 its set is a bitmap, 2 joins the walk's
@@ -354,8 +356,10 @@ pp_status launch_traceback(pp_instance *inst, int batch, const DpWork &work, con
     const int skips = inst->trace_skips >= 3 ? 3 : 1;
     // CTAs per item to write out a set that the reduction has found: 8 chunks a thread
     const int parts = work.red ? std::min(32, (inst->n + 2047) / 2048) : 1;
+    cudaError_t err = cudaSuccess;
     auto go = [&](auto kern) {
-        kern<<<dim3(batch, parts), 256, 0, st>>>(inst->n, work, g.C, g.P, g.kpad, item_budget, inst->d_order, chosen, a);
+        err = launch_chained(kern, dim3(batch, parts), dim3(256), 0, st, 1, inst->n, work, g.C, g.P, g.kpad, item_budget,
+                             inst->d_order, chosen, a);
     };
     if (skips == 3) {
         if (bynode) unit ? go(k_traceback<3, true, true>) : go(k_traceback<3, true, false>);
@@ -364,7 +368,7 @@ pp_status launch_traceback(pp_instance *inst, int batch, const DpWork &work, con
         if (bynode) unit ? go(k_traceback<1, true, true>) : go(k_traceback<1, true, false>);
         else unit ? go(k_traceback<1, false, true>) : go(k_traceback<1, false, false>);
     }
-    PP_CUDA(cudaGetLastError());
+    PP_CUDA(err);
     return PP_OK;
 }
 
