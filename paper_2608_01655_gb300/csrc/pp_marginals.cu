@@ -32,6 +32,32 @@ __device__ __forceinline__ void block_add64(int64_t v, int64_t *dst)
     }
 }
 
+// Values of kReq requesters at once, so that a thread has that many loads in
+// flight: one requester at a time, a thread waited for memory W times (1 + |H|)
+// (20,000 chunks, 16 workers, 8 items: 58 and 61 us for marginals and objective).
+constexpr int kReq = 8;
+// g_{l,m}(i) of the requesters m0 .. m0 + kReq - 1 (0 past the last)
+__device__ __forceinline__ void load_req(int32_t n, int32_t W, int32_t l, int32_t m0, int32_t i,
+                                         const int64_t *__restrict__ g, int64_t (&x)[kReq])
+{
+    const int64_t *q = g + ((size_t)l * W + m0) * n + i;
+#pragma unroll
+    for (int u = 0; u < kReq; ++u) x[u] = m0 + u < W ? __ldg(q + (size_t)u * n) : 0;
+}
+// their largest over the holders, 0 without one
+__device__ __forceinline__ void best_of(int32_t n, int32_t W, uint32_t holders, int32_t m0, int32_t i,
+                                        const int64_t *__restrict__ g, int64_t (&v)[kReq])
+{
+#pragma unroll
+    for (int u = 0; u < kReq; ++u) v[u] = 0;
+    for (uint32_t o = holders; o; o &= o - 1) {
+        int64_t x[kReq];
+        load_req(n, W, __ffs((int)o) - 1, m0, i, g, x);
+#pragma unroll
+        for (int u = 0; u < kReq; ++u) v[u] = x[u] > v[u] ? x[u] : v[u];
+    }
+}
+
 // Marginal of one chunk at preorder position i for worker h; `others` is the
 // holder mask without bit h.
 template <int MODE>
@@ -46,17 +72,12 @@ __device__ __forceinline__ int64_t marginal_at(int32_t n, int32_t W, int32_t h, 
         return p;
     } else {
         int64_t p = 0;
-        for (int32_t m = 0; m < W; ++m) {
-            int64_t mine = g[((size_t)h * W + m) * n + i];
-            int64_t v = 0;
-            uint32_t o = others;
-            while (o) {
-                int l = __ffs(o) - 1;
-                o &= o - 1;
-                int64_t x = g[((size_t)l * W + m) * n + i];
-                v = x > v ? x : v;
-            }
-            p += mine > v ? mine - v : 0;
+        for (int32_t m0 = 0; m0 < W; m0 += kReq) {
+            int64_t mine[kReq], v[kReq];
+            load_req(n, W, h, m0, i, g, mine);
+            best_of(n, W, others, m0, i, g, v);
+#pragma unroll
+            for (int u = 0; u < kReq; ++u) p += mine[u] > v[u] ? mine[u] - v[u] : 0;
         }
         return p;
     }
@@ -311,8 +332,14 @@ __global__ void __launch_bounds__(256) k_objective(int32_t n, int32_t W,
         uint32_t mk = 0;
         if (FROM_BYTES) {
             const int32_t b = order[i];
-            for (int32_t m = 0; m < W; ++m)
-                if (chosen[((size_t)item * W + m) * n + b]) mk |= 1u << m;
+            for (int32_t m0 = 0; m0 < W; m0 += kReq) {
+                uint8_t c[kReq];
+#pragma unroll
+                for (int u = 0; u < kReq; ++u)
+                    c[u] = m0 + u < W ? __ldg(chosen + ((size_t)item * W + m0 + u) * n + b) : 0;
+#pragma unroll
+                for (int u = 0; u < kReq; ++u) mk |= c[u] ? 1u << (m0 + u) : 0u;
+            }
         } else {
             mk = mask[(size_t)item * n + i];
         }
@@ -326,16 +353,11 @@ __global__ void __launch_bounds__(256) k_objective(int32_t n, int32_t W,
             }
             acc += delta[i];
         } else {
-            for (int32_t m = 0; m < W; ++m) {
-                int64_t best = 0;
-                uint32_t o = mk;
-                while (o) {
-                    int h = __ffs(o) - 1;
-                    o &= o - 1;
-                    int64_t x = g[((size_t)h * W + m) * n + i];
-                    best = x > best ? x : best;
-                }
-                acc += best;
+            for (int32_t m0 = 0; m0 < W; m0 += kReq) {
+                int64_t v[kReq];
+                best_of(n, W, mk, m0, i, g, v);
+#pragma unroll
+                for (int u = 0; u < kReq; ++u) acc += v[u];
             }
         }
     }
