@@ -127,7 +127,7 @@ constexpr int32_t kDevOk = PP_OK;
 
 // Layout of the exact reduction (pp_reduce.cu): host tables while an instance
 // is built, and their sizes.  CL = 0: this tree is not reduced.
-constexpr int32_t kReduceMinRows = 1024;    // below, the sweep is as short as the reduction
+constexpr int32_t kReduceMinRows = 128;     // below, the sweep is as short (501 rows: 79 us swept, 40 reduced)
 struct ReduceTables {
     struct Info {
         int32_t x, y;
