@@ -1016,7 +1016,7 @@ static std::atomic<bool> g_injected[64];      // pp_test_inject has silenced a w
 
 bool reduce_on(const pp_instance *inst)
 {
-    return inst->red.CL > 0 && !inst->tune_noprune && !(inst->device < 64 && g_injected[inst->device].load());
+    return inst->red.bins > 0 && !inst->tune_noprune && !(inst->device < 64 && g_injected[inst->device].load());
 }
 
 size_t dp_work_bytes(const pp_instance *inst, int batch, int words)
@@ -1025,7 +1025,7 @@ size_t dp_work_bytes(const pp_instance *inst, int batch, int words)
     const size_t nb = (size_t)(n + 63) / 64 * 64, B = (size_t)std::max(batch, 1), N = (size_t)std::max(n, 1);
     return align256(B * nb * words * 4) + 4 * align256(B * N * 4) + 2 * align256(B * (N + 1) * 4) +
            align256(B * 4) + align256(B * N * 8) +
-           (inst->red.CL ? 2 * align256(B * 4) + align256(B * 8) + 2 * align256(B * ((N + 31) / 32) * 4) +
+           (inst->red.bins ? 2 * align256(B * 4) + align256(B * 8) + 2 * align256(B * ((N + 31) / 32) * 4) +
                                B * reduce_item_bytes(inst)
                          : 0);
 }

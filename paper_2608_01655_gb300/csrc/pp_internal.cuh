@@ -115,6 +115,7 @@ struct DpWork {
     uint32_t *taken = nullptr;     // [batch][ceil(n / 32)] by preorder position
     uint32_t *undecided = nullptr; // [batch][ceil(n / 32)]
     char *red_scratch = nullptr;   // [batch][reduce_item_bytes]
+    int items = 0;                 // items in flight together with this launch's (0: only those)
     int64_t *clear = nullptr;      // [batch] or null: zeroed by the reduction (the planner's next held sums)
 };
 size_t dp_work_bytes(const pp_instance *inst, int batch, int words);
@@ -135,14 +136,21 @@ struct ReduceTables {
     struct Stream {
         int32_t tile, tiles;
     };
-    int CL = 0, max_kids = 0;
+    struct Cluster {
+        int cl, acc;                // CTAs of an item; accumulators of a CTA, at most
+    };
+    int bins = 0, max_kids = 0;
     std::vector<Info> info;
     std::vector<int32_t> pos;
+    std::vector<uint8_t> form;
+    std::vector<Cluster> cluster;   // largest first
     std::vector<Stream> stream;
     std::vector<int32_t> lev, binlev, binslot, nacc;
 };
 struct ReduceShape {
-    int CL = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_acc = 0, acc_smem = 0, max_kids = 0;
+    int bins = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_kids = 0;
+    int ncl = 0, cl[8] = {}, acc[8] = {}, acc_global = 0;      // cluster sizes, largest first
+    int wide = 0;                   // clusters above the portable size that fit the device
 };
 
 struct Scratch {
@@ -179,7 +187,7 @@ struct pp_instance {
     int64_t *d_tr = nullptr;            // by node id: mode 0 [W][n] f_m(b), mode 1 [W][W][n] f_{m<-h}(b)
     int64_t *d_g = nullptr;             // mode 1: [W][W][n] Lambda_m(b) q_{m<-h}(b) at [h][m][i] (Eq. 5)
     int32_t *d_status = nullptr;        // device status word
-    pp::ReduceShape red;                // exact reduction's layout (pp_reduce.cu); CL = 0: none
+    pp::ReduceShape red;                // exact reduction's layout (pp_reduce.cu); no bins: none
     void *d_red = nullptr;              // its tables
     pp::Scratch stack;                  // skip-row stack spill of pp_tree_dp
     pp::Scratch plan;                   // pp_plan_run working set
@@ -261,6 +269,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
 size_t reduce_tables_bytes(const ReduceTables &R);
 void reduce_tables_pack(const ReduceTables &R, char *dst);
 ReduceShape reduce_shape(const ReduceTables &R);
+pp_status reduce_device(ReduceShape *r);
 size_t reduce_item_bytes(const pp_instance *inst);
 // whether launches of this instance try the reduction first (not without
 // pruning, and not while pp_test_inject makes a warp of the sweep silent)

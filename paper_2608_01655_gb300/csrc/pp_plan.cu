@@ -436,6 +436,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 uint32_t *mk = pb.mask + (size_t)x * N;
                 int64_t *pf = pb.profit + (size_t)x * N;
                 DpWork wx = dp_work_item(inst, work, x, g.words);
+                wx.items = S;
                 int64_t *held = nullptr;
                 if ((s = held_sums(x, b, sx, &wx, &held))) return s;
                 if ((s = smark(q0, sx))) return s;

@@ -36,10 +36,12 @@
 // log2(n) + 1 for every tree shape (6 to 9 on the prefix trees here, whose
 // depth is 72 and more).  Rows are laid out by (bin, level, path), bottom of
 // the path first, in tiles of 32 (one per warp step).  A bin is a set of
-// whole subtrees of at most n / (2 CL) rows, one bin per CTA of the cluster,
-// so that levels are separated by block barriers only; the few nodes above
-// all bins form a last bin that one warp of every CTA walks for itself, after
-// the cluster barrier that ends an evaluation.
+// whole subtrees of at most n / (2 bins) rows; a CTA of the item's cluster
+// walks one bin or several side by side, so that levels are separated by block
+// barriers only.  The few nodes above all bins form a last bin that one warp
+// of every CTA walks for itself, after the cluster barrier that ends an
+// evaluation.  How many CTAs share an item is decided at the launch, from the
+// items that are in flight together.
 #include <algorithm>
 #include <climits>
 #include <cstring>
@@ -70,6 +72,8 @@ constexpr int kMaxKids = 65535;             // light children of a row: its 16-b
 constexpr int kRing = 3;                    // tiles of a warp in flight or in use
 constexpr int kMaxTiles = 64;               // of a warp, all levels together
 constexpr size_t kRingBytes = (size_t)kWarps * kRing * 512;
+constexpr int kMaxBins = 16;
+constexpr int kReduceCtas = 128;            // of all items in flight: 16 clusters of 8 find room, and no more
 constexpr int kMaxTop = 256;                // rows of the last bin (every CTA walks it)
 // the search's 32-bit units: the first price is 2^11 to 2^12 of them
 constexpr int kUnitBits = 11;
@@ -83,14 +87,16 @@ constexpr int kCont = 32, kTop = 64, kUp = 128, kWeightShift = 8;
 constexpr int kNone = 0xffff;
 
 struct Tab {
-    int n, CL, nslots, ntop;
+    int n, bins, CL, nslots, ntop;
     const int2 *info;
     const int *pos;              // position of the slot's row (-1 pad)
+    const uint8_t *form;         // of a tile: 1 on level 0 (paths without light children), 3 there and its first
+                                 // path comes from the tile before, 0 above
     const int2 *stream;          // first tile, tiles: what one warp walks in sequence
     const int *lev;              // stream boundaries of the levels
-    const int *binlev;           // [CL + 2] boundaries of a bin's entries in lev
-    const int *binslot;          // [CL + 2] first slot of a bin
-    const int *nacc;             // [CL + 1] accumulators of a bin
+    const int *binlev;           // [bins + 2] boundaries of a bin's entries in lev
+    const int *binslot;          // [bins + 2] first slot of a bin
+    const int *nacc;             // [bins + 1] accumulators of a bin
 };
 
 struct Scal {                    // per item, zeroed by the kernel
@@ -220,10 +226,16 @@ __device__ __forceinline__ T acc_ld(const T *p)
     else return *p;
 }
 
-// The tiles that a warp walks, (level << 16) + tile, its lanes' slots (info
-// and a value) copied to shared memory two tiles ahead.  Asynchronous copies:
-// registers loaded for the next trip of a loop are waited for at its back
-// edge, which puts L2's latency (300 to 500 cycles) on every tile.
+// An entry of a warp's list of tiles: bits 0-15 the tile of the CTA's, 16-20
+// its level, 21-25 its bin
+__device__ __forceinline__ int tile_of(unsigned en) { return (int)(en & 0xffffu); }
+__device__ __forceinline__ int level_of(unsigned en) { return (int)(en >> 16 & 31u); }
+__device__ __forceinline__ int bin_of(unsigned en) { return (int)(en >> 21); }
+
+// The tiles that a warp walks, its lanes' slots (info and a value) copied to
+// shared memory two tiles ahead.  Asynchronous copies: registers loaded for
+// the next trip of a loop are waited for at its back edge, which puts L2's
+// latency (300 to 500 cycles) on every tile.
 template <typename V, int DIR>
 struct Feed {
     const int2 *info;                        // of this lane's slot of the bin's first tile
@@ -246,7 +258,7 @@ struct Feed {
     __device__ __forceinline__ void issue(int x, int to)
     {
         if (x >= 0 && x < n) {
-            const int slot = (int)(list[x] & 0xffffu) * 32;
+            const int slot = tile_of(list[x]) * 32;
             asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(ri + to * 32)),
                          "l"(__cvta_generic_to_global(info + slot)) : "memory");
             asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(rv + to * 32)),
@@ -314,7 +326,7 @@ __device__ __forceinline__ STile search_tile(int code, int p, int2 kids, int lam
 // light children read it).
 template <bool GLOBAL>
 __device__ __forceinline__ int search_bin(const int2 *info, const int *val, const unsigned *list, int n, unsigned *keep,
-                                          int nlev, const Acc &own, int na, int2 *tops, int lam, int clip,
+                                          int nlev, const Acc &own, const int *base, int na, int2 *tops, int lam, int clip,
                                           unsigned char *ring, int &rootZ)
 {
     const int lane = threadIdx.x & 31;
@@ -323,12 +335,13 @@ __device__ __forceinline__ int search_bin(const int2 *info, const int *val, cons
     unsigned prev = 0;
     while (feed.more()) {
         const unsigned en = feed.entry();
-        for (; lev < (int)(en >> 16); ++lev) __syncthreads();
+        for (; lev < level_of(en); ++lev) __syncthreads();
         int2 c;
         int p;
         feed.take(c, p);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
-        const int2 kids = acc_ld<GLOBAL>(own.s + min(ac, na));
+        const int a0 = base[bin_of(en)];
+        const int2 kids = acc_ld<GLOBAL>(own.s + min(a0 + ac, na));
         if (en != prev + 1) carryY = carryZ = 0;         // not the same path's next tile
         prev = en;
         const STile r = search_tile(c.x, p, kids, lam, carryY, carryZ);
@@ -339,7 +352,7 @@ __device__ __forceinline__ int search_bin(const int2 *info, const int *val, cons
         if ((c.x & kTop) && r.f > 0) {
             if (up == kNone) rootZ += r.z;
             else if (c.x & kUp) pair_add(tops + up, min(r.f, clip), r.z);
-            else pair_add(own.s + up, min(r.f, clip), r.z);
+            else pair_add(own.s + a0 + up, min(r.f, clip), r.z);
         }
     }
     for (++lev; lev < nlev; ++lev) __syncthreads();
@@ -347,18 +360,29 @@ __device__ __forceinline__ int search_bin(const int2 *info, const int *val, cons
 }
 
 // The last bin, by one warp (every CTA does it for itself): its tiles in
-// order; `loc`: what the bins have added, then its own paths.
-__device__ __forceinline__ int search_top(const Tab &t, const Scratch1 &g, const int2 *tops, int2 *loc, int lam, int clip)
+// order; `loc`: what the bins have added, then its own paths.  The slots come
+// from shared memory if there are at most kTopSlots (two trips to L2 less a
+// price).
+constexpr int kTopSlots = 256;
+__device__ __forceinline__ int search_top(const Tab &t, const Scratch1 &g, const int4 *slots, const int2 *tops, int2 *loc,
+                                          int lam, int clip)
 {
     const int lane = threadIdx.x & 31;
     for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(tops + i);
     __syncwarp();
     int rootZ = 0, carryY = 0, carryZ = 0;
-    for (int s = t.binslot[t.CL] + lane; s < t.nslots; s += 32) {
-        const int2 c = __ldg(t.info + s);
+    const int s0 = t.binslot[t.bins], ns = t.nslots - s0;
+    for (int s = lane; s < ns; s += 32) {
+        int4 c;
+        if (ns <= kTopSlots) {
+            c = slots[s];
+        } else {
+            const int2 i = __ldg(t.info + s0 + s);
+            c = make_int4(i.x, i.y, __ldcg(g.unit + s0 + s), 0);
+        }
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const int2 kids = ac != kNone ? loc[ac] : make_int2(0, 0);
-        const STile r = search_tile(c.x, __ldcg(g.unit + s), kids, lam, carryY, carryZ);
+        const STile r = search_tile(c.x, c.z, kids, lam, carryY, carryZ);
         if ((c.x & kTop) && r.f > 0) {
             if (up == kNone) rootZ += r.z;
             else pair_add(loc + up, min(r.f, clip), r.z);
@@ -397,7 +421,7 @@ __device__ __forceinline__ int64_t exact_tile(int code, int64_t p, int64_t kids,
 // f of every row of a bin to f, the roots' share of L to rootY
 template <bool GLOBAL>
 __device__ __forceinline__ void exact_bin(const int2 *info, const int64_t *val, int64_t *fout, int4 *topl,
-                                          const unsigned *list, int n, int nlev, const Acc &own, int na, int64_t lam,
+                                          const unsigned *list, int n, int nlev, const Acc &own, const int *base, int na, int64_t lam,
                                           unsigned char *ring, int64_t &rootY)
 {
     const int lane = threadIdx.x & 31;
@@ -407,20 +431,21 @@ __device__ __forceinline__ void exact_bin(const int2 *info, const int64_t *val, 
     unsigned prev = 0;
     while (feed.more()) {
         const unsigned en = feed.entry();
-        for (; lev < (int)(en >> 16); ++lev) __syncthreads();
+        for (; lev < level_of(en); ++lev) __syncthreads();
         int2 c;
         int64_t p;
         feed.take(c, p);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
-        const int64_t kids = limbs(acc_ld<GLOBAL>(own.limb + min(ac, na)));
+        const int a0 = base[bin_of(en)];
+        const int64_t kids = limbs(acc_ld<GLOBAL>(own.limb + min(a0 + ac, na)));
         if (en != prev + 1) carryY = 0;
         prev = en;
         const int64_t f = exact_tile(c.x, p, kids, lam, carryY);
-        fout[(en & 0xffffu) * 32 + lane] = f;
+        fout[tile_of(en) * 32 + lane] = f;
         if ((c.x & kTop) && f > 0) {
             if (up == kNone) rootY += f;
             else if (c.x & kUp) limb_add(topl + up, f);
-            else limb_add(own.limb + up, f);
+            else limb_add(own.limb + a0 + up, f);
         }
     }
     for (++lev; lev < nlev; ++lev) __syncthreads();
@@ -432,7 +457,7 @@ __device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, in
     for (int i = lane; i < t.ntop; i += 32) loc[i] = __ldcg(g.topl + i);
     __syncwarp();
     int64_t rootY = 0, carryY = 0;
-    for (int s = t.binslot[t.CL] + lane; s < t.nslots; s += 32) {
+    for (int s = t.binslot[t.bins] + lane; s < t.nslots; s += 32) {
         const int2 c = __ldg(t.info + s);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const int64_t kids = ac != kNone ? limbs(loc[ac]) : 0;
@@ -492,7 +517,7 @@ __device__ __forceinline__ int loss_code(float a, float b)
 // losses of one bin, levels from the top down, and their histogram
 template <bool GLOBAL>
 __device__ __forceinline__ void loss_bin(const int2 *info, const int64_t *fin, uint16_t *key, const unsigned *list, int n,
-                                         int nlev, const Acc &own, const float2 *topd, unsigned char *ring,
+                                         int nlev, const Acc &own, const int *base, const float2 *topd, unsigned char *ring,
                                          unsigned *hist)
 {
     const int lane = threadIdx.x & 31;
@@ -501,23 +526,24 @@ __device__ __forceinline__ void loss_bin(const int2 *info, const int64_t *fin, u
     float ca = 0.f, cb = 0.f;
     while (feed.more()) {
         const unsigned en = feed.entry();
-        for (; lev > (int)(en >> 16); --lev) __syncthreads();
+        for (; lev > level_of(en); --lev) __syncthreads();
         int2 c;
         int64_t f;
         feed.take(c, f);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const bool child = (c.x & kTop) && up != kNone;
+        const int a0 = base[bin_of(en)];
         float2 from = make_float2(0.f, 0.f);
         if (child) {
             if (c.x & kUp) from = topd[up];
-            else from = acc_ld<GLOBAL>(own.down + up);
+            else from = acc_ld<GLOBAL>(own.down + a0 + up);
         }
         float a, b;                          // (a path that goes on does so in the tile just done)
         loss_tile(c.x, f, child, from, ca, cb, a, b);
-        if (ac != kNone) own.down[ac] = make_float2(a, b);
+        if (ac != kNone) own.down[a0 + ac] = make_float2(a, b);
         const int code = (c.x >> kWeightShift) ? loss_code(a, b) : kKeyPad;      // (a pad weighs nothing)
         if (code != kKeyPad) atomicAdd(hist + (code & 0x7fff), 1u);
-        key[(en & 0xffffu) * 32 + lane] = (uint16_t)code;
+        key[tile_of(en) * 32 + lane] = (uint16_t)code;
     }
     for (; lev > 0; --lev) __syncthreads();
 }
@@ -526,7 +552,7 @@ __device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, float2
 {
     const int lane = threadIdx.x & 31;
     float ca = 0.f, cb = 0.f;
-    for (int s = t.nslots - 32 + lane; s >= t.binslot[t.CL]; s -= 32) {
+    for (int s = t.nslots - 32 + lane; s >= t.binslot[t.bins]; s -= 32) {
         const int2 c = __ldg(t.info + s);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const bool child = (c.x & kTop) && up != kNone;
@@ -810,7 +836,9 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     __shared__ unsigned char leaf[kWarps * kMaxTiles];   // tiles of level 0: see the gather
     __shared__ unsigned lists[3][kWarps][kMaxTiles];    // a warp's tiles: all; two that the search shortens in turn
     __shared__ int4 s_top[kMaxTop];          // the last bin's own sums, then what it passes down
+    __shared__ int4 slots[kTopSlots];        // of the last bin: info, profit in units
     __shared__ int sh[kWarps];
+    __shared__ int base[kMaxBins + 1];       // of a bin's accumulators among the CTA's
     __shared__ int s_a, s_b, s_flag, s_lam;
     __shared__ int64_t s_val;
     const Tab &t = A.t;
@@ -841,15 +869,26 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         }
         return;
     }
-    const int na = t.nacc[cr];
-    const int lo = t.binslot[cr], hi = t.binslot[cr + 1];
+    const int per = t.bins / CL, bin0 = cr * per;            // this CTA's bins
+    const int lo = t.binslot[bin0], hi = t.binslot[bin0 + per];
+    if (tid < 32) {
+        const int mine = lane < per ? __ldg(t.nacc + bin0 + lane) : 0;
+        int x = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(kAll, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane <= per) base[lane] = x - mine;
+    }
+    __syncthreads();
+    const int na = base[per];
     const Acc own = acc_at(SMEM ? (char *)smem : g.own + (size_t)(lo + cr) * kAccBytes, na + 1);   // (one reads as zero)
     unsigned char *ring = smem + (SMEM ? up16((size_t)(na + 1) * kAccBytes) : 0);
     unsigned *hist = (unsigned *)(ring + kRingBytes);
-    const bool has_top = t.binslot[CL] < t.nslots;
+    const int top0 = t.binslot[t.bins];
+    const bool has_top = top0 < t.nslots;
     const int2 *info = t.info + lo;
-    const int l0 = t.binlev[cr], nlev = t.binlev[cr + 1] - 1 - l0;
-    const int top0 = t.binslot[CL];
     auto sync_all = [&] {
         if (CL > 1) cluster_sync();
         else __syncthreads();
@@ -863,17 +902,45 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         for (int i = tid; i < t.ntop; i += kThreads) g.topl[i] = make_int4(0, 0, 0, 0);
     }
     for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
-    int tiles = 0;                           // of this warp
-    for (int l = 0; l < nlev; ++l) {
-        const int q = __ldg(t.lev + l0 + l) + warp;
-        if (q >= __ldg(t.lev + l0 + l + 1)) continue;
-        const int2 x = __ldg(t.stream + q);
-        for (int i = lane; i < x.y; i += 32) lists[0][warp][tiles + i] = ((unsigned)l << 16) + (unsigned)(x.x - (lo >> 5) + i);
-        tiles += x.y;
+    // this warp's tiles: of every level the bins' streams go round the warps
+    int tiles = 0, nlev = 0;
+    {
+        const int e0 = __ldg(t.binlev + bin0), e1 = __ldg(t.binlev + bin0 + per);
+        const int q0 = __ldg(t.lev + e0);
+        // (at most kMaxBins (kMaxLevels + 1) entries, then at most kWarps kMaxTiles streams)
+        int *lev = (int *)ring;
+        int2 *stream = (int2 *)(ring + kMaxBins * (kMaxLevels + 1) * 4);
+        const int ns = __ldg(t.lev + e1 - 1) - q0;
+        for (int i = tid; i < e1 - e0; i += kThreads) lev[i] = __ldg(t.lev + e0 + i) - q0;
+        for (int i = tid; i < ns; i += kThreads) stream[i] = __ldg(t.stream + q0 + i);
+        const int from = lane < per ? __ldg(t.binlev + bin0 + lane) - e0 : 0;       // a lane per bin
+        const int levels = lane < per ? __ldg(t.binlev + bin0 + lane + 1) - 1 - e0 - from : 0;
+        nlev = __reduce_max_sync(kAll, levels);
+        __syncthreads();
+        for (int l = 0, at = 0; l < nlev; ++l) {
+            int first = 0, c = 0;
+            if (l < levels) {
+                first = lev[from + l];
+                c = lev[from + l + 1] - first;
+            }
+            int x = c;
+#pragma unroll
+            for (int o = 1; o < kMaxBins; o <<= 1) {
+                const int y = __shfl_up_sync(kAll, x, o);
+                if (lane >= o) x += y;
+            }
+            const int j = (warp - at - (x - c)) & (kWarps - 1);     // which of the bin's streams is this warp's
+            for (unsigned m = __ballot_sync(kAll, j < c); m; m &= m - 1) {
+                const int bb = __ffs((int)m) - 1;
+                const int2 st = stream[__shfl_sync(kAll, first + j, bb)];
+                for (int i = lane; i < st.y; i += 32)
+                    lists[0][warp][tiles + i] = (unsigned)bb << 21 | (unsigned)l << 16 | (unsigned)(st.x - (lo >> 5) + i);
+                tiles += st.y;
+            }
+            at += __shfl_sync(kAll, x, kMaxBins - 1);
+        }
     }
-    // the slots of level 0 (paths without light children) end here
-    const int leaf_end = nlev > 1 ? min(hi, __ldg(&t.stream[__ldg(t.lev + l0 + 1)].x) * 32) : hi;
-    for (int i = tid; i < (leaf_end - lo) >> 5; i += kThreads) leaf[i] = 0;
+    for (int i = tid; i < (hi - lo) >> 5; i += kThreads) leaf[i] = 0;
     sync_all();
 
     // ---- gather the profits into the slots; weights by profit per slot
@@ -883,10 +950,14 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     auto gather = [&](int from, int to) {
         constexpr int U = 4;                 // loads in flight per thread
         for (int s0 = from + tid; s0 < to; s0 += U * kThreads) {
-            int x[U];
+            int x[U], form[U];
             int64_t p[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) x[u] = s0 + u * kThreads < to ? __ldg(t.pos + s0 + u * kThreads) : -1;
+            for (int u = 0; u < U; ++u) {
+                const int s = s0 + u * kThreads;
+                x[u] = s < to ? __ldg(t.pos + s) : -1;
+                form[u] = s < to ? __ldg(t.form + (s >> 5)) : 0;
+            }
             if (A.order)
 #pragma unroll
                 for (int u = 0; u < U; ++u)
@@ -899,12 +970,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 if (s >= to) break;
                 g.prof[s] = p[u];
                 mx = p[u] > mx ? p[u] : mx;
-                // a warp's slots are a tile; bit 0: no profit in it, bit 1: its
-                // first path comes from the tile before
-                if (!__any_sync(kAll, p[u] > 0) && s < leaf_end) {
-                    const bool cont = __any_sync(kAll, __ldg(&t.info[s].x) & kCont);
-                    if (lane == 0) leaf[(s - lo) >> 5] = cont ? 3 : 1;
-                }
+                // a warp's slots are a tile; its form if there is no profit in it
+                if (!__any_sync(kAll, p[u] > 0) && form[u] && lane == 0) leaf[(s - lo) >> 5] = (unsigned char)form[u];
                 if (p[u] > 0 && ((s >> 5) & ((1 << every) - 1)) == 0) {
                     const int w = __ldg(&t.info[s].x) >> kWeightShift;
                     const int c = w == 1 ? code_of(p[u]) : code_of((int64_t)((float)p[u] / (float)w));
@@ -914,7 +981,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         }
     };
     gather(lo, hi);
-    if (cr == 0 && has_top) gather(t.binslot[CL], t.nslots);
+    if (cr == 0 && has_top) gather(top0, t.nslots);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const int64_t y = __shfl_xor_sync(kAll, mx, o);
@@ -930,18 +997,18 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         // leaf tiles without a profit leave the lists: at any price nothing in
         // them is taken (on the planner's later sweeps, most of the tree)
         int kept = 0;
-        unsigned prev = 0;
+        int prev = -2;
         bool pd = false;
         for (int i = 0; i < tiles; ++i) {
             const unsigned en = lists[0][warp][i];
-            const int fl = en >> 16 ? 0 : leaf[en];
-            const bool d = (fl & 1) && (!(fl & 2) || (pd && en == prev + 1));
+            const int q = tile_of(en), fl = leaf[q];
+            const bool d = (fl & 1) && (!(fl & 2) || (pd && q == prev + 1));
             __syncwarp();
-            if (d) g.key[lo + en * 32 + lane] = kKeyPad;
+            if (d) g.key[lo + q * 32 + lane] = kKeyPad;
             else if (lane == 0) lists[0][warp][kept] = lists[1][warp][kept] = en;
             kept += !d;
             pd = d;
-            prev = en;
+            prev = q;
         }
         tiles = kept;
     }
@@ -982,7 +1049,13 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             }
         };
         to_units(lo, hi);
-        if (cr == 0 && has_top) to_units(top0, t.nslots);
+        if (has_top && t.nslots - top0 > kTopSlots) {
+            if (cr == 0) to_units(top0, t.nslots);
+        } else if (tid < t.nslots - top0) {
+            const int64_t p = __ldcg(g.prof + top0 + tid) >> shift;
+            const int2 i = __ldg(t.info + top0 + tid);
+            slots[tid] = make_int4(i.x, i.y, (int)(p > kClipRow ? kClipRow : p < -kClipRow ? -kClipRow : p), 0);
+        }
         bool low = false;                    // the last price was a lower bound
         int at = 1, alive = tiles, kept = 0;
         for (int ev = 0;; ++ev) {
@@ -997,16 +1070,17 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             int2 *tops = g.tops + ev % 3 * t.ntop;
             int rz = 0;
             __syncthreads();
-            kept = search_bin<!SMEM>(info, g.unit + lo, lists[at][warp], alive, lists[at ^ 3][warp], nlev, own, na, tops,
+            kept = search_bin<!SMEM>(info, g.unit + lo, lists[at][warp], alive, lists[at ^ 3][warp], nlev, own, base, na, tops,
                                      price, A.clip_kid, ring, rz);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(kAll, rz, o);
             if (lane == 0 && rz) atomicAdd(&g.s->sumZ[ev], (unsigned long long)rz);
             sync_all();
             if (warp == 0) {
-                int z = has_top ? search_top(t, g, tops, (int2 *)s_top, price, A.clip_kid) : 0;
+                const int bins = lane == 0 ? (int)__ldcg(&g.s->sumZ[ev]) : 0;
+                int z = has_top ? search_top(t, g, slots, tops, (int2 *)s_top, price, A.clip_kid) : 0;
                 if (lane == 0) {
-                    z += (int)__ldcg(&g.s->sumZ[ev]);
+                    z += bins;
                     int nx = price;
                     s_flag = next_price(sr, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
                     s_lam = nx;
@@ -1025,7 +1099,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
         for (int i = tid; i <= na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
         __syncthreads();
         int64_t ry = 0;
-        exact_bin<!SMEM>(info, g.prof + lo, g.f + lo, g.topl, lists[0][warp], tiles, nlev, own, na, lam, ring, ry);
+        exact_bin<!SMEM>(info, g.prof + lo, g.f + lo, g.topl, lists[0][warp], tiles, nlev, own, base, na, lam, ring, ry);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ry += __shfl_xor_sync(kAll, ry, o);
         if (lane == 0 && ry) atomicAdd(&g.s->sumL, (unsigned long long)ry);
@@ -1047,7 +1121,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             if (warp == 0) loss_top(t, g, (float2 *)s_top, hist, cr == 0);
             __syncthreads();
         }
-        loss_bin<!SMEM>(info, g.f + lo, g.key + lo, lists[0][warp], tiles, nlev, own, (const float2 *)s_top, ring, hist);
+        loss_bin<!SMEM>(info, g.f + lo, g.key + lo, lists[0][warp], tiles, nlev, own, base, (const float2 *)s_top, ring, hist);
         __syncthreads();
         for (int i = tid; i < kBins; i += kThreads)
             if (hist[i]) atomicAdd(ghist + i, hist[i]);
@@ -1125,7 +1199,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 }
             };
             classify(lo, hi);
-            if (cr == 0 && has_top) classify(t.binslot[CL], t.nslots);
+            if (cr == 0 && has_top) classify(top0, t.nslots);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 vf += __shfl_xor_sync(kAll, vf, o);
@@ -1364,7 +1438,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             }
         };
         mark(lo, hi);
-        if (cr == 0 && has_top) mark(t.binslot[CL], t.nslots);
+        if (cr == 0 && has_top) mark(top0, t.nslots);
     }
     if (cr == 0 && tid == 0) {
         *red = state;
@@ -1378,8 +1452,13 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
 // ---------------------------------------------------------------------------
 // host: the layout (see the top of the file), one device block per instance
 // ---------------------------------------------------------------------------
-// CTAs of an item's cluster
-static int cluster_of(int n) { return n <= 8192 ? 1 : n <= 24576 ? 4 : n <= 98304 ? 6 : 8; }
+// Bins of a tree: the most CTAs that can share an item.  One price costs
+// 12.4 us on 6 CTAs and 8.6 on 8 (50,000 rows), 19.5 on 8 and 11.3 on 16
+// (200,000 rows): 32 warps on four schedulers issue some 150 instructions a
+// tile each.  But more bins put more rows into the last one and more padding
+// into the tiles: at 10,000 rows 8 CTAs are 6% slower than 6.  Below 1,536
+// rows one CTA is as fast as any cluster.
+static int bins_of(int n) { return n <= 1536 ? 1 : n <= 12288 ? 6 : 16; }
 
 bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::vector<int32_t> &next,
                          const std::vector<int32_t> &wpre, int64_t total_weight, int32_t max_weight,
@@ -1388,7 +1467,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     ReduceTables &R = *out;
     R = ReduceTables();
     if (n < kReduceMinRows || max_weight > kMaxWeight || total_weight >= ((int64_t)1 << 30)) return false;
-    int CL = cluster_of(n);
+    int NB = bins_of(n);
     // rows of a subtree that stays in one bin: half a CTA's share, more
     // if that leaves too many rows above the bins
     std::vector<int32_t> kids(n, 0), heavy(n, -1), best(n, 0);
@@ -1399,14 +1478,14 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
         R.max_kids = std::max(R.max_kids, kids[p]);
     }
     int limit = n;
-    if (CL > 1) {
-        limit = std::max(64, n / (2 * CL));
+    if (NB > 1) {
+        limit = std::max(64, n / (2 * NB));
         for (;; limit *= 2) {
             int above = 0;
             for (int32_t i = 0; i < n; ++i) above += next[i] - i > limit;
             if (above <= kMaxTop) break;
             if (limit >= n / 2) {
-                CL = 1;
+                NB = 1;
                 limit = n;
                 break;
             }
@@ -1415,11 +1494,11 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     auto is_top = [&](int i) { return next[i] - i > limit; };
     // bins: subtrees below the limit, each to the emptiest bin
     std::vector<int32_t> bin(n), level(n, 0), acc(n, -1);
-    std::vector<int64_t> load(CL, 0);
+    std::vector<int64_t> load(NB, 0);
     for (int32_t i = 0; i < n; ++i) {
         const int p = par[i];
-        if (is_top(i)) bin[i] = CL;
-        else if (p >= 0 && bin[p] != CL) bin[i] = bin[p];
+        if (is_top(i)) bin[i] = NB;
+        else if (p >= 0 && bin[p] != NB) bin[i] = bin[p];
         else {
             const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
             bin[i] = b;
@@ -1431,7 +1510,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
             heavy[p] = i;
         }
     }
-    R.nacc.assign(CL + 1, 0);
+    R.nacc.assign(NB + 1, 0);
     int maxlev = 0;
     for (int32_t i = n - 1; i >= 0; --i) {
         const int p = par[i];
@@ -1441,12 +1520,12 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
         else if (bin[p] == bin[i]) level[p] = std::max(level[p], level[i] + 1);
         if (heavy[p] != i && acc[p] < 0) acc[p] = R.nacc[bin[p]]++;
     }
-    for (int b = 0; b <= CL; ++b)
+    for (int b = 0; b <= NB; ++b)
         if (R.nacc[b] >= kNone) return false;
     // path tops grouped by (bin, level)
     const int nl = maxlev + 1;
     if (nl > kMaxLevels) return false;
-    std::vector<int32_t> start((size_t)(CL + 1) * nl + 1, 0), rows((size_t)(CL + 1) * nl, 0), tops, len(n, 0);
+    std::vector<int32_t> start((size_t)(NB + 1) * nl + 1, 0), rows((size_t)(NB + 1) * nl, 0), tops, len(n, 0);
     for (int32_t i = n - 1; i >= 0; --i) len[i] = 1 + (heavy[i] >= 0 ? len[heavy[i]] : 0);
     auto path_top = [&](int i) { return par[i] < 0 || heavy[par[i]] != i; };
     for (int32_t i = 0; i < n; ++i)
@@ -1465,8 +1544,8 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     }
     R.info.reserve((size_t)n + 32 * 64);
     R.pos.reserve((size_t)n + 32 * 64);
-    std::vector<int32_t> path;
-    for (int b = 0; b <= CL; ++b) {
+    std::vector<int32_t> path, to(tops.size()), mine[kWarps];
+    for (int b = 0; b <= NB; ++b) {
         R.binslot.push_back((int32_t)R.info.size());
         R.binlev.push_back((int32_t)R.lev.size());
         int levels = nl;
@@ -1474,78 +1553,94 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
         for (int l = 0; l < levels; ++l) {
             const size_t q = (size_t)b * nl + l;
             R.lev.push_back((int32_t)R.stream.size());
-            // streams, at most one per warp of the CTA: the fewest tiles each
-            // (one, where the level has rows for no more) that take every path,
-            // next fit; a longer path has a stream of its own
-            int room = (rows[q] + 32 * kWarps - 1) / (32 * kWarps) * 32;
+            // streams, at most one per warp: the fewest tiles each (one, where
+            // the level has rows for no more) that take every path, in the
+            // first stream with room (the next stream only: 15% more tiles);
+            // a longer path has a stream of its own
+            int room = (rows[q] + 32 * kWarps - 1) / (32 * kWarps) * 32, streams = 0;
+            int used[kWarps];
             for (;; room += 32) {
-                int streams = 0, used = room + 1;
-                for (int x = start[q]; x < start[q + 1] && streams <= kWarps; ++x) {
-                    if (used + len[tops[x]] > room) {
-                        ++streams;
-                        used = 0;
-                    }
-                    used += len[tops[x]];
+                streams = 0;
+                bool fits = true;
+                for (int x = start[q]; x < start[q + 1] && fits; ++x) {
+                    const int l1 = len[tops[x]];
+                    int y = 0;
+                    while (y < streams && used[y] + l1 > room) ++y;
+                    fits = y < kWarps;
+                    if (!fits) break;
+                    if (y == streams) used[streams++] = 0;
+                    used[y] += l1;
+                    to[x] = y;
                 }
-                if (streams <= kWarps) break;
+                if (fits) break;
             }
-            int in_stream = 0, tile0 = (int)(R.info.size() / 32);
-            auto close = [&] {
-                if (in_stream == 0) return;
+            for (int x = start[q]; x < start[q + 1]; ++x) mine[to[x]].push_back(tops[x]);
+            for (int st = 0; st < streams; ++st) {
+                const int tile0 = (int)(R.info.size() / 32);
+                for (int topn : mine[st]) {
+                    path.clear();
+                    for (int v = topn; v >= 0; v = heavy[v]) path.push_back(v);
+                const int first = (int)R.info.size();            // the path's first slot
+                    for (int y = (int)path.size() - 1; y >= 0; --y) {
+                        const int v = path[y];
+                        const int s = (int)R.info.size(), t0 = s & ~31;
+                        int code = (s - std::max(first, t0)) | (first < t0 ? kCont : 0) | (v == topn ? kTop : 0) |
+                                   (wpre[v] << kWeightShift);
+                        int up = kNone;
+                        if (v == topn && par[v] >= 0) {
+                            up = acc[par[v]];
+                            if (bin[par[v]] != bin[v]) code |= kUp;
+                        }
+                        if (s == t0) R.form.push_back(l == 0 ? (first < t0 ? 3 : 1) : 0);
+                        R.info.push_back({code, (acc[v] < 0 ? kNone : acc[v]) | (int)((unsigned)up << 16)});
+                        R.pos.push_back(v);
+                    }
+                }
                 while (R.info.size() % 32) {
                     R.info.push_back({0, kNone | (int)((unsigned)kNone << 16)});
                     R.pos.push_back(-1);
                 }
-                const int tile1 = (int)(R.info.size() / 32);
-                R.stream.push_back({tile0, tile1 - tile0});
-                tile0 = tile1;
-                in_stream = 0;
-            };
-            for (int x = start[q]; x < start[q + 1]; ++x) {
-                const int topn = tops[x];
-                path.clear();
-                for (int v = topn; v >= 0; v = heavy[v]) path.push_back(v);
-                if (in_stream > 0 && in_stream + (int)path.size() > room) close();
-                int first = (int)R.info.size();            // the path's first slot
-                for (int y = (int)path.size() - 1; y >= 0; --y) {
-                    const int v = path[y];
-                    const int s = (int)R.info.size(), t0 = s & ~31;
-                    int code = (s - std::max(first, t0)) | (first < t0 ? kCont : 0) | (v == topn ? kTop : 0) |
-                               (wpre[v] << kWeightShift);
-                    int up = kNone;
-                    if (v == topn && par[v] >= 0) {
-                        up = acc[par[v]];
-                        if (bin[par[v]] != bin[v]) code |= kUp;
-                    }
-                    R.info.push_back({code, (acc[v] < 0 ? kNone : acc[v]) | (int)((unsigned)up << 16)});
-                    R.pos.push_back(v);
-                }
-                in_stream += (int)path.size();
+                R.stream.push_back({tile0, (int)(R.info.size() / 32) - tile0});
+                mine[st].clear();
             }
-            close();
         }
         R.lev.push_back((int32_t)R.stream.size());
     }
     R.binslot.push_back((int32_t)R.info.size());
     R.binlev.push_back((int32_t)R.lev.size());
-    // a warp's tiles have to fit its list
-    for (int b = 0; b < CL; ++b)
-        for (int w = 0; w < kWarps; ++w) {
-            int tiles = 0;
-            for (int l = R.binlev[b]; l + 1 < R.binlev[b + 1]; ++l)
-                if (R.lev[l] + w < R.lev[l + 1]) tiles += R.stream[R.lev[l] + w].tiles;
-            if (tiles > kMaxTiles) return false;
+    // the cluster sizes: every warp's tiles have to fit its list (streams go
+    // round the warps as the kernel deals them)
+    for (int cl = NB; cl >= 1; --cl) {
+        if (NB % cl) continue;
+        const int per = NB / cl;
+        int most = 0, acc_most = 0;
+        for (int r = 0; r < cl; ++r) {
+            int tiles[kWarps] = {}, at = 0, accs = 0;
+            for (int l = 0; l < kMaxLevels; ++l)
+                for (int b = r * per; b < (r + 1) * per; ++b) {
+                    const int e = R.binlev[b] + l;
+                    if (e + 1 >= R.binlev[b + 1]) continue;
+                    for (int x = R.lev[e]; x < R.lev[e + 1]; ++x) tiles[at++ % kWarps] += R.stream[x].tiles;
+                }
+            for (int b = r * per; b < (r + 1) * per; ++b) accs += R.nacc[b];
+            most = std::max(most, *std::max_element(tiles, tiles + kWarps));
+            acc_most = std::max(acc_most, accs);
         }
-    R.CL = CL;
+        if (most > kMaxTiles || acc_most >= kNone) break;
+        R.cluster.push_back({cl, acc_most});
+    }
+    if (R.cluster.empty()) return false;
+    R.bins = NB;
     return true;
 }
 
 static size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// device block: info | positions | streams | levels | binlev | binslot | nacc
+// device block: info | positions | forms | streams | levels | binlev | binslot | nacc
 size_t reduce_tables_bytes(const ReduceTables &R)
 {
-    return al(R.info.size() * 8) + al(R.info.size() * 4) + al(R.stream.size() * 8) + al(R.lev.size() * 4) + al(R.binlev.size() * 4) +
+    return al(R.info.size() * 8) + al(R.info.size() * 4) + al(R.form.size()) + al(R.stream.size() * 8) +
+           al(R.lev.size() * 4) + al(R.binlev.size() * 4) +
            al(R.binslot.size() * 4) + al(R.nacc.size() * 4);
 }
 
@@ -1557,6 +1652,7 @@ void reduce_tables_pack(const ReduceTables &R, char *dst)
     };
     put(R.info.data(), R.info.size() * 8);
     put(R.pos.data(), R.info.size() * 4);
+    put(R.form.data(), R.form.size());
     put(R.stream.data(), R.stream.size() * 8);
     put(R.lev.data(), R.lev.size() * 4);
     put(R.binlev.data(), R.binlev.size() * 4);
@@ -1575,38 +1671,77 @@ static Tab device_tab(const pp_instance *inst)
     };
     Tab t;
     t.n = inst->n;
-    t.CL = r.CL;
+    t.bins = r.bins;
     t.nslots = r.nslots;
     t.ntop = r.ntop;
     t.info = (const int2 *)take((size_t)r.nslots * 8);
     t.pos = (const int *)take((size_t)r.nslots * 4);
+    t.form = (const uint8_t *)take((size_t)r.nslots / 32);
     t.stream = (const int2 *)take((size_t)r.nstreams * 8);
     t.lev = (const int *)take((size_t)r.nlev * 4);
-    t.binlev = (const int *)take((size_t)(r.CL + 2) * 4);
-    t.binslot = (const int *)take((size_t)(r.CL + 2) * 4);
-    t.nacc = (const int *)take((size_t)(r.CL + 1) * 4);
+    t.binlev = (const int *)take((size_t)(r.bins + 2) * 4);
+    t.binslot = (const int *)take((size_t)(r.bins + 2) * 4);
+    t.nacc = (const int *)take((size_t)(r.bins + 1) * 4);
     return t;
 }
+
+// shared memory of the scans, with up to `acc` accumulators of a CTA there
+static size_t scan_bytes(int acc, bool acc_smem)
+{
+    return (acc_smem ? up16((size_t)(acc + 1) * kAccBytes) : 0) + kRingBytes + kBins * 4;
+}
+constexpr size_t kAccLimit = (size_t)192 << 10;
+constexpr int kPortable = 8;     // CTAs of a cluster that every device takes
 
 ReduceShape reduce_shape(const ReduceTables &R)
 {
     ReduceShape s;
-    s.CL = R.CL;
+    s.bins = R.bins;
     s.nslots = (int)R.info.size();
     s.nstreams = (int)R.stream.size();
     s.nlev = (int)R.lev.size();
-    s.ntop = R.nacc[R.CL];
+    s.ntop = R.nacc[R.bins];
     s.max_kids = R.max_kids;
-    s.max_acc = *std::max_element(R.nacc.begin(), R.nacc.end() - 1);
-    s.acc_smem = up16((size_t)(s.max_acc + 1) * kAccBytes) + kRingBytes + kBins * 4 <= (size_t)(192 << 10);
+    for (const auto &c : R.cluster) {
+        s.cl[s.ncl] = c.cl;
+        s.acc[s.ncl++] = c.acc;
+        if (scan_bytes(c.acc, true) > kAccLimit) s.acc_global = 1;
+    }
     return s;
 }
 
 // scratch of one item in the DP workspace, 0 when the instance has no reduction
 size_t reduce_item_bytes(const pp_instance *inst)
 {
-    if (!inst->red.CL) return 0;
-    return al(carve(nullptr, inst->red.nslots, inst->red.ntop, !inst->red.acc_smem, nullptr));
+    if (!inst->red.bins) return 0;
+    return al(carve(nullptr, inst->red.nslots, inst->red.ntop, inst->red.acc_global, nullptr));
+}
+
+// clusters above the portable size: how many the device holds at once
+pp_status reduce_device(ReduceShape *r)
+{
+    r->wide = 0;
+    if (!r->ncl || r->cl[0] <= kPortable) return PP_OK;
+    const bool acc_smem = scan_bytes(r->acc[0], true) <= kAccLimit;
+    const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;
+    const size_t smem = std::max(scan_bytes(r->acc[0], acc_smem), up16(sizeof(Rows)) + kPool);
+    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(r->cl[0]);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = r->cl[0];
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&r->wide, kern, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        r->wide = 0;
+    }
+    return PP_OK;
 }
 
 pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, bool by_node,
@@ -1630,11 +1765,20 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.total_weight = inst->total_weight;
     a.max_weight = inst->max_weight;
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
-    const size_t scan = (r.acc_smem ? up16((size_t)(r.max_acc + 1) * kAccBytes) : 0) + kRingBytes + kBins * 4;
-    const size_t smem = std::max(scan, up16(sizeof(Rows)) + kPool);
-    const auto kern = r.acc_smem ? k_reduce<true> : k_reduce<false>;
+    // As many CTAs per item as the items in flight leave SMs for (whole plans,
+    // 16 CTAs an item against 8: 2 starts of 200,000 rows 11.9 and 15.7 ms, 8
+    // starts of 20,000 10.4 and 11.1 although one start in eight waits; 16
+    // starts of 50,000 41.7 and 29.3, half of them waiting)
+    const int items = std::max(work.items, batch);
+    int x = 0;
+    while (x + 1 < r.ncl && ((r.cl[x] > kPortable && items * 7 > r.wide * 8) || r.cl[x] * items > kReduceCtas)) ++x;
+    a.t.CL = r.cl[x];
+    const bool acc_smem = scan_bytes(r.acc[x], true) <= kAccLimit;
+    const size_t smem = std::max(scan_bytes(r.acc[x], acc_smem), up16(sizeof(Rows)) + kPool);
+    const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;
     PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PP_CUDA(launch_chained(kern, dim3(r.CL * batch), dim3(kThreads), smem, st, r.CL, a));
+    if (r.cl[x] > kPortable) PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    PP_CUDA(launch_chained(kern, dim3(r.cl[x] * batch), dim3(kThreads), smem, st, r.cl[x], a));
     return PP_OK;
 }
 

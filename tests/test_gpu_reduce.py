@@ -59,7 +59,7 @@ def _check(pp, oracle_lib, parent, weight, profits, budgets, by_rows):
 @pytest.mark.parametrize("shape", ["random", "star", "caterpillar", "mixed"])
 @pytest.mark.parametrize("n,wmax", [(1024, 1), (1055, 3), (6144, 1), (6145, 2), (12289, 9), (24577, 1)])
 def test_reduced_optimum_and_set(pp, oracle_lib, shape, n, wmax):
-    """One CTA to eight, weights on and above the wavefront kernel's limit;
+    """Layouts of one bin, six and sixteen, weights on and above the wavefront kernel's limit;
     per batch: profits over several decades, few values (ties), mostly zero,
     negative ones, a budget of one slot and one that does not bind."""
     rng = np.random.default_rng(n + wmax)
@@ -78,6 +78,19 @@ def test_reduced_optimum_and_set(pp, oracle_lib, shape, n, wmax):
         if shape == "mixed":
             assert r[0] <= n // 4                # few rows are left undecided
     _check(pp, oracle_lib, parent, weight, wide, budgets, rows)
+
+
+@pytest.mark.parametrize("n", [128, 501, 1537, 12289])
+@pytest.mark.parametrize("batch", [1, 9, 17, 33, 65])
+def test_cluster_sizes(pp, oracle_lib, n, batch):
+    """The items of a launch decide how many CTAs share one, and so how many
+    bins a CTA walks."""
+    rng = np.random.default_rng(n + batch)
+    parent = _tree(rng, "mixed", n)
+    profits = np.exp(rng.uniform(0, 18, size=(batch, n))).astype(np.int64)
+    profits[:, rng.random(n) < 0.3] = 0
+    budgets = rng.integers(1, 90, size=batch)
+    _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, budgets, lambda r: None)
 
 
 def test_ties_and_zero_budget_and_long_paths(pp, oracle_lib):
