@@ -57,11 +57,12 @@ constexpr int kThreads = 1024;              // per CTA
 constexpr int kWarps = kThreads / 32;
 constexpr int kMaxLevels = 20;              // of a bin (heavy paths: log2 of its rows, plus one)
 constexpr int kMaxEvals = 16;               // prices tried per item
-constexpr int kPasses = 4;                  // thresholds tried per item
+constexpr int kPasses = 5;                  // thresholds tried per item
 constexpr int kRowCap = 1024;               // undecided rows the on-chip DP takes
-constexpr int kFirstRows = 320;             // most rows of the first threshold
+constexpr int kFirstRows = 192;             // most rows of the first threshold
+constexpr int kMoreRows = 640;              // of the next, where the first gave no V or a poor one
 constexpr int kColCap = 1024;               // its columns (budget left over)
-constexpr int kPool = 96 << 10;             // its decisions, stack and row buffers, bytes
+constexpr int kPool = 112 << 10;            // its decisions, stack and row buffers, bytes
 constexpr int kKeyBase = (127 << 5) - 1;    // float bits >> 18 of 1.0, minus 1
 constexpr int kBins = 2048;                 // keys of 0 .. 2^62
 constexpr int kKeyPad = 0xffff;
@@ -700,7 +701,7 @@ struct __align__(16) Row {
 struct Rows {                                // in sweep order (last position first)
     Row row[kRowCap + 8];                    // (read up to eight at a time)
     int2 step[kRowCap];                      // the walk's: weight, row that a skip goes to (-1 past the last)
-    int pos[kRowCap], last[kRowCap];
+    int pos[kRowCap], last[kRowCap + 8];
     unsigned leaf[kRowCap / 32];             // bit: a skip goes to the next row
 };
 constexpr int kPush = 1, kReload = 2, kZeroTop = 4, kFromCur = 8;
@@ -753,9 +754,9 @@ __device__ __forceinline__ void dp_rows(const Rows &R, int T, int act, int guard
 // Unit weights and at most 128 columns: one warp, C columns per lane (column
 // j = 1 + lane * C + c) in registers, the column shift a shuffle, no barrier:
 // 24 to 40 ns a row against 90 with a barrier per row.  Instead of decision
-// bits it keeps, per row and column, the first row taken from there on
-// (following skips changes nothing), so the walk takes one step per chunk.
-constexpr int kNoRow = 0xffff;
+// bits it keeps, per row and column, the first row taken from there on, plus
+// 1 (0: none; following skips changes nothing), so the walk takes one step per
+// chunk.
 constexpr int kUnitCols = 128;
 template <int C>
 __device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint16_t *stf, uint16_t *first,
@@ -768,7 +769,7 @@ __device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint
 #pragma unroll
     for (int c = 0; c < C; ++c) {
         cur[c] = top[c] = 0;
-        fc[c] = ft[c] = kNoRow;
+        fc[c] = ft[c] = 0;
     }
     constexpr int U = 4;                     // rows unrolled (no-op rows past the last)
     constexpr int kOps = kPush | kReload | kZeroTop;
@@ -790,7 +791,7 @@ __device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint
                 const int64_t tv = x[u].p + (c ? cur[c > 0 ? c - 1 : 0] : up);
                 const bool take = tv > sk;
                 cur[c] = take ? tv : sk;
-                fc[c] = take ? r0 + u : same ? fc[c] : ft[c];
+                fc[c] = take ? r0 + u + 1 : same ? fc[c] : ft[c];
             }
             uint16_t *fo = first + (r0 + u) * cols + lane * C;
             if (C == 4) *(uint2 *)fo = make_uint2(fc[0] | fc[C > 1 ? 1 : 0] << 16, fc[C > 2 ? 2 : 0] | fc[C > 3 ? 3 : 0] << 16);
@@ -809,7 +810,7 @@ __device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint
 #pragma unroll
                     for (int c = 0; c < C; ++c) {
                         top[c] = re ? stk[at + 32 * c] : 0;
-                        ft[c] = re ? stf[at + 32 * c] : kNoRow;
+                        ft[c] = re ? stf[at + 32 * c] : 0;
                     }
                 }
             }
@@ -1165,13 +1166,13 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     bool sure = false;           // the key comes from a V: no row above it is undecided
     if (!give_up) {
         int T = 0;
-        // first the rows whose loss is within 0.15 of the price of a chunk's
+        // first the rows whose loss is within 0.1 of the price of a chunk's
         // slots (most gaps are), at most kFirstRows; none at price 0 (see
         // kleft < 0 below)
         if (lam == 0) {
             key = -1;
         } else {
-            T = up_to(kFirstRows, code_of((int64_t)(0.15f * (float)lam * ((float)A.total_weight / (float)n))), key);
+            T = up_to(kFirstRows, code_of((int64_t)(0.1f * (float)lam * ((float)A.total_weight / (float)n))), key);
         }
         for (; pass < kPasses; ++pass) {
             const bool big = T > kRowCap;                         // the same in every CTA
@@ -1224,6 +1225,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                 if (kleft < 0) {                        // too few rows undecided: take more by rank
                     out = 2;
                     up_to(kFirstRows, kBins, okey);
+                    if (okey <= key) up_to(kMoreRows, kBins, okey);
                     if (okey <= key) up_to(kRowCap, kBins, okey);
                     if (okey <= key) out = 3;
                 } else {
@@ -1319,7 +1321,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                     const int pitch = cols + 1 + guard;
                     const size_t need = (size_t)2 * pitch * 8 + (size_t)levels * cols * 8 + (size_t)((T + 31) / 32) * cols * 4;
                     const int C = kc <= 32 ? 1 : kc <= 64 ? 2 : 4;   // columns per lane of the one-warp kernel
-                    const size_t uneed = (size_t)levels * 32 * C * 10 + (size_t)(T + 4) * 32 * C * 2;
+                    const size_t uneed = (size_t)levels * 32 * C * 10 + (size_t)(T + 6) * 32 * C * 2 + 16;
                     const bool unit = A.max_weight == 1 && kc <= kUnitCols && uneed <= (size_t)kPool;
                     const int ucols = 32 * C;
                     if (kc > kColCap || (!unit && need > (size_t)kPool)) {
@@ -1329,8 +1331,11 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                         int64_t *stk = rowb + 2 * pitch;             // [levels][cols]
                         uint32_t *bits = (uint32_t *)(stk + (size_t)levels * cols);   // [T / 32][cols]
                         int64_t *ustk = (int64_t *)pool;             // [levels][ucols]
-                        uint16_t *first = (uint16_t *)(ustk + (size_t)levels * ucols);       // [T][ucols]
+                        // [T + 4][ucols], two rows of zeros (and a little) before
+                        uint16_t *first = (uint16_t *)(ustk + (size_t)levels * ucols) + 8 + 2 * ucols;
                         uint16_t *stf = first + (size_t)(T + 4) * ucols;     // [levels][ucols]
+                        if (unit)
+                            for (int i = tid; i < 8 + 2 * ucols; i += kThreads) first[i - 8 - 2 * ucols] = 0;
                         if (!unit) {
                             for (int i = tid; i < 2 * pitch; i += kThreads) rowb[i] = i % pitch < guard ? -2 * kBig : 0;
                             for (int r = tid; r < T; r += kThreads)
@@ -1361,13 +1366,24 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                             // next row that is taken or whose skip is no leaf's
                             if (tid == 0) {
                                 int r = T - 1, j = kc;
-                                int m = 0;                   // rows taken, listed in R.last
-                                while (unit && r >= 0 && j > 0) {
-                                    const int f = first[r * ucols + j - 1];
-                                    if (f == kNoRow) break;
-                                    R.last[m++] = f;
-                                    r = f - 1;
-                                    --j;
+                                int m = 0;                   // rows taken (plus 1), listed in R.last
+                                if (unit) {
+                                    // Four steps a trip, nothing tested in between (a branch a
+                                    // step: 94 ns each, so 26): after a 0 the walk stays in
+                                    // the zeros.  What it reads left of
+                                    // column 1, after kc steps, is not listed.
+                                    for (; m < kc; m += 4) {
+                                        int v = 0;
+#pragma unroll
+                                        for (int u = 0; u < 4; ++u) {
+                                            v = first[r * ucols + j - 1];
+                                            R.last[m + u] = v;
+                                            r = v - 2;
+                                            --j;
+                                        }
+                                        if (v == 0) break;
+                                    }
+                                    m = min(m + 4, kc);
                                 }
                                 while (!unit && r >= 0 && j > 0) {
                                     const int blk = r >> 5;
@@ -1376,7 +1392,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                                     const int rr = (r & ~31) + 31 - __clz((int)cand);      // below the block if none
                                     const int2 st = R.step[max(rr, 0)];
                                     const bool none = cand == 0, take = (cand & word) >> (rr & 31) & 1u;
-                                    if (!none && take) R.last[m++] = rr;
+                                    if (!none && take) R.last[m++] = rr + 1;
                                     j -= !none && take ? st.x : 0;
                                     r = none || take ? rr - !none : st.y;
                                 }
@@ -1387,17 +1403,20 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
                             }
                             __syncthreads();
                             for (int i = tid; i < s_a; i += kThreads) {
-                                const int x = R.pos[R.last[i]];
+                                if (R.last[i] == 0) continue;
+                                const int x = R.pos[R.last[i] - 1];
                                 atomicOr(taken + (x >> 5), 1u << (x & 31));
                             }
                         } else {
                             out = 5;
                             okey = vkey = vkey < 0 ? need_key : min(vkey, need_key);
                             int same;
-                            if (pass == 0 && up_to(INT_MAX, okey, same) > kRowCap) {
-                                // a V from more rows may need fewer
+                            if (pass < kPasses - 2 && up_to(INT_MAX, okey, same) > kRowCap) {
+                                // a V from more rows may need fewer (an item of 50,000
+                                // rows: 16,299 left by the V of 591 rows, 1,447 by that of
+                                // 1,010; the sweep of the former took 1.5 ms)
                                 int more;
-                                up_to(2 * kFirstRows, kBins, more);
+                                up_to(T < kMoreRows * 7 / 8 ? kMoreRows : kRowCap, kBins, more);
                                 if (more > key) {
                                     out = 2;
                                     okey = more;
