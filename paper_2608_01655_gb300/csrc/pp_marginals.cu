@@ -227,9 +227,12 @@ __device__ __forceinline__ int64_t top2_share(int32_t n, int32_t W, int32_t h, i
 }
 
 // A lane per chunk; a changed chunk's tables, and a stale marginal unless many
-// lanes have one, are the whole warp's work, a lane per requester: one lane
+// lanes have one, are the work of G lanes, a lane per requester: one lane
 // alone waited for memory W times (and W times per holder in a rebuild), which
-// was 53 us a pass whatever n.
+// was 53 us a pass whatever n.  Changed chunks lie next to one another
+// (subtrees), so a warp's 32 chunks are four runs of 8 (a sector of masks)
+// from the four quarters of the order, and 32 / G chunks are done at once.
+template <int G>                             // lanes per chunk: the power of two from W on, at least 8
 __global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W, const int32_t *__restrict__ worker,
                                                          const uint32_t *__restrict__ mask,
                                                          const int64_t *__restrict__ g, Top2 t,
@@ -255,9 +258,22 @@ __global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W, co
     int64_t *marg = t.marg + tb + (size_t)h * n;
     uint32_t *seen = t.seen + (size_t)item * n, *stale = t.stale + (size_t)item * n;
     int64_t held = 0;
-    for (int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
-        const int32_t i = i0 + lane;
+    constexpr int kAtOnce = 32 / G;
+    const int m = lane % G;                  // requester, where lanes share a chunk
+    const int32_t units = (n + 31) / 32, dw = gridDim.x * blockDim.x / 32;
+    for (int32_t x0 = (blockIdx.x * blockDim.x + threadIdx.x) / 32; x0 < units; x0 += dw) {
+        const int32_t i = ((lane >> 3) * units + x0) * 8 + (lane & 7);
         const bool in = i < n;
+        // the lane whose chunk this lane's group takes of the lanes in `c` (-1: none)
+        auto mine = [&](unsigned c) {
+            for (int q = 0; q < lane / G; ++q) c &= c - 1;
+            return __ffs((int)c) - 1;
+        };
+        auto rest = [](unsigned c) {
+#pragma unroll
+            for (int q = 0; q < kAtOnce; ++q) c &= c - 1;
+            return c;
+        };
         const uint32_t mk = in ? M[i] : 0, was = in ? seen[i] : 0, st = in ? stale[i] : 0;
         int64_t p = in ? marg[i] : 0;
         uint32_t s = st;
@@ -265,26 +281,30 @@ __global__ void __launch_bounds__(256) k_marginals_top2(int32_t n, int32_t W, co
             seen[i] = mk;
             s |= ~(mk ^ was);
         }
-        for (unsigned c = __ballot_sync(kAllLanes, mk != was); c; c &= c - 1) {
-            const int src = __ffs((int)c) - 1;
-            const uint32_t now = __shfl_sync(kAllLanes, mk, src), x = now ^ __shfl_sync(kAllLanes, was, src);
-            if (lane < W) top2_apply(n, W, __ffs(x) - 1, lane, i0 + src, now, (now & x) != 0, tb, g, t);
+        for (unsigned c = __ballot_sync(kAllLanes, mk != was); c; c = rest(c)) {
+            const int src = mine(c);
+            const uint32_t now = __shfl_sync(kAllLanes, mk, src & 31), x = now ^ __shfl_sync(kAllLanes, was, src & 31);
+            const int32_t at = __shfl_sync(kAllLanes, i, src & 31);
+            if (src >= 0 && m < W) top2_apply(n, W, __ffs(x) - 1, m, at, now, (now & x) != 0, tb, g, t);
         }
         __syncwarp();                        // the tables' new entries, before the shares below
         const bool old = (s >> h) & 1u;
-        const unsigned c = __ballot_sync(kAllLanes, old);
-        if (__popc(c) <= 8) {
-            for (unsigned o = c; o; o &= o - 1) {
-                const int src = __ffs((int)o) - 1;
-                int64_t v = lane < W ? top2_share(n, W, h, lane, i0 + src, tb, g, t) : 0;
+        const unsigned all = __ballot_sync(kAllLanes, old);
+        if (__popc(all) <= 8) {
+            for (unsigned c = all; c; c = rest(c)) {
+                const int src = mine(c);
+                const int32_t at = __shfl_sync(kAllLanes, i, src & 31);
+                int64_t v = src >= 0 && m < W ? top2_share(n, W, h, m, at, tb, g, t) : 0;
 #pragma unroll
-                for (int q = 16; q > 0; q >>= 1) v += __shfl_xor_sync(kAllLanes, v, q);
-                if (lane == src) p = v;
+                for (int q = G / 2; q > 0; q >>= 1) v += __shfl_xor_sync(kAllLanes, v, q);
+                const int rank = __popc(c & ((1u << lane) - 1));       // which group took this lane's chunk
+                v = __shfl_sync(kAllLanes, v, rank * G & 31);
+                if ((c >> lane & 1u) && rank < kAtOnce) p = v;
             }
         } else if (old) {
             p = 0;
 #pragma unroll 4
-            for (int32_t m = 0; m < W; ++m) p += top2_share(n, W, h, m, i, tb, g, t);
+            for (int32_t r = 0; r < W; ++r) p += top2_share(n, W, h, r, i, tb, g, t);
         }
         if (old) {
             marg[i] = p;
@@ -306,7 +326,8 @@ pp_status launch_marginals_top2(pp_instance *inst, int batch, const int32_t *wor
     int cap = (2 * inst->sm_count * 8 + batch - 1) / batch;
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    PP_CUDA(launch_chained(k_marginals_top2, dim3(bx, batch), dim3(256), 0, st, 1, inst->n, inst->W, worker, mask,
+    const auto kern = inst->W <= 8 ? k_marginals_top2<8> : inst->W <= 16 ? k_marginals_top2<16> : k_marginals_top2<32>;
+    PP_CUDA(launch_chained(kern, dim3(bx, batch), dim3(256), 0, st, 1, inst->n, inst->W, worker, mask,
                            inst->d_g, t2, item_active, profit, oldsum, inst->d_status));
     return PP_OK;
 }

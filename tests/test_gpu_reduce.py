@@ -111,3 +111,18 @@ def test_ties_and_zero_budget_and_long_paths(pp, oracle_lib):
         def swept(r, want=want, m=m):
             assert (r[0] == m) == want
         _check(pp, oracle_lib, _tree(rng, "chain", m), np.ones(m, np.int32), p, [m], swept)
+
+
+@pytest.mark.parametrize("n", [31, 257, 1030])
+@pytest.mark.parametrize("W", [1, 8, 9, 16, 17, 32])
+def test_kept_marginals_of_every_lane_group(pp, oracle_lib, n, W):
+    """Plans from top-2 tables at the widths where 8, 16 and 32 lanes share a
+    chunk, over orders that do not fill their four quarters: many chunks change
+    per update, so several are done at once, in one lane group and the next."""
+    rng = np.random.default_rng(n * 40 + W)
+    inst = wl.random_small(rng, n, W, 1, k_max=max(2, n // 4), w_max=2, demand_max=20)
+    o = oracle_lib.plan(oracle_lib.Problem.from_instance(inst), 2, 2)
+    with pp.Instance.from_workload(inst) as ppi:
+        g = pp.pp_plan_run(ppi, 2, None, 2, marginals=2)
+    assert g.used_top2 and g.objective == o.objective
+    np.testing.assert_array_equal(g.placement, o.placement)
