@@ -199,7 +199,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 return s;
             if ((s = mark())) return s;
             if ((s = mark())) return s;   // no traceback for the standalone scores
-            launches += 3 + (gw.split ? 1 : 0) + (work.red ? 1 : 0);     // a split DP is two launches
+            launches += 3 + (gw.split ? 1 : 0);     // a split DP is two launches
             dp_launches += 1;
             std::vector<int64_t> score(W);
             standalone_cells = (int64_t)n * sumk;
@@ -356,7 +356,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
             a.greedy = greedy;
             if ((r = launch_traceback(inst, S, work, g, kb, nullptr, &a, st))) return r;
             if ((r = mark())) return r;
-            launches += 4 + (g.split ? 1 : 0) + (work.red ? 1 : 0);
+            launches += 4 + (g.split ? 1 : 0);
             dp_launches += 1;
             return PP_OK;
         };
@@ -469,7 +469,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 a.greedy = pass == 0;
                 if ((s = launch_traceback(inst, b, wx, g1, kb, nullptr, &a, sx))) return s;
                 if ((s = smark(q0, sx))) return s;
-                launches += 4 + (work.red ? 1 : 0);
+                launches += 4;
                 if (pass > 0 && t == W - 1) {
                     k_sweep_end<<<(b + 31) / 32, 32, 0, sx>>>(b, pb.active + x, pb.improved + x, pb.sweeps + x);
                     PP_CUDA(cudaGetLastError());

@@ -46,7 +46,7 @@
 #include <climits>
 #include <cstring>
 
-#include "pp_internal.cuh"
+#include "pp_prune.cuh"
 
 namespace pp {
 
@@ -124,6 +124,9 @@ struct Args {
     int64_t total_weight;
     int32_t max_weight;
     int32_t clip_kid;            // the search's bound on what a light child adds
+    const int2 *pspan;           // the pruned sweep's: see prune_item
+    int32_t stack_depth;
+    int32_t *status;
 };
 
 __host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
@@ -828,10 +831,17 @@ __device__ __forceinline__ void dp_unit(const Rows &R, int T, int64_t *stk, uint
         if (kc == 1 + lane * C + c) *result = cur[c];
 }
 
+// the rows of an item that stays unsolved (not inlined: its registers are not
+// the reduction's)
+__device__ __noinline__ void prune_left(const Args &A, int item, const uint32_t *ud)
+{
+    prune_item(A.t.n, item, A.profit, A.order, A.next, A.pspan, A.wpre, A.w, ud, 1, A.stack_depth, A.status, A.rows_kept);
+}
+
 }  // namespace
 
 template <bool SMEM>                         // accumulators of the bins in shared memory
-__global__ void __launch_bounds__(kThreads) k_reduce(Args A)
+__global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Args A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned char leaf[kWarps * kMaxTiles];   // tiles of level 0: see the gather
@@ -851,8 +861,9 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
     int32_t *red = A.w.red + item;
     if (A.item_active && !A.item_active[item]) return;      // uniform over the cluster
     const int32_t kreq = A.item_budget[item];
-    if (kreq < 0 || kreq > A.max_budget) {                  // the pruned sweep's kernel reports it
+    if (kreq < 0 || kreq > A.max_budget) {                  // the DP's kernel reports it
         if (cr == 0 && tid == 0) *red = 0;
+        prune_left(A, item, nullptr);
         return;
     }
     const int64_t k = kreq < A.total_weight ? kreq : A.total_weight;     // more changes nothing
@@ -1466,6 +1477,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(Args A)
             A.w.base[item] = (int64_t)__ldcg(&g.s->vfix[pass]);
         }
     }
+    if (state != 1) prune_left(A, item, state == 2 ? freeb : nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -1783,6 +1795,9 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.item_bytes = reduce_item_bytes(inst);
     a.total_weight = inst->total_weight;
     a.max_weight = inst->max_weight;
+    a.pspan = inst->d_pspan;
+    a.stack_depth = inst->stack_depth;
+    a.status = inst->d_status;
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
     // As many CTAs per item as the items in flight leave SMs for (whole plans,
     // 16 CTAs an item against 8: 2 starts of 200,000 rows 11.9 and 15.7 ms, 8
