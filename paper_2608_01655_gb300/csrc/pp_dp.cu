@@ -1079,7 +1079,7 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
 
 // Skip-row stack levels below shared memory, per item (the larger need of the
 // two launches of a split).
-static int dp_global_levels(const pp_instance *inst, const DpGeom &g)
+int dp_global_levels(const pp_instance *inst, const DpGeom &g)
 {
     return std::max(0, inst->stack_depth - (g.split ? std::min(g.L_smem, g.L_smem2) : g.L_smem));
 }

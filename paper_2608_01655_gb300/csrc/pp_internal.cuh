@@ -204,6 +204,8 @@ struct pp_instance {
     std::vector<cudaStream_t> plan_streams;
     std::vector<cudaEvent_t> plan_join;
     cudaEvent_t plan_fork = nullptr;
+    cudaStream_t sg_stream = nullptr;        // safeguard candidates beside a plan
+    cudaEvent_t sg_fork = nullptr, sg_join = nullptr;
     std::vector<cudaEvent_t> phase_events;      // timing events of pp_plan_run, reused across calls
 };
 
@@ -278,6 +280,8 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
                         const int32_t *item_budget, const int32_t *item_active, int64_t *best, const DpWork &work,
                         cudaStream_t st, int32_t max_budget, unsigned long long *rows_kept);
 // scratch for the skip-row stack of `items` item slots of geometry g
+// levels of the stack of skipped rows that do not fit in shared memory
+int dp_global_levels(const pp_instance *inst, const DpGeom &g);
 pp_status ensure_dp_stack(pp_instance *inst, const DpGeom &g, int items);
 
 pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,
@@ -323,14 +327,22 @@ pp_status launch_traceback(pp_instance *inst, int batch, const DpWork &work, con
                            const int32_t *item_budget, uint8_t *chosen, const AcceptArgs *acc,
                            cudaStream_t st);
 
-// Safeguard candidates (requester-side): Independent, Popularity, LocalDedup
-// holder masks [3][n] in preorder (device, in inst->sg, valid until the next
-// call) and their objectives (host [3]).  Adds its kernel launches and DP
-// cells to the counters.
 pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t R, uint8_t *placement,
                     int64_t *objective, pp_plan_stats *stats, cudaStream_t st, bool orders_only = false);
 
-pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **masks, int64_t *obj,
-                          int *launches, int64_t *cells, int *dp_launches);
+// Safeguard candidates (requester-side): Independent, Popularity, LocalDedup
+// holder masks in preorder (in inst->sg, valid until the next call), their
+// objectives, and what they cost.
+struct SafeguardRun {
+    const uint32_t *masks = nullptr;     // [3][n], device
+    const int64_t *obj = nullptr;        // [3], device
+    int launches = 0, dp_launches = 0;
+    int64_t cells = 0;
+    bool enqueued = false;
+};
+// `beside`: other work of the instance runs meanwhile, so enqueue nothing if the
+// DP's stack of skipped rows, which that work may use, would be needed
+pp_status safeguards_enqueue(pp_instance *inst, cudaStream_t st, SafeguardRun *run, bool beside);
+pp_status safeguards_read(const SafeguardRun &run, cudaStream_t st, int64_t *obj);
 
 }  // namespace pp

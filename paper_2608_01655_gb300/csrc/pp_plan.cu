@@ -146,6 +146,29 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
 
     // optional per-phase timing: events around every launch, read once at the end
     const bool timing = stats && stats->time_phases;
+
+    // The safeguard candidates need nothing of the starts, and LocalDedup is W
+    // dependent updates of one item: they run beside the starts on a stream of
+    // their own (RAG plan, 8 workers: 3.93 ms after them, 2.69 beside; not when
+    // phases are timed).
+    const bool safeguards = inst->mode == PP_TRANSFER_REQUESTER && !(stats && stats->no_safeguards) && !orders_only;
+    SafeguardRun sg;
+    struct Settle {                          // nothing stays in flight on that stream
+        cudaStream_t stream = nullptr;
+        ~Settle() { if (stream) cudaStreamSynchronize(stream); }
+    } settle;
+    if (safeguards && !timing) {
+        if (!inst->sg_stream) {
+            PP_CUDA(cudaEventCreateWithFlags(&inst->sg_fork, cudaEventDisableTiming));
+            PP_CUDA(cudaEventCreateWithFlags(&inst->sg_join, cudaEventDisableTiming));
+            PP_CUDA(cudaStreamCreateWithFlags(&inst->sg_stream, cudaStreamNonBlocking));
+        }
+        PP_CUDA(cudaEventRecord(inst->sg_fork, st));
+        PP_CUDA(cudaStreamWaitEvent(inst->sg_stream, inst->sg_fork, 0));
+        settle.stream = inst->sg_stream;
+        if ((s = safeguards_enqueue(inst, inst->sg_stream, &sg, true))) return s;
+        PP_CUDA(cudaEventRecord(inst->sg_join, inst->sg_stream));
+    }
     int32_t dp_launches = 0;
     std::vector<cudaEvent_t> ev;        // lock step: every mark; per-start streams: the standalone step
     size_t pool_used = 0;
@@ -511,15 +534,20 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     const uint32_t *best_mask = pb.mask + (size_t)bs * n;
     // requester-side safeguard candidates S, S+1, S+2 (ties stay with the lower index)
     int64_t so[3] = {0, 0, 0};
-    if (inst->mode == PP_TRANSFER_REQUESTER && !(stats && stats->no_safeguards)) {
-        const uint32_t *sgm = nullptr;
-        if ((s = safeguards_impl(inst, st, &sgm, so, &launches, &cells, &dp_launches))) return s;
+    if (safeguards) {
+        if (sg.enqueued) PP_CUDA(cudaStreamWaitEvent(st, inst->sg_join, 0));
+        else if ((s = safeguards_enqueue(inst, st, &sg, false))) return s;
+        if ((s = safeguards_read(sg, st, so))) return s;      // waits for them
+        settle.stream = nullptr;
+        launches += sg.launches;
+        cells += sg.cells;
+        dp_launches += sg.dp_launches;
         dp_count += 3 * W;
         for (int c = 0; c < 3; ++c)
             if (so[c] > best_obj) {
                 best_obj = so[c];
                 bs = S + c;
-                best_mask = sgm + (size_t)c * n;
+                best_mask = sg.masks + (size_t)c * n;
             }
     }
     std::vector<uint32_t> mk(std::max(n, 1));

@@ -52,8 +52,7 @@ __global__ void k_or_rows(int32_t n, int32_t W, int32_t C, const uint32_t *__res
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **masks, int64_t *obj,
-                          int *launches, int64_t *cells, int *dp_launches)
+pp_status safeguards_enqueue(pp_instance *inst, cudaStream_t st, SafeguardRun *run, bool beside)
 {
     if (inst->mode != PP_TRANSFER_REQUESTER)
         return fail(PP_EINVAL, "safeguard candidates are defined for the requester-side objective only");
@@ -68,6 +67,8 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
     DpGeom gB, g1;
     if (!dp_geometry(inst, maxk, &gB, B) || !dp_geometry(inst, maxk, &g1, 1))
         return fail(PP_EINVAL, "budget too large for the DP kernel");
+    run->enqueued = !beside || (dp_global_levels(inst, gB) <= 0 && dp_global_levels(inst, g1) <= 0);
+    if (!run->enqueued) return PP_OK;
     const size_t N = (size_t)std::max(n, 1);
     // rows [B][n] | cand [3][n] | profit [B][n] | best [B] | objd [3] | ints [5][B] | DP work
     const size_t o_rows = 0, o_cand = o_rows + a256(4 * N * B), o_prof = o_cand + a256(4 * N * 3);
@@ -136,12 +137,18 @@ pp_status safeguards_impl(pp_instance *inst, cudaStream_t st, const uint32_t **m
     }
     if ((s = launch_objective(inst, 3, cand, nullptr, objd, st))) return s;
     nl += 1;
-    PP_CUDA(cudaMemcpyAsync(obj, objd, 8 * 3, cudaMemcpyDeviceToHost, st));
+    run->masks = cand;
+    run->obj = objd;
+    run->launches = nl;
+    run->cells = 3 * (int64_t)n * sumk;
+    run->dp_launches = (n > 0 && W > 0) ? 1 + W : 0;
+    return PP_OK;
+}
+
+pp_status safeguards_read(const SafeguardRun &run, cudaStream_t st, int64_t *obj)
+{
+    PP_CUDA(cudaMemcpyAsync(obj, run.obj, 8 * 3, cudaMemcpyDeviceToHost, st));
     PP_CUDA(cudaStreamSynchronize(st));
-    *masks = cand;
-    if (launches) *launches += nl;
-    if (cells) *cells += 3 * (int64_t)n * sumk;
-    if (dp_launches) *dp_launches += (n > 0 && W > 0) ? 1 + W : 0;
     return PP_OK;
 }
 
@@ -156,9 +163,11 @@ extern "C" pp_status pp_safeguards(pp_instance *inst, uint8_t *placement, int64_
     PP_CUDA(cudaGetDevice(&cur));
     if (cur != inst->device) return fail(PP_EINVAL, "the instance's device must be the current device");
     cudaStream_t st = (cudaStream_t)stream;
-    const uint32_t *masks = nullptr;
-    pp_status s = safeguards_impl(inst, st, &masks, objective, nullptr, nullptr, nullptr);
+    SafeguardRun run;
+    pp_status s = safeguards_enqueue(inst, st, &run, false);
     if (s != PP_OK) return s;
+    if ((s = safeguards_read(run, st, objective)) != PP_OK) return s;
+    const uint32_t *masks = run.masks;
     const int32_t n = inst->n, W = inst->W;
     std::memset(placement, 0, (size_t)3 * W * n);
     if (n == 0) return PP_OK;

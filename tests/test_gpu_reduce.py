@@ -126,3 +126,17 @@ def test_kept_marginals_of_every_lane_group(pp, oracle_lib, n, W):
         g = pp.pp_plan_run(ppi, 2, None, 2, marginals=2)
     assert g.used_top2 and g.objective == o.objective
     np.testing.assert_array_equal(g.placement, o.placement)
+
+
+@pytest.mark.parametrize("starts,schedule", [(1, 0), (3, 0), (3, 1), (9, 2)])
+def test_safeguards_beside_the_starts(pp, oracle_lib, starts, schedule):
+    """Candidates computed on their own stream while the starts run are those
+    computed after them (a plan whose phases are timed), call after call."""
+    inst = wl.random_small(np.random.default_rng(starts), 900, 5, 0, k_max=200, w_max=2, demand_max=50)
+    o = oracle_lib.plan(oracle_lib.Problem.from_instance(inst), starts, 2)
+    with pp.Instance.from_workload(inst) as ppi:
+        for timed in (False, True, False, False):
+            g = pp.pp_plan_run(ppi, starts, None, 2, schedule=schedule, time_phases=timed)
+            assert list(g.safeguard_objective) == o.safeguard_objective.tolist()
+            assert g.objective == o.objective and g.best_start == o.best_start
+            np.testing.assert_array_equal(g.placement, o.placement)
