@@ -286,10 +286,15 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         t2.stale = reinterpret_cast<uint32_t *>(carve(4 * sn));
         t2.l1 = reinterpret_cast<int8_t *>(carve(tw));
         t2.marg = reinterpret_cast<int64_t *>(carve(8 * tw));
-        // v1 = v2 = 0 and no masks seen: nobody holds anything yet; l1 = -1 and
-        // every marginal stale
+        // v1 = v2 = 0 and no masks seen: nobody holds anything yet; l1 = -1
         PP_CUDA(cudaMemsetAsync(t2.v1, 0, (char *)t2.stale - (char *)t2.v1, st));
-        PP_CUDA(cudaMemsetAsync(t2.stale, 0xFF, (char *)t2.marg - (char *)t2.stale, st));
+        PP_CUDA(cudaMemsetAsync(t2.l1, 0xFF, tw, st));
+        // every worker's marginals against an empty placement are the profits
+        // of the standalone scores, where those were computed; else all are stale
+        // (each greedy update of a start read 33 W bytes a chunk for its own)
+        PP_CUDA(cudaMemsetAsync(t2.stale, standalone_cells > 0 ? 0 : 0xFF, 4 * sn, st));
+        for (int32_t x = 0; x < S && standalone_cells > 0; ++x)
+            PP_CUDA(cudaMemcpyAsync(t2.marg + (size_t)x * W * n, pb.profit, 8 * (size_t)W * n, cudaMemcpyDeviceToDevice, st));
     }
     PP_CUDA(cudaMemsetAsync(pb.improved, 0, 4 * S, st));
     PP_CUDA(cudaMemsetAsync(pb.oldsum, 0, 16 * (size_t)B, st));
