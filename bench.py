@@ -13,13 +13,15 @@ W = 16 workers, k = 4,096 slots, 16 starts, 6 rounds), inputs resident in HBM.
   e2e       the same metric through the C ABI from pinned host buffers:
             pp_instance_create (upload + tables) + pp_plan_run (placement
             back to the host) + pp_instance_destroy, every step
-  roofline  the tree-DP step (dominant): the algorithmic bytes of the paper's
-            table algorithm (decision bits n(k+1)/8, p/w/next 16n, every
-            pushed skip row written and read once 16(k+1) per push, the
-            traceback's at most n states 8n) per DP, times the DPs of a step,
+  roofline  the tree-DP step (dominant): the bytes that any exact update has to
+            move per DP (p/w/next 16n, the set n/8), times the DPs of a step,
             over the step's CUDA-event time, against the measured HBM copy
-            bandwidth; the dependent row chain that actually limits the kernel
-            is reported beside it (t_row_min)
+            bandwidth.  The bytes of the paper's table algorithm (decision bits
+            n(k+1)/8, p/w/next 16n, every pushed skip row written and read once
+            16(k+1) per push, the traceback's at most n states 8n) are reported
+            beside it, over the same time: the exact reduction decides most
+            chunks without forming their rows, so that ratio is above the
+            bandwidth.  What limits the step is latency (limiter)
   cpu_baseline  the CPU oracle's whole plan of the same workload on the
             host's cores (one thread per start), outside the timed region
   configs   the same measurements for all five synthetic workloads (tiny,
@@ -289,8 +291,9 @@ def _probe_read_gbs(torch, stream, nbytes, iters):
 
 def _t_row_min(pp, torch, inst, ppi, res, S, stream):
     """Per-row time of the smallest DP launch shape (one warp per DP, 32
-    columns, no hand-off between warps) on the plan's last marginals: the
-    dependent row chain alone."""
+    columns, no hand-off between warps) on the plan's last marginals, over
+    every row of the tree (no reduction, no pruning): the dependent row chain
+    alone."""
     n = inst.n
     masks = np.zeros((S, n), np.uint32)
     for m in range(inst.W):
@@ -300,7 +303,7 @@ def _t_row_min(pp, torch, inst, ppi, res, S, stream):
     prof = torch.zeros((S, n), dtype=torch.int64, device="cuda")
     pp.pp_marginals(ppi, workers, masks_t, prof)
     kk = 32
-    pp.pp_tune_dp(ppi, 1, 1, False, False)
+    pp.pp_tune_dp(ppi, 1, 1, False, True)
     try:
         bud = torch.full((S,), kk, dtype=torch.int32, device="cuda")
         best = torch.zeros(S, dtype=torch.int64, device="cuda")
@@ -415,7 +418,7 @@ def plan_summary(inst, res, times, phase, e2e_times, h2d, d2h, l2_gbs, hbm_gbs):
         "bstream_frac_of_l2": items * tb["bstream_bytes_per_dp"] / dp_t / 1e9 / l2_gbs,
         "objective": res.objective, "best_start": res.best_start,
         "sweeps": res.per_start_sweeps.tolist(), "dp_count": res.dp_count, "dp_cells": res.dp_cells,
-        "dp_rows_swept": res.dp_rows_swept, "schedule": "per-start streams" if res.schedule == 2 else "lock step",
+        "dp_rows_swept": res.dp_rows_swept, "schedule": "starts on streams" if res.schedule == 2 else "lock step",
     }
     return out
 
@@ -570,7 +573,8 @@ def run_native(args):
     cells_swept = rows_swept * k
     tb = table_bytes(inst.parent, k)
     bmin_step = items * tb["bmin_bytes_per_dp"]
-    achieved = bmin_step / dp_t / 1e9
+    update_bytes = 16 * inst.n + (inst.n + 7) // 8              # p, w, next read; the set written
+    achieved = items * update_bytes / dp_t / 1e9
     l2_gbs = _probe_read_gbs(torch, stream, 32 << 20, 200)     # 32 MiB: resident in L2
     hbm_read_gbs = _probe_read_gbs(torch, stream, 4 << 30, 3)  # 4 GiB: far larger than L2
     t_row_min = _t_row_min(pp, torch, inst, ppi, res, S_mine, stream)
@@ -585,17 +589,23 @@ def run_native(args):
         "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
         "traffic": traffic,
         "peak_source": f"MEASURED_PEAKS.json hbm_gbs ({peak_kind} copy bandwidth)",
-        "achieved_source": ("algorithmic bytes of the paper's table algorithm per DP (bmin_bytes_per_dp: "
-                            "n(k+1)/8 decision bits + 16n p/w/next + 16(k+1) per skip-row push + 8n "
-                            "traceback) x DPs per step / the step's CUDA-event time"),
+        "achieved_source": ("bytes any exact update moves per DP (16n p/w/next + n/8 for the set) x DPs per "
+                            "step / the step's CUDA-event time"),
+        "update_bytes_per_dp": update_bytes,
+        "table_algorithm": {
+            "gbs": bmin_step / dp_t / 1e9, "over_hbm": bmin_step / dp_t / 1e9 / hbm_peak,
+            "source": ("bytes of the paper's table algorithm per DP (bmin_bytes_per_dp: n(k+1)/8 decision bits + "
+                       "16n p/w/next + 16(k+1) per skip-row push + 8n traceback) over the same time; the "
+                       "exact reduction never forms that table, so this is work avoided, not bandwidth")},
         "traffic_source": ("DRAM bytes per swept cell of a one-kernel ncu capture of the batched DP on the "
                            "small profile case, times the step's swept cells" if traffic is not None else
                            "no capture of the current DP sources"),
-        "limiter": ("latency: the dependent row chain of Eq. 9 (one warp's rows follow one another; "
-                    "t_dp_over_rows_x_t_row_min compares the step with that chain alone)"),
-        "kernel": ("k_prune + k_tree_dp_wave (one tree-DP step of the plan: every start's DP on its own "
-                   "stream, concurrently; duration = mean over starts of the start's DP events)"
-                   if per_start else "k_prune + k_tree_dp_wave (one batched tree-DP launch of the plan)"),
+        "limiter": ("latency: the levels of heavy paths in every price evaluation of the reduction, barriers "
+                    "between them, then the dependent rows of the undecided chunks (t_row_min_ns: one row of "
+                    "the sweep that is left out for the others)"),
+        "kernel": ("k_reduce + k_tree_dp_wave (one tree-DP step of the plan: the starts on streams, "
+                   "concurrently; duration = mean over the streams' DP events)"
+                   if per_start else "k_reduce + k_tree_dp_wave (one batched tree-DP launch of the plan)"),
         "launches": nl * args.steps, "launch_ms": 1000 * dp_t, "items_per_launch": items,
         **tb,
         "bmin_bytes_per_launch": bmin_step,
@@ -605,8 +615,7 @@ def run_native(args):
         "bstream_frac_of_l2": items * tb["bstream_bytes_per_dp"] / dp_t / 1e9 / l2_gbs,
         "l2_read_gbs_probe": l2_gbs, "hbm_read_gbs_probe": hbm_read_gbs,
         "t_row_min_ns": 1e9 * t_row_min,
-        "t_row_min_source": "one warp per DP, 32 columns, the same rows (pp_tune_dp(inst, 1, 1))",
-        "t_dp_over_rows_x_t_row_min": dp_t / ((rows_swept / items) * t_row_min),
+        "t_row_min_source": "one warp per DP, 32 columns, every row (pp_tune_dp(inst, 1, 1, no_prune))",
         "alu_model": {"achieved_tcells": cells_swept / dp_t / 1e12, "peak_tcells": alu_peak / 1e12,
                       "frac": cells_swept / dp_t / alu_peak,
                       "source": (f"derived, not measured: {SM_COUNT} SMs x {INT32_LANES_PER_SM} int32 ALU lanes x "
@@ -669,7 +678,7 @@ def run_native(args):
             "gpu_launches": res.kernel_launches * args.steps,
             "clocks": clocks,
             "plan": {"objective": best_obj, "best_start": best_start,
-                     "schedule": "per-start streams" if per_start else "lock step",
+                     "schedule": "starts on streams" if per_start else "lock step",
                      "hw_queues_assumed": res.hw_queues,
                      "dp_count": res.dp_count, "dp_cells": res.dp_cells,
                      "dp_launches": nl, "dp_rows_swept": res.dp_rows_swept,
@@ -739,7 +748,7 @@ def main():
                     help="skip the other four workloads and the side timings")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--schedule", choices=["auto", "lock", "per-start"], default="auto",
-                    help="plan schedule: automatic (per-start streams when the hardware queues allow), "
+                    help="plan schedule: automatic (groups of starts on eight streams), "
                          "lock step, or per-start streams")
     ap.add_argument("--profile-dp", type=int, default=0, metavar="B",
                     help="only launch the tree DP and traceback of B items twice (a small case for ncu) and exit")

@@ -75,10 +75,10 @@ typedef struct {
                                       pruning), summed */
     int32_t time_phases;           /* in: nonzero = time the phases below with CUDA events */
     float phase_ms[3];             /* out (if time_phases): device time of the marginal,
-                                      tree-DP (with its row pruning) and traceback launches,
-                                      summed over the plan's steps (per-start streams: the
-                                      mean over starts of each start's sum) */
-    int32_t dp_launches;           /* out: tree-DP steps (lock step: batched launches; per-start
+                                      tree-DP (with reduction and pruning) and traceback
+                                      launches, summed over the plan's steps (starts on
+                                      streams: the mean over streams of each one's sum) */
+    int32_t dp_launches;           /* out: tree-DP steps (lock step: batched launches; starts on
                                       streams: the mean over starts of executed updates),
                                       the standalone-score launch included */
     int32_t no_safeguards;         /* in: nonzero = leave out the safeguard candidates */
@@ -89,18 +89,20 @@ typedef struct {
                                       (Section IV-C); results are identical */
     int32_t used_top2;             /* out: 1 if the top-2 tables were used */
     int32_t schedule;              /* in: 0 automatic, 1 lock step (all starts advance together,
-                                      one batched launch per step), 2 per-start streams (each
-                                      start on its own stream, never waiting for a slower
-                                      one).  Automatic takes per-start streams when S > 1 and
-                                      CUDA_DEVICE_MAX_CONNECTIONS (read at the call; it acts
-                                      when the CUDA context is created) gives every stream its
-                                      own hardware queue, min(S, 32), else lock step.
-                                      out: the schedule used (1 or 2).  Results are identical */
+                                      one batched launch per step), 2 one stream per start
+                                      (none waits for a slower one).  Automatic with S > 1: up
+                                      to eight groups of starts, each group in lock step on a
+                                      stream of its own; where the exact reduction is off, one
+                                      stream per start if CUDA_DEVICE_MAX_CONNECTIONS (read at
+                                      the call; it acts when the CUDA context is created) gives
+                                      every stream its own hardware queue, min(S, 32), else
+                                      lock step.  out: 1 lock step, 2 starts on streams.
+                                      Results are identical */
     int32_t hw_queues;             /* out: the hardware queue count the automatic schedule assumed
                                       (CUDA_DEVICE_MAX_CONNECTIONS as read at the call, 8 when
                                       unset).  The driver reads that variable only when the CUDA
                                       context is created, so a context created before it was set
-                                      may have fewer queues: the per-start schedule then runs
+                                      may have fewer queues: one stream per start then runs
                                       slower, with the same results */
 } pp_plan_stats;
 
@@ -208,8 +210,8 @@ pp_status pp_marginals(pp_instance *inst, int32_t batch, const int32_t *worker,
  * `max_budget`: the decision bits plus the rows of the pruned sweep (rows
  * strictly below a chunk whose strict descendants all have profit <= 0 never
  * change a kept row's value or decision, so the DP skips them) and of the
- * exact reduction (chunks that are the same in every optimal set need no DP).  Returns 0 for
- * batch <= 0 or an invalid max_budget.
+ * exact reduction (chunks that are the same in every optimal set need no DP).
+ * Returns 0 for batch <= 0 or an invalid max_budget.
  */
 size_t pp_dp_bits_size(const pp_instance *inst, int32_t batch, int32_t max_budget);
 
@@ -304,9 +306,10 @@ pp_status pp_objective(pp_instance *inst, int32_t batch, const uint8_t *chosen, 
  * pp_plan_run -- Algorithm 1 (procedure PrefixPlace): for each start order,
  * one WorkerGreedy pass (Theorem 3), then at most max_rounds refinement
  * sweeps; a sweep with no accepted update ends that start.  Starts run
- * batched in lock step, or each on its own stream (stats->schedule).  With the requester-side objective the Independent, Popularity
- * and LocalDedup placements (pp_safeguards) join the candidates as indices
- * S, S+1, S+2 unless stats->no_safeguards is set.
+ * batched in lock step, or on several streams (stats->schedule).  With the
+ * requester-side objective the Independent, Popularity and LocalDedup
+ * placements (pp_safeguards) join the candidates as indices S, S+1, S+2 unless
+ * stats->no_safeguards is set; they are computed beside the starts.
  *   n_starts      S >= 1
  *   orders        host [S][W] permutations of 0..W-1, or NULL for the default:
  *                 S == 1 the identity; otherwise start 0 = standalone-score
@@ -373,7 +376,7 @@ pp_status pp_dp_stack_bytes(const pp_instance *inst, size_t *out);
  * sweeps (no counterpart in the paper): CTAs per cluster (1..8, 0 =
  * automatic), columns per thread (power of two up to 16, 0 = automatic),
  * force_flat != 0 selects the one-CTA kernel, no_prune != 0 sweeps every row
- * instead of the pruned sweep (results are the same either way).  Later
+ * instead of reducing and pruning (results are the same either way).  Later
  * pp_dp_bits_size / pp_tree_dp / pp_traceback / pp_plan_run calls on this
  * instance use it, so set it before sizing workspaces; other instances are
  * not affected.  Not thread-safe against concurrent calls on the same

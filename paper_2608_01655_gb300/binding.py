@@ -14,11 +14,11 @@ from dataclasses import dataclass
 
 import numpy as np
 
-# The plan's per-start schedule puts each start on its own CUDA stream; the
-# driver maps streams onto CUDA_DEVICE_MAX_CONNECTIONS hardware queues (8 by
-# default), and streams sharing a queue wait on one another's launches.  The
-# variable acts when the CUDA context is created, so it is set here, before
-# that, unless the caller has chosen a value.
+# A plan puts its starts on several CUDA streams; the driver maps streams onto
+# CUDA_DEVICE_MAX_CONNECTIONS hardware queues (8 by default), and streams
+# sharing a queue wait on one another's launches.  The variable acts when the
+# CUDA context is created, so it is set here, before that, unless the caller
+# has chosen a value.
 os.environ.setdefault("CUDA_DEVICE_MAX_CONNECTIONS", "32")
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -219,7 +219,7 @@ def pp_tree_dp_noalloc(inst: Instance, profit, budget, max_budget: int, best, bi
 
 
 def pp_dp_rows_swept(inst: Instance, batch: int, max_budget: int, bits, stream=None) -> np.ndarray:
-    """Rows each item of the last DP on `bits` swept after pruning."""
+    """Rows each item of the last DP on `bits` swept after reduction and pruning."""
     rows = np.zeros(max(int(batch), 1), np.int32)
     _check(_lib.pp_dp_rows_swept(inst.handle, int(batch), int(max_budget), _dev(bits), _host(rows),
                                  _stream(stream)))
@@ -253,7 +253,7 @@ class PlanResult:
     dp_launches: int = 0
     safeguard_objective: tuple = ()     # Independent, Popularity, LocalDedup (requester-side)
     used_top2: bool = False             # source-dependent marginals from top-2 holder tables
-    schedule: int = 0                   # 1 lock step, 2 per-start streams
+    schedule: int = 0                   # 1 lock step, 2 starts on streams
     hw_queues: int = 0                  # hardware queues the automatic schedule assumed
 
 
@@ -261,8 +261,9 @@ def pp_plan_run(inst: Instance, n_starts: int, orders=None, max_rounds: int = 0,
                 time_phases: bool = False, safeguards: bool = True, marginals: int = 0,
                 schedule: int = 0) -> PlanResult:
     """marginals (source-dependent): 0 automatic, 1 holder scan, 2 top-2 tables.
-    schedule: 0 automatic, 1 lock step (one batched launch per step), 2 one
-    stream per start; the results are identical."""
+    schedule: 0 automatic (groups of starts on up to eight streams), 1 lock step
+    (one batched launch per step), 2 one stream per start; the results are
+    identical."""
     S, W, n = int(n_starts), inst.W, inst.n
     placement = np.zeros((W, max(n, 1)), np.uint8)
     obj = _i64(0)

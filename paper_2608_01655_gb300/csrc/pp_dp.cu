@@ -21,7 +21,9 @@
 //   warp g lagging warp g-1 by a sub-block of rows.  Every wait is bounded in
 //   time and reports PP_ETIMEOUT through the status word.
 // k_tree_dp_flat (any weight): one CTA per DP, row i+1 staged in shared memory
-//   and one __syncthreads per row.
+//   and one barrier per row.
+// Both sweep what the exact reduction (pp_reduce.cu) leaves: nothing for the
+// items that it solves, and the rows of pp_prune.cuh for the others.
 //
 // Skip rows: next(i) = i+1 is the row just computed (registers), next(i) = n
 // is the zero row, and any other next(i) is the top of the skip-row stack,

@@ -89,7 +89,8 @@ struct DpGeom {
 // profits, kept-row counts).  A row is dropped when every strict descendant
 // of its parent has a non-positive profit: such a parent's interior is never
 // taken and leaves D[parent+1] = D[next(parent)], so dropping those rows
-// changes no value and no bit of a kept row (see k_prune).
+// changes no value and no bit of a kept row (see pp_prune.cuh).  Then the exact
+// reduction's: states, sets as bitmaps, scratch.
 // For the traceback, per kept row t (kept index, sweep order): skip[t] = kept
 // index of next(row t), -1 when next(row t) = n; wsuf[t] = sum of the
 // weights of kept rows t..nkept-1.
@@ -199,7 +200,7 @@ struct pp_instance {
     // lower priority), forked from and joined back to the caller's stream
     cudaStream_t split_hi = nullptr, split_lo = nullptr;
     cudaEvent_t split_fork = nullptr, split_join_hi = nullptr, split_join_lo = nullptr;
-    // pp_plan_run without lock step: one stream per start (up to kPlanStreams),
+    // pp_plan_run without lock step: a stream per start or group (up to kPlanStreams),
     // forked from and joined back to the caller's stream
     std::vector<cudaStream_t> plan_streams;
     std::vector<cudaEvent_t> plan_join;

@@ -34,7 +34,8 @@ __global__ void k_sweep_end(int S, int32_t *active, int32_t *improved, int32_t *
 
 // streams of the per-start schedule (starts beyond share them round-robin)
 constexpr int kPlanStreams = 32;
-constexpr int kGroupStreams = 8;        // streams of groups of starts (the driver's default hardware queues)
+constexpr int kGroupStreams = 8;        // streams of groups of starts: the driver's default hardware queues (16 starts
+                                        // of 50,000 chunks in 4, 5 and 8 groups: 29.9, 30.0 and 27.6 ms)
 
 static pp_status ensure_plan_streams(pp_instance *inst, int ns)
 {
@@ -170,7 +171,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         PP_CUDA(cudaEventRecord(inst->sg_join, inst->sg_stream));
     }
     int32_t dp_launches = 0;
-    std::vector<cudaEvent_t> ev;        // lock step: every mark; per-start streams: the standalone step
+    std::vector<cudaEvent_t> ev;        // lock step: every mark; on streams: the standalone step
     size_t pool_used = 0;
     auto take = [&](cudaEvent_t *e) -> pp_status {
         if (pool_used == inst->phase_events.size()) {
@@ -338,20 +339,20 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         launches += 1;
         return PP_OK;
     };
-    // lock step unless asked for per-start streams, or (automatic) unless every
-    // start's stream gets a hardware queue of its own: streams that share a
-    // queue wait on one another's launches, which costs more than lock step
     const int32_t sched = stats ? stats->schedule : 0;
     // With the exact reduction an update is short, and launches count: the
     // automatic schedule puts groups of starts on kGroupStreams streams, each
-    // group in lock step (paper-scale plan, 16 starts: one group 52.6 ms, one
-    // stream per start 72 ms with 8 hardware queues and 37 ms with 32)
+    // group in lock step (16 starts of 50,000 chunks, when this was chosen: one
+    // group 52.6 ms, one stream per start 72 ms with 8 hardware queues and 37
+    // with 32, eight groups 39).  Without it: one stream per start if every
+    // stream gets a hardware queue of its own, else lock step (streams that
+    // share a queue wait on one another's launches)
     const bool grouped = sched == 0 && work.red && S > 1;
     const int gs = grouped ? (S + kGroupStreams - 1) / kGroupStreams : 1;      // starts per stream
     const bool lockstep = S == 1 || sched == 1 ||
                           (sched == 0 && !grouped && hardware_queues() < std::min<int>(S, kPlanStreams));
-    int32_t start_steps = 0;            // per-start streams: updates launched per start
-    std::vector<std::vector<cudaEvent_t>> sev;   // per-start streams: each start's phase events
+    int32_t start_steps = 0;            // on streams: updates launched per start
+    std::vector<std::vector<cudaEvent_t>> sev;   // on streams: each stream's phase events
     if (lockstep) {
         auto step = [&](int t, int greedy) -> pp_status {
             const int32_t *wk = pb.work + (size_t)t * B;

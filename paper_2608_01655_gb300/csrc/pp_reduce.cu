@@ -22,12 +22,13 @@
 // their keys (an order-preserving 11-bit code of the loss), so every test
 // errs on the side of keeping a row.
 //
-// A prefix tree of 50,000 chunks with the planner's profits leaves 10 to 1,500
+// A prefix tree of 50,000 chunks with the planner's profits leaves 30 to 600
 // undecided rows of the 16,000 to 37,000 that the pruned sweep keeps, and a
-// budget of a few hundred slots instead of 4,096.  More undecided rows than
-// fit on chip (chunks in long chains that are worth taking only whole) go to
-// pp_dp.cu's kernels with what is left of the budget; where no V is found
-// (ties that leave nearly everything undecided) those kernels get every row.
+// budget of a few hundred slots instead of 4,096: 0.19 ms an item, where that
+// sweep took 1.3.  More undecided rows than fit on chip (chunks in long chains
+// that are worth taking only whole) go to pp_dp.cu's kernels with what is left
+// of the budget; where no V is found (ties that leave nearly everything
+// undecided) those kernels get every row.
 //
 // Layout.  f is a Lindley recursion along every heavy path of the tree
 // (y_i = max(0, d_i + y_(i+1)), d_i the row's own term plus its light
@@ -756,7 +757,7 @@ __device__ __forceinline__ void dp_rows(const Rows &R, int T, int act, int guard
 
 // Unit weights and at most 128 columns: one warp, C columns per lane (column
 // j = 1 + lane * C + c) in registers, the column shift a shuffle, no barrier:
-// 24 to 40 ns a row against 90 with a barrier per row.  Instead of decision
+// 38 to 80 ns a row (C and stack rows) against 98 with a barrier per row.  Instead of decision
 // bits it keeps, per row and column, the first row taken from there on, plus
 // 1 (0: none; following skips changes nothing), so the walk takes one step per
 // chunk.
