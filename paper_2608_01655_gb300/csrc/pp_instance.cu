@@ -243,6 +243,8 @@ extern "C" pp_status pp_instance_destroy(pp_instance *inst)
     for (cudaStream_t x : inst->plan_streams) cudaStreamDestroy(x);
     for (cudaEvent_t x : inst->plan_join) cudaEventDestroy(x);
     if (inst->plan_fork) cudaEventDestroy(inst->plan_fork);
+    if (inst->sweep_flags) cudaFreeHost(inst->sweep_flags);
+    for (cudaEvent_t x : inst->sweep_events) cudaEventDestroy(x);
     if (inst->sg_stream) cudaStreamDestroy(inst->sg_stream);
     if (inst->sg_fork) cudaEventDestroy(inst->sg_fork);
     if (inst->sg_join) cudaEventDestroy(inst->sg_join);

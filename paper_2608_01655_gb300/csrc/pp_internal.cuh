@@ -205,6 +205,9 @@ struct pp_instance {
     std::vector<cudaStream_t> plan_streams;
     std::vector<cudaEvent_t> plan_join;
     cudaEvent_t plan_fork = nullptr;
+    int32_t *sweep_flags = nullptr;          // pinned host memory: starts that go on
+    int sweep_flags_count = 0;
+    std::vector<cudaEvent_t> sweep_events;
     cudaStream_t sg_stream = nullptr;        // safeguard candidates beside a plan
     cudaEvent_t sg_fork = nullptr, sg_join = nullptr;
     std::vector<cudaEvent_t> phase_events;      // timing events of pp_plan_run, reused across calls

@@ -22,7 +22,8 @@ constexpr size_t kTop2MaxBytes = (size_t)24 << 30;
 constexpr size_t kTop2Bytes = 17 + 8;
 
 // per-sweep bookkeeping: a start that accepted nothing is done
-__global__ void k_sweep_end(int S, int32_t *active, int32_t *improved, int32_t *sweeps)
+// (`seen`, if given: host memory, what the starts are now)
+__global__ void k_sweep_end(int S, int32_t *active, int32_t *improved, int32_t *sweeps, int32_t *seen)
 {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < S && active[s]) {
@@ -30,6 +31,7 @@ __global__ void k_sweep_end(int S, int32_t *active, int32_t *improved, int32_t *
         active[s] = improved[s];
         improved[s] = 0;                // for the next sweep
     }
+    if (s < S && seen) seen[s] = active[s];
 }
 
 // streams of the per-start schedule (starts beyond share them round-robin)
@@ -48,6 +50,24 @@ static pp_status ensure_plan_streams(pp_instance *inst, int ns)
         inst->plan_join.push_back(e);
     }
     if (!inst->plan_fork) PP_CUDA(cudaEventCreateWithFlags(&inst->plan_fork, cudaEventDisableTiming));
+    return PP_OK;
+}
+
+// host flags that k_sweep_end writes, and an event per group for two sweeps
+static pp_status ensure_sweep_flags(pp_instance *inst, int starts, int events)
+{
+    if (inst->sweep_flags_count < starts) {
+        if (inst->sweep_flags) cudaFreeHost(inst->sweep_flags);
+        inst->sweep_flags = nullptr;
+        inst->sweep_flags_count = 0;
+        PP_CUDA(cudaHostAlloc((void **)&inst->sweep_flags, sizeof(int32_t) * starts, cudaHostAllocMapped));
+        inst->sweep_flags_count = starts;
+    }
+    while ((int)inst->sweep_events.size() < events) {
+        cudaEvent_t e;
+        PP_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+        inst->sweep_events.push_back(e);
+    }
     return PP_OK;
 }
 
@@ -351,7 +371,6 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     const int gs = grouped ? (S + kGroupStreams - 1) / kGroupStreams : 1;      // starts per stream
     const bool lockstep = S == 1 || sched == 1 ||
                           (sched == 0 && !grouped && hardware_queues() < std::min<int>(S, kPlanStreams));
-    int32_t start_steps = 0;            // on streams: updates launched per start
     std::vector<std::vector<cudaEvent_t>> sev;   // on streams: each stream's phase events
     if (lockstep) {
         auto step = [&](int t, int greedy) -> pp_status {
@@ -412,7 +431,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 if ((s = step(t, 0))) return s;
             dp_count += nact * W;
             cells += (int64_t)nact * n * sumk;
-            k_sweep_end<<<(S + 127) / 128, 128, 0, st>>>(S, pb.active, pb.improved, pb.sweeps);
+            k_sweep_end<<<(S + 127) / 128, 128, 0, st>>>(S, pb.active, pb.improved, pb.sweeps, nullptr);
             PP_CUDA(cudaGetLastError());
             launches += 1;
             PP_CUDA(cudaMemcpyAsync(act.data(), pb.active, 4 * S, cudaMemcpyDeviceToHost, st));
@@ -424,8 +443,8 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
         // slower start of another group (in lock step each step waits for the
         // start with the most kept rows).  Each update is the same kernels on
         // the group's slice of every buffer, in the batch's launch shape (no
-        // split).  All R sweeps are enqueued; a start whose sweep accepted
-        // nothing is inactive from then on and its later kernels return at once.
+        // split).  A start whose sweep accepted nothing is inactive from then on
+        // and its later kernels return at once.
         const int ngroups = (S + gs - 1) / gs, NS = std::min(ngroups, kPlanStreams);
         if ((s = ensure_plan_streams(inst, NS))) return s;
         if ((s = ensure_dp_stack(inst, g, S))) return s;   // one stack slot per start, allocated up front
@@ -454,10 +473,34 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
             return PP_OK;
         };
         const size_t N = (size_t)std::max(n, 1);
-        for (int q = 0; q < W * (1 + R); ++q) {
+        // From the third sweep on the host waits for the last but one before
+        // it enqueues the next, and leaves out the groups that are done (the
+        // launches of a sweep that does nothing cost 2.3 us each, and the
+        // device has a sweep in hand meanwhile)
+        const bool look = R >= 4;
+        if (look && (s = ensure_sweep_flags(inst, S, 2 * ngroups))) return s;
+        std::vector<char> done(ngroups, 0);
+        int left = ngroups;
+        if (look) std::fill(inst->sweep_flags, inst->sweep_flags + S, 1);
+        for (int q = 0; q < W * (1 + R) && left > 0; ++q) {
             const int pass = q / W, t = q % W;
             if (q == 0 && reuse) continue;
+            if (look && t == 0 && pass >= 3) {
+                for (int q0 = 0; q0 < ngroups; ++q0) {
+                    if (done[q0]) continue;
+                    PP_CUDA(cudaEventSynchronize(inst->sweep_events[(pass & 1) * ngroups + q0]));
+                    const volatile int32_t *f = inst->sweep_flags + q0 * gs;
+                    bool any = false;
+                    for (int y = 0; y < std::min(gs, S - q0 * gs); ++y) any = any || f[y];
+                    if (!any) {
+                        done[q0] = 1;
+                        --left;
+                    }
+                }
+                if (left == 0) break;
+            }
             for (int q0 = 0; q0 < ngroups; ++q0) {
+                if (done[q0]) continue;
                 const int x = q0 * gs, b = std::min(gs, S - x);       // starts x .. x + b - 1
                 cudaStream_t sx = inst->plan_streams[q0 % NS];
                 const int32_t *wk = pb.work + (size_t)t * B + x;
@@ -500,14 +543,15 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
                 if ((s = smark(q0, sx))) return s;
                 launches += 4;
                 if (pass > 0 && t == W - 1) {
-                    k_sweep_end<<<(b + 31) / 32, 32, 0, sx>>>(b, pb.active + x, pb.improved + x, pb.sweeps + x);
+                    k_sweep_end<<<(b + 31) / 32, 32, 0, sx>>>(b, pb.active + x, pb.improved + x, pb.sweeps + x,
+                                                              look ? inst->sweep_flags + x : nullptr);
                     PP_CUDA(cudaGetLastError());
+                    if (look) PP_CUDA(cudaEventRecord(inst->sweep_events[(pass & 1) * ngroups + q0], sx));
                     launches += 1;
                 }
             }
             parity ^= 1;
         }
-        start_steps = W * (1 + R);
         for (int x = 0; x < NS; ++x) {
             PP_CUDA(cudaEventRecord(inst->plan_join[x], inst->plan_streams[x]));
             PP_CUDA(cudaStreamWaitEvent(st, inst->plan_join[x], 0));
