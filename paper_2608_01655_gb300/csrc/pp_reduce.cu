@@ -1046,7 +1046,9 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     }
 
     // ---- the price
-    const bool give_up = maxp > kBig / (k > A.max_weight ? k : A.max_weight);
+    // lambda k, and lambda times the weight of a tile's 32 rows (what a scan sums
+    // before it takes the maximum), have to stay within int64
+    const bool give_up = maxp > kBig / (k > 32 * A.max_weight ? k : 32 * A.max_weight);
     int64_t lam = 0, L = 0;
     if (!give_up) {
         const float guess = cum[0] <= k ? 0.f : fminf(fmaxf(price_of_rank(cum, (float)k), 1.f), (float)maxp);

@@ -113,6 +113,27 @@ def test_ties_and_zero_budget_and_long_paths(pp, oracle_lib):
         _check(pp, oracle_lib, _tree(rng, "chain", m), np.ones(m, np.int32), p, [m], swept)
 
 
+@pytest.mark.parametrize("wmax", [1, 9])
+@pytest.mark.parametrize("top", [10 ** 9, (1 << 55) - 1, 1 << 56, 1 << 57, 279496122328932600, 558992244657865200, 1 << 59, 1 << 60])
+def test_profits_up_to_the_bound(pp, oracle_lib, top, wmax):
+    """Few profits with ties between them (absolute sum below 2^62) and chains
+    without any: a price of that size times a tile's 32 rows leaves int64."""
+    rng = np.random.default_rng(wmax)
+    parent = [-1] * 32 + [19, 4, 8, 4, 35, 2, 12, 37, 0, 30, 3, 32, 13, 17, 10, 34, 35, 12, 25, 13, 35, 30, 22, 29, 31,
+                          18, 36, 22, 19, 33, 22, 35, 53, 26, 5, 22]
+    for above, length in ((16, 31), (67, 31), (35, 41), (68, 2), (5, 58)):
+        parent += [above] + list(range(len(parent), len(parent) + length - 1))
+    n = len(parent)
+    profits = np.zeros((3, n), np.int64)
+    profits[0, [14, 55, 155, 197][: 4 if top < 1 << 60 else 3]] = top
+    profits[1, [14, 55, 197]] = top
+    profits[2, [14, 55]] = top
+    profits[2, :14] = -1
+    weight = rng.integers(1, wmax + 1, size=n).astype(np.int32)
+    _check(pp, oracle_lib, np.array(parent, np.int32), weight, np.tile(profits, (5, 1)),
+           np.repeat([1, 2, 3, 5, 40], 3) * wmax, lambda r: None)
+
+
 @pytest.mark.parametrize("n", [31, 257, 1030])
 @pytest.mark.parametrize("W", [1, 8, 9, 16, 17, 32])
 def test_kept_marginals_of_every_lane_group(pp, oracle_lib, n, W):
