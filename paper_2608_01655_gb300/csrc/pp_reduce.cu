@@ -970,7 +970,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
             for (int u = 0; u < U; ++u) {
                 const int s = s0 + u * kThreads;
                 x[u] = s < to ? __ldg(t.pos + s) : -1;
-                form[u] = s < to ? __ldg(t.form + (s >> 5)) : 0;
+                form[u] = s < min(to, hi) ? __ldg(t.form + (s >> 5)) : 0;      // (the last bin's tiles are in no list)
             }
             if (A.order)
 #pragma unroll

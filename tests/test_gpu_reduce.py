@@ -113,6 +113,24 @@ def test_ties_and_zero_budget_and_long_paths(pp, oracle_lib):
         _check(pp, oracle_lib, _tree(rng, "chain", m), np.ones(m, np.int32), p, [m], swept)
 
 
+@pytest.mark.parametrize("n,batch", [(60000, 40), (66000, 40), (72001, 40), (72001, 17), (140000, 20)])
+def test_many_tiles_in_few_ctas(pp, oracle_lib, n, batch):
+    """More than 2,048 tiles before the last bin, whose rows have no profit, on
+    two CTAs an item (and four), accumulators in shared memory and beyond."""
+    rng = np.random.default_rng(n)
+    parent = np.array([-1] + [int(rng.integers(max(0, v - 60), v)) if rng.random() < 0.95 else int(rng.integers(min(v, 40)))
+                              for v in range(1, n)], np.int32)
+    profits = np.exp(rng.uniform(0, 18, size=(2, n))).astype(np.int64)
+    profits[:, rng.random(n) < 0.5] = 0
+    size = np.ones(n, np.int64)
+    for v in range(n - 1, 0, -1):
+        size[parent[v]] += size[v]
+    profits[:, size > 200] = 0
+    profits[1] -= 3
+    _check(pp, oracle_lib, parent, np.ones(n, np.int32), np.tile(profits, (batch // 2 + 1, 1))[:batch],
+           np.resize([400, 60, 7, 150], batch), lambda r: None)
+
+
 @pytest.mark.parametrize("wmax", [1, 9])
 @pytest.mark.parametrize("top", [10 ** 9, (1 << 55) - 1, 1 << 56, 1 << 57, 279496122328932600, 558992244657865200, 1 << 59, 1 << 60])
 def test_profits_up_to_the_bound(pp, oracle_lib, top, wmax):
