@@ -54,6 +54,7 @@ def _check(pp, oracle_lib, parent, weight, profits, budgets, by_rows):
                 assert int(best[b]) == ob, b
                 np.testing.assert_array_equal(chosen[b].cpu().numpy(), oc, err_msg=str(b))
         by_rows(pp.pp_dp_rows_swept(ppi, B, maxb, bits))
+    return chosen.cpu().numpy()
 
 
 @pytest.mark.parametrize("shape", ["random", "star", "caterpillar", "mixed"])
@@ -179,3 +180,102 @@ def test_safeguards_beside_the_starts(pp, oracle_lib, starts, schedule):
             assert list(g.safeguard_objective) == o.safeguard_objective.tolist()
             assert g.objective == o.objective and g.best_start == o.best_start
             np.testing.assert_array_equal(g.placement, o.placement)
+
+
+def _down(x):
+    """Sums of two float32 values (exact in float64) rounded down to float32."""
+    y = x.astype(np.float32)
+    return np.where(y.astype(np.float64) > x, np.nextafter(y, np.float32(-np.inf)), y).astype(np.float64)
+
+
+def _doubling_sums(a):
+    """Sums from each row of a path to its top ([trials][rows], bottom first)
+    by a doubling scan of float32 values in tiles of 32, top tile first."""
+    out, carry = np.empty_like(a), None
+    for t0 in range((a.shape[1] - 1) // 32 * 32, -1, -32):
+        x = _down(a[:, t0:t0 + 32])
+        m = x.shape[1]
+        for o in (1, 2, 4, 8, 16):
+            y = x.copy()
+            if o < m:
+                y[:, :m - o] = _down(x[:, :m - o] + x[:, o:])
+            x = y
+        if carry is not None:
+            x = _down(x + carry[:, None])
+        carry = x[:, 0]
+        out[:, t0:t0 + 32] = x
+    return out
+
+
+def _rounded_apart(rng, m, tail, wmax, extra):
+    """A path of m rows that lose value at the price 2^40, above a row that
+    gains; `tail` rows below that one.  Losses of the m rows are such that the
+    gaining row's and its parent's, equal by themselves, lie on two sides of a
+    key's edge, the first threshold's, if they are sums of a doubling scan.  The
+    gaining row without its parent would fill the budget that is left."""
+    lam, g = 1 << 40, 1 << 34
+    wt = rng.integers(1, wmax + 1, size=m)               # from the gaining row's parent up
+    slots = int(wt[1:].sum()) + 1
+    k = max(200, 21 * slots * slots)                     # |S| = k - slots is near enough to k
+    big, pairs = k - slots, slots - 1
+    n = m + 1 + tail + 2 * pairs + big + extra
+    t = np.float32(0.1) * np.float32(lam) * (np.float32(n - m + int(wt.sum())) / np.float32(n))
+    e = int(np.floor(np.log2(t)))
+    edge = int((int(t / 2.0 ** e * 32) + 1) * 2.0 ** (e - 5))          # 32 keys an octave
+    hit = []
+    while len(hit) == 0:
+        cut = np.sort(rng.integers(1, edge, size=(4000, m - 1)), axis=1)
+        a = np.diff(np.concatenate([np.zeros((4000, 1), np.int64), cut, np.full((4000, 1), edge)], axis=1), axis=1)
+        a = a >> 12 << 12
+        a[:, 0] += edge - a.sum(1)
+        s = _doubling_sums(np.concatenate([np.full((4000, tail), lam - 5.0), np.zeros((4000, 1)), a], axis=1))
+        hit = np.flatnonzero((s[:, tail + 1] >= edge) & (s[:, tail] < edge))
+    a = a[hit[0]]
+    parent, profit, weight = [], [], []
+
+    def add(above, value, w=1):
+        parent.append(above)
+        profit.append(int(value))
+        weight.append(int(w))
+        return len(parent) - 1
+    at = -1
+    for i in range(m - 1, -1, -1):
+        at = add(at, lam * int(wt[i]) - int(a[i]) - (g if i == 0 else 0), wt[i])
+    at = add(at, lam + g)
+    for _ in range(tail):
+        at = add(at, 5)
+    for _ in range(pairs):
+        add(add(-1, 0), lam + g)
+    for i in range(big):
+        add(-1, (2 << 40) + 12345 * i)
+    while len(parent) < n:
+        add(-1, 5 + len(parent) % 97)
+    return np.array(parent, np.int32), np.array(weight, np.int32), np.array(profit, np.int64), k
+
+
+def _assert_closed(parent, chosen):
+    below = parent >= 0
+    assert not np.any(chosen[:, below] > chosen[:, parent[below]])
+
+
+@pytest.mark.parametrize("m,tail,wmax,extra", [
+    (3, 0, 1, 60), (3, 28, 1, 60), (4, 10, 1, 60), (5, 27, 1, 60), (8, 28, 1, 60), (8, 60, 1, 2000), (14, 25, 1, 9000),
+    (4, 0, 3, 60), (5, 28, 3, 60), (8, 28, 2, 60)])
+def test_rounded_losses_keep_rows_together(pp, oracle_lib, m, tail, wmax, extra):
+    """Losses above 2^24 are rounded: a row is never undecided below one that is
+    decided out, in a tile and across its edge, on one CTA and on several."""
+    for seed in range(3):
+        parent, weight, profit, k = _rounded_apart(np.random.default_rng(seed), m, tail, wmax, extra)
+        chosen = _check(pp, oracle_lib, parent, weight, profit[None], [k], lambda r: None)
+        _assert_closed(parent, chosen)
+
+
+def test_three_losses_in_two_orders(pp, oracle_lib):
+    """The same with the numbers written out: 13 * 2^33 = a + a + c, budget 200."""
+    lam, g, a = 1 << 40, 1 << 34, (1 << 35) + (1 << 12)
+    c = 13 * (1 << 33) - 2 * a
+    parent = np.array([-1, 0, 1, 2, -1, 4, -1, 6] + [-1] * 257, np.int32)
+    profit = np.array([lam - c, lam - a, lam - a - g, lam + g, 0, lam + g, 0, lam + g] +
+                      [(2 << 40) + 12345 * i for i in range(197)] + [5 + i for i in range(60)], np.int64)
+    chosen = _check(pp, oracle_lib, parent, np.ones(265, np.int32), profit[None], [200], lambda r: None)
+    _assert_closed(parent, chosen)
