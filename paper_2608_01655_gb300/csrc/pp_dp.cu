@@ -189,7 +189,7 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
         // item of rank s by kept rows, most first (ties to the lower index,
         // inactive items last), so the narrower second launch gets the
         // smallest sweeps; every CTA of a cluster computes the same item
-        __shared__ int s_item;
+        int *const s_item = reinterpret_cast<int *>(smem);      // (the rings' place, not yet in use)
         if (threadIdx.x < 32) {
             const int x = threadIdx.x;
             const int key = x < batch && (!item_active || item_active[x]) && !(red && red[x] == 1) ? nkept[x] : -1;
@@ -199,10 +199,11 @@ k_tree_dp_wave(int32_t n, int32_t nblk, const int64_t *__restrict__ rowp,
                 rank += ky > key || (ky == key && y < x);
             }
             const unsigned m = __ballot_sync(kFull, x < batch && rank == slot_base + item);
-            if (x == 0) s_item = m ? __ffs((int)m) - 1 : -1;
+            if (x == 0) *s_item = m ? __ffs((int)m) - 1 : -1;
         }
         __syncthreads();
-        item = s_item;
+        item = *s_item;
+        __syncthreads();
         if (item < 0) return;           // no such slot: uniform over the cluster
     }
     const int NT = blockDim.x;
@@ -794,6 +795,17 @@ static int max_smem_optin(const pp_instance *inst)
     return v;
 }
 
+// The largest dynamic shared memory of a kernel is an attribute of the process,
+// not of a launch: it is always set to the device's limit (the DP kernels have
+// no static shared memory), so no thread lowers it between another's setting
+// and launch.
+static bool allow_smem(const void *fn, int smem_max)
+{
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+}
+
 // Split launch: measured on GB300 (152 SMs), the placement of clusters of 8
 // CTAs at one CTA per SM finds room for 15 of them; a 16th cluster then shares
 // SMs with other items and slows them and itself by ~25% per row.  When the
@@ -809,10 +821,6 @@ static void split_geometry(const pp_instance *inst, int batch, const void *fn, c
     cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, inst->device);
     const size_t excl = std::max(g->smem, (size_t)per_sm / 2);   // two CTAs never fit in one SM
     if (excl > (size_t)smem_max) return;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)excl) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
     cudaLaunchConfig_t cfg = cfg0;
     cfg.dynamicSmemBytes = excl;
     int m1 = 0;
@@ -828,10 +836,7 @@ static void split_geometry(const pp_instance *inst, int batch, const void *fn, c
     const int L2 = (int)std::min<size_t>((size_t)inst->stack_depth, ((size_t)smem_max - fixed2) / level2);
     const size_t smem2 = std::max(fixed2 + (size_t)L2 * level2, excl);
     const void *fn2 = wave_kernel_for(g->C, g->WMAX, L2 < inst->stack_depth);
-    if (!fn2 || cudaFuncSetAttribute(fn2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
+    if (!fn2 || !allow_smem(fn2, smem_max)) return;
     cudaLaunchConfig_t cfg2 = cfg0;
     cfg2.gridDim = dim3(CL2 * (batch - m1));
     cfg2.blockDim = dim3(WPC2 * 32);
@@ -897,10 +902,7 @@ static bool wave_geometry(const pp_instance *inst, int64_t k, int batch, DpGeom 
         const void *fn = wave_kernel_for(C, WMAX, L_smem < inst->stack_depth);
         if (!fn) continue;
         const size_t smem = fixed + (size_t)L_smem * level;
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-            cudaGetLastError();
-            continue;
-        }
+        if (!allow_smem(fn, smem_max)) continue;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CL * std::max(batch, 1));
         cfg.blockDim = dim3(WPC * 32);
@@ -985,7 +987,8 @@ static pp_status launch_flat_c(pp_instance *inst, int batch, const int32_t *item
                                const int32_t *item_active, const DpGeom &g, int64_t *best,
                                const DpWork &work, int64_t *gstack, int L_glob, cudaStream_t st)
 {
-    PP_CUDA(cudaFuncSetAttribute(k_tree_dp_flat<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+    if (!allow_smem((const void *)k_tree_dp_flat<C>, max_smem_optin(inst)))
+        return fail(PP_ECUDA, "shared memory of the one-CTA DP kernel");
     PP_CUDA(launch_chained(k_tree_dp_flat<C>, dim3(batch), dim3(g.T), g.smem, st, 1, inst->n, work, inst->d_wpre,
                            item_budget, max_budget, item_active, best, gstack, g.L_smem, L_glob, inst->d_status));
     return PP_OK;
@@ -1030,8 +1033,7 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
                           cudaStream_t s) -> pp_status {
             const void *fn = wave_kernel_for(g.C, g.WMAX, L_smem < inst->stack_depth);
             if (!fn) return fail(PP_EINVAL, "unsupported DP geometry");
-            PP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            cudaLaunchConfig_t cfg = {};
+            cudaLaunchConfig_t cfg = {};          // (dp_geometry has allowed the kernel its shared memory)
             cfg.gridDim = dim3(CL * items);
             cfg.blockDim = dim3(WPC * 32);
             cfg.dynamicSmemBytes = smem;

@@ -1767,16 +1767,26 @@ size_t reduce_item_bytes(const pp_instance *inst)
     return al(carve(nullptr, inst->red.nslots, inst->red.ntop, inst->red.acc_global, nullptr));
 }
 
-// clusters above the portable size: how many the device holds at once
+// Once per instance: the kernels' attributes, and how many clusters above the
+// portable size the device holds at once.  Attributes belong to the process, so
+// every instance sets the same: all the shared memory that the device allows.
 pp_status reduce_device(ReduceShape *r)
 {
     r->wide = 0;
-    if (!r->ncl || r->cl[0] <= kPortable) return PP_OK;
+    if (!r->ncl) return PP_OK;
+    int dev = 0, limit = 0;
+    PP_CUDA(cudaGetDevice(&dev));
+    PP_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    for (const void *fn : {(const void *)k_reduce<true>, (const void *)k_reduce<false>}) {
+        cudaFuncAttributes at;
+        PP_CUDA(cudaFuncGetAttributes(&at, fn));
+        PP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, limit - (int)at.sharedSizeBytes));
+        PP_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    }
+    if (r->cl[0] <= kPortable) return PP_OK;
     const bool acc_smem = scan_bytes(r->acc[0], true) <= kAccLimit;
     const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;
     const size_t smem = std::max(scan_bytes(r->acc[0], acc_smem), up16(sizeof(Rows)) + kPool);
-    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(r->cl[0]);
     cfg.blockDim = dim3(kThreads);
@@ -1829,8 +1839,6 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     const bool acc_smem = scan_bytes(r.acc[x], true) <= kAccLimit;
     const size_t smem = std::max(scan_bytes(r.acc[x], acc_smem), up16(sizeof(Rows)) + kPool);
     const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;
-    PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (r.cl[x] > kPortable) PP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     PP_CUDA(launch_chained(kern, dim3(r.cl[x] * batch), dim3(kThreads), smem, st, r.cl[x], a));
     return PP_OK;
 }

@@ -2,6 +2,8 @@
 bit against the oracle: trees around its tile, stream and cluster boundaries,
 budgets that bind or do not, ties that leave it more undecided rows than it
 takes, and paths too long for it.  Everything is integer: equality."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -279,3 +281,46 @@ def test_three_losses_in_two_orders(pp, oracle_lib):
                       [(2 << 40) + 12345 * i for i in range(197)] + [5 + i for i in range(60)], np.int64)
     chosen = _check(pp, oracle_lib, parent, np.ones(265, np.int32), profit[None], [200], lambda r: None)
     _assert_closed(parent, chosen)
+
+
+def test_two_instances_on_two_threads(pp, oracle_lib):
+    """Launches of instances whose kernels take different amounts of shared
+    memory (the sweep's, for weights on both sides of the wavefront kernel's
+    limit, and the reduction's) do not disturb one another."""
+    errors = []
+
+    def work(n, wmax, k, seed, noprune):
+        parent = _tree(np.random.default_rng(seed), "random", n)
+        weight = np.random.default_rng(seed).integers(1, wmax + 1, size=n).astype(np.int32)
+        profit = np.exp(np.random.default_rng(seed + 1).uniform(0, 18, n)).astype(np.int64)
+        best0, set0 = oracle_lib.rooted_dp(parent, weight, profit, k)
+        inst = wl.Instance("t", n, 1, parent, weight, np.ones((1, n), np.int64), np.ones((1, n), np.int64),
+                           np.ones((1, n), np.int64), 0, np.array([1], np.int32), 1, 1)
+
+        def go():
+            try:
+                stream = torch.cuda.Stream()
+                with pp.Instance.from_workload(inst) as ppi, torch.cuda.stream(stream):
+                    pp.pp_tune_dp(ppi, 0, 0, False, noprune)
+                    prof = torch.from_numpy(profit[None].copy()).cuda()
+                    bud = torch.full((1,), k, dtype=torch.int32, device="cuda")
+                    best = torch.zeros(1, dtype=torch.int64, device="cuda")
+                    bits = torch.zeros(pp.pp_dp_bits_size(ppi, 1, k) // 4, dtype=torch.int32, device="cuda")
+                    chosen = torch.zeros((1, n), dtype=torch.uint8, device="cuda")
+                    for _ in range(400):
+                        pp.pp_tree_dp(ppi, prof, bud, k, best, bits, stream=stream)
+                        pp.pp_traceback(ppi, bits, bud, k, chosen, stream=stream)
+                    ppi.sync()
+                    stream.synchronize()
+                    assert int(best[0]) == best0
+                    np.testing.assert_array_equal(chosen[0].cpu().numpy(), set0)
+            except Exception as e:                        # noqa: BLE001
+                errors.append(repr(e))
+        return threading.Thread(target=go)
+    threads = [work(300, 9, 500, 1, True), work(301, 9, 1000, 2, True), work(700, 1, 60, 3, True), work(701, 1, 600, 4, True),
+               work(1500, 1, 50, 5, False), work(12000, 1, 50, 6, False)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
