@@ -412,8 +412,8 @@ static pp_status create_impl(int32_t n, int32_t W, const int32_t *parent, const 
         }
         if ((s = upload(&inst->d_pspan, span.data(), n, st))) return s;
         std::vector<char> rt;
+        if (inst->red.bins && (s = reduce_device(&inst->red))) return s;
         if (inst->red.bins) {
-            if ((s = reduce_device(&inst->red))) return s;
             rt.resize(reduce_tables_bytes(red));
             reduce_tables_pack(red, rt.data());
             char *d = nullptr;

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "pp_reduce_shape.h"
 #include "prefixplace.h"
 
 namespace pp {
@@ -128,7 +129,7 @@ DpWork dp_work_item(const pp_instance *inst, const DpWork &w, int item, int word
 constexpr int32_t kDevOk = PP_OK;
 
 // Layout of the exact reduction (pp_reduce.cu): host tables while an instance
-// is built, and their sizes.  CL = 0: this tree is not reduced.
+// is built (their sizes: pp_reduce_shape.h).
 constexpr int32_t kReduceMinRows = 128;     // below, the sweep is as short (501 rows: 79 us swept, 40 reduced)
 struct ReduceTables {
     struct Info {
@@ -147,11 +148,6 @@ struct ReduceTables {
     std::vector<Cluster> cluster;   // largest first
     std::vector<Stream> stream;
     std::vector<int32_t> lev, binlev, binslot, nacc;
-};
-struct ReduceShape {
-    int bins = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_kids = 0;
-    int ncl = 0, cl[8] = {}, acc[8] = {}, acc_global = 0;      // cluster sizes, largest first
-    int wide = 0;                   // clusters above the portable size that fit the device
 };
 
 struct Scratch {

@@ -78,8 +78,6 @@ constexpr int kRing = 3;                    // tiles of a warp in flight or in u
 constexpr int kMaxTiles = 64;               // of a warp, all levels together
 constexpr size_t kRingBytes = (size_t)kWarps * kRing * 512;
 constexpr int kMaxBins = 16;
-constexpr int kReduceCtas = 128;            // of all items in flight (16 clusters of 8, 15 of which run at a time on 152
-                                            // SMs: a batch of 16 685 us; all at once on 6 CTAs each, 712)
 constexpr int kMaxTop = 256;                // rows of the last bin (every CTA walks it)
 // the search's 32-bit units: the first price is 2^11 to 2^12 of them
 constexpr int kUnitBits = 11;
@@ -1741,7 +1739,6 @@ static size_t scan_bytes(int acc, bool acc_smem)
     return (acc_smem ? up16((size_t)(acc + 1) * kAccBytes) : 0) + kRingBytes + kBins * 4;
 }
 constexpr size_t kAccLimit = (size_t)192 << 10;
-constexpr int kPortable = 8;     // CTAs of a cluster that every device takes
 
 ReduceShape reduce_shape(const ReduceTables &R)
 {
@@ -1772,7 +1769,6 @@ size_t reduce_item_bytes(const pp_instance *inst)
 // every instance sets the same: all the shared memory that the device allows.
 pp_status reduce_device(ReduceShape *r)
 {
-    r->wide = 0;
     if (!r->ncl) return PP_OK;
     int dev = 0, limit = 0;
     PP_CUDA(cudaGetDevice(&dev));
@@ -1797,10 +1793,12 @@ pp_status reduce_device(ReduceShape *r)
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&r->wide, kern, &cfg) != cudaSuccess) {
+    int wide = 0;
+    if (cudaOccupancyMaxActiveClusters(&wide, kern, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        r->wide = 0;
+        wide = 0;
     }
+    set_wide(*r, wide);
     return PP_OK;
 }
 
@@ -1828,13 +1826,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.stack_depth = inst->stack_depth;
     a.status = inst->d_status;
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
-    // As many CTAs per item as the items in flight leave SMs for (whole plans,
-    // 16 CTAs an item against 8: 2 starts of 200,000 rows 11.9 and 15.7 ms, 8
-    // starts of 20,000 10.4 and 11.1 although one start in eight waits; 16
-    // starts of 50,000 41.7 and 29.3, half of them waiting)
-    const int items = std::max(work.items, batch);
-    int x = 0;
-    while (x + 1 < r.ncl && ((r.cl[x] > kPortable && items * 7 > r.wide * 8) || r.cl[x] * items > kReduceCtas)) ++x;
+    const int x = cluster_index(r, std::max(work.items, batch));
     a.t.CL = r.cl[x];
     const bool acc_smem = scan_bytes(r.acc[x], true) <= kAccLimit;
     const size_t smem = std::max(scan_bytes(r.acc[x], acc_smem), up16(sizeof(Rows)) + kPool);
