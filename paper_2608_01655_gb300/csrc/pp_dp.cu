@@ -687,6 +687,7 @@ k_prune(int32_t n, const int64_t *__restrict__ profit, const int32_t *__restrict
     chain_release();
     const int item = blockIdx.x / (int)cluster_nctarank();
     if (item_active && !item_active[item]) return;       // uniform over the cluster
+    if (w.red && threadIdx.x == 0 && cluster_ctarank() == 0) w.red[item] = 0;
     prune_item(n, item, profit, BYNODE ? order : nullptr, next, pspan, wpre, w, nullptr, prune, stack_depth, status,
                rows_kept);
 }
@@ -731,7 +732,8 @@ DpWork dp_work_split(const pp_instance *inst, void *base, int batch, int words)
     w.wsuf = reinterpret_cast<int32_t *>(take(B * (N + 1) * 4));
     w.rowp = reinterpret_cast<int64_t *>(take(B * N * 8));
     w.rowm = reinterpret_cast<int32_t *>(take(B * N * 4));
-    if (reduce_on(inst)) {
+    if (inst->red.bins) {
+        w.reduce = reduce_on(inst);
         w.red = reinterpret_cast<int32_t *>(take(B * 4));
         w.left = reinterpret_cast<int32_t *>(take(B * 4));
         w.base = reinterpret_cast<int64_t *>(take(B * 8));
@@ -757,6 +759,7 @@ DpWork dp_work_item(const pp_instance *inst, const DpWork &w, int item, int word
     o.rowp = w.rowp + it * N;
     o.rowm = w.rowm + it * N;
     if (w.red) {
+        o.reduce = w.reduce;
         o.red = w.red + it;
         o.left = w.left + it;
         o.base = w.base + it;
@@ -1007,7 +1010,7 @@ static pp_status launch_dp_kernels(pp_instance *inst, int batch, const int64_t *
     // does not solve (a launch of its own for that stood idle between the others
     // of nearly every update: RAG plan 4.06 -> 3.93 ms, 20,000 chunks 9.07 -> 8.81
     // without it)
-    if (work.red) {
+    if (work.reduce) {
         pp_status s = launch_reduce(inst, batch, profit, by_node, item_budget, item_active, best, work, st, max_budget,
                                     rows_kept);
         if (s != PP_OK) return s;

@@ -105,18 +105,21 @@ struct DpWork {
     int32_t *wsuf = nullptr;       // [batch][n + 1]
     int64_t *rowp = nullptr;       // [batch][n] profit of each kept row, sweep order
     int32_t *rowm = nullptr;       // [batch][n] wave-kernel metadata of each kept row
-    // exact reduction (pp_reduce.cu), null when the launch does without it.
+    // exact reduction (pp_reduce.cu), null when the tree has none.
     // red[item] = 1: solved, the optimal set is `taken` and nkept[item] the
     // number of rows that were undecided; the pruned sweep's kernels leave
     // it alone.  2: those kernels sweep only the rows in `undecided`, with the
     // budget left[item]; base[item] is the value of the decided rows, which
-    // are in `taken`.  0: they sweep all rows.
+    // are in `taken`.  0: they sweep all rows.  A launch without the reduction
+    // writes 0 too, so what reads the workspace later does not depend on the
+    // switches then.
     int32_t *red = nullptr;        // [batch]
     int32_t *left = nullptr;       // [batch]
     int64_t *base = nullptr;       // [batch]
     uint32_t *taken = nullptr;     // [batch][ceil(n / 32)] by preorder position
     uint32_t *undecided = nullptr; // [batch][ceil(n / 32)]
     char *red_scratch = nullptr;   // [batch][reduce_item_bytes]
+    bool reduce = false;           // launches on this workspace try the reduction
     int items = 0;                 // items in flight together with this launch's (0: only those)
     int64_t *clear = nullptr;      // [batch] or null: zeroed by the reduction (the planner's next held sums)
 };

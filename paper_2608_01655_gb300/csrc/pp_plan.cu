@@ -326,7 +326,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     auto held_sums = [&](int first, int count, cudaStream_t sx, DpWork *w, int64_t **cur) -> pp_status {
         *cur = pb.oldsum + (size_t)parity * B + first;
         int64_t *other = pb.oldsum + (size_t)(parity ^ 1) * B + first;
-        if (w->red) w->clear = other;
+        if (w->reduce) w->clear = other;
         else PP_CUDA(cudaMemsetAsync(other, 0, sizeof(int64_t) * count, sx));
         return PP_OK;
     };
@@ -367,7 +367,7 @@ pp_status plan_impl(pp_instance *inst, int32_t S, const int32_t *orders, int32_t
     // with 32, eight groups 39).  Without it: one stream per start if every
     // stream gets a hardware queue of its own, else lock step (streams that
     // share a queue wait on one another's launches)
-    const bool grouped = sched == 0 && work.red && S > 1;
+    const bool grouped = sched == 0 && work.reduce && S > 1;
     const int gs = grouped ? (S + kGroupStreams - 1) / kGroupStreams : 1;      // starts per stream
     const bool lockstep = S == 1 || sched == 1 ||
                           (sched == 0 && !grouped && hardware_queues() < std::min<int>(S, kPlanStreams));

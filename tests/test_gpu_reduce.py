@@ -283,6 +283,35 @@ def test_three_losses_in_two_orders(pp, oracle_lib):
     _assert_closed(parent, chosen)
 
 
+@pytest.mark.parametrize("solved_by_reduction", [True, False])
+def test_workspace_is_read_as_it_was_written(pp, oracle_lib, solved_by_reduction):
+    """Switching the reduction off or on between the DP and its traceback does
+    not change what the workspace holds."""
+    rng = np.random.default_rng(8)
+    n, k = 900, 120
+    parent = _tree(rng, "mixed", n)
+    weight = rng.integers(1, 3, size=n).astype(np.int32)
+    profit = np.exp(rng.uniform(0, 18, size=(2, n))).astype(np.int64)
+    inst = wl.Instance("t", n, 1, parent, weight, np.ones((1, n), np.int64), np.ones((1, n), np.int64),
+                       np.ones((1, n), np.int64), 0, np.array([1], np.int32), 1, 1)
+    with pp.Instance.from_workload(inst) as ppi:
+        prof = torch.from_numpy(profit).cuda()
+        bud = torch.full((2,), k, dtype=torch.int32, device="cuda")
+        best = torch.zeros(2, dtype=torch.int64, device="cuda")
+        bits = torch.zeros(pp.pp_dp_bits_size(ppi, 2, k) // 4, dtype=torch.int32, device="cuda")
+        chosen = torch.zeros((2, n), dtype=torch.uint8, device="cuda")
+        pp.pp_tune_dp(ppi, 0, 0, False, not solved_by_reduction)
+        pp.pp_tree_dp(ppi, prof, bud, k, best, bits)
+        pp.pp_tune_dp(ppi, 0, 0, False, solved_by_reduction)
+        pp.pp_traceback(ppi, bits, bud, k, chosen)
+        ppi.sync()
+        assert (pp.pp_dp_rows_swept(ppi, 2, k, bits) < n).all() == solved_by_reduction
+        for b in range(2):
+            ob, oc = oracle_lib.rooted_dp(parent, weight, profit[b], k)
+            assert int(best[b]) == ob
+            np.testing.assert_array_equal(chosen[b].cpu().numpy(), oc)
+
+
 def test_two_instances_on_two_threads(pp, oracle_lib):
     """Launches of instances whose kernels take different amounts of shared
     memory (the sweep's, for weights on both sides of the wavefront kernel's
