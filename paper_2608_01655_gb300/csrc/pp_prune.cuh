@@ -45,10 +45,12 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
 // i is kept iff it is a root or its parent has one.  A kept row i that is
 // itself an identity (p_i <= 0 and no positive strict descendant: D[i] =
 // D[next(i)], all bits "skip") is dropped as well.  For an item that the
-// reduction has cut down (`ud`: its undecided rows) only those are kept: decided
-// rows inside the optimal set are closed upwards and those outside it
+// reduction has cut down (`ud`: its undecided rows) only those of them are kept:
+// decided rows inside the optimal set are closed upwards and those outside it
 // downwards, so the undecided rows in preorder form a forest of their own,
-// with the same subtree ends.
+// with the same subtree ends, in which a row without a positive profit at or
+// below it is never worth taking either (a caterpillar of 1,600 chunks with a
+// tenth of the profits: 1,568 undecided rows, 883 of them kept).
 // Kept rows are listed in sweep order (decreasing i); every position records
 // the first kept row at or after it in preorder, so a skip to a dropped row
 // lands where the all-"skip" walk through it would.
@@ -115,7 +117,7 @@ __device__ __forceinline__ int cluster_exclusive_scan(int v, int *total, int *sl
 // thread, one block scan per tile), and the slices are joined by a scan over
 // the cluster's CTAs.
 // (as many CTAs as the cluster has, 1024 threads each; `order`: profits are by
-// node id; `ud`: bitmap of the only rows to keep)
+// node id; `ud`: bitmap of the only rows to keep, of those that pruning keeps)
 __device__ __forceinline__ void prune_item(int32_t n, int item, const int64_t *__restrict__ profit,
                                            const int32_t *__restrict__ order, const int32_t *__restrict__ next,
                                            const int2 *__restrict__ pspan, const int32_t *__restrict__ wpre,
@@ -139,9 +141,8 @@ __device__ __forceinline__ void prune_item(int32_t n, int item, const int64_t *_
     };
     int lo, hi, total;
 
-    // prefix counts of positive profits, preorder (the reduction has already
-    // chosen the rows otherwise)
-    slice(ud ? 0 : n, lo, hi);
+    // prefix counts of positive profits, preorder
+    slice(n, lo, hi);
     int mine = 0;
     for (int i = lo + t; i < hi; i += T) mine += pval(i) > 0;
     block_exclusive_scan(mine, &total, sh);
@@ -167,14 +168,14 @@ __device__ __forceinline__ void prune_item(int32_t n, int item, const int64_t *_
         }
         carry += tt;
     }
-    if (cr == 0 && t == 0 && !ud) cnt[n] = npos;
+    if (cr == 0 && t == 0) cnt[n] = npos;
     cluster_sync_all();                                   // cnt complete for every CTA
 
     // kept rows in sweep order r = n - 1 - i, their kept index, their total weight
     auto keep = [&](int r) -> bool {
         if (!prune) return true;
         const int i = n - 1 - r;
-        if (ud) return (ud[i >> 5] >> (i & 31)) & 1u;
+        if (ud && !((ud[i >> 5] >> (i & 31)) & 1u)) return false;
         const int2 sp = pspan[i];
         if (!(sp.x < 0 || cnt[sp.y] - cnt[sp.x] > 0)) return false;
         // an identity row (p <= 0 and no positive strict descendant, so D[i] =

@@ -283,6 +283,25 @@ def test_three_losses_in_two_orders(pp, oracle_lib):
     _assert_closed(parent, chosen)
 
 
+@pytest.mark.parametrize("n,k", [(12000, 600), (20000, 1000)])
+def test_rows_left_to_the_sweep_are_pruned(pp, oracle_lib, n, k):
+    """A tenth of the profits: whatever the reduction leaves undecided, no row
+    is swept that pruning alone would drop."""
+    rng = np.random.default_rng(n)
+    parent = _tree(rng, "random", n)
+    profits = np.exp(rng.uniform(0, 18, size=(4, n))).astype(np.int64)
+    profits[rng.random((4, n)) < 0.9] = 0
+    positive = profits > 0                       # at or below a row
+    for v in range(n - 1, 0, -1):
+        if parent[v] >= 0:
+            positive[:, parent[v]] |= positive[:, v]
+
+    def rows(r):
+        assert (r <= positive.sum(axis=1)).all() and r.max() > 1024
+    chosen = _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, [k] * 4, rows)
+    _assert_closed(parent, chosen)
+
+
 @pytest.mark.parametrize("solved_by_reduction", [True, False])
 def test_workspace_is_read_as_it_was_written(pp, oracle_lib, solved_by_reduction):
     """Switching the reduction off or on between the DP and its traceback does
