@@ -620,7 +620,8 @@ __device__ int block_scan(int v, int *total, int *sh)
 // interpolating logarithms (|S| falls like a power).  3 to 6 prices; a search
 // from price 0 by the tangents of L took 9 to 10.
 // ---------------------------------------------------------------------------
-enum : int { kGo = 0, kStop = 1, kSlack = 2 };
+enum : int { kGo = 0, kStop = 1, kSlack = 2, kCoarser = 3 };
+constexpr int kCoarserBits = 6;
 
 struct Search {                              // prices in units
     float x0, x1, z0, z1;                    // price and |S| of the ends with |S| > k and <= k
@@ -652,7 +653,10 @@ __device__ float price_of_rank(const int *cum, float rank)
 }
 
 // what to do after the price `lam` (units of 2^shift) gave |S| = Z: try `nx`
-// (kGo), stop and use `nx` (kStop), or the budget does not bind (kSlack)
+// (kGo), stop and use `nx` (kStop), the budget does not bind (kSlack), or go on
+// in units of 2^(shift + kCoarserBits) with `nx` of them (kCoarser): where few
+// chunks have a profit whole paths are taken for one, and the price may be far
+// above the k-th largest profit per slot, which the units were chosen by
 __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int lam, float Z, int &nx)
 {
     if (Z > k) {
@@ -670,6 +674,11 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
     if ((Z - k) * (Z - k) <= 0.05f * k) {    // |S| is so near k that L is flat
         nx = lam;
         return kStop;
+    }
+    if (lam == kClipPrice && Z > k && evals < kMaxEvals) {
+        b.x0 *= 1.f / (1 << kCoarserBits);
+        nx = lam >> (kCoarserBits - 3);
+        return kCoarser;
     }
     float x;
     if (b.have == 3) {
@@ -866,6 +875,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     __shared__ int sh[kWarps];
     __shared__ int base[kMaxBins + 1];       // of a bin's accumulators among the CTA's
     __shared__ int s_a, s_b, s_flag, s_lam;
+    __shared__ Search s_search;
     __shared__ int64_t s_val;
     const Tab &t = A.t;
     const int CL = t.CL, cr = CL > 1 ? cluster_rank() : 0;
@@ -1065,62 +1075,67 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     int64_t lam = 0, L = 0;
     if (!give_up) {
         const float guess = cum[0] <= k ? 0.f : fminf(fmaxf(price_of_rank(cum, (float)k), 1.f), (float)maxp);
-        const int shift = max(0, (int)(__float_as_uint(fmaxf(guess, 1.f)) >> 23) - 127 - kUnitBits);
-        const int maxlam = (int)min((maxp >> shift) + 1, (int64_t)kClipPrice);
+        int shift = max(0, (int)(__float_as_uint(fmaxf(guess, 1.f)) >> 23) - 127 - kUnitBits);
         int price = (int)(guess * exp2f((float)-shift));
-        Search sr;
-        sr.have = sr.side = 0;
-        sr.x0 = sr.x1 = sr.z0 = sr.z1 = 0.f;
+        if (tid == 0) s_search = Search();   // (shared: only that thread uses it)
         auto to_units = [&](int from, int to) {
             for (int s = from + tid; s < to; s += kThreads) {
                 const int64_t p = g.prof[s] >> shift;
                 g.unit[s] = (int)(p > kClipRow ? kClipRow : p < -kClipRow ? -kClipRow : p);
             }
         };
-        to_units(lo, hi);
-        if (has_top && t.nslots - top0 > kTopSlots) {
-            if (cr == 0) to_units(top0, t.nslots);
-        } else if (tid < t.nslots - top0) {
-            const int64_t p = __ldcg(g.prof + top0 + tid) >> shift;
-            const int2 i = __ldg(t.info + top0 + tid);
-            slots[tid] = make_int4(i.x, i.y, (int)(p > kClipRow ? kClipRow : p < -kClipRow ? -kClipRow : p), 0);
-        }
         bool low = false;                    // the last price was a lower bound
         int at = 1, alive = tiles, kept = 0;
-        for (int ev = 0;; ++ev) {
-            for (int i = tid; i <= na; i += kThreads) own.s[i] = make_int2(0, 0);
-            // (the set that the last price but one's sums were read from)
-            if (low) {                       // fewer tiles to walk from now on
-                at ^= 3;
-                alive = kept;
+        int ev = 0;
+        for (;;) {
+            const int maxlam = (int)min((maxp >> shift) + 1, (int64_t)kClipPrice);
+            to_units(lo, hi);
+            if (has_top && t.nslots - top0 > kTopSlots) {
+                if (cr == 0) to_units(top0, t.nslots);
+            } else if (tid < t.nslots - top0) {
+                const int64_t p = __ldcg(g.prof + top0 + tid) >> shift;
+                const int2 i = __ldg(t.info + top0 + tid);
+                slots[tid] = make_int4(i.x, i.y, (int)(p > kClipRow ? kClipRow : p < -kClipRow ? -kClipRow : p), 0);
             }
-            if (cr == 0)
-                for (int i = tid; i < t.ntop; i += kThreads) g.tops[(ev + 1) % 3 * t.ntop + i] = make_int2(0, 0);
-            int2 *tops = g.tops + ev % 3 * t.ntop;
-            int rz = 0;
-            __syncthreads();
-            kept = search_bin<!SMEM>(info, g.unit + lo, lists[at][warp], alive, lists[at ^ 3][warp], nlev, own, base, na, tops,
-                                     price, A.clip_kid, ring, rz);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(kAll, rz, o);
-            if (lane == 0 && rz) atomicAdd(&g.s->sumZ[ev], (unsigned long long)rz);
-            sync_all();
-            if (warp == 0) {
-                const int bins = lane == 0 ? (int)__ldcg(&g.s->sumZ[ev]) : 0;
-                int z = has_top ? search_top(t, g, slots, tops, (int2 *)s_top, price, A.clip_kid) : 0;
-                if (lane == 0) {
-                    z += bins;
-                    int nx = price;
-                    s_flag = next_price(sr, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
-                    s_lam = nx;
-                    s_a = z > k;
+            for (;; ++ev) {
+                for (int i = tid; i <= na; i += kThreads) own.s[i] = make_int2(0, 0);
+                // (the set that the last price but one's sums were read from)
+                if (low) {                       // fewer tiles to walk from now on
+                    at ^= 3;
+                    alive = kept;
                 }
+                if (cr == 0)
+                    for (int i = tid; i < t.ntop; i += kThreads) g.tops[(ev + 1) % 3 * t.ntop + i] = make_int2(0, 0);
+                int2 *tops = g.tops + ev % 3 * t.ntop;
+                int rz = 0;
+                __syncthreads();
+                kept = search_bin<!SMEM>(info, g.unit + lo, lists[at][warp], alive, lists[at ^ 3][warp], nlev, own, base, na, tops,
+                                         price, A.clip_kid, ring, rz);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) rz += __shfl_xor_sync(kAll, rz, o);
+                if (lane == 0 && rz) atomicAdd(&g.s->sumZ[ev], (unsigned long long)rz);
+                sync_all();
+                if (warp == 0) {
+                    const int bins = lane == 0 ? (int)__ldcg(&g.s->sumZ[ev]) : 0;
+                    int z = has_top ? search_top(t, g, slots, tops, (int2 *)s_top, price, A.clip_kid) : 0;
+                    if (lane == 0) {
+                        z += bins;
+                        int nx = price;
+                        s_flag = next_price(s_search, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
+                        s_lam = nx;
+                        s_a = z > k;
+                    }
+                }
+                __syncthreads();
+                price = s_lam;
+                low = s_a;
+                if (s_flag != kGo) break;
+                __syncthreads();
             }
-            __syncthreads();
-            price = s_lam;
-            low = s_a;
-            if (s_flag != kGo) break;
-            __syncthreads();
+            if (s_flag != kCoarser) break;
+            ++ev;
+            shift += kCoarserBits;
+            sync_all();                      // no CTA reads the old units any more
         }
         if (s_flag == kSlack) price = 0;
         lam = (int64_t)price << shift;

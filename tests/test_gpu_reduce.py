@@ -283,23 +283,41 @@ def test_three_losses_in_two_orders(pp, oracle_lib):
     _assert_closed(parent, chosen)
 
 
-@pytest.mark.parametrize("n,k", [(12000, 600), (20000, 1000)])
+def _few_profits(rng, n, B):
+    profits = np.exp(rng.uniform(0, 18, size=(B, n))).astype(np.int64)
+    profits[rng.random((B, n)) < 0.9] = 0
+    return profits
+
+
+@pytest.mark.parametrize("n,k", [(1600, 80), (1900, 95)])
 def test_rows_left_to_the_sweep_are_pruned(pp, oracle_lib, n, k):
     """A tenth of the profits: whatever the reduction leaves undecided, no row
     is swept that pruning alone would drop."""
     rng = np.random.default_rng(n)
-    parent = _tree(rng, "random", n)
-    profits = np.exp(rng.uniform(0, 18, size=(4, n))).astype(np.int64)
-    profits[rng.random((4, n)) < 0.9] = 0
+    parent = _tree(rng, "caterpillar", n)
+    profits = _few_profits(rng, n, 12)
     positive = profits > 0                       # at or below a row
     for v in range(n - 1, 0, -1):
         if parent[v] >= 0:
             positive[:, parent[v]] |= positive[:, v]
 
     def rows(r):
-        assert (r <= positive.sum(axis=1)).all() and r.max() > 1024
-    chosen = _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, [k] * 4, rows)
+        swept = r > 1024                         # more than the DP on chip takes
+        assert (r[swept] <= positive.sum(axis=1)[swept]).all()
+    chosen = _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, [k] * 12, rows)
     _assert_closed(parent, chosen)
+
+
+@pytest.mark.parametrize("shape,n,k", [("random", 1600, 80), ("random", 12000, 600), ("mixed", 4000, 200)])
+def test_price_far_above_the_first_guess(pp, oracle_lib, shape, n, k):
+    """Few chunks with a profit, whole paths taken for one: the price is a
+    hundred times the k-th largest profit, and is found all the same."""
+    rng = np.random.default_rng(n + 1)
+    parent = _tree(rng, shape, n)
+
+    def rows(r):
+        assert (r <= 1024).all() and np.median(r) <= 256
+    _check(pp, oracle_lib, parent, np.ones(n, np.int32), _few_profits(rng, n, 6), [k] * 6, rows)
 
 
 @pytest.mark.parametrize("solved_by_reduction", [True, False])
