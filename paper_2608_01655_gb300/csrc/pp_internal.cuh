@@ -143,6 +143,7 @@ struct ReduceTables {
     };
     struct Cluster {
         int cl, acc;                // CTAs of an item; accumulators of a CTA, at most
+        int path;                   // tiles in sequence: over the levels, the most of one warp
     };
     int bins = 0, max_kids = 0;
     std::vector<Info> info;

@@ -65,6 +65,8 @@ constexpr int kPasses = 5;                  // thresholds tried per item
 constexpr int kRowCap = 1024;               // undecided rows the on-chip DP takes
 constexpr int kFirstRows = 192;             // most rows of the first threshold
 constexpr int kMoreRows = 640;              // of the next, where the first gave no V or a poor one
+constexpr float kPassUs = 6.f;              // a threshold without its DP, and a row of the DP, us
+constexpr float kRowUs = 0.08f, kWeightedRowUs = 0.11f;
 constexpr int kColCap = 1024;               // its columns (budget left over)
 constexpr int kPool = 112 << 10;            // its decisions, stack and row buffers, bytes
 constexpr int kKeyBase = (127 << 5) - 1;    // float bits >> 18 of 1.0, minus 1
@@ -127,6 +129,8 @@ struct Args {
     int64_t total_weight;
     int32_t max_weight;
     int32_t clip_kid;            // the search's bound on what a light child adds
+    float price_us, sweep_us[2]; // of one price; of a sweep of all rows, at most 128 columns and more
+    int32_t evals[2];            // prices tried at most
     const int2 *pspan;           // the pruned sweep's: see prune_item
     int32_t stack_depth;
     int32_t *status;
@@ -657,7 +661,8 @@ __device__ float price_of_rank(const int *cum, float rank)
 // in units of 2^(shift + kCoarserBits) with `nx` of them (kCoarser): where few
 // chunks have a profit whole paths are taken for one, and the price may be far
 // above the k-th largest profit per slot, which the units were chosen by
-__device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int lam, float Z, int &nx)
+__device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int max_evals,
+                          int lam, float Z, int &nx)
 {
     if (Z > k) {
         b.x0 = (float)lam;
@@ -675,7 +680,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         nx = lam;
         return kStop;
     }
-    if (lam == kClipPrice && Z > k && evals < kMaxEvals) {
+    if (lam == kClipPrice && Z > k && evals < max_evals) {
         b.x0 *= 1.f / (1 << kCoarserBits);
         nx = lam >> (kCoarserBits - 3);
         return kCoarser;
@@ -684,7 +689,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
     if (b.have == 3) {
         // L's slope is k - |S|, so these bound what a better price could still give
         const float d = b.x1 - b.x0, e0 = (b.z0 - k) * d, e1 = (k - b.z1) * d;
-        if (fminf(e0, e1) <= 0.1f * b.x0 || d <= 1.f || evals >= kMaxEvals) {
+        if (fminf(e0, e1) <= 0.1f * b.x0 || d <= 1.f || evals >= max_evals) {
             nx = (int)(e0 < e1 ? b.x0 : b.x1);
             return kStop;
         }
@@ -699,7 +704,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         }
         x = fminf(fmaxf(x, b.x0 + 1.f), b.x1 - 1.f);
     } else {
-        if (evals >= kMaxEvals) {
+        if (evals >= max_evals) {
             nx = lam;
             return kStop;
         }
@@ -876,6 +881,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     __shared__ int base[kMaxBins + 1];       // of a bin's accumulators among the CTA's
     __shared__ int s_a, s_b, s_flag, s_lam;
     __shared__ Search s_search;
+    __shared__ float s_spent;
     __shared__ int64_t s_val;
     const Tab &t = A.t;
     const int CL = t.CL, cr = CL > 1 ? cluster_rank() : 0;
@@ -1071,8 +1077,10 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     // ---- the price
     // lambda k, and lambda times the weight of a tile's 32 rows (what a scan sums
     // before it takes the maximum), have to stay within int64
-    const bool give_up = maxp > kBig / (k > 32 * A.max_weight ? k : 32 * A.max_weight);
+    bool give_up = maxp > kBig / (k > 32 * A.max_weight ? k : 32 * A.max_weight);
     int64_t lam = 0, L = 0;
+    // what may be spent before the item is left to the sweep (see sweep_us)
+    auto limit = [&] { return k > 128 ? A.sweep_us[1] : A.sweep_us[0]; };
     if (!give_up) {
         const float guess = cum[0] <= k ? 0.f : fminf(fmaxf(price_of_rank(cum, (float)k), 1.f), (float)maxp);
         int shift = max(0, (int)(__float_as_uint(fmaxf(guess, 1.f)) >> 23) - 127 - kUnitBits);
@@ -1121,7 +1129,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                     if (lane == 0) {
                         z += bins;
                         int nx = price;
-                        s_flag = next_price(s_search, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
+                        s_flag = next_price(s_search, cum, (float)k, maxlam, exp2f((float)shift), ev + 1,
+                                            k > 128 ? A.evals[1] : A.evals[0], price, (float)z, nx);
                         s_lam = nx;
                         s_a = z > k;
                     }
@@ -1139,6 +1148,11 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
         }
         if (s_flag == kSlack) price = 0;
         lam = (int64_t)price << shift;
+        const float spent = (float)(ev + 3) * A.price_us;
+        give_up = spent + kPassUs > limit();
+        if (tid == 0) s_spent = spent;
+    }
+    if (!give_up) {
         // ---- exactly there: f of every row, L
         for (int i = tid; i <= na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
         __syncthreads();
@@ -1207,6 +1221,13 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
 
     int verdict = 3, key = 0, pass = 0, vkey = -1;      // vkey: the smallest sure key so far (first CTA)
     bool sure = false;           // the key comes from a V: no row above it is undecided
+    // time of a threshold with T rows, and the rows that what is left to spend
+    // allows for one more after it (one that is sure to succeed is not refused)
+    auto pass_us = [&](int T) { return kPassUs + (float)T * (A.max_weight > 1 ? kWeightedRowUs : kRowUs); };
+    auto rows_left = [&](float more) {
+        const float us = limit() - s_spent - more - kPassUs;
+        return (int)fminf(fmaxf(us * (A.max_weight > 1 ? 1.f / kWeightedRowUs : 1.f / kRowUs), 0.f), (float)kRowCap);
+    };
     if (!give_up) {
         int T = 0;
         // first the rows whose loss is within 0.1 of the price of a chunk's
@@ -1215,10 +1236,10 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
         if (lam == 0) {
             key = -1;
         } else {
-            T = up_to(kFirstRows, code_of((int64_t)(0.1f * (float)lam * ((float)A.total_weight / (float)n))), key);
+            T = up_to(min(kFirstRows, rows_left(0.f)), code_of((int64_t)(0.1f * (float)lam * ((float)A.total_weight / (float)n))), key);
         }
         for (; pass < kPasses; ++pass) {
-            const bool big = T > kRowCap;                         // the same in every CTA
+            const bool big = T > (sure ? kRowCap : rows_left(0.f));       // the same in every CTA
             verdict = 3;
             if (big && !sure) break;
             // ---- decided rows: value and weight of those in; the others' positions
@@ -1267,9 +1288,10 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                 int out = 0, okey = 0;       // 1 solved, 2 again with okey (5: which is sure), 3 not reducible, 4 to the sweep
                 if (kleft < 0) {                        // too few rows undecided: take more by rank
                     out = 2;
-                    up_to(kFirstRows, kBins, okey);
-                    if (okey <= key) up_to(kMoreRows, kBins, okey);
-                    if (okey <= key) up_to(kRowCap, kBins, okey);
+                    const int most = rows_left(kPassUs);
+                    up_to(min(kFirstRows, most), kBins, okey);
+                    if (okey <= key) up_to(min(kMoreRows, most), kBins, okey);
+                    if (okey <= key) up_to(most, kBins, okey);
                     if (okey <= key) out = 3;
                 } else {
                     // rows in sweep order from the bitmap
@@ -1459,7 +1481,8 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                                 // rows: 16,299 left by the V of 591 rows, 1,447 by that of
                                 // 1,010; the sweep of the former took 1.5 ms)
                                 int more;
-                                up_to(T < kMoreRows * 7 / 8 ? kMoreRows : kRowCap, kBins, more);
+                                const int most = rows_left(pass_us(T));
+                                up_to(T < kMoreRows * 7 / 8 ? min(kMoreRows, most) : most, kBins, more);
                                 if (more > key) {
                                     out = 2;
                                     okey = more;
@@ -1477,6 +1500,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                     g.s->verdict[pass] = out;
                 }
             }
+            if (tid == 0) s_spent += pass_us(T);
             sync_all();
             verdict = __ldcg(&g.s->verdict[pass]);
             if (verdict != 2 && verdict != 5) break;
@@ -1676,21 +1700,26 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
     for (int cl = NB; cl >= 1; --cl) {
         if (NB % cl) continue;
         const int per = NB / cl;
-        int most = 0, acc_most = 0;
+        int most = 0, acc_most = 0, longest = 0;
         for (int r = 0; r < cl; ++r) {
-            int tiles[kWarps] = {}, at = 0, accs = 0;
-            for (int l = 0; l < kMaxLevels; ++l)
+            int tiles[kWarps] = {}, at = 0, accs = 0, path = 0;
+            for (int l = 0; l < kMaxLevels; ++l) {
+                int level[kWarps] = {};
                 for (int b = r * per; b < (r + 1) * per; ++b) {
                     const int e = R.binlev[b] + l;
                     if (e + 1 >= R.binlev[b + 1]) continue;
-                    for (int x = R.lev[e]; x < R.lev[e + 1]; ++x) tiles[at++ % kWarps] += R.stream[x].tiles;
+                    for (int x = R.lev[e]; x < R.lev[e + 1]; ++x) level[at++ % kWarps] += R.stream[x].tiles;
                 }
+                for (int q = 0; q < kWarps; ++q) tiles[q] += level[q];
+                path += *std::max_element(level, level + kWarps);
+            }
+            longest = std::max(longest, path);
             for (int b = r * per; b < (r + 1) * per; ++b) accs += R.nacc[b];
             most = std::max(most, *std::max_element(tiles, tiles + kWarps));
             acc_most = std::max(acc_most, accs);
         }
         if (most > kMaxTiles || acc_most >= kNone) break;
-        R.cluster.push_back({cl, acc_most});
+        R.cluster.push_back({cl, acc_most, longest});
     }
     if (R.cluster.empty()) return false;
     R.bins = NB;
@@ -1763,9 +1792,11 @@ ReduceShape reduce_shape(const ReduceTables &R)
     s.nstreams = (int)R.stream.size();
     s.nlev = (int)R.lev.size();
     s.ntop = R.nacc[R.bins];
+    s.toptiles = (s.nslots - R.binslot[R.bins]) / 32;
     s.max_kids = R.max_kids;
     for (const auto &c : R.cluster) {
         s.cl[s.ncl] = c.cl;
+        s.path[s.ncl] = c.path;
         s.acc[s.ncl++] = c.acc;
         if (scan_bytes(c.acc, true) > kAccLimit) s.acc_global = 1;
     }
@@ -1843,6 +1874,11 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
     const int x = cluster_index(r, std::max(work.items, batch));
     a.t.CL = r.cl[x];
+    a.price_us = price_us(r, x);
+    for (int many = 0; many < 2; ++many) {
+        a.sweep_us[many] = sweep_us(inst->n, inst->max_weight, many);
+        a.evals[many] = std::min(kMaxEvals, std::max(3, (int)(a.sweep_us[many] / a.price_us) - 2));
+    }
     const bool acc_smem = scan_bytes(r.acc[x], true) <= kAccLimit;
     const size_t smem = std::max(scan_bytes(r.acc[x], acc_smem), up16(sizeof(Rows)) + kPool);
     const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;

@@ -9,8 +9,8 @@ constexpr int kReduceCtas = 128;            // of all items in flight (16 cluste
 
 // Layout of an instance's reduction.  bins = 0: this tree is not reduced.
 struct ReduceShape {
-    int bins = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, max_kids = 0;
-    int ncl = 0, cl[8] = {}, acc[8] = {}, acc_global = 0;      // cluster sizes, largest first
+    int bins = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, toptiles = 0, max_kids = 0;
+    int ncl = 0, cl[8] = {}, acc[8] = {}, path[8] = {}, acc_global = 0;      // cluster sizes, largest first
     int wide = 0;                   // clusters above the portable size that fit the device
 };
 
@@ -26,6 +26,7 @@ inline void set_wide(ReduceShape &r, int wide)
     for (int x = drop; x < r.ncl; ++x) {
         r.cl[x - drop] = r.cl[x];
         r.acc[x - drop] = r.acc[x];
+        r.path[x - drop] = r.path[x];
     }
     r.ncl -= drop;
     if (r.ncl == 0) r.bins = 0;
@@ -40,6 +41,27 @@ inline int cluster_index(const ReduceShape &r, int items)
     int x = 0;
     while (x + 1 < r.ncl && ((r.cl[x] > kPortable && items * 7 > r.wide * 8) || r.cl[x] * items > kReduceCtas)) ++x;
     return x;
+}
+
+// Microseconds of one price for an item on r.cl[x] CTAs, by the tiles that
+// follow one another (measured: 3.3 on a star of 800 rows, one tile; 5.0 on a
+// random tree of 800, 6 tiles; 12.5 on a chain of 800, 25; 6.0 on a random tree
+// of 1,600 on 6 CTAs, 4 and 2 in the last bin; 10.9 on chains of 256, 18 and 1).
+// The exact evaluation with the losses takes two.
+inline float price_us(const ReduceShape &r, int x)
+{
+    return 2.6f + 0.4f * (float)(r.path[x] + r.toptiles) + (r.cl[x] > 1 ? 1.f : 0.f);
+}
+
+// What a sweep of n rows takes, in microseconds: pruning and walk, then 0.035 to
+// 0.045 a row of at most 128 columns of unit weights, 0.065 to 0.1 of more
+// (`many`), 0.18 to 0.4 with weights (0.25 here: they sooner pay).  No more is
+// spent on an item before it is left to the sweep, so that one which the
+// reduction cannot solve takes about twice as long as without it at most (with
+// 16 prices and three DPs for every item, up to 5.6 times).
+inline float sweep_us(int n, int max_weight, bool many)
+{
+    return 25.f + (float)n * (max_weight > 1 ? 0.25f : many ? 0.07f : 0.04f);
 }
 
 }  // namespace pp
