@@ -714,6 +714,10 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
             x = price_of_rank(cum, k * c / Z) / unit;
             const float step = evals == 1 ? 0.015f : evals == 2 ? 0.04f : evals == 3 ? 0.1f : 0.3f;
             x = above ? fmaxf(x, l1) * (1.f + step) : fminf(x, l1) * (1.f - step);
+        } else if (!above && evals < 5) {
+            // nothing is worth that much, a little less (close profits) or much
+            // less (for what lies above it)
+            x = l1 * (evals == 1 ? 0.96f : evals == 2 ? 0.5f : 0.25f);
         } else {
             x = above ? (float)maxlam : 0.f;
         }

@@ -320,6 +320,19 @@ def test_price_far_above_the_first_guess(pp, oracle_lib, shape, n, k):
     _check(pp, oracle_lib, parent, np.ones(n, np.int32), _few_profits(rng, n, 6), [k] * 6, rows)
 
 
+@pytest.mark.parametrize("shape,n,k", [("star", 12000, 600), ("mixed", 12000, 600), ("mixed", 1600, 80), ("random", 800, 40)])
+def test_price_just_below_the_first_guess(pp, oracle_lib, shape, n, k):
+    """Profits within a tenth of one another: the price lies within that tenth,
+    and the search does not go through zero and use up its prices."""
+    rng = np.random.default_rng(n + 2)
+    parent = _tree(rng, shape, n)
+    profits = rng.integers(10 ** 6, 10 ** 6 + 10 ** 5, size=(4, n))
+
+    def rows(r):
+        assert (r <= 640).all(), r
+    _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, [k] * 4, rows)
+
+
 @pytest.mark.parametrize("k", [40, 160])
 def test_items_that_do_not_reduce_stop_early(pp, oracle_lib, k):
     """Nothing to gain on a chain that pays all at its end, and a price takes
