@@ -22,8 +22,8 @@
 // their keys (an order-preserving 11-bit code of the loss rounded down), so
 // every test errs on the side of keeping a row.  The rows kept also have to
 // hang together: below a row that is decided out every row is, as it is for
-// the losses themselves (lin grows down a path), and the rounded ones are made
-// to grow likewise (loss_tile).
+// the losses themselves (lin grows down a path) and for the rounded ones, which
+// are sums of whole numbers (loss_tile).
 //
 // A prefix tree of 50,000 chunks with the planner's profits leaves 30 to 600
 // undecided rows of the 16,000 to 37,000 that the pruned sweep keeps, and a
@@ -144,17 +144,21 @@ __host__ __device__ inline size_t up16(size_t x) { return (x + 15) & ~(size_t)15
 // compare-and-swap loop.  Integer sums do not depend on the order of the
 // additions.  `down` is what the light children read on the way down.
 constexpr size_t kAccBytes = 8 + 16 + 8;
+struct Down {                    // what a row passes to its light children: lin (units), lout
+    int a;
+    float b;
+};
 struct Acc {
     int4 *limb;
     int2 *s;                     // search: value, size
-    float2 *down;                // lin, lout
+    Down *down;
 };
 __host__ __device__ inline Acc acc_at(char *base, size_t count)
 {
     Acc a;
     a.limb = (int4 *)base;
     a.s = (int2 *)(base + count * 16);
-    a.down = (float2 *)(base + count * 24);
+    a.down = (Down *)(base + count * 24);
     return a;
 }
 
@@ -486,16 +490,17 @@ __device__ __forceinline__ int64_t exact_top(const Tab &t, const Scratch1 &g, in
 }
 
 // ---- one tile of the losses, from the top of a path down: `a` the sum of
-// max(0, -f) over the path from the root, `b` the smallest f on it.  In
-// floats rounded down: a loss is only ever underestimated, which keeps rows.
-// The scan adds in an order that differs from lane to lane, so a row's rounded
-// sum may lie below its parent's, and a row would be undecided under a parent
-// that is decided out.  The largest of the sums from the top down to the row
-// is what the row gets: each of them is a lower bound of the row's loss, and no
-// row's is below its parent's.  (Where a sum starts from the parent's value,
-// here and at a tile's edge, rounding down leaves it at least that.)  Five more
-// shuffles a tile: 16 items of 50,000 rows 586.5 -> 589.3 us.
-__device__ __forceinline__ void loss_tile(int code, int64_t f, bool child, float2 up, float &ca, float &cb, float &a,
+// max(0, -f) over the path from the root, `b` the smallest f on it.  Sums in
+// units of 2^shift, each row's share rounded down to them and no more than
+// kLossCap: a loss is only ever underestimated, which keeps rows.  Below a row
+// that is decided out every row has to be, so no row's sum may lie below its
+// parent's: whole numbers add up to the same in any order (sums of floats did
+// not, and a row stayed undecided under a parent that was out; with a running
+// maximum over them, five more shuffles a tile, the paper-scale plan took 27.73
+// ms, with whole numbers 27.53).
+constexpr int kLossCap = 1 << 30;
+constexpr int kLossBits = 20;                // of a price times a mean weight: 0.1 of it, the first threshold, is 2^17
+__device__ __forceinline__ void loss_tile(int code, int64_t f, int shift, bool child, Down up, int &ca, float &cb, int &a,
                                           float &b)
 {
     const int lane = threadIdx.x & 31;
@@ -504,49 +509,48 @@ __device__ __forceinline__ void loss_tile(int code, int64_t f, bool child, float
     const unsigned after = lane < 31 ? starts >> (lane + 1) : 0u;
     const int rem = after ? __ffs((int)after) - 1 : 31 - lane;    // lanes to the right in this path
     b = __ll2float_rd(f);
-    a = f < 0 ? __ll2float_rd(-f) : 0.f;
+    const unsigned long long loss = f < 0 ? (unsigned long long)-f >> shift : 0;
+    a = loss < kLossCap ? (int)loss : kLossCap;
     if (child) {                             // a path's top below some row: `up` is that row's
-        a = __fadd_rd(a, up.x);
-        b = fminf(b, up.y);
+        a = min(a + up.a, kLossCap);
+        b = fminf(b, up.b);
     }
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const float a2 = __shfl_down_sync(kAll, a, o), b2 = __shfl_down_sync(kAll, b, o);
+        const int a2 = __shfl_down_sync(kAll, a, o);
+        const float b2 = __shfl_down_sync(kAll, b, o);
         if (rem >= o) {
-            a = __fadd_rd(a, a2);
+            a = min(a + a2, kLossCap);
             b = fminf(b, b2);
         }
     }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float a2 = __shfl_down_sync(kAll, a, o);
-        if (rem >= o) a = fmaxf(a, a2);
-    }
     if (!((tops >> (lane + rem)) & 1u)) {       // the path goes on in the next tile
-        a = __fadd_rd(a, ca);
+        a = min(a + ca, kLossCap);
         b = fminf(b, cb);
     }
     ca = __shfl_sync(kAll, a, 0);
     cb = __shfl_sync(kAll, b, 0);
 }
 // key of a row (15 bits) and whether it is in S (bit 15)
-__device__ __forceinline__ int loss_code(float a, float b)
+__device__ __forceinline__ int loss_code(int a, float b, int shift)
 {
-    const float v = b > 0.f ? b : a;
-    const int k = v < 1.f ? 0 : min((int)(__float_as_uint(v) >> 18) - kKeyBase, kBins - 1);
-    return k | (b > 0.f ? 0x8000 : 0);
+    const bool in = b > 0.f;
+    const float v = in ? b : __int2float_rd(a);
+    const int k = v < 1.f ? 0 : min((int)(__float_as_uint(v) >> 18) - kKeyBase + (in ? 0 : 32 * shift), kBins - 1);
+    return k | (in ? 0x8000 : 0);
 }
 
 // losses of one bin, levels from the top down, and their histogram
 template <bool GLOBAL>
 __device__ __forceinline__ void loss_bin(const int2 *info, const int64_t *fin, uint16_t *key, const unsigned *list, int n,
-                                         int nlev, const Acc &own, const int *base, const float2 *topd, unsigned char *ring,
-                                         unsigned *hist)
+                                         int nlev, const Acc &own, const int *base, const Down *topd, int shift,
+                                         unsigned char *ring, unsigned *hist)
 {
     const int lane = threadIdx.x & 31;
     Feed<int64_t, -1> feed(info, fin, list, n, ring);
     int lev = nlev - 1;
-    float ca = 0.f, cb = 0.f;
+    int ca = 0;
+    float cb = 0.f;
     while (feed.more()) {
         const unsigned en = feed.entry();
         for (; lev > level_of(en); --lev) __syncthreads();
@@ -556,34 +560,40 @@ __device__ __forceinline__ void loss_bin(const int2 *info, const int64_t *fin, u
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const bool child = (c.x & kTop) && up != kNone;
         const int a0 = base[bin_of(en)];
-        float2 from = make_float2(0.f, 0.f);
+        Down from = {0, 0.f};
         if (child) {
             if (c.x & kUp) from = topd[up];
-            else from = acc_ld<GLOBAL>(own.down + a0 + up);
+            else {
+                const int2 d = acc_ld<GLOBAL>((const int2 *)(own.down + a0 + up));
+                from = {d.x, __int_as_float(d.y)};
+            }
         }
-        float a, b;                          // (a path that goes on does so in the tile just done)
-        loss_tile(c.x, f, child, from, ca, cb, a, b);
-        if (ac != kNone) own.down[a0 + ac] = make_float2(a, b);
-        const int code = (c.x >> kWeightShift) ? loss_code(a, b) : kKeyPad;      // (a pad weighs nothing)
+        int a;                               // (a path that goes on does so in the tile just done)
+        float b;
+        loss_tile(c.x, f, shift, child, from, ca, cb, a, b);
+        if (ac != kNone) own.down[a0 + ac] = {a, b};
+        const int code = (c.x >> kWeightShift) ? loss_code(a, b, shift) : kKeyPad;      // (a pad weighs nothing)
         if (code != kKeyPad) atomicAdd(hist + (code & 0x7fff), 1u);
         key[tile_of(en) * 32 + lane] = (uint16_t)code;
     }
     for (; lev > 0; --lev) __syncthreads();
 }
 // the last bin, by one warp; one CTA (`write`) keeps its keys
-__device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, float2 *topd, unsigned *hist, bool write)
+__device__ __forceinline__ void loss_top(const Tab &t, const Scratch1 &g, Down *topd, int shift, unsigned *hist, bool write)
 {
     const int lane = threadIdx.x & 31;
-    float ca = 0.f, cb = 0.f;
+    int ca = 0;
+    float cb = 0.f;
     for (int s = t.nslots - 32 + lane; s >= t.binslot[t.bins]; s -= 32) {
         const int2 c = __ldg(t.info + s);
         const int ac = c.y & 0xffff, up = (unsigned)c.y >> 16;
         const bool child = (c.x & kTop) && up != kNone;
-        float a, b;
-        loss_tile(c.x, g.f[s], child, child ? topd[up] : make_float2(0.f, 0.f), ca, cb, a, b);
-        if (ac != kNone) topd[ac] = make_float2(a, b);
+        int a;
+        float b;
+        loss_tile(c.x, g.f[s], shift, child, child ? topd[up] : Down{0, 0.f}, ca, cb, a, b);
+        if (ac != kNone) topd[ac] = {a, b};
         if (write) {
-            const int code = (c.x >> kWeightShift) ? loss_code(a, b) : kKeyPad;
+            const int code = (c.x >> kWeightShift) ? loss_code(a, b, shift) : kKeyPad;
             if (code != kKeyPad) atomicAdd(hist + (code & 0x7fff), 1u);
             g.key[s] = (uint16_t)code;
         }
@@ -1177,13 +1187,16 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     // ---- losses and their histogram
     unsigned *ghist = g.hist + kBins;
     if (!give_up) {
+        // (at price 0 the largest profit stands for it)
+        const float unit = lam > 0 ? (float)lam * ((float)A.total_weight / (float)n) : (float)maxp;
+        const int shift = max(0, (int)(__float_as_uint(fmaxf(unit, 1.f)) >> 23) - 127 - kLossBits);
         for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
         __syncthreads();
         if (has_top) {
-            if (warp == 0) loss_top(t, g, (float2 *)s_top, hist, cr == 0);
+            if (warp == 0) loss_top(t, g, (Down *)s_top, shift, hist, cr == 0);
             __syncthreads();
         }
-        loss_bin<!SMEM>(info, g.f + lo, g.key + lo, lists[0][warp], tiles, nlev, own, base, (const float2 *)s_top, ring, hist);
+        loss_bin<!SMEM>(info, g.f + lo, g.key + lo, lists[0][warp], tiles, nlev, own, base, (const Down *)s_top, shift, ring, hist);
         __syncthreads();
         for (int i = tid; i < kBins; i += kThreads)
             if (hist[i]) atomicAdd(ghist + i, hist[i]);
