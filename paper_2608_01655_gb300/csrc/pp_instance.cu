@@ -308,7 +308,7 @@ static pp_status build_host_tables(int32_t n, int32_t W, const int32_t *parent, 
         }
     }
     if (build_reduce_tables(n, inst->h_par, inst->h_next, inst->h_wpre, inst->total_weight, inst->max_weight, red))
-        inst->red = reduce_shape(*red);
+        inst->red = reduce_shape(*red, n, inst->max_weight);
     return PP_OK;
 }
 

@@ -274,7 +274,7 @@ bool build_reduce_tables(int32_t n, const std::vector<int32_t> &par, const std::
                          ReduceTables *out);
 size_t reduce_tables_bytes(const ReduceTables &R);
 void reduce_tables_pack(const ReduceTables &R, char *dst);
-ReduceShape reduce_shape(const ReduceTables &R);
+ReduceShape reduce_shape(const ReduceTables &R, int32_t n, int32_t max_weight);
 pp_status reduce_device(ReduceShape *r);
 size_t reduce_item_bytes(const pp_instance *inst);
 // whether launches of this instance try the reduction first (not without

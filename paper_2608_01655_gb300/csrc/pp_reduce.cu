@@ -127,10 +127,10 @@ struct Args {
     DpWork w;
     size_t item_bytes;           // of w.red_scratch
     int64_t total_weight;
+    float mean_weight;           // of a row
     int32_t max_weight;
     int32_t clip_kid;            // the search's bound on what a light child adds
-    float price_us, sweep_us[2]; // of one price; of a sweep of all rows, at most 128 columns and more
-    int32_t evals[2];            // prices tried at most
+    Spending spending;
     const int2 *pspan;           // the pruned sweep's: see prune_item
     int32_t stack_depth;
     int32_t *status;
@@ -634,12 +634,14 @@ __device__ int block_scan(int v, int *total, int *sh)
 // interpolating logarithms (|S| falls like a power).  3 to 6 prices; a search
 // from price 0 by the tangents of L took 9 to 10.
 // ---------------------------------------------------------------------------
-enum : int { kGo = 0, kStop = 1, kSlack = 2, kCoarser = 3 };
+enum : int { kGo = 0, kStop = 1, kSlack = 2, kCoarser = 3, kTooDear = 4 };
 constexpr int kCoarserBits = 6;
 
 struct Search {                              // prices in units
     float x0, x1, z0, z1;                    // price and |S| of the ends with |S| > k and <= k
     int have, side;                          // bit 0, 1: that end is there; steps in a row to one side
+    int max_evals;                           // prices that may be tried
+    float left;                              // us that may still be spent before the item is left to the sweep
 };
 
 // weight of the rows worth at least lam per slot, and its inverse (cum[c]:
@@ -671,8 +673,7 @@ __device__ float price_of_rank(const int *cum, float rank)
 // in units of 2^(shift + kCoarserBits) with `nx` of them (kCoarser): where few
 // chunks have a profit whole paths are taken for one, and the price may be far
 // above the k-th largest profit per slot, which the units were chosen by
-__device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int max_evals,
-                          int lam, float Z, int &nx)
+__device__ int next_price(Search &b, const int *cum, float k, int maxlam, float unit, int evals, int lam, float Z, int &nx)
 {
     if (Z > k) {
         b.x0 = (float)lam;
@@ -690,7 +691,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         nx = lam;
         return kStop;
     }
-    if (lam == kClipPrice && Z > k && evals < max_evals) {
+    if (lam == kClipPrice && Z > k && evals < b.max_evals) {
         b.x0 *= 1.f / (1 << kCoarserBits);
         nx = lam >> (kCoarserBits - 3);
         return kCoarser;
@@ -699,7 +700,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
     if (b.have == 3) {
         // L's slope is k - |S|, so these bound what a better price could still give
         const float d = b.x1 - b.x0, e0 = (b.z0 - k) * d, e1 = (k - b.z1) * d;
-        if (fminf(e0, e1) <= 0.1f * b.x0 || d <= 1.f || evals >= max_evals) {
+        if (fminf(e0, e1) <= 0.1f * b.x0 || d <= 1.f || evals >= b.max_evals) {
             nx = (int)(e0 < e1 ? b.x0 : b.x1);
             return kStop;
         }
@@ -714,7 +715,7 @@ __device__ int next_price(Search &b, const int *cum, float k, int maxlam, float 
         }
         x = fminf(fmaxf(x, b.x0 + 1.f), b.x1 - 1.f);
     } else {
-        if (evals >= max_evals) {
+        if (evals >= b.max_evals) {
             nx = lam;
             return kStop;
         }
@@ -895,7 +896,6 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     __shared__ int base[kMaxBins + 1];       // of a bin's accumulators among the CTA's
     __shared__ int s_a, s_b, s_flag, s_lam;
     __shared__ Search s_search;
-    __shared__ float s_spent;
     __shared__ int64_t s_val;
     const Tab &t = A.t;
     const int CL = t.CL, cr = CL > 1 ? cluster_rank() : 0;
@@ -1090,16 +1090,20 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
 
     // ---- the price
     // lambda k, and lambda times the weight of a tile's 32 rows (what a scan sums
-    // before it takes the maximum), have to stay within int64
-    bool give_up = maxp > kBig / (k > 32 * A.max_weight ? k : 32 * A.max_weight);
+    // before it takes the maximum), have to stay within int64 (a product: the
+    // division, with one of the mean weight further on, was 0.8 us an item)
+    const unsigned long long slots_most = k > 32 * A.max_weight ? k : 32 * A.max_weight, top_profit = maxp;
+    const bool too_large = __umul64hi(top_profit, slots_most) != 0 || top_profit * slots_most > (unsigned long long)kBig;
     int64_t lam = 0, L = 0;
-    // what may be spent before the item is left to the sweep (see sweep_us)
-    auto limit = [&] { return k > 128 ? A.sweep_us[1] : A.sweep_us[0]; };
-    if (!give_up) {
+    if (!too_large) {
         const float guess = cum[0] <= k ? 0.f : fminf(fmaxf(price_of_rank(cum, (float)k), 1.f), (float)maxp);
         int shift = max(0, (int)(__float_as_uint(fmaxf(guess, 1.f)) >> 23) - 127 - kUnitBits);
         int price = (int)(guess * exp2f((float)-shift));
-        if (tid == 0) s_search = Search();   // (shared: only that thread uses it)
+        if (tid == 0) {                      // (shared; the search's thread)
+            s_search = Search();
+            s_search.max_evals = A.spending.evals[k > 128];
+            s_search.left = A.spending.sweep[k > 128];
+        }
         auto to_units = [&](int from, int to) {
             for (int s = from + tid; s < to; s += kThreads) {
                 const int64_t p = g.prof[s] >> shift;
@@ -1143,8 +1147,12 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                     if (lane == 0) {
                         z += bins;
                         int nx = price;
-                        s_flag = next_price(s_search, cum, (float)k, maxlam, exp2f((float)shift), ev + 1,
-                                            k > 128 ? A.evals[1] : A.evals[0], price, (float)z, nx);
+                        s_flag = next_price(s_search, cum, (float)k, maxlam, exp2f((float)shift), ev + 1, price, (float)z, nx);
+                        if (s_flag == kStop || s_flag == kSlack) {
+                            // (the exact evaluation and the losses take two prices)
+                            s_search.left -= (float)(ev + 3) * A.spending.price;
+                            if (s_search.left < kPassUs) s_flag = kTooDear;
+                        }
                         s_lam = nx;
                         s_a = z > k;
                     }
@@ -1162,33 +1170,31 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
         }
         if (s_flag == kSlack) price = 0;
         lam = (int64_t)price << shift;
-        const float spent = (float)(ev + 3) * A.price_us;
-        give_up = spent + kPassUs > limit();
-        if (tid == 0) s_spent = spent;
-    }
-    if (!give_up) {
-        // ---- exactly there: f of every row, L
-        for (int i = tid; i <= na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
-        __syncthreads();
-        int64_t ry = 0;
-        exact_bin<!SMEM>(info, g.prof + lo, g.f + lo, g.topl, lists[0][warp], tiles, nlev, own, base, na, lam, ring, ry);
+        if (s_flag != kTooDear) {
+            // ---- exactly there: f of every row, L
+            for (int i = tid; i <= na; i += kThreads) own.limb[i] = make_int4(0, 0, 0, 0);
+            __syncthreads();
+            int64_t ry = 0;
+            exact_bin<!SMEM>(info, g.prof + lo, g.f + lo, g.topl, lists[0][warp], tiles, nlev, own, base, na, lam, ring, ry);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ry += __shfl_xor_sync(kAll, ry, o);
-        if (lane == 0 && ry) atomicAdd(&g.s->sumL, (unsigned long long)ry);
-        sync_all();
-        if (warp == 0) {
-            ry = has_top ? exact_top(t, g, s_top, lam) : 0;
-            if (lane == 0) s_val = (int64_t)__ldcg(&g.s->sumL) + ry + lam * k;
+            for (int o = 16; o > 0; o >>= 1) ry += __shfl_xor_sync(kAll, ry, o);
+            if (lane == 0 && ry) atomicAdd(&g.s->sumL, (unsigned long long)ry);
+            sync_all();
+            if (warp == 0) {
+                ry = has_top ? exact_top(t, g, s_top, lam) : 0;
+                if (lane == 0) s_val = (int64_t)__ldcg(&g.s->sumL) + ry + lam * k;
+            }
+            __syncthreads();
+            L = s_val;
         }
-        __syncthreads();
-        L = s_val;
     }
+    const bool give_up = too_large || s_flag == kTooDear;
 
     // ---- losses and their histogram
     unsigned *ghist = g.hist + kBins;
     if (!give_up) {
         // (at price 0 the largest profit stands for it)
-        const float unit = lam > 0 ? (float)lam * ((float)A.total_weight / (float)n) : (float)maxp;
+        const float unit = lam > 0 ? (float)lam * A.mean_weight : (float)maxp;
         const int shift = max(0, (int)(__float_as_uint(fmaxf(unit, 1.f)) >> 23) - 127 - kLossBits);
         for (int i = tid; i < kBins; i += kThreads) hist[i] = 0;
         __syncthreads();
@@ -1242,7 +1248,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
     // allows for one more after it (one that is sure to succeed is not refused)
     auto pass_us = [&](int T) { return kPassUs + (float)T * (A.max_weight > 1 ? kWeightedRowUs : kRowUs); };
     auto rows_left = [&](float more) {
-        const float us = limit() - s_spent - more - kPassUs;
+        const float us = s_search.left - more - kPassUs;
         return (int)fminf(fmaxf(us * (A.max_weight > 1 ? 1.f / kWeightedRowUs : 1.f / kRowUs), 0.f), (float)kRowCap);
     };
     if (!give_up) {
@@ -1253,7 +1259,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
         if (lam == 0) {
             key = -1;
         } else {
-            T = up_to(min(kFirstRows, rows_left(0.f)), code_of((int64_t)(0.1f * (float)lam * ((float)A.total_weight / (float)n))), key);
+            T = up_to(min(kFirstRows, rows_left(0.f)), code_of((int64_t)(0.1f * (float)lam * A.mean_weight)), key);
         }
         for (; pass < kPasses; ++pass) {
             const bool big = T > (sure ? kRowCap : rows_left(0.f));       // the same in every CTA
@@ -1517,7 +1523,7 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
                     g.s->verdict[pass] = out;
                 }
             }
-            if (tid == 0) s_spent += pass_us(T);
+            if (tid == 0) s_search.left -= pass_us(T);
             sync_all();
             verdict = __ldcg(&g.s->verdict[pass]);
             if (verdict != 2 && verdict != 5) break;
@@ -1801,7 +1807,7 @@ static size_t scan_bytes(int acc, bool acc_smem)
 }
 constexpr size_t kAccLimit = (size_t)192 << 10;
 
-ReduceShape reduce_shape(const ReduceTables &R)
+ReduceShape reduce_shape(const ReduceTables &R, int32_t n, int32_t max_weight)
 {
     ReduceShape s;
     s.bins = R.bins;
@@ -1817,14 +1823,15 @@ ReduceShape reduce_shape(const ReduceTables &R)
         s.acc[s.ncl++] = c.acc;
         if (scan_bytes(c.acc, true) > kAccLimit) s.acc_global = 1;
     }
+    s.item_bytes = al(carve(nullptr, s.nslots, s.ntop, s.acc_global, nullptr));
+    set_spending(s, n, max_weight, kMaxEvals);
     return s;
 }
 
 // scratch of one item in the DP workspace, 0 when the instance has no reduction
 size_t reduce_item_bytes(const pp_instance *inst)
 {
-    if (!inst->red.bins) return 0;
-    return al(carve(nullptr, inst->red.nslots, inst->red.ntop, inst->red.acc_global, nullptr));
+    return inst->red.bins ? inst->red.item_bytes : 0;
 }
 
 // Once per instance: the kernels' attributes, and how many clusters above the
@@ -1884,6 +1891,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.w = work;
     a.item_bytes = reduce_item_bytes(inst);
     a.total_weight = inst->total_weight;
+    a.mean_weight = (float)inst->total_weight / (float)inst->n;
     a.max_weight = inst->max_weight;
     a.pspan = inst->d_pspan;
     a.stack_depth = inst->stack_depth;
@@ -1891,11 +1899,7 @@ pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, boo
     a.clip_kid = std::min(1 << 22, (1 << 30) / std::max(1, r.max_kids));
     const int x = cluster_index(r, std::max(work.items, batch));
     a.t.CL = r.cl[x];
-    a.price_us = price_us(r, x);
-    for (int many = 0; many < 2; ++many) {
-        a.sweep_us[many] = sweep_us(inst->n, inst->max_weight, many);
-        a.evals[many] = std::min(kMaxEvals, std::max(3, (int)(a.sweep_us[many] / a.price_us) - 2));
-    }
+    a.spending = r.spending[x];
     const bool acc_smem = scan_bytes(r.acc[x], true) <= kAccLimit;
     const size_t smem = std::max(scan_bytes(r.acc[x], acc_smem), up16(sizeof(Rows)) + kPool);
     const auto kern = acc_smem ? k_reduce<true> : k_reduce<false>;

@@ -1,17 +1,29 @@
 // How many CTAs share an item of the exact reduction: plain C++, no device.
 #pragma once
 
+#include <algorithm>
+#include <cstddef>
+
 namespace pp {
 
 constexpr int kPortable = 8;     // CTAs of a cluster that every device takes
 constexpr int kReduceCtas = 128;            // of all items in flight (16 clusters of 8, 15 of which run at a time on 152
                                             // SMs: a batch of 16 685 us; all at once on 6 CTAs each, 712)
 
+// What an item may cost, in microseconds, see set_spending.
+struct Spending {
+    float price = 0.f;              // of one price
+    float sweep[2] = {};            // of a sweep of all rows: at most 128 columns, more
+    int evals[2] = {};              // prices tried at most
+};
+
 // Layout of an instance's reduction.  bins = 0: this tree is not reduced.
 struct ReduceShape {
     int bins = 0, nslots = 0, nstreams = 0, nlev = 0, ntop = 0, toptiles = 0, max_kids = 0;
     int ncl = 0, cl[8] = {}, acc[8] = {}, path[8] = {}, acc_global = 0;      // cluster sizes, largest first
     int wide = 0;                   // clusters above the portable size that fit the device
+    Spending spending[8];           // by cluster size
+    size_t item_bytes = 0;          // scratch of one item
 };
 
 // `wide` clusters of the largest size, above the portable one, run at a time:
@@ -27,6 +39,7 @@ inline void set_wide(ReduceShape &r, int wide)
         r.cl[x - drop] = r.cl[x];
         r.acc[x - drop] = r.acc[x];
         r.path[x - drop] = r.path[x];
+        r.spending[x - drop] = r.spending[x];
     }
     r.ncl -= drop;
     if (r.ncl == 0) r.bins = 0;
@@ -43,25 +56,27 @@ inline int cluster_index(const ReduceShape &r, int items)
     return x;
 }
 
-// Microseconds of one price for an item on r.cl[x] CTAs, by the tiles that
-// follow one another (measured: 3.3 on a star of 800 rows, one tile; 5.0 on a
-// random tree of 800, 6 tiles; 12.5 on a chain of 800, 25; 6.0 on a random tree
-// of 1,600 on 6 CTAs, 4 and 2 in the last bin; 10.9 on chains of 256, 18 and 1).
-// The exact evaluation with the losses takes two.
-inline float price_us(const ReduceShape &r, int x)
+// No more is spent on an item before it is left to the sweep than a sweep of
+// all rows would take, so that one which the reduction cannot solve takes about
+// twice as long as without it at most (with 16 prices and three DPs for every
+// item, up to 5.6 times).
+// A price, by the tiles that follow one another: 3.3 us on a star of 800 rows
+// (one tile), 5.0 on a random tree of 800 (6), 12.5 on a chain of 800 (25), 6.0
+// on a random tree of 1,600 on 6 CTAs (4, and 2 in the last bin), 10.9 on
+// chains of 256 (18 and 1).  The exact evaluation with the losses takes two.
+// A sweep: pruning and walk, then 0.035 to 0.045 us a row of at most 128
+// columns of unit weights, 0.065 to 0.1 of more, 0.18 to 0.4 with weights
+// (0.25 here: they sooner pay).
+inline void set_spending(ReduceShape &r, int n, int max_weight, int max_evals)
 {
-    return 2.6f + 0.4f * (float)(r.path[x] + r.toptiles) + (r.cl[x] > 1 ? 1.f : 0.f);
-}
-
-// What a sweep of n rows takes, in microseconds: pruning and walk, then 0.035 to
-// 0.045 a row of at most 128 columns of unit weights, 0.065 to 0.1 of more
-// (`many`), 0.18 to 0.4 with weights (0.25 here: they sooner pay).  No more is
-// spent on an item before it is left to the sweep, so that one which the
-// reduction cannot solve takes about twice as long as without it at most (with
-// 16 prices and three DPs for every item, up to 5.6 times).
-inline float sweep_us(int n, int max_weight, bool many)
-{
-    return 25.f + (float)n * (max_weight > 1 ? 0.25f : many ? 0.07f : 0.04f);
+    for (int x = 0; x < r.ncl; ++x) {
+        Spending &s = r.spending[x];
+        s.price = 2.6f + 0.4f * (float)(r.path[x] + r.toptiles) + (r.cl[x] > 1 ? 1.f : 0.f);
+        for (int many = 0; many < 2; ++many) {
+            s.sweep[many] = 25.f + (float)n * (max_weight > 1 ? 0.25f : many ? 0.07f : 0.04f);
+            s.evals[many] = std::min(max_evals, std::max(3, (int)(s.sweep[many] / s.price) - 2));
+        }
+    }
 }
 
 }  // namespace pp
