@@ -398,6 +398,63 @@ def test_workspace_is_read_as_it_was_written(pp, oracle_lib, solved_by_reduction
             np.testing.assert_array_equal(chosen[b].cpu().numpy(), oc)
 
 
+@pytest.mark.parametrize("shape,n,wmax", [("mixed", 6000, 1), ("random", 12000, 3), ("star", 6000, 9)])
+def test_some_rows_decided_and_the_rest_swept(pp, oracle_lib, shape, n, wmax):
+    """Ten profits close to one another: more rows stay undecided than the DP on
+    chip takes and fewer than pruning alone leaves, so the sweep joins the
+    decided rows, on the wavefront kernel and the one-CTA kernel."""
+    rng = np.random.default_rng(n + wmax)
+    parent = _tree(rng, shape, n)
+    weight = rng.integers(1, wmax + 1, size=n).astype(np.int32)
+    profits = np.stack([rng.integers(10 ** 6, 10 ** 6 + 10 ** 5, n), rng.integers(1000, 1010, n)]).astype(np.int64)
+
+    def rows(r):
+        assert 1024 < r[1] < n
+    chosen = _check(pp, oracle_lib, parent, weight, profits, [n // 20 * wmax] * 2, rows)
+    _assert_closed(parent, chosen)
+
+
+@pytest.mark.parametrize("shape,n,k", [("random", 100, 20), ("mixed", 2000, 256), ("mixed", 20000, 1000), ("star", 3000, 300)])
+def test_update_chain_in_a_graph(pp, oracle_lib, shape, n, k):
+    """The allocation-free DP and its traceback, chained by programmatic
+    dependent launch, captured in a CUDA graph and replayed on new profits:
+    trees with and without the reduction, items that it solves and leaves."""
+    rng = np.random.default_rng(n)
+    parent = _tree(rng, shape, n)
+    inst = wl.Instance("t", n, 1, parent, np.ones(n, np.int32), np.ones((1, n), np.int64), np.ones((1, n), np.int64),
+                       np.ones((1, n), np.int64), 0, np.array([1], np.int32), 1, 1)
+    with pp.Instance.from_workload(inst) as ppi:
+        prof = torch.zeros((3, n), dtype=torch.int64, device="cuda")
+        bud = torch.tensor([k, k // 2, 0], dtype=torch.int32, device="cuda")
+        best = torch.zeros(3, dtype=torch.int64, device="cuda")
+        bits = torch.zeros(pp.pp_dp_bits_size(ppi, 3, k) // 4, dtype=torch.int32, device="cuda")
+        chosen = torch.zeros((3, n), dtype=torch.uint8, device="cuda")
+
+        def chain():
+            for _ in range(2):                   # a chain, not one call: the second follows the first's last kernel
+                pp.pp_tree_dp_noalloc(ppi, prof, bud, k, best, bits)
+                pp.pp_traceback(ppi, bits, bud, k, chosen)
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            chain()
+        side.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            chain()
+        for _ in range(2):
+            p = np.exp(rng.uniform(0, 18, size=(3, n))).astype(np.int64)
+            p[1] = rng.integers(1, 3, size=n)
+            prof.copy_(torch.from_numpy(p))
+            chosen.fill_(7)
+            graph.replay()
+            torch.cuda.synchronize()
+            ppi.sync()
+            for b, kb in enumerate((k, k // 2, 0)):
+                ob, oc = oracle_lib.rooted_dp(parent, np.ones(n, np.int32), p[b], kb)
+                assert int(best[b]) == ob
+                np.testing.assert_array_equal(chosen[b].cpu().numpy(), oc)
+
+
 def test_two_instances_on_two_threads(pp, oracle_lib):
     """Launches of instances whose kernels take different amounts of shared
     memory (the sweep's, for weights on both sides of the wavefront kernel's
