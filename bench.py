@@ -6,7 +6,7 @@ pass, up to R refinement sweeps over S starts, objective + argmax) of the
 headline workload, the paper-scale synthetic instance (n = 50,000 chunks,
 W = 16 workers, k = 4,096 slots, 16 starts, 6 rounds), inputs resident in HBM.
 
-  value     Eq. 9 cell updates executed (sum over DPs of n * k_h) per second of
+  value     Eq. 9 cell updates of the DPs that ran (sum over them of n * k_h) per second of
             device time, summed over ranks; L2 is flushed between steps, and the
             timed plans carry no per-launch events (the phase breakdown comes
             from the warm-up plans)
@@ -391,7 +391,7 @@ def measure_e2e(pp, torch, inst, S, R, orders, warmup, steps, flush, sched, sg, 
 
 def plan_summary(inst, res, times, phase, e2e_times, h2d, d2h, l2_gbs, hbm_gbs):
     """Per-workload figures: plan time with inputs resident and with upload,
-    executed and swept cells/s, per-update latency, and the table
+    table and swept cells/s, per-update latency, and the table
     algorithm's B_min / B_stream bytes over the DP step's time as fractions
     of the HBM copy and L2 read bandwidths."""
     k = int(inst.budget.max())
@@ -406,7 +406,7 @@ def plan_summary(inst, res, times, phase, e2e_times, h2d, d2h, l2_gbs, hbm_gbs):
         "steps": len(times), "plan_ms": 1000 * plan_s,
         "plan_ms_with_upload": 1000 * sum(e2e_times) / len(e2e_times) if e2e_times else None,
         "e2e_steps": len(e2e_times), "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
-        "cells_per_s_executed": res.dp_cells / plan_s,
+        "cells_per_s_table": res.dp_cells / plan_s,
         "cells_per_s_swept": res.dp_rows_swept * k / plan_s,
         "update_ms": sum(phase) / (nl * len(times)),
         "dp_step_ms": 1000 * dp_t, "dps_per_step": items,
@@ -502,7 +502,7 @@ def oracle_leg(inst, res):
                 "sample": f"{count} concurrent worker updates (marginals + Eq. 9 DP + backtrack, "
                           f"{inst.n} x {int(inst.budget.max())} cells each), {secs:.1f} s",
                 "plan_s_extrapolated": res.dp_cells / rate,
-                "extrapolation": "the GPU plan's executed cells at the sample's rate"}
+                "extrapolation": "the GPU plan's table cells at the sample's rate"}
     threads = min(inst.starts, cores)
     r, secs = oracle_plan(inst, threads)
     return {"kind": "oracle plan", "cores": threads, "value": r.cells / secs, "unit": UNIT, "plan_s": secs,

@@ -283,9 +283,9 @@ bool reduce_on(const pp_instance *inst);
 pp_status launch_reduce(pp_instance *inst, int batch, const int64_t *profit, bool by_node,
                         const int32_t *item_budget, const int32_t *item_active, int64_t *best, const DpWork &work,
                         cudaStream_t st, int32_t max_budget, unsigned long long *rows_kept);
-// scratch for the skip-row stack of `items` item slots of geometry g
 // levels of the stack of skipped rows that do not fit in shared memory
 int dp_global_levels(const pp_instance *inst, const DpGeom &g);
+// scratch for the skip-row stack of `items` item slots of geometry g
 pp_status ensure_dp_stack(pp_instance *inst, const DpGeom &g, int items);
 
 pp_status launch_marginals(pp_instance *inst, int batch, const int32_t *worker,

@@ -25,13 +25,14 @@
 // the losses themselves (lin grows down a path) and for the rounded ones, which
 // are sums of whole numbers (loss_tile).
 //
-// A prefix tree of 50,000 chunks with the planner's profits leaves 30 to 600
-// undecided rows of the 16,000 to 37,000 that the pruned sweep keeps, and a
-// budget of a few hundred slots instead of 4,096: 0.19 ms an item, where that
-// sweep took 1.3.  More undecided rows than fit on chip (chunks in long chains
-// that are worth taking only whole) go to pp_dp.cu's kernels with what is left
-// of the budget; where no V is found (ties that leave nearly everything
-// undecided) those kernels get every row.
+// A prefix tree of 50,000 chunks with the planner's profits leaves 222
+// undecided rows (the mean of a plan's updates) of the 16,000 to 37,000 that the
+// pruned sweep keeps, and a budget of a few hundred slots instead of 4,096: 0.17
+// ms an item, where that sweep took 1.3.  More undecided rows than fit on chip
+// (chunks in long chains that are worth taking only whole) go to pp_dp.cu's
+// kernels with what is left of the budget; where no V is found (ties that leave
+// nearly everything undecided), or none before as much time is spent as they
+// take, those kernels get every row.
 //
 // Layout.  f is a Lindley recursion along every heavy path of the tree
 // (y_i = max(0, d_i + y_(i+1)), d_i the row's own term plus its light
@@ -631,7 +632,7 @@ __device__ int block_scan(int v, int *total, int *sh)
 // Its first guess is the k-th largest profit per slot (chunks taken without
 // their prefixes: within ~15% on the prefix trees here), the second scales
 // that curve through the first point, then the bracket is closed by
-// interpolating logarithms (|S| falls like a power).  3 to 6 prices; a search
+// interpolating logarithms (|S| falls like a power).  3 to 7 prices; a search
 // from price 0 by the tangents of L took 9 to 10.
 // ---------------------------------------------------------------------------
 enum : int { kGo = 0, kStop = 1, kSlack = 2, kCoarser = 3, kTooDear = 4 };
