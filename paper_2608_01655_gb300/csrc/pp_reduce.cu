@@ -913,6 +913,11 @@ __global__ void __launch_bounds__(kThreads) k_reduce(const __grid_constant__ Arg
         return;
     }
     const int64_t k = kreq < A.total_weight ? kreq : A.total_weight;     // more changes nothing
+    if (A.spending.evals[k > 128] == 0 && k > 0) {           // (the same in every CTA)
+        if (cr == 0 && tid == 0) *red = 0;
+        prune_left(A, item, nullptr);
+        return;
+    }
     Scratch1 g;
     carve(A.w.red_scratch + (size_t)item * A.item_bytes, t.nslots, t.ntop, !SMEM, &g);
     const int words = (n + 31) / 32;

@@ -14,7 +14,7 @@ constexpr int kReduceCtas = 128;            // of all items in flight (16 cluste
 struct Spending {
     float price = 0.f;              // of one price
     float sweep[2] = {};            // of a sweep of all rows: at most 128 columns, more
-    int evals[2] = {};              // prices tried at most
+    int evals[2] = {};              // prices tried at most (0: the sweep takes the item)
 };
 
 // Layout of an instance's reduction.  bins = 0: this tree is not reduced.
@@ -67,6 +67,9 @@ inline int cluster_index(const ReduceShape &r, int items)
 // A sweep: pruning and walk, then 0.035 to 0.045 us a row of at most 128
 // columns of unit weights, 0.065 to 0.1 of more, 0.18 to 0.4 with weights
 // (0.25 here: they sooner pay).
+// A tree whose sweep takes less than six prices is left to it at once: three
+// prices, the exact evaluation and a DP would not fit (chains of 400 and 800
+// rows, 128 columns at most: 105 to 130 us with the prices, 64 to 78 without).
 inline void set_spending(ReduceShape &r, int n, int max_weight, int max_evals)
 {
     for (int x = 0; x < r.ncl; ++x) {
@@ -74,7 +77,7 @@ inline void set_spending(ReduceShape &r, int n, int max_weight, int max_evals)
         s.price = 2.6f + 0.4f * (float)(r.path[x] + r.toptiles) + (r.cl[x] > 1 ? 1.f : 0.f);
         for (int many = 0; many < 2; ++many) {
             s.sweep[many] = 25.f + (float)n * (max_weight > 1 ? 0.25f : many ? 0.07f : 0.04f);
-            s.evals[many] = std::min(max_evals, std::max(3, (int)(s.sweep[many] / s.price) - 2));
+            s.evals[many] = s.sweep[many] < 6 * s.price ? 0 : std::min(max_evals, (int)(s.sweep[many] / s.price) - 2);
         }
     }
 }

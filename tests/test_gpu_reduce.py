@@ -333,11 +333,12 @@ def test_price_just_below_the_first_guess(pp, oracle_lib, shape, n, k):
     _check(pp, oracle_lib, parent, np.ones(n, np.int32), profits, [k] * 4, rows)
 
 
-@pytest.mark.parametrize("k", [40, 160])
-def test_items_that_do_not_reduce_stop_early(pp, oracle_lib, k):
+@pytest.mark.parametrize("k,most", [(40, 2.0), (160, 2.8)])
+def test_items_that_do_not_reduce_stop_early(pp, oracle_lib, k, most):
     """Nothing to gain on a chain that pays all at its end, and a price takes
-    its 25 tiles in turn: the call may take about twice the sweep of all rows
-    (which is what the pruned sweep takes here), and took 3.4 to 3.8 times."""
+    its 25 tiles in turn: up to 128 columns the sweep is left to it at once,
+    with more the call may take about twice the sweep of all rows (which is
+    what the pruned sweep takes here).  It took 3.4 to 3.8 times."""
     rng = np.random.default_rng(k)
     n = 800
     parent = _tree(rng, "chain", n)
@@ -366,7 +367,7 @@ def test_items_that_do_not_reduce_stop_early(pp, oracle_lib, k):
                 b.synchronize()
                 times.append(a.elapsed_time(b))
             took.append(float(np.median(times[5:])))
-    assert took[1] <= 2.8 * took[0], took
+    assert took[1] <= most * took[0], took
 
 
 @pytest.mark.parametrize("solved_by_reduction", [True, False])
