@@ -69,7 +69,7 @@ inline int cluster_index(const ReduceShape &r, int items)
 // (0.25 here: they sooner pay).
 // A tree whose sweep takes less than six prices is left to it at once: three
 // prices, the exact evaluation and a DP would not fit (chains of 400 and 800
-// rows, 128 columns at most: 105 to 130 us with the prices, 64 to 78 without).
+// rows, 128 columns at most: 85 and 115 us with the prices, 55 and 72 without).
 inline void set_spending(ReduceShape &r, int n, int max_weight, int max_evals)
 {
     for (int x = 0; x < r.ncl; ++x) {
